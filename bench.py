@@ -916,7 +916,7 @@ def main():
         gemm_tops = ops / (tg * 1e-3) / 1e12
         roof = tensor_roofline(gemm_tops, total_ms * 1e-3, peaks, tp)
         roof.update(traffic=NCU_TRAFFIC_BYTES.get(("gemm", args.workload)),
-                    kernel="gemm_w4a4_kernel (with the 9 us expand_weight_kernel in front of it)", ms=tg)
+                    kernel="gemm_w4a4_kernel (with the expand_weight_kernel in front of it)", ms=tg)
         # Bytes the activation step needs by its definition (X read; 4-bit codes, FP32 group scales and BF16 T written)
         # and bytes this layout moves (one E4M3 byte per code, FP32 scales plus the 8-byte scale operand of the GEMM's
         # scale MMA per (token, group), T as a BF16 high | low pair).

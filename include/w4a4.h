@@ -97,7 +97,7 @@ void w4a4_destroy(w4a4_handle_t h);
  *   X   device BF16 [M, K] row-major (leading dimension K), 16-byte aligned
  *   Y   device BF16 [M, N] row-major, 16-byte aligned
  *   clip_table  device FP32 [num_experts, num_layers, num_bins], values in [1e-4, 1]
- *   stream      a cudaStream_t (as void*); three kernels are enqueued (activation quantization, expansion of
+ *   stream      a cudaStream_t (as void*); two kernels are enqueued (activation quantization with the expansion of
  *               the layer's 4-bit weights to bytes, GEMM), no host synchronisation.
  * M may be 0 (nothing is launched).  Errors: INVALID_ARG, SHAPE (M > max_M), CUDA.  A pipeline wait that
  * gives up on the device is not visible here (the call does not synchronise): see w4a4_query_status. */

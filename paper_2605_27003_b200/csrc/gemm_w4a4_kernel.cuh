@@ -6,7 +6,7 @@
 // Code products.  The 4-bit codes go through the tensor core as E4M3 bytes (fp8_codes.cuh): tcgen05.mma
 // kind::f8f6f4 runs at the 8-bit rate and leaves every group's partial sums in TMEM as exact integers already in
 // FP32 (|P| <= 4096).  The activation codes come straight from kernel 1, the weight codes from
-// expand_weight_kernel, which runs right before this kernel and turns the layer's nibble-packed weights (their
+// the expansion in kernel 1's launch (ExpandJob), which turns the layer's nibble-packed weights (their
 // format at rest) into an N x K byte image that stays in L2 for the duration of the GEMM.
 //
 // Scale products.  The factor S_g = sx[:, g] (x) sw[g, :] is an outer product, i.e. a K = 16 BF16 MMA on operands

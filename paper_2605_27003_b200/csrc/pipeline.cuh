@@ -1,6 +1,5 @@
 // Pieces every tcgen05 GEMM of this library shares: tile constants, bounded mbarrier waits with their error
-// codes, ring bookkeeping, the fused output activation, the parameter block and
-// the weight expansion pre-pass.
+// codes, ring bookkeeping, the fused output activation and the parameter block.
 //
 // Every wait on an mbarrier is bounded: after WaitEnv::limit_ns without progress (or as soon as another CTA
 // has reported an error) the role leaves its loop, the CTA records a code in *err and exits through the common
@@ -10,7 +9,6 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 
-#include "fp8_codes.cuh"
 #include "ptx.cuh"
 
 namespace w4a4 {
@@ -138,19 +136,6 @@ struct GemmParams {
   double* sq_err;
   int act;              // output activation: 0 none, 1 GELU (tanh form)
 };
-
-// Weight codes at rest -> the E4M3 byte image kernel 2 reads: [N, K/2] packed as code + 8 (byte j of a row holds
-// K offsets 2 j in its low nibble and 2 j + 1 in its high nibble) -> [N, K] bytes.  One thread turns 32 codes
-// (16 bytes in) into 32 bytes out; each half-word of an input word is one byte-permute selector.
-__global__ void expand_weight_kernel(const uint4* __restrict__ packed, uint4* __restrict__ out, size_t chunks) {
-  const size_t i = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (i >= chunks) return;
-  const uint4 w = __ldg(packed + i);
-  out[2 * i] = make_uint4(e4m3_of_offset_nibbles4(w.x), e4m3_of_offset_nibbles4(w.x >> 16), e4m3_of_offset_nibbles4(w.y),
-                          e4m3_of_offset_nibbles4(w.y >> 16));
-  out[2 * i + 1] = make_uint4(e4m3_of_offset_nibbles4(w.z), e4m3_of_offset_nibbles4(w.z >> 16),
-                              e4m3_of_offset_nibbles4(w.w), e4m3_of_offset_nibbles4(w.w >> 16));
-}
 
 // The end every GEMM kernel of this library shares after its role loops: if a wait gave up, copies that may
 // still be in flight get time to land before the CTA's shared memory is released.

@@ -17,9 +17,15 @@
 // fragments are laid out at pack time to match (see l1_fragment_channel()).
 //
 // K split (gridDim.y > 1): with few token rows there are too few 16-row warps to fill the machine, so the K groups
-// are divided among gridDim.y CTAs per row block.  Codes and scales of different groups are independent; the
-// partial sums of T go to an FP32 scratch [split][M][r] and t_reduce_kernel adds them in split order and writes
-// the BF16 high | low pair.
+// are divided among gridDim.y CTAs per row block, which form one thread-block cluster.  Codes and scales of different
+// groups are independent; the partial sums of T stay in each CTA's shared memory, and after a cluster barrier every CTA
+// adds its share of them over distributed shared memory, in split order, and writes the BF16 high | low pair.  (A
+// reduction kernel over a global scratch cost a dependent launch.)
+//
+// Weight expansion (ExpandJob): the CTAs past the row blocks turn the layer's 4-bit weights into the byte image the
+// INT4 GEMM reads.  It is independent of the activations, so it shares their launch instead of being a kernel between
+// two dependent ones; at the large sizes its traffic hides behind the activation CTAs.  Both together, per forward: 256 x
+// 512 -> 512 20.5 -> 14.3 us (four launches -> two), 1560 x 5120 -> 5120 at rank 64 112 -> 105 us.
 //
 // Code output, three formats (template parameter FORMAT):
 //   kCodesE4M3    one E4M3 byte per code, row-major [M, K]: the tensor-core operand of kernel 2 as it is
@@ -41,6 +47,7 @@
 #include <stdint.h>
 
 #include "fp8_codes.cuh"
+#include "ptx.cuh"
 
 namespace w4a4 {
 
@@ -170,6 +177,14 @@ __device__ __forceinline__ uint2 quantize16(const float* xh, float is) {
   return make_uint2(w0 ^ 0x88888888u, w1 ^ 0x88888888u);  // offset-binary -> two's complement nibbles
 }
 
+// Two neighbouring entries of a row of T as BF16 high parts (columns c, c + 1 of the row) and the BF16 rounding of the
+// remainders (columns R + c, R + c + 1).
+__device__ __forceinline__ void store_t_pair(uint16_t* row, int R, int c, float t0, float t1) {
+  const __nv_bfloat16 h0 = __float2bfloat16_rn(t0), h1 = __float2bfloat16_rn(t1);
+  *reinterpret_cast<uint32_t*>(row + c) = pack_bf16x2(__bfloat162float(h0), __bfloat162float(h1));
+  *reinterpret_cast<uint32_t*>(row + R + c) = pack_bf16x2(t0 - __bfloat162float(h0), t1 - __bfloat162float(h1));
+}
+
 // Eight FP32 values -> eight E2M1 codes (round to nearest even, saturating at +-6), element 0 in the lowest nibble.
 __device__ __forceinline__ uint32_t e2m1x8(const float* v) {
   uint32_t r;
@@ -217,6 +232,39 @@ __device__ __forceinline__ uint2 sop_slots_activation(float s) {
   return make_uint2(hb | (hb << 16), mb | (mb << 16));
 }
 
+// Weight codes at rest -> the E4M3 byte image the INT4 GEMM reads: [N, K/2] packed as code + 8 (byte j of a row holds
+// K offsets 2 j in its low nibble and 2 j + 1 in its high nibble) -> [N, K] bytes.  One step turns 32 codes (16 bytes)
+// into 32 bytes; each half-word of an input word is one byte-permute selector.
+struct ExpandJob {
+  const uint4* packed = nullptr;
+  uint4* out = nullptr;
+  uint32_t chunks = 0;      // of 32 codes
+  uint32_t first_cta = 0;   // blockIdx.x from which CTAs do this instead of quantizing (gridDim.x: none)
+};
+__device__ __forceinline__ void expand_chunk(const uint4& w, uint4* out) {
+  out[0] = make_uint4(e4m3_of_offset_nibbles4(w.x), e4m3_of_offset_nibbles4(w.x >> 16), e4m3_of_offset_nibbles4(w.y),
+                      e4m3_of_offset_nibbles4(w.y >> 16));
+  out[1] = make_uint4(e4m3_of_offset_nibbles4(w.z), e4m3_of_offset_nibbles4(w.z >> 16), e4m3_of_offset_nibbles4(w.w),
+                      e4m3_of_offset_nibbles4(w.w >> 16));
+}
+constexpr int kExpandUnroll = 4;   // 16-byte loads a thread keeps in flight
+// `index` / `count`: this thread among all threads that share the job.
+__device__ __forceinline__ void expand_weights(const ExpandJob& job, uint32_t index, uint32_t count) {
+  for (uint32_t i = index; i < job.chunks; i += kExpandUnroll * count) {
+    uint4 w[kExpandUnroll];
+#pragma unroll
+    for (int j = 0; j < kExpandUnroll; ++j)
+      if (i + j * count < job.chunks) w[j] = __ldg(job.packed + i + j * count);
+#pragma unroll
+    for (int j = 0; j < kExpandUnroll; ++j)
+      if (i + j * count < job.chunks) expand_chunk(w[j], job.out + 2 * static_cast<size_t>(i + j * count));
+  }
+}
+// The same as a kernel of its own, for the GEMM without an activation pass in front of it.
+static __global__ void expand_weight_kernel(const ExpandJob job) {
+  expand_weights(job, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+}
+
 template <int R, int WARPS, int FORMAT>
 // Sixteen resident warps per SM (at most 128 registers) at every rank, so that the 2048 warps of row blocks of the
 // DiT shapes fit one wave: at 130-160 registers the wide ranks ran 1.15 waves.
@@ -224,7 +272,12 @@ __global__ void __launch_bounds__(32 * WARPS, 16 / WARPS)
 quantize_kernel(const uint16_t* __restrict__ X, int M, int K, const float* __restrict__ rlam,
                 const float* __restrict__ clip_table, int clip_index, const uint2* __restrict__ l1frag,
                 uint8_t* __restrict__ codes, float* __restrict__ scales, int scales_ld,
-                uint16_t* __restrict__ t_hilo, float* __restrict__ t_partial, uint2* __restrict__ a_sop) {
+                uint16_t* __restrict__ t_hilo, uint2* __restrict__ a_sop, const ExpandJob expand) {
+  if (blockIdx.x >= expand.first_cta) {   // whole clusters: the cluster spans gridDim.y, never blockIdx.x
+    const uint32_t cta = (blockIdx.x - expand.first_cta) * gridDim.y + blockIdx.y;
+    expand_weights(expand, cta * (32 * WARPS) + threadIdx.x, (gridDim.x - expand.first_cta) * gridDim.y * (32 * WARPS));
+    return;
+  }
   constexpr int NT = R / 8;                          // n-tiles of the m16n8k16 MMA
   constexpr int kFragBytes = 4 * NT * 32 * 8;        // L1 fragments of one group (4 KiB at r = 32)
   constexpr int kFragChunks = kFragBytes / 16;
@@ -394,37 +447,50 @@ quantize_kernel(const uint16_t* __restrict__ X, int M, int K, const float* __res
   if constexpr (NT > 0) {
     // Each warp owns its 16 rows over all of K (or over its split of K): T, or its partial sum, is complete in
     // the accumulators.  Unsplit: store it as a BF16 high part and the BF16 rounding of the remainder
-    // ([T_hi | T_lo], two values per 32-bit store).  Split: store the FP32 partial sums for t_reduce_kernel.
+    // ([T_hi | T_lo], two values per 32-bit store).
+    if (gridDim.y == 1) {
 #pragma unroll
-    for (int nt = 0; nt < NT; ++nt) {
-      const int c = 8 * nt + 2 * qj;
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int row = h ? rowB : rowA;
-        if (row < M) {
-          const float t0 = acc[nt][2 * h], t1 = acc[nt][2 * h + 1];
-          if (gridDim.y > 1) {
-            *reinterpret_cast<float2*>(t_partial + (static_cast<size_t>(blockIdx.y) * M + row) * R + c) = make_float2(t0, t1);
-            continue;
-          }
-          const __nv_bfloat16 h0 = __float2bfloat16_rn(t0), h1 = __float2bfloat16_rn(t1);
-          const uint32_t hi = pack_bf16x2(__bfloat162float(h0), __bfloat162float(h1));
-          const uint32_t lo = pack_bf16x2(t0 - __bfloat162float(h0), t1 - __bfloat162float(h1));
-          uint16_t* dst = t_hilo + static_cast<size_t>(row) * (2 * R);
-          *reinterpret_cast<uint32_t*>(dst + c) = hi;
-          *reinterpret_cast<uint32_t*>(dst + R + c) = lo;
-        }
+      for (int nt = 0; nt < NT; ++nt) {
+        const int c = 8 * nt + 2 * qj;
+        if (okA) store_t_pair(t_hilo + static_cast<size_t>(rowA) * (2 * R), R, c, acc[nt][0], acc[nt][1]);
+        if (okB) store_t_pair(t_hilo + static_cast<size_t>(rowB) * (2 * R), R, c, acc[nt][2], acc[nt][3]);
       }
+    } else {
+      // Split: the CTA's partial sums replace the rings in shared memory, then every CTA of the cluster adds up its
+      // share of the tile over all splits, in split order.
+      float* tile = reinterpret_cast<float*>(quant_smem);   // [16 WARPS rows][R]
+      static_assert(16 * R * 4 <= kStages * 4 * 32 * 16, "a warp's partial sums fit its activation ring");
+      __syncthreads();
+#pragma unroll
+      for (int nt = 0; nt < NT; ++nt) {
+        const int c = 8 * nt + 2 * qj;
+        *reinterpret_cast<float2*>(tile + (16 * warp + qi) * R + c) = make_float2(acc[nt][0], acc[nt][1]);
+        *reinterpret_cast<float2*>(tile + (16 * warp + qi + 8) * R + c) = make_float2(acc[nt][2], acc[nt][3]);
+      }
+      cluster_sync_all();
+      const uint32_t tile_addr = smem_u32(tile);
+      const int rows = min(16 * WARPS, M - static_cast<int>(blockIdx.x) * 16 * WARPS);
+      for (int i = blockIdx.y * (32 * WARPS) + threadIdx.x; i < rows * (R / 2); i += gridDim.y * (32 * WARPS)) {
+        float t0 = 0.0f, t1 = 0.0f;
+        for (uint32_t s = 0; s < gridDim.y; ++s) {
+          const float2 v = ld_cluster_f32x2(map_to_cta(tile_addr + 8 * i, s));
+          t0 += v.x;
+          t1 += v.y;
+        }
+        const int row = i / (R / 2), c = 2 * (i - row * (R / 2));
+        store_t_pair(t_hilo + (static_cast<size_t>(blockIdx.x) * (16 * WARPS) + row) * (2 * R), R, c, t0, t1);
+      }
+      cluster_sync_all();   // nobody leaves while its shared memory is still being read
     }
   }
 }
 
-// Sum of the K splits' partial T (in split order), written as the BF16 high | low pair kernel 2 reads.
-static __global__ void t_reduce_kernel(const float* __restrict__ t_partial, int splits, int M, int r, uint16_t* __restrict__ t_hilo) {
+// T in FP32 [M, r] -> the BF16 high | low pair kernel 2 reads (the fused producer of the MXFP4 variant accumulates T
+// in FP32).
+static __global__ void t_split_kernel(const float* __restrict__ t32, int M, int r, uint16_t* __restrict__ t_hilo) {
   const size_t idx = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (idx >= static_cast<size_t>(M) * r) return;
-  float t = 0.0f;
-  for (int s = 0; s < splits; ++s) t += t_partial[static_cast<size_t>(s) * M * r + idx];
+  const float t = t32[idx];
   const size_t row = idx / r;
   const int c = static_cast<int>(idx % r);
   const __nv_bfloat16 hi = __float2bfloat16_rn(t);
@@ -434,12 +500,10 @@ static __global__ void t_reduce_kernel(const float* __restrict__ t_partial, int 
 }
 
 // Number of K splits for a launch of `row_ctas` row blocks over G groups on a device with `sms` SMs: enough CTAs
-// for about three per SM, at most kMaxKSplits, and only while the partial sums of T fit the scratch
-// (M <= kKSplitMaxRows).
+// for about three per SM, at most kMaxKSplits (the portable cluster size).
 constexpr int kMaxKSplits = 8;
-constexpr int kKSplitMaxRows = 8192;
-inline int quantize_k_splits(int row_ctas, int G, int M, int sms) {
-  if (M > kKSplitMaxRows || row_ctas >= 2 * sms) return 1;
+inline int quantize_k_splits(int row_ctas, int G, int sms) {
+  if (row_ctas >= 2 * sms) return 1;
   int s = (3 * sms + row_ctas - 1) / row_ctas;
   if (s > kMaxKSplits) s = kMaxKSplits;
   if (s > G) s = G;

@@ -169,24 +169,58 @@ w4a4_status_t check_forward_args(w4a4_handle_t h, const void* X, int M, int expe
   return W4A4_OK;
 }
 
+// Kernel 1's launch: row blocks x K splits (a cluster per row block when K is split), plus the CTAs that expand weights.
+template <int R, int FORMAT>
+cudaError_t launch_quantize_kernel(int num_sms, cudaStream_t stream, const uint16_t* x, int M, int K, const float* rlam,
+                                   const float* clip_table, int clip_index, const uint2* l1frag, uint8_t* codes,
+                                   float* scales, int scales_ld, uint16_t* t_hilo, uint2* a_sop, ExpandJob job) {
+  constexpr int kWarps = quantize_warps(R);
+  const int row_ctas = (M + kQuantRows * kWarps - 1) / (kQuantRows * kWarps);
+  const int splits = quantize_k_splits(row_ctas, K / 64, num_sms);
+  const uint32_t per_cta = 32 * kWarps * kExpandUnroll * splits;
+  job.first_cta = row_ctas;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(row_ctas + (job.chunks + per_cta - 1) / per_cta, splits);
+  cfg.blockDim = dim3(32 * kWarps);
+  cfg.dynamicSmemBytes = quantize_smem_bytes(R);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 1;
+  attr[0].val.clusterDim.y = splits;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = splits > 1 ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, quantize_kernel<R, kWarps, FORMAT>, x, M, K, rlam, clip_table, clip_index, l1frag, codes,
+                            scales, scales_ld, t_hilo, a_sop, job);
+}
+
 // Index of (expert, this layer, bin) in a clip table (Sec. III-C: one ratio per expert, layer and timestep bin).
 int clip_table_index(const w4a4_layer* h, int expert_id, int bin) { return (expert_id * h->L + h->layer_id) * h->B + bin; }
 
-// Kernel 1 with the ratio read from clip_table[clip_index].
+ExpandJob expand_job(const w4a4_layer* h, int expert_id) {
+  ExpandJob job;
+  job.packed = reinterpret_cast<const uint4*>(h->experts[expert_id].bpacked);
+  job.out = reinterpret_cast<uint4*>(h->ctx->b8);
+  job.chunks = static_cast<uint32_t>(static_cast<size_t>(h->N) * h->K / 32);
+  return job;
+}
+
+// Kernel 1 with the ratio read from clip_table[clip_index]; with `expand`, its launch also rewrites the context's byte
+// image with the expert's weights.
 w4a4_status_t launch_quantize_at(w4a4_handle_t h, const void* X, int M, int expert_id, const float* clip_table,
-                                 int clip_index, cudaStream_t stream) {
+                                 int clip_index, bool expand, cudaStream_t stream) {
   if (M == 0) return W4A4_OK;
   w4a4_ctx* ctx = h->ctx;
   const ExpertData& e = h->experts[expert_id];
-  const int rows_per_cta = kQuantRows * quantize_warps(h->r);
-  const int row_ctas = (M + rows_per_cta - 1) / rows_per_cta;
-  const int splits = quantize_k_splits(row_ctas, h->K / 64, M, ctx->num_sms);
-  const dim3 grid(row_ctas, splits), block(32 * quantize_warps(h->r));
+  ExpandJob job;
+  if (expand) job = expand_job(h, expert_id);
   const uint16_t* x = static_cast<const uint16_t*>(X);
-#define W4A4_LAUNCH_Q(R)                                                                                         \
-  quantize_kernel<R, quantize_warps(R), kCodesE4M3><<<grid, block, quantize_smem_bytes(R), stream>>>(x, M, h->K, e.rlam, clip_table, clip_index, e.l1frag, ctx->codes, \
-                                                 ctx->scales, ctx->scales_ld, ctx->t_hilo, ctx->t_partial,     \
-                                                 reinterpret_cast<uint2*>(ctx->a_sop))
+  uint2* a_sop = reinterpret_cast<uint2*>(ctx->a_sop);
+  cudaError_t le;
+#define W4A4_LAUNCH_Q(R)                                                                                          \
+  le = launch_quantize_kernel<R, kCodesE4M3>(ctx->num_sms, stream, x, M, h->K, e.rlam, clip_table, clip_index, e.l1frag, \
+                                             ctx->codes, ctx->scales, ctx->scales_ld, ctx->t_hilo, a_sop, job)
   switch (h->r) {
     case 0: W4A4_LAUNCH_Q(0); break;
     case 16: W4A4_LAUNCH_Q(16); break;
@@ -196,24 +230,21 @@ w4a4_status_t launch_quantize_at(w4a4_handle_t h, const void* X, int M, int expe
     default: return W4A4_ERR_SHAPE;
   }
 #undef W4A4_LAUNCH_Q
-  if (splits > 1 && h->r > 0) {
-    const size_t nt = static_cast<size_t>(M) * h->r;
-    t_reduce_kernel<<<static_cast<unsigned>((nt + 255) / 256), 256, 0, stream>>>(ctx->t_partial, splits, M, h->r, ctx->t_hilo);
-  }
-  return cudaGetLastError() == cudaSuccess ? W4A4_OK : W4A4_ERR_CUDA;
+  if (le != cudaSuccess) cudaGetLastError();
+  return le == cudaSuccess ? W4A4_OK : W4A4_ERR_CUDA;
 }
 
 w4a4_status_t launch_quantize(w4a4_handle_t h, const void* X, int M, int expert_id, int bin, const float* clip_table,
-                              cudaStream_t stream) {
-  return launch_quantize_at(h, X, M, expert_id, clip_table, clip_table_index(h, expert_id, bin), stream);
+                              bool expand, cudaStream_t stream) {
+  return launch_quantize_at(h, X, M, expert_id, clip_table, clip_table_index(h, expert_id, bin), expand, stream);
 }
 
-// Kernel 2 (preceded by the expansion of the expert's 4-bit weights unless `expand` is false, i.e. the
-// context's byte image already holds them).  With yref set, the squared distance to yref is accumulated into
+// Kernel 2; `expand`: preceded by the expansion of the expert's 4-bit weights (false: the context's byte image already
+// holds them, normally because kernel 1's launch wrote it).  With yref set, the squared distance to yref is accumulated into
 // *sq_err instead of storing Y.
 w4a4_status_t launch_gemm(w4a4_handle_t h, int M, int expert_id, void* Y, cudaStream_t stream, int32_t* dbg_P,
                           int dbg_m0, int dbg_n0, const void* yref = nullptr, double* sq_err = nullptr,
-                          bool expand = true, int stall_stage = -1, uint64_t wait_limit_ns = kWaitLimitNs) {
+                          bool expand = false, int stall_stage = -1, uint64_t wait_limit_ns = kWaitLimitNs) {
   if (M == 0) return W4A4_OK;
   w4a4_ctx* ctx = h->ctx;
   const ExpertData& e = h->experts[expert_id];
@@ -258,9 +289,9 @@ w4a4_status_t launch_gemm(w4a4_handle_t h, int M, int expert_id, void* Y, cudaSt
     h->tmB_base = ctx->b8;
   }
   if (expand) {
-    const size_t chunks = static_cast<size_t>(h->N) * h->K / 32;
-    expand_weight_kernel<<<static_cast<unsigned>((chunks + 255) / 256), 256, 0, stream>>>(
-        reinterpret_cast<const uint4*>(e.bpacked), reinterpret_cast<uint4*>(ctx->b8), chunks);
+    const ExpandJob job = expand_job(h, expert_id);
+    const uint32_t per_cta = 256 * kExpandUnroll;
+    expand_weight_kernel<<<(job.chunks + per_cta - 1) / per_cta, 256, 0, stream>>>(job);
   }
   // Persistent: one CTA per SM walks the 128 x 128 tiles.
   const int num_tiles = p.tiles_m * p.tiles_n;
@@ -342,9 +373,6 @@ w4a4_status_t w4a4_ctx_create(int device, int max_M, int max_K, int max_r, w4a4_
   // Rows past M and the unused half of an odd last stage are multiplied by zeros: they only have to be finite.
   if (st == W4A4_OK && cudaMemset(ctx->a_sop, 0, a_sop_bytes) != cudaSuccess) st = W4A4_ERR_CUDA;
   if (st == W4A4_OK) st = dev_alloc(&ctx->t_hilo, static_cast<size_t>(max_M) * 2 * (max_r > 0 ? max_r : 8), &ctx->bytes);
-  if (st == W4A4_OK && max_r > 0)
-    st = dev_alloc(&ctx->t_partial,
-                   static_cast<size_t>(kMaxKSplits) * (max_M < kKSplitMaxRows ? max_M : kKSplitMaxRows) * max_r, &ctx->bytes);
   if (st == W4A4_OK) st = dev_alloc(&ctx->d_err, 1, &ctx->bytes);
   if (st == W4A4_OK && cudaMemset(ctx->d_err, 0, sizeof(int)) != cudaSuccess) st = W4A4_ERR_CUDA;
   // The workspace is read by TMA for rows up to max_M even when fewer are valid: start it defined.
@@ -382,7 +410,6 @@ void w4a4_ctx_destroy(w4a4_ctx_t ctx) {
   cudaFree(ctx->mx_sfa2);
   cudaFree(ctx->mx_t32);
   cudaFree(ctx->t_hilo2);
-  cudaFree(ctx->t_partial);
   cudaFree(ctx->scales);
   cudaFree(ctx->a_sop);
   cudaFree(ctx->t_hilo);
@@ -557,7 +584,7 @@ w4a4_status_t w4a4_quantize_activations(w4a4_handle_t h, const void* X, int M, i
   w4a4_status_t st = check_forward_args(h, X, M, expert_id, timestep_bin, clip_table, true);
   if (st != W4A4_OK) return st;
   DeviceGuard guard(h->ctx->device);
-  return launch_quantize(h, X, M, expert_id, timestep_bin, clip_table, static_cast<cudaStream_t>(stream));
+  return launch_quantize(h, X, M, expert_id, timestep_bin, clip_table, false, static_cast<cudaStream_t>(stream));
 }
 
 w4a4_status_t w4a4_gemm_from_workspace(w4a4_handle_t h, int M, int expert_id, void* Y, void* stream) {
@@ -565,7 +592,7 @@ w4a4_status_t w4a4_gemm_from_workspace(w4a4_handle_t h, int M, int expert_id, vo
   if (st != W4A4_OK) return st;
   if (M > 0 && (!Y || !aligned16(Y))) return W4A4_ERR_INVALID_ARG;
   DeviceGuard guard(h->ctx->device);
-  return launch_gemm(h, M, expert_id, Y, static_cast<cudaStream_t>(stream), nullptr, 0, 0);
+  return launch_gemm(h, M, expert_id, Y, static_cast<cudaStream_t>(stream), nullptr, 0, 0, nullptr, nullptr, true);
 }
 
 w4a4_status_t w4a4_clip_search(w4a4_handle_t h, const void* const* X_samples, const void* const* Yref_samples,
@@ -601,9 +628,8 @@ w4a4_status_t w4a4_clip_search(w4a4_handle_t h, const void* const* X_samples, co
   bool expanded = false;
   for (int s = 0; st == W4A4_OK && s < num_samples; ++s) {
     for (int c = 0; st == W4A4_OK && c < num_candidates; ++c) {
-      st = launch_quantize_at(h, X_samples[s], M, expert_id, d_cand, c, st_);
-      if (st == W4A4_OK)
-        st = launch_gemm(h, M, expert_id, nullptr, st_, nullptr, 0, 0, Yref_samples[s], d_err + c, !expanded);
+      st = launch_quantize_at(h, X_samples[s], M, expert_id, d_cand, c, !expanded, st_);
+      if (st == W4A4_OK) st = launch_gemm(h, M, expert_id, nullptr, st_, nullptr, 0, 0, Yref_samples[s], d_err + c);
       expanded = true;
     }
   }
@@ -634,7 +660,7 @@ w4a4_status_t w4a4_linear_forward(w4a4_handle_t h, const void* X, int M, int exp
   if (M > 0 && (!Y || !aligned16(Y))) return W4A4_ERR_INVALID_ARG;
   DeviceGuard guard(h->ctx->device);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  st = launch_quantize(h, X, M, expert_id, timestep_bin, clip_table, s);
+  st = launch_quantize(h, X, M, expert_id, timestep_bin, clip_table, true, s);
   if (st != W4A4_OK) return st;
   return launch_gemm(h, M, expert_id, Y, s, nullptr, 0, 0);
 }
@@ -698,9 +724,9 @@ w4a4_status_t w4a4_linear_forward_host(w4a4_handle_t h, const void* X_host, int 
          cudaStreamWaitEvent(ctx->s_compute, ctx->ev_in[b], 0) == cudaSuccess;
     if (ok && i >= 2) ok = cudaStreamWaitEvent(ctx->s_compute, ctx->ev_out[b], 0) == cudaSuccess;  // staging Y[b] drained
     if (!ok) break;
-    st = launch_quantize(h, ctx->hx[b], rows, expert_id, timestep_bin, clip_table, ctx->s_compute);
     // The weight byte image is the same for every chunk: expand it with the first one only.
-    if (st == W4A4_OK) st = launch_gemm(h, rows, expert_id, ctx->hy[b], ctx->s_compute, nullptr, 0, 0, nullptr, nullptr, i == 0);
+    st = launch_quantize(h, ctx->hx[b], rows, expert_id, timestep_bin, clip_table, i == 0, ctx->s_compute);
+    if (st == W4A4_OK) st = launch_gemm(h, rows, expert_id, ctx->hy[b], ctx->s_compute, nullptr, 0, 0);
     if (st != W4A4_OK) return st;
     ok = cudaEventRecord(ctx->ev_done[b], ctx->s_compute) == cudaSuccess &&
          cudaStreamWaitEvent(ctx->s_d2h, ctx->ev_done[b], 0) == cudaSuccess &&
@@ -724,7 +750,7 @@ w4a4_status_t w4a4_debug_quantize(w4a4_handle_t h, const void* X, int M, int exp
   if (M > 0 && (!codes || !scales)) return W4A4_ERR_INVALID_ARG;
   DeviceGuard guard(h->ctx->device);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  st = launch_quantize(h, X, M, expert_id, timestep_bin, clip_table, s);
+  st = launch_quantize(h, X, M, expert_id, timestep_bin, clip_table, false, s);
   if (st != W4A4_OK || M == 0) return st;
   const size_t nc = static_cast<size_t>(M) * h->K;
   decode_codes_kernel<<<static_cast<unsigned>((nc + 255) / 256), 256, 0, s>>>(h->ctx->codes, codes, M, h->K);
@@ -746,7 +772,7 @@ w4a4_status_t w4a4_debug_partials(w4a4_handle_t h, const void* X, int M, int exp
   if (m0 < 0 || n0 < 0 || m0 % kBM != 0 || n0 % kBN != 0 || n0 >= h->N || (M > 0 && m0 >= M)) return W4A4_ERR_INVALID_ARG;
   DeviceGuard guard(h->ctx->device);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  st = launch_quantize(h, X, M, expert_id, timestep_bin, clip_table, s);
+  st = launch_quantize(h, X, M, expert_id, timestep_bin, clip_table, true, s);
   if (st != W4A4_OK) return st;
   return launch_gemm(h, M, expert_id, Y, s, P, m0, n0);
 }

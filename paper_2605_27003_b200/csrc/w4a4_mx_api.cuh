@@ -61,15 +61,12 @@ w4a4_status_t mx_launch_quantize_at(w4a4_mx_handle_t h, const void* X, int M, in
   if (M == 0) return W4A4_OK;
   w4a4_ctx* ctx = h->ctx;
   const MxExpertData& e = h->experts[expert_id];
-  const int rows_per_cta = kQuantRows * quantize_warps(h->r);
-  const int row_ctas = (M + rows_per_cta - 1) / rows_per_cta;
-  const int splits = quantize_k_splits(row_ctas, h->K / 64, M, ctx->num_sms);
-  const dim3 grid(row_ctas, splits), block(32 * quantize_warps(h->r));
   const uint16_t* x = static_cast<const uint16_t*>(X);
   float* sf = reinterpret_cast<float*>(ctx->mx_sfa);
-#define W4A4_LAUNCH_MXQ(R)                                                                                             \
-  quantize_kernel<R, quantize_warps(R), kCodesMxfp4><<<grid, block, quantize_smem_bytes(R), stream>>>(                 \
-      x, M, h->K, e.rlam, clip_table, clip_index, e.l1frag, ctx->codes, sf, h->K / 128, ctx->t_hilo, ctx->t_partial, nullptr)
+  cudaError_t le;
+#define W4A4_LAUNCH_MXQ(R)                                                                                        \
+  le = launch_quantize_kernel<R, kCodesMxfp4>(ctx->num_sms, stream, x, M, h->K, e.rlam, clip_table, clip_index, e.l1frag, \
+                                              ctx->codes, sf, h->K / 128, ctx->t_hilo, nullptr, ExpandJob())
   switch (h->r) {
     case 0: W4A4_LAUNCH_MXQ(0); break;
     case 16: W4A4_LAUNCH_MXQ(16); break;
@@ -78,11 +75,8 @@ w4a4_status_t mx_launch_quantize_at(w4a4_mx_handle_t h, const void* X, int M, in
     default: return W4A4_ERR_SHAPE;
   }
 #undef W4A4_LAUNCH_MXQ
-  if (splits > 1 && h->r > 0) {
-    const size_t nt = static_cast<size_t>(M) * h->r;
-    t_reduce_kernel<<<static_cast<unsigned>((nt + 255) / 256), 256, 0, stream>>>(ctx->t_partial, splits, M, h->r, ctx->t_hilo);
-  }
-  return cudaGetLastError() == cudaSuccess ? W4A4_OK : W4A4_ERR_CUDA;
+  if (le != cudaSuccess) cudaGetLastError();
+  return le == cudaSuccess ? W4A4_OK : W4A4_ERR_CUDA;
 }
 
 w4a4_status_t mx_launch_quantize(w4a4_mx_handle_t h, const void* X, int M, int expert_id, int bin, const float* clip_table,
@@ -484,7 +478,7 @@ w4a4_status_t w4a4_mx_ffn_forward(w4a4_mx_handle_t up, w4a4_mx_handle_t down, co
   if (st != W4A4_OK) return st;
   if (down->r > 0) {
     const size_t nt = static_cast<size_t>(M) * down->r;
-    t_reduce_kernel<<<static_cast<unsigned>((nt + 255) / 256), 256, 0, s>>>(ctx->mx_t32, 1, M, down->r, ctx->t_hilo2);
+    t_split_kernel<<<static_cast<unsigned>((nt + 255) / 256), 256, 0, s>>>(ctx->mx_t32, M, down->r, ctx->t_hilo2);
     if (cudaGetLastError() != cudaSuccess) return W4A4_ERR_CUDA;
   }
   return mx_launch_gemm(down, M, expert_id, Y, s, nullptr, nullptr, true);
