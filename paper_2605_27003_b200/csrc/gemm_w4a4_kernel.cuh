@@ -238,7 +238,6 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   const WaitEnv env{p.err, s_abort, p.wait_limit_ns};
 
   if (threadIdx.x == 0) {
-    *s_abort = (*reinterpret_cast<volatile int*>(p.err) != 0) ? 1 : 0;
     for (int i = 0; i < kGemmStages; ++i) {
       mbar_init(bar_op_full + 8 * i, 1);
       mbar_init(bar_op_empty + 8 * i, 2);    // the code-MMA warp and the scale-MMA warp
@@ -266,6 +265,9 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     tmem_relinquish();
     tc_fence_before_sync();
   }
+  // Everything above overlaps the end of the kernel before this one; its results are needed from here on.
+  grid_dependency_wait();
+  if (threadIdx.x == 0) *s_abort = (*reinterpret_cast<volatile int*>(p.err) != 0) ? 1 : 0;
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);

@@ -73,6 +73,28 @@ struct DeviceGuard {
   }
 };
 
+// A launch that may start its prologue while the kernel before it on the stream finishes (programmatic dependent launch;
+// the kernel calls grid_dependency_wait()), with a cluster of `cluster` CTAs if that is not 1 x 1.
+struct OverlappedLaunch {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[2];
+  OverlappedLaunch(dim3 grid, dim3 block, size_t smem, cudaStream_t stream, dim3 cluster = dim3(1)) {
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster.x;
+    attr[1].val.clusterDim.y = cluster.y;
+    attr[1].val.clusterDim.z = cluster.z;
+    cfg.attrs = attr;
+    cfg.numAttrs = cluster.x * cluster.y * cluster.z > 1 ? 2 : 1;
+  }
+  OverlappedLaunch(const OverlappedLaunch&) = delete;
+};
+
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 template <typename T>

@@ -137,7 +137,6 @@ mx_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   const WaitEnv env{p.err, s_abort, kWaitLimitNs};
 
   if (threadIdx.x == 0) {
-    *s_abort = (*reinterpret_cast<volatile int*>(p.err) != 0) ? 1 : 0;
     for (int i = 0; i < kMxStages; ++i) {
       mbar_init(bar_full + 8 * i, 1);
       mbar_init(bar_empty + 8 * i, 1);
@@ -158,6 +157,9 @@ mx_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     tmem_relinquish();
     tc_fence_before_sync();
   }
+  // Everything above overlaps the end of the kernel before this one; its results are needed from here on.
+  grid_dependency_wait();
+  if (threadIdx.x == 0) *s_abort = (*reinterpret_cast<volatile int*>(p.err) != 0) ? 1 : 0;
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
@@ -479,7 +481,6 @@ mx_gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
   const int cluster_id = blockIdx.x >> 1, num_clusters = gridDim.x >> 1;
   const WaitEnv env{p.err, s_abort, kWaitLimitNs};
   if (threadIdx.x == 0) {
-    *s_abort = (*reinterpret_cast<volatile int*>(p.err) != 0) ? 1 : 0;
     for (int i = 0; i < STAGES; ++i) {
       mbar_init(bar_full + 8 * i, 1);
       mbar_init(bar_empty + 8 * i, 1);
@@ -511,6 +512,9 @@ mx_gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     tmem_alloc2(smem_u32(tmem_slot), 512);
     tc_fence_before_sync();
   }
+  // Everything above overlaps the end of the kernel before this one; its results are needed from here on.
+  grid_dependency_wait();
+  if (threadIdx.x == 0) *s_abort = (*reinterpret_cast<volatile int*>(p.err) != 0) ? 1 : 0;
   __syncthreads();
   cluster_sync_all();  // both CTAs' barriers and TMEM exist before anything crosses over
   tc_fence_after_sync();

@@ -273,6 +273,7 @@ quantize_kernel(const uint16_t* __restrict__ X, int M, int K, const float* __res
                 const float* __restrict__ clip_table, int clip_index, const uint2* __restrict__ l1frag,
                 uint8_t* __restrict__ codes, float* __restrict__ scales, int scales_ld,
                 uint16_t* __restrict__ t_hilo, uint2* __restrict__ a_sop, const ExpandJob expand) {
+  grid_dependency_wait();
   if (blockIdx.x >= expand.first_cta) {   // whole clusters: the cluster spans gridDim.y, never blockIdx.x
     const uint32_t cta = (blockIdx.x - expand.first_cta) * gridDim.y + blockIdx.y;
     expand_weights(expand, cta * (32 * WARPS) + threadIdx.x, (gridDim.x - expand.first_cta) * gridDim.y * (32 * WARPS));
@@ -444,6 +445,10 @@ quantize_kernel(const uint16_t* __restrict__ X, int M, int K, const float* __res
     if (++stage == kStages) stage = 0;
   }
 
+  // The GEMM's CTAs may come in now, as room allows.  (Letting them in from the start takes shared memory from nobody but
+  // measured the same; the GEMM itself lets nobody in before its end: the next forward's activation CTAs then sat beside
+  // it, 78 -> 84 us at 1560 x 5120 -> 13824 MXFP4.)
+  grid_dependency_launch();
   if constexpr (NT > 0) {
     // Each warp owns its 16 rows over all of K (or over its split of K): T, or its partial sum, is complete in
     // the accumulators.  Unsplit: store it as a BF16 high part and the BF16 rounding of the remainder

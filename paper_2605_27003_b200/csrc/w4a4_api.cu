@@ -179,19 +179,9 @@ cudaError_t launch_quantize_kernel(int num_sms, cudaStream_t stream, const uint1
   const int splits = quantize_k_splits(row_ctas, K / 64, num_sms);
   const uint32_t per_cta = 32 * kWarps * kExpandUnroll * splits;
   job.first_cta = row_ctas;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(row_ctas + (job.chunks + per_cta - 1) / per_cta, splits);
-  cfg.blockDim = dim3(32 * kWarps);
-  cfg.dynamicSmemBytes = quantize_smem_bytes(R);
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = 1;
-  attr[0].val.clusterDim.y = splits;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = splits > 1 ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, quantize_kernel<R, kWarps, FORMAT>, x, M, K, rlam, clip_table, clip_index, l1frag, codes,
+  const OverlappedLaunch l(dim3(row_ctas + (job.chunks + per_cta - 1) / per_cta, splits), dim3(32 * kWarps), quantize_smem_bytes(R),
+                           stream, dim3(1, splits));
+  return cudaLaunchKernelEx(&l.cfg, quantize_kernel<R, kWarps, FORMAT>, x, M, K, rlam, clip_table, clip_index, l1frag, codes,
                             scales, scales_ld, t_hilo, a_sop, job);
 }
 
@@ -298,12 +288,11 @@ w4a4_status_t launch_gemm(w4a4_handle_t h, int M, int expert_id, void* Y, cudaSt
   const dim3 grid(num_tiles < ctx->num_sms ? num_tiles : ctx->num_sms), block(kGemmThreads);
   const CUtensorMap& tmT = h->r > 0 ? h->tmT : h->tmA;   // unused when r == 0
   const CUtensorMap& tmL2 = h->r > 0 ? e.tmL2 : h->tmB;
-  if (dbg_P || stall_stage >= 0) {
-    gemm_w4a4_kernel<true><<<grid, block, kGemmSmemBytes, stream>>>(h->tmA, h->tmB, tmT, tmL2, h->tmSopA, e.tmSopB, p);
-  } else {
-    gemm_w4a4_kernel<false><<<grid, block, kGemmSmemBytes, stream>>>(h->tmA, h->tmB, tmT, tmL2, h->tmSopA, e.tmSopB, p);
-  }
-  const cudaError_t le = cudaGetLastError();
+  const OverlappedLaunch l(grid, block, kGemmSmemBytes, stream);
+  cudaError_t le;
+  if (dbg_P || stall_stage >= 0) le = cudaLaunchKernelEx(&l.cfg, gemm_w4a4_kernel<true>, h->tmA, h->tmB, tmT, tmL2, h->tmSopA, e.tmSopB, p);
+  else le = cudaLaunchKernelEx(&l.cfg, gemm_w4a4_kernel<false>, h->tmA, h->tmB, tmT, tmL2, h->tmSopA, e.tmSopB, p);
+  if (le != cudaSuccess) cudaGetLastError();
   return le == cudaSuccess ? W4A4_OK : W4A4_ERR_CUDA;
 }
 

@@ -120,18 +120,7 @@ w4a4_status_t mx_launch_gemm(w4a4_mx_handle_t h, int M, int expert_id, void* Y, 
   if (p.tiles_m >= 2 && ctx->num_sms >= 2) {
     const int runs = ((p.tiles_m + 1) / 2) * ((p.tiles_n + p.run - 1) / p.run);
     const int ctas = 2 * runs < ctx->num_sms ? 2 * runs : (ctx->num_sms & ~1);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(ctas);
-    cfg.blockDim = block;
-    cfg.dynamicSmemBytes = kMx2SmemBytes;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    OverlappedLaunch l(dim3(ctas), block, next ? kMx2FuseSmemBytes : kMx2SmemBytes, stream, dim3(2));
     const CUtensorMap& tmL2h = h->r > 0 ? e.tmL2half : e.tmBhalf;
     MxNextParams nx = {};
     cudaError_t le;
@@ -143,11 +132,10 @@ w4a4_status_t mx_launch_gemm(w4a4_mx_handle_t h, int M, int expert_id, void* Y, 
       nx.sfa = ctx->mx_sfa2;
       nx.t32 = ctx->mx_t32;
       nx.r2 = next->r;
-      cfg.dynamicSmemBytes = kMx2FuseSmemBytes;
       const CUtensorMap& tmL1T = next->r > 0 ? ne.tmL1T : e.tmBhalf;
-      le = cudaLaunchKernelEx(&cfg, mx_gemm2_kernel<true>, tmA, e.tmBhalf, tmT, tmL2h, tmSFA, e.tmSFB, tmL1T, p, nx);
+      le = cudaLaunchKernelEx(&l.cfg, mx_gemm2_kernel<true>, tmA, e.tmBhalf, tmT, tmL2h, tmSFA, e.tmSFB, tmL1T, p, nx);
     } else {
-      le = cudaLaunchKernelEx(&cfg, mx_gemm2_kernel<false>, tmA, e.tmBhalf, tmT, tmL2h, tmSFA, e.tmSFB, e.tmBhalf, p, nx);
+      le = cudaLaunchKernelEx(&l.cfg, mx_gemm2_kernel<false>, tmA, e.tmBhalf, tmT, tmL2h, tmSFA, e.tmSFB, e.tmBhalf, p, nx);
     }
     if (le != cudaSuccess) {
       cudaGetLastError();
@@ -156,8 +144,12 @@ w4a4_status_t mx_launch_gemm(w4a4_mx_handle_t h, int M, int expert_id, void* Y, 
     return W4A4_OK;
   }
   if (next) return W4A4_ERR_SHAPE;   // the fused form runs on CTA pairs only
-  mx_gemm_kernel<<<grid, block, kMxSmemBytes, stream>>>(tmA, e.tmB, tmT, tmL2, p);
-  return cudaGetLastError() == cudaSuccess ? W4A4_OK : W4A4_ERR_CUDA;
+  const OverlappedLaunch l(grid, block, kMxSmemBytes, stream);
+  if (cudaLaunchKernelEx(&l.cfg, mx_gemm_kernel, tmA, e.tmB, tmT, tmL2, p) != cudaSuccess) {
+    cudaGetLastError();
+    return W4A4_ERR_CUDA;
+  }
+  return W4A4_OK;
 }
 
 }  // namespace
