@@ -20,7 +20,7 @@
 // shared-memory images (no-swizzle K-major canonical layout: [8-row group][8 rows][16 bytes]); kernel 1 writes the
 // token side next to the FP32 scales, the channel side is built once at pack time.  The low-rank product T L2 goes
 // through the same path as one more "group" that opens a tile: its P is the BF16 product [T_hi | T_lo] [L2 | L2]^T,
-// its S is the constant 1 (an MMA on a tile of ones), so the epilogue has a single loop.
+// which the epilogue takes as the accumulators' first value.
 //
 // Persistent, one CTA (640 threads) per SM, 128 x 128 tiles, column tile fastest (the CTAs running at any moment
 // share a few row blocks of A and a super-column of B through L2).  TMEM: two slots of 256 columns, one per group in flight:
@@ -40,14 +40,15 @@
 //               second half is in registers.  Measured alternatives (all four loads in one round trip; the second
 //               half's loads issued ahead of the first half's arithmetic; warps of a scheduler skewed against one
 //               another) were slower.
-// What bounds the kernel is the round trip of a TMEM slot (two slots, so two round trips overlap): epilogue releases it
-// -> issuing warps see that -> MMAs run -> commit -> epilogue sees that -> loads.  A lone warp's dependent instructions
+// What bounds the kernel is the serial chain of an epilogue warp per group: wait, load, 8 multiply-adds, load, release, 8
+// multiply-adds (a stand-alone copy of the hand-over runs at 330-340 clocks per group with the MMAs and without them; the
+// loads and multiply-adds alone at 200; this kernel at ~355).  A lone warp's dependent instructions
 // cost 10-15 cycles each and a branch on a fresh mbarrier result ~70, so the hops are written as single instruction
 // sequences without branches: wait_issue_* (try_wait, then fence, MMAs and commit predicated on its answer),
 // wait_then_ld16 (try_wait, then fence and first TMEM load predicated on its answer), descriptors computed before the wait, and
 // predicated instead of branched single-lane instructions (umma_*_if, mbar_arrive_if).  A wait that outlasts the
 // try_wait falls back to the bounded wait of pipeline.cuh and the same instructions issued from C++.
-// Tile order: column tiles are walked in super-columns (GemmParams::sc_tiles column tiles wide, all row blocks of a
+// Tile order: column tiles are walked in super-columns (GemmParams::order, all row blocks of a
 // super-column before the next) sized so that the weight bytes a wave of CTAs touches stay in L2; with the plain
 // row-major order the 71 MB weight image of the FFN shapes streamed from DRAM once per 1.4 row blocks.
 // Every role loops warp-uniformly (waits are voted, only the TMA / tcgen05 instructions are predicated on one elected
@@ -71,16 +72,28 @@ constexpr uint32_t kSopATile = kBM * 16;              // 2 KiB: 128 token rows x
 constexpr uint32_t kSopBTile = 2 * kBN * 16;          // 4 KiB: per group 128 channel rows x one 16-byte chunk
 constexpr uint32_t kStageBytes = kOpATile + kOpBTile + kSopATile + kSopBTile;   // 38 KiB
 constexpr uint32_t kLrStageBytes = kOpATile + kOpBTile;   // a low-rank stage: T tile and L2 rows
-constexpr uint32_t kConstTile = 2048;                 // tiles of zeros and of ones: 128 rows x 16 bytes
+constexpr uint32_t kZeroTile = 2048;                  // tile of zeros: 128 rows x 16 bytes
+constexpr uint32_t kOutTile = 32 * 2 * kEpiCols;      // an epilogue warp's 32 x 32 outputs in BF16
 constexpr uint32_t kGemmNumBarriers = 2 * kGemmStages + 2 * kTmemSlots;
-constexpr uint32_t kGemmSmemBytes = 1024 + kGemmStages * kStageBytes + 2 * kConstTile + kGemmNumBarriers * 8 + 16;
+constexpr uint32_t kGemmSmemBytes = 1024 + kGemmStages * kStageBytes + kZeroTile + kEpiWarps * kOutTile + kGemmNumBarriers * 8 + 16;
 static_assert(kGemmSmemBytes <= 232448, "shared memory budget of one CTA");
 static_assert(kStageBytes % 1024 == 0, "operand tiles must stay 1024-byte aligned");
 
-// Register budgets: the launch bound fixes 96 registers per thread for all 20 warps (five per scheduler: one control
-// warp and four epilogue warps).  Moving registers from the control warps to the epilogue with setmaxnreg was
-// measured and does not pay: at 104 the time is the same, at 112 the compiler's freer scheduling of the TMEM loads
-// against the multiply-adds made the kernel 7 % slower.
+// Register budgets.  640 threads are launched with 96 registers each; the control warpgroup gives most of its share to the
+// epilogue's four.  What the compiler makes of the epilogue's loop decides the kernel (clocks per 128 x 128 tile at K = 5120
+// | 13824, the same on every SM and at every clock): ring position as slot + parity with a wrap, 96 registers 34261 |
+// 88083; as a counter whose bits are slot and parity 31314 | 79971; with 112 registers 30529 | 78045.
+constexpr int kGemmRegs = 96, kControlRegs = 32, kEpilogueRegs = 112;
+static_assert((kGemmThreads - 32 * kEpiWarps) * kControlRegs + 32 * kEpiWarps * kEpilogueRegs <= kGemmThreads * kGemmRegs,
+              "a larger sum would wait forever for registers that the launch does not have");
+
+// Uses of the TMEM slots, counted: use u takes slot u % kTmemSlots.
+struct SlotUse {
+  uint32_t u = 0;
+  static_assert(kTmemSlots == 2, "slot and parity are bits 0 and 1 of the counter");
+  __device__ __forceinline__ uint32_t slot() const { return u & 1u; }
+  __device__ __forceinline__ uint32_t parity() const { return (u >> 1) & 1u; }
+};
 
 // Wait for a TMEM slot and issue its MMAs in one branch-free instruction sequence: one try_wait (it blocks in hardware
 // for a while before it gives up), then the fence, the MMAs and the commit predicated on its answer.  A branch on the
@@ -148,17 +161,13 @@ __device__ __forceinline__ uint32_t wait_then_ld16(uint32_t bar, uint32_t parity
 
 // Tile raster: column tiles are walked in super-columns of `sc` tiles (all row blocks of one super-column before the
 // next), so that the weight bytes a wave of CTAs touches stay in L2.  sc == tiles_n: plain row-major order.
-__device__ __forceinline__ void tile_coords(int tile, int tiles_m, int tiles_n, int sc, int& tm, int& tn) {
-  const int per_sc = tiles_m * sc;
-  const int full = tiles_n / sc;
-  int s_idx = tile / per_sc, rem = tile - s_idx * per_sc, width = sc;
-  if (s_idx >= full) {
-    s_idx = full;
-    rem = tile - full * per_sc;
-    width = tiles_n - full * sc;
-  }
-  tm = rem / width;
-  tn = s_idx * sc + (rem - tm * width);
+__device__ __forceinline__ void tile_coords(uint32_t tile, const TileOrder& o, int& tm, int& tn) {
+  const uint32_t s_idx = o.per_sc.quotient(tile);        // full super-columns before this tile, or all of them
+  const uint32_t rem = tile - s_idx * o.per_sc.divisor;
+  const bool last = s_idx >= o.full;                      // the narrower super-column that may end the order
+  const uint32_t row = last ? o.last_width.quotient(rem) : o.width.quotient(rem);
+  tm = static_cast<int>(row);
+  tn = static_cast<int>(s_idx * o.width.divisor + rem - row * (last ? o.last_width.divisor : o.width.divisor));
 }
 
 // Ties a fragment to the tcgen05.wait::ld in front of it: the registers count as written there, so nothing that
@@ -189,6 +198,18 @@ __device__ __forceinline__ void fma_fragment(const uint32_t (&pv)[16], const uin
   }
 }
 
+__device__ __forceinline__ uint32_t bf16x2_bits(float2 v) {
+  const __nv_bfloat162 b = __floats2bfloat162_rn(v.x, v.y);
+  return *reinterpret_cast<const uint32_t*>(&b);
+}
+
+// acc + (a0 - b0)^2 + (a1 - b1)^2 for two pairs of BF16 values.
+__device__ __forceinline__ float sq_diff_bf16x2(uint32_t a, uint32_t b, float acc) {
+  const float d0 = __uint_as_float(a << 16) - __uint_as_float(b << 16);
+  const float d1 = __uint_as_float(a & 0xffff0000u) - __uint_as_float(b & 0xffff0000u);
+  return fmaf(d1, d1, fmaf(d0, d0, acc));
+}
+
 // One scale as two BF16 pieces: s = h + m up to 2^-16 relative.
 __device__ __forceinline__ uint32_t scale_pieces(float s) {
   const __nv_bfloat16 h = __float2bfloat16_rn(s);
@@ -217,10 +238,10 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   extern __shared__ uint8_t smem_raw[];
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* smem = smem_raw + (smem_base - smem_u32(smem_raw));
-  // Constant tiles, above every operand tile so that the descriptors' chunk distances are positive.
-  const uint32_t ones_base = smem_base + kGemmStages * kStageBytes;   // rows [1, 0, 0, 0, 0, 0, 0, 0]: S = 1 for the low-rank entry
-  const uint32_t zero_base = ones_base + kConstTile;                  // second K chunk of every scale MMA
-  const uint32_t bar_base = zero_base + kConstTile;
+  // Above every operand tile so that the descriptors' chunk distances are positive.
+  const uint32_t zero_base = smem_base + kGemmStages * kStageBytes;   // second K chunk of every scale MMA
+  const uint32_t out_base = zero_base + kZeroTile;                    // the epilogue warps' output tiles
+  const uint32_t bar_base = out_base + kEpiWarps * kOutTile;
   const uint32_t bar_op_full = bar_base;
   const uint32_t bar_op_empty = bar_op_full + 8 * kGemmStages;
   const uint32_t bar_tmem_full = bar_op_empty + 8 * kGemmStages;
@@ -234,7 +255,6 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   const int n_int_stages = (G + 1) >> 1;
   const int n_lr_stages = p.r > 0 ? (2 * p.r + 63) / 64 : 0;
   const int num_tiles = p.tiles_m * p.tiles_n;
-  const int sc_tiles = p.sc_tiles;
   const WaitEnv env{p.err, s_abort, p.wait_limit_ns};
 
   if (threadIdx.x == 0) {
@@ -257,9 +277,9 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       tma_prefetch_desc(&tmL2);
     }
   }
-  for (uint32_t i = threadIdx.x; i < 2 * kConstTile / 16; i += blockDim.x)
-    reinterpret_cast<uint4*>(smem + (ones_base - smem_base))[i] = i < kConstTile / 16 ? make_uint4(0x3F80u, 0u, 0u, 0u) : make_uint4(0u, 0u, 0u, 0u);
-  fence_proxy_async_smem();   // the tensor core reads these tiles through the async proxy
+  for (uint32_t i = threadIdx.x; i < kZeroTile / 16; i += blockDim.x)
+    reinterpret_cast<uint4*>(smem + (zero_base - smem_base))[i] = make_uint4(0u, 0u, 0u, 0u);
+  fence_proxy_async_smem();   // the tensor core reads the tile through the async proxy
   if (warp == 2) {
     tmem_alloc(smem_u32(tmem_slot), 512);
     tmem_relinquish();
@@ -277,6 +297,7 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   // Per tile the issuing warps and the epilogue walk the same list of TMEM slot uses: [the low-rank entry, if r > 0]
   // followed by one entry per group.
   if (warp < kEpiWarp0) {
+    setmaxnreg_dec<kControlRegs>();
     if (live && warp == 0) {
       // ------------------------------------------------------------------ TMA producer (all lanes loop, one issues)
       const bool issuer = elect_one_lane();
@@ -285,7 +306,7 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       int stage_no = 0;
       for (int tile = blockIdx.x; ok && tile < num_tiles; tile += gridDim.x) {
         int tm, tn;
-        tile_coords(tile, p.tiles_m, p.tiles_n, sc_tiles, tm, tn);
+        tile_coords(tile, p.order, tm, tn);
         const int m0 = tm * kBM, n0 = tn * kBN;
         for (int st = 0; st < n_lr_stages + n_int_stages; ++st) {
           ok = __all_sync(0xffffffffu, bounded_wait<64>(bar_op_empty + 8 * op.slot, op.parity ^ 1u, env, kErrProducerWait));
@@ -381,7 +402,7 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       }
     } else if (live && warp == 3) {
       // ------------------------------------------------------------------ scale-MMA issuer
-      // Walks the same slot uses as the code-MMA warp: S = 1 for the low-rank entry, S_g for the groups.
+      // Walks the same slot uses as the code-MMA warp.
       constexpr uint32_t idesc_bf16 = umma_idesc(1, 1, kBM, kBN);
       const bool issuer = elect_one_lane();
       const uint32_t go = issuer ? 1u : 0u;
@@ -394,13 +415,9 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           ok = __all_sync(0xffffffffu, bounded_wait<0, 1>(bar_tmem_empty + 8 * tm.slot, tm.parity ^ 1u, env, kErrMmaWait));
           if (!ok) break;
           tc_fence_after_sync();
-          if (issuer) {
-            const uint64_t ones = umma_desc_k_plain(ones_base, zero_base - ones_base, 128);
-            umma_f16(tmem_base + tm.slot * 2 * kBN + kBN, ones, ones, idesc_bf16, 0u);
-            umma_commit(bar_tmem_full + 8 * tm.slot);
-          }
+          if (issuer) mbar_arrive(bar_tmem_full + 8 * tm.slot);   // the entry has no scale products, nor its stages anything for this warp
           tm.advance();
-          for (int l = 0; ok && l < n_lr_stages; ++l) {   // the low-rank stages hold nothing for this warp: sign off
+          for (int l = 0; ok && l < n_lr_stages; ++l) {
             ok = __all_sync(0xffffffffu, bounded_wait<0, 1>(bar_op_full + 8 * op.slot, op.parity, env, kErrMmaWait));
             if (!ok) break;
             if (issuer) mbar_arrive(bar_op_empty + 8 * op.slot);
@@ -434,6 +451,7 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       }
     }
   } else {
+    setmaxnreg_inc<kEpilogueRegs>();
     if (live) {
       // ------------------------------------------------------------------ epilogue warps
       // Warp ew owns TMEM lanes 32 * (ew % 4) .. +31 (token rows) and the 32-column block ew / 4; a thread owns one
@@ -441,30 +459,52 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       const int ew = warp - kEpiWarp0;
       const int quarter = ew & 3, colblk = ew >> 2;
       const uint32_t t_lane = tmem_base + (static_cast<uint32_t>(32 * quarter) << 16) + kEpiCols * colblk;
-      const int entries = G + (n_lr_stages > 0 ? 1 : 0);
-      Ring<kTmemSlots> tm;
+      const uint32_t out_tile = out_base + kOutTile * ew;
+      SlotUse use;
       bool ok = true;
       for (int tile = blockIdx.x; ok && tile < num_tiles; tile += gridDim.x) {
         int tm_e, tn_e;
-        tile_coords(tile, p.tiles_m, p.tiles_n, sc_tiles, tm_e, tn_e);
+        tile_coords(tile, p.order, tm_e, tn_e);
         const int m0 = tm_e * kBM, n0 = tn_e * kBN;
         const bool dbg_tile = DEBUG && p.dbg_P != nullptr && m0 == p.dbg_m0 && n0 == p.dbg_n0;
+        // Lane l holds the bias of the block's channel l; it reaches the other lanes through shared memory at the end.
+        const float bias_lane = p.bias ? __ldg(p.bias + n0 + kEpiCols * colblk + lane) : 0.0f;
         float2 acc[16];  // pair k: channels ch0 + 2 k, ch0 + 2 k + 1
+        if (n_lr_stages > 0) {   // the low-rank entry opens the tile: the accumulators start as T L2
+          const uint32_t t = t_lane + use.slot() * 2 * kBN;
+          uint32_t pv[16], qv[16];
+          ok = __all_sync(0xffffffffu, bounded_wait(bar_tmem_full + 8 * use.slot(), use.parity(), env, kErrEpilogueWait));
+          if (!ok) break;
+          tc_fence_after_sync();
+          tmem_ld_32x32b_x16(t, pv);
+          tmem_ld_32x32b_x16(t + 16, qv);
+          tmem_wait_ld();
+          tie_fragment(pv);
+          tie_fragment(qv);
+          tc_fence_before_sync();
+          mbar_arrive_if(lane == 0 ? 1u : 0u, bar_tmem_empty + 8 * use.slot());
+          ++use.u;
 #pragma unroll
-        for (int j = 0; j < 16; ++j) acc[j] = make_float2(0.0f, 0.0f);
-        for (int e = 0; e < entries; ++e) {
-          const uint32_t t = t_lane + tm.slot * 2 * kBN;
+          for (int j = 0; j < 8; ++j) {
+            acc[j] = make_float2(__uint_as_float(pv[2 * j]), __uint_as_float(pv[2 * j + 1]));
+            acc[8 + j] = make_float2(__uint_as_float(qv[2 * j]), __uint_as_float(qv[2 * j + 1]));
+          }
+        } else {
+#pragma unroll
+          for (int j = 0; j < 16; ++j) acc[j] = make_float2(0.0f, 0.0f);
+        }
+        for (int g = 0; g < G; ++g) {
+          const uint32_t t = t_lane + use.slot() * 2 * kBN;
           uint32_t pv[16], sv[16];
-          if (!__all_sync(0xffffffffu, wait_then_ld16(bar_tmem_full + 8 * tm.slot, tm.parity, t, pv) != 0)) {
-            ok = __all_sync(0xffffffffu, bounded_wait(bar_tmem_full + 8 * tm.slot, tm.parity, env, kErrEpilogueWait));
+          if (!__all_sync(0xffffffffu, wait_then_ld16(bar_tmem_full + 8 * use.slot(), use.parity(), t, pv) != 0)) {
+            ok = __all_sync(0xffffffffu, bounded_wait(bar_tmem_full + 8 * use.slot(), use.parity(), env, kErrEpilogueWait));
             if (!ok) break;
             tc_fence_after_sync();
             tmem_ld_32x32b_x16(t, pv);
           }
           int32_t* d0 = nullptr;
           if (DEBUG) {
-            const int g = e - (n_lr_stages > 0 ? 1 : 0);
-            if (dbg_tile && g >= 0) d0 = p.dbg_P + (static_cast<size_t>(32 * quarter + lane) * G + g) * kBN + kEpiCols * colblk;
+            if (dbg_tile) d0 = p.dbg_P + (static_cast<size_t>(32 * quarter + lane) * G + g) * kBN + kEpiCols * colblk;
           }
           tmem_ld_32x32b_x16(t + kBN, sv);
           tmem_wait_ld();
@@ -476,73 +516,66 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           tmem_wait_ld();
           tie_fragment(pv);
           tie_fragment(sv);
-          // The whole slot is in registers: hand it back to the MMA warps.
+          // The whole slot is in registers (loads and waits are warp-wide): hand it back to the MMA warps.
           tc_fence_before_sync();
-          __syncwarp();
-          mbar_arrive_if(lane == 0 ? 1u : 0u, bar_tmem_empty + 8 * tm.slot);
-          tm.advance();
+          mbar_arrive_if(lane == 0 ? 1u : 0u, bar_tmem_empty + 8 * use.slot());
+          ++use.u;
           fma_fragment<DEBUG>(pv, sv, acc + 8, DEBUG && d0 ? d0 + 16 : nullptr);
         }
         if (!ok) break;
-        const int row = m0 + 32 * quarter + lane;
-        const int ch0 = n0 + kEpiCols * colblk;
-        if (p.yref != nullptr) {
+        // The tile's end: bias, activation, BF16, then through shared memory so that a warp's 16-byte accesses to Y (or to
+        // the reference) cover eight rows x 64 bytes instead of 32 rows x 16.
+        __syncwarp();
+        sts_f32(out_tile + 4 * lane, bias_lane);
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < kEpiCols / 4; ++i) {
+          const float4 b = lds_f32x4(out_tile + 16 * i);
+          acc[2 * i].x += b.x, acc[2 * i].y += b.y, acc[2 * i + 1].x += b.z, acc[2 * i + 1].y += b.w;
+        }
+        if (p.act != 0) {  // uniform over the grid
+#pragma unroll
+          for (int j = 0; j < 16; ++j) acc[j] = make_float2(apply_activation(acc[j].x, p.act), apply_activation(acc[j].y, p.act));
+        }
+        __syncwarp();
+        // Output tile: 64-byte rows, 16-byte chunk c at c ^ (row / 2 % 4): conflict free for both sides.
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          uint4 o;
+          o.x = bf16x2_bits(acc[4 * c]), o.y = bf16x2_bits(acc[4 * c + 1]), o.z = bf16x2_bits(acc[4 * c + 2]), o.w = bf16x2_bits(acc[4 * c + 3]);
+          sts_u32x4(out_tile + 64 * lane + 16 * (c ^ ((lane >> 1) & 3)), o);
+        }
+        __syncwarp();
+        const int row = m0 + 32 * quarter + (lane >> 2);   // and rows + 8, + 16, + 24
+        const size_t at = static_cast<size_t>(row) * p.N + n0 + kEpiCols * colblk + 8 * (lane & 3);
+        const size_t step = 8 * static_cast<size_t>(p.N);
+        uint4 y[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          y[j] = lds_u32x4(out_tile + 512 * j + 64 * (lane >> 2) + 16 * ((lane ^ (lane >> 3)) & 3));
+        if (p.yref == nullptr) {
+          uint16_t* yp = p.Y + at;
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            if (row + 8 * j < p.M) *reinterpret_cast<uint4*>(yp + j * step) = y[j];
+        } else {
           // Eq. 10's objective: || Y_ref - Y_hat ||^2 over the tile, with Y_hat rounded to BF16 exactly as the
           // forward would store it.  FP32 within the thread and the warp, FP64 across warps and tiles.
-          float e = 0.0f;
-          if (row < p.M) {
-            const uint4* yr = reinterpret_cast<const uint4*>(p.yref + static_cast<size_t>(row) * p.N + ch0);
+          float sq = 0.0f;
+          const uint16_t* rp = p.yref + at;
 #pragma unroll
-            for (int i = 0; i < kEpiCols / 8; ++i) {
-              float4 b0 = make_float4(0.f, 0.f, 0.f, 0.f), b1 = b0;
-              if (p.bias) {
-                b0 = __ldg(reinterpret_cast<const float4*>(p.bias + ch0) + 2 * i);
-                b1 = __ldg(reinterpret_cast<const float4*>(p.bias + ch0) + 2 * i + 1);
-              }
-              const uint4 ref = __ldg(yr + i);
-              const float2 a0 = acc[4 * i], a1 = acc[4 * i + 1], a2 = acc[4 * i + 2], a3 = acc[4 * i + 3];
-              const float yh[8] = {a0.x + b0.x, a0.y + b0.y, a1.x + b0.z, a1.y + b0.w,
-                                   a2.x + b1.x, a2.y + b1.y, a3.x + b1.z, a3.y + b1.w};
-              const uint32_t rw[4] = {ref.x, ref.y, ref.z, ref.w};
-#pragma unroll
-              for (int c = 0; c < 8; ++c) {
-                const float y_hat = __bfloat162float(__float2bfloat16_rn(apply_activation(yh[c], p.act)));
-                const float y_ref = __uint_as_float((c & 1) ? (rw[c >> 1] & 0xffff0000u) : (rw[c >> 1] << 16));
-                const float d = y_ref - y_hat;
-                e = fmaf(d, d, e);
-              }
+          for (int j = 0; j < 4; ++j) {
+            if (row + 8 * j < p.M) {
+              const uint4 ref = __ldg(reinterpret_cast<const uint4*>(rp + j * step));
+              sq = sq_diff_bf16x2(ref.x, y[j].x, sq);
+              sq = sq_diff_bf16x2(ref.y, y[j].y, sq);
+              sq = sq_diff_bf16x2(ref.z, y[j].z, sq);
+              sq = sq_diff_bf16x2(ref.w, y[j].w, sq);
             }
           }
 #pragma unroll
-          for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
-          if (lane == 0) atomicAdd(p.sq_err, static_cast<double>(e));
-        } else if (row < p.M) {
-          // The thread's channels are contiguous bytes of its output row.
-          uint4* yrow = reinterpret_cast<uint4*>(p.Y + static_cast<size_t>(row) * p.N + ch0);
-#pragma unroll
-          for (int i = 0; i < kEpiCols / 8; ++i) {  // 8 channels per 16-byte store
-            float4 b0 = make_float4(0.f, 0.f, 0.f, 0.f), b1 = b0;
-            if (p.bias) {
-              b0 = __ldg(reinterpret_cast<const float4*>(p.bias + ch0) + 2 * i);
-              b1 = __ldg(reinterpret_cast<const float4*>(p.bias + ch0) + 2 * i + 1);
-            }
-            const float2 a0 = acc[4 * i], a1 = acc[4 * i + 1], a2 = acc[4 * i + 2], a3 = acc[4 * i + 3];
-            float y[8] = {a0.x + b0.x, a0.y + b0.y, a1.x + b0.z, a1.y + b0.w, a2.x + b1.x, a2.y + b1.y, a3.x + b1.z, a3.y + b1.w};
-            if (p.act != 0) {  // uniform over the grid
-#pragma unroll
-              for (int c = 0; c < 8; ++c) y[c] = apply_activation(y[c], p.act);
-            }
-            __nv_bfloat162 o0 = __floats2bfloat162_rn(y[0], y[1]);
-            __nv_bfloat162 o1 = __floats2bfloat162_rn(y[2], y[3]);
-            __nv_bfloat162 o2 = __floats2bfloat162_rn(y[4], y[5]);
-            __nv_bfloat162 o3 = __floats2bfloat162_rn(y[6], y[7]);
-            uint4 o;
-            o.x = *reinterpret_cast<uint32_t*>(&o0);
-            o.y = *reinterpret_cast<uint32_t*>(&o1);
-            o.z = *reinterpret_cast<uint32_t*>(&o2);
-            o.w = *reinterpret_cast<uint32_t*>(&o3);
-            yrow[i] = o;
-          }
+          for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+          if (lane == 0) atomicAdd(p.sq_err, static_cast<double>(sq));
         }
       }
       tmem_wait_ld();   // a role that gave up may still have loads in flight

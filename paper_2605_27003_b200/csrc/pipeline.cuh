@@ -119,12 +119,34 @@ __device__ __forceinline__ float apply_activation(float y, int act) {
   return y;
 }
 
+// n / divisor by one high multiplication and a shift, for n < 2^31 (round-up method: Granlund and Montgomery, "Division by
+// invariant integers using multiplication", 1994).  A plain division cost the epilogue's tile change ~300 clocks each.
+struct FastDiv {
+  uint32_t divisor = 1, mul = 0, shift = 0;
+  FastDiv() = default;
+  explicit FastDiv(uint32_t d) : divisor(d) {
+    while ((1ull << shift) < d) ++shift;
+    mul = static_cast<uint32_t>((((1ull << shift) - d) << 32) / d + 1);
+  }
+  __device__ uint32_t quotient(uint32_t n) const { return (__umulhi(n, mul) + n) >> shift; }
+};
+
+// Order of the INT4 GEMM's output tiles: super-columns of `width` column tiles, all row blocks of one before the next;
+// width == number of column tiles: plain row-major order.
+struct TileOrder {
+  FastDiv per_sc, width, last_width;   // tiles of a full super-column; its width; the width of what is left (if anything)
+  uint32_t full = 0;                   // full super-columns
+  TileOrder() = default;
+  TileOrder(int tiles_m, int tiles_n, int sc)
+      : per_sc(static_cast<uint32_t>(tiles_m) * sc), width(sc), last_width(tiles_n % sc ? tiles_n % sc : sc), full(tiles_n / sc) {}
+};
+
 struct GemmParams {
   const float* bias;    // [N] or nullptr
   uint16_t* Y;          // [M, N] BF16
   int M, N, K, r;
   int tiles_m, tiles_n;
-  int sc_tiles;         // column tiles per super-column of the tile order (tiles_n: plain row-major order)
+  TileOrder order;
   int* err;
   uint64_t wait_limit_ns;
   int32_t* dbg_P;       // debug tap: [kBM, G, kBN] or nullptr

@@ -260,7 +260,7 @@ w4a4_status_t launch_gemm(w4a4_handle_t h, int M, int expert_id, void* Y, cudaSt
       sc = (p.tiles_n + ns - 1) / ns;
     }
     if (ctx->debug_sc_tiles > 0) sc = ctx->debug_sc_tiles < p.tiles_n ? ctx->debug_sc_tiles : p.tiles_n;
-    p.sc_tiles = sc;
+    p.order = TileOrder(p.tiles_m, p.tiles_n, sc);
   }
   p.err = ctx->d_err;
   p.wait_limit_ns = wait_limit_ns;
@@ -376,7 +376,11 @@ w4a4_status_t w4a4_ctx_create(int device, int max_M, int max_K, int max_r, w4a4_
                          static_cast<int>(quantize_smem_bytes(96)));
     const cudaError_t e1 = cudaFuncSetAttribute(gemm_w4a4_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmemBytes);
     const cudaError_t e2 = cudaFuncSetAttribute(gemm_w4a4_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmemBytes);
-    if (e1 != cudaSuccess || e2 != cudaSuccess) {
+    // The kernel redistributes its launch's registers: it must have been compiled with as many as it hands out.
+    cudaFuncAttributes a1, a2;
+    const bool regs_ok = cudaFuncGetAttributes(&a1, gemm_w4a4_kernel<false>) == cudaSuccess && a1.numRegs == kGemmRegs &&
+                         cudaFuncGetAttributes(&a2, gemm_w4a4_kernel<true>) == cudaSuccess && a2.numRegs == kGemmRegs;
+    if (e1 != cudaSuccess || e2 != cudaSuccess || !regs_ok) {
       cudaGetLastError();
       st = W4A4_ERR_CUDA;
     }
