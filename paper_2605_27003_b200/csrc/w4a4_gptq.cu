@@ -6,16 +6,20 @@
 // layer's calibration inputs.  Here:
 //
 //   1. H (upper triangle) = X_hat^T X_hat by a tiled FP64 GEMM; dead channels and damping on the diagonal.
-//   2. U without ever forming H^-1: factor H = V V^T with V UPPER triangular (a Cholesky factorization taken from
-//      the last channel to the first, blocked by 64: diagonal block, panel solve, rank-64 update), then U = V^-1
-//      (blocked triangular inverse, bottom up).  H^-1 = V^-T V^-1 = U^T U with U upper and a positive diagonal,
-//      which is the unique factor the algorithm asks for.
-//   3. The sweep, one 64-channel group at a time: one thread per output channel holds the group's 64 weights in
-//      registers, takes the group scale, quantizes channel after channel and applies the in-group updates; the
-//      group's scaled errors then update all later channels by one more GEMM (the algorithm's lazy batch).
+//   2. H = V V^T with V UPPER triangular: a Cholesky factorization taken from the last channel to the first, blocked by 64.
+//      U = V^-1 is the factor the algorithm asks for (H^-1 = V^-T V^-1), but neither H^-1 nor U is formed: with e_k the
+//      algorithm's scaled errors and z = U^T e, i.e. V^T z = e, forward substitution gives the compensated weight of
+//      channel j as
+//          w_j = W_j - sum_{k<j} U_kj e_k = W_j + sum_{k<j} (V_kj / V_jj) z_k ,      z_k = W_k - q_k ,
+//      the difference between the ORIGINAL weight and the value its code stands for (the form of the same procedure
+//      published as LDLQ: Chee et al., "QuIP", 2023, Sec. 3).  So the sweep needs L = V with its columns divided by the
+//      diagonal, and K^3 / 3 multiply-adds of a triangular inverse are not there.  A group's scale is taken from its weights
+//      as compensated for the channels before the group only; with t_j = sum_{k before the group} L_kj z_k these are
+//      W_g + L_gg^-T t_g, which needs the inverse of L's 64 x 64 diagonal blocks.
+//   3. The sweep, 256 channels (a lazy batch) per launch, and one product for the channels after the batch.
 //
-// Nothing here waits on another block: every dependency is a kernel boundary, on the caller's stream or on an event
-// between it and one side stream of the call's own.
+// One stream, and nothing here waits on another block: every dependency is a kernel boundary.  (Large products beside the
+// serial steps on a second stream gave nothing: sharing the FP64 pipe stretches the serial chains by as much as is hidden.)
 #include "../../include/w4a4.h"
 
 #include <cuda_runtime.h>
@@ -25,25 +29,46 @@
 namespace {
 
 constexpr int kNb = 64;     // block of the factorization = quantization group = lazy batch
-constexpr int kBand = 512;  // columns per band of the factorization, rows per band of the triangular inverse
+constexpr int kBand = 512;  // columns per band of the factorization
 constexpr int kLazy = 256;  // input channels per lazy batch of the sweep
 
 // ---------------------------------------------------------------------------------------------------------
-// C[m, n] = beta * C[m, n] + alpha * sum_k A(m, k) * B(k, n), every operand addressed by two strides so that a
-// transposed or sub-matrix operand costs nothing.  (16 TM) x 64 tile per block in 16-deep slices, double-buffered in
-// shared memory by asynchronous copies; eight warps, each a (4 TM) x 32 corner as 8 x 8 x 4 FP64 tensor-core steps.  Structure flags: kUpperOut -- blocks whose tile lies entirely below the diagonal return at once (only the
-// upper triangle of C is wanted); kAUpper -- A(m, k) = 0 for k < m, so the sum starts at the tile's first row;
-// kBUpper -- B(k, n) = 0 for k > n, so the sum ends at the tile's last column.
+// C = beta C + alpha A B in FP64, C row-major.  Each operand is stored with one of its two indices contiguous: k (AK,
+// BK) or the output index (A(m, k) at A[k lda + m], B(k, n) at B[k ldb + n]).  M and N are multiples of 64, Kd of 16,
+// leading dimensions and offsets multiples of two elements.
+//
+// BM x 64 tile per block, eight warps, each a (BM / 4) x 32 corner as 8 x 8 x 4 FP64 tensor-core steps; 16-deep slices in a
+// ring of four, filled by 16-byte asynchronous copies three slices ahead, one barrier per slice.  The FP64 tensor path
+// is the bound (37.0 TFLOP/s measured for every instruction shape): a slice of a 128 x 64 tile takes it ~2000 clocks and
+// brings in 24 KiB, far below what shared memory and L2 deliver.
+//
+// With `upper_out`, blocks whose tile lies entirely below the diagonal (column index + diag_shift) return at once (only the
+// upper triangle of C is wanted).
 // ---------------------------------------------------------------------------------------------------------
-constexpr int kBN = 64, kBK = 16;
-enum : int { kUpperOut = 1, kAUpper = 2, kBUpper = 4 };
+constexpr int kBN = 64, kBK = 16, kGemmRing = 4;
 
-// 8-byte asynchronous copy global -> shared; with `valid` false nothing is read and zeros are written.
-__device__ __forceinline__ void async_copy8(double* smem_dst, const double* gmem_src, bool valid) {
+struct GemmArgs {
+  int M, N, Kd;
+  const double* A;
+  long lda;
+  const double* B;
+  long ldb;
+  double* C;
+  long ldc;
+  double alpha, beta;   // +1 or -1; 0 or 1
+  bool upper_out = false;
+  int diag_shift = 0;
+};
+
+// 16-byte asynchronous copy global -> shared; with `valid` false nothing is read and zeros are written.
+__device__ __forceinline__ void async_copy16(double* smem_dst, const double* gmem_src, bool valid) {
   const unsigned dst = static_cast<unsigned>(__cvta_generic_to_shared(smem_dst));
-  const int src_bytes = valid ? 8 : 0;
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(gmem_src), "r"(src_bytes) : "memory");
+  const int src_bytes = valid ? 16 : 0;
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(gmem_src), "r"(src_bytes) : "memory");
 }
+__device__ __forceinline__ void async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int LEFT>
+__device__ __forceinline__ void async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(LEFT) : "memory"); }
 
 // D (8 x 8) += A (8 x 4) B (4 x 8) on the FP64 tensor core; per lane one element of A and B, two of D.
 __device__ __forceinline__ void dmma_8x8x4(double (&d)[2], double a, double b) {
@@ -52,323 +77,533 @@ __device__ __forceinline__ void dmma_8x8x4(double (&d)[2], double a, double b) {
                : "d"(a), "d"(b));
 }
 
-template <int TM>
-__global__ void __launch_bounds__(256, 2) dgemm_kernel(int M, int N, int Kd, const double* __restrict__ A, long sa_m,
-                                                    long sa_k, const double* __restrict__ B, long sb_k, long sb_n,
-                                                    double* __restrict__ C, long sc_m, long sc_n, double alpha,
-                                                    double beta, int flags) {
-  constexpr int BM = 16 * TM;
-  constexpr int MT = TM / 2;  // 8 x 8 tensor-core tiles per warp along M (four along N)
-  // Two slices of each operand: the next one arrives while this one is used.  Element (k, x) sits at column
-  // x ^ ((k & 3) << 2): a fragment load touches four k rows times four neighbouring columns per half warp, and the
-  // swap of 4-column groups by k spreads them over all banks.
-  __shared__ __align__(16) double As[2][kBK][BM];
-  __shared__ __align__(16) double Bs[2][kBK][kBN];
+// Place of element (k, x) in a slice of X output indices.  A fragment load of a half warp touches four k and four x:
+// the swap of groups of four (by k where x is contiguous, by x where k is) spreads them over all banks and keeps the pairs
+// of a 16-byte copy together.
+template <int X, bool KFAST>
+__device__ __forceinline__ int slice_at(int k, int x) {
+  return KFAST ? x * kBK + ((((k >> 2) ^ (x & 3)) << 2) | (k & 3)) : k * X + (x ^ ((k & 3) << 2));
+}
+
+// One operand's share of a slice: X * 16 elements by 256 threads, two per copy.  `src` points at this thread's first pair
+// of the slice.
+template <int X, bool KFAST>
+__device__ __forceinline__ void fetch_operand(double* dst, const double* src, long ld, int x_valid) {
+  const int tid = threadIdx.x;
+#pragma unroll
+  for (int i = 0; i < X / 32; ++i) {
+    if (KFAST) {
+      const int x = (tid >> 3) + 32 * i, k = 2 * (tid & 7);
+      async_copy16(dst + slice_at<X, true>(k, x), src + 32 * i * ld, x < x_valid);
+    } else {
+      constexpr int kPerPass = 512 / X;   // k rows covered by one pass of the 256 threads
+      const int x = 2 * (tid % (X / 2)), k = tid / (X / 2) + kPerPass * i;
+      async_copy16(dst + slice_at<X, false>(k, x), src + static_cast<long>(kPerPass * i) * ld, x < x_valid);
+    }
+  }
+}
+template <int X, bool KFAST>
+__device__ __forceinline__ const double* operand_start(const double* p, long ld, int x0, int k0) {
+  const int tid = threadIdx.x;
+  return KFAST ? p + static_cast<long>(x0 + (tid >> 3)) * ld + k0 + 2 * (tid & 7)
+               : p + static_cast<long>(k0 + tid / (X / 2)) * ld + x0 + 2 * (tid % (X / 2));
+}
+
+constexpr size_t dgemm_smem_bytes(int BM) { return static_cast<size_t>(kGemmRing) * (BM + kBN) * kBK * sizeof(double); }
+
+template <int BM, bool AK, bool BK>
+__global__ void __launch_bounds__(256, 2) dgemm_kernel(const GemmArgs g) {
+  constexpr int MT = BM / 32;  // 8 x 8 tensor-core tiles per warp along M (four along N)
+  extern __shared__ __align__(16) double slices[];
+  double* const As = slices;
+  double* const Bs = slices + kGemmRing * BM * kBK;
   const int m0 = blockIdx.y * BM, n0 = blockIdx.x * kBN;
-  if ((flags & kUpperOut) && m0 >= n0 + kBN) return;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (g.upper_out && m0 >= n0 + g.diag_shift + kBN) return;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int wm = (warp & 3) * (8 * MT), wn = (warp >> 2) * 32;  // the warp's corner inside the block's tile
   const int fr = lane >> 2, fk = lane & 3;                      // fragment row (or column) and k index of this lane
-  const bool a_m_fast = (sa_m == 1), b_n_fast = (sb_n == 1);
-  const int k_begin = (flags & kAUpper) ? m0 : 0;  // m0 is a multiple of 16
-  const int k_end = (flags & kBUpper) ? min(Kd, n0 + kBN) : Kd;
-  // One slice of both operands, global -> shared without passing through registers; elements outside the
-  // operands are written as zeros (source size 0).
-  auto fetch_slice = [&](int buf, int k0) {
-#pragma unroll
-    for (int i = 0; i < TM; ++i) {
-      const int e = tid + i * 256;
-      const int am = a_m_fast ? (e % BM) : (e >> 4), ak = a_m_fast ? (e / BM) : (e & 15);
-      const bool in = (m0 + am < M && k0 + ak < Kd);
-      async_copy8(&As[buf][ak][am ^ ((ak & 3) << 2)], in ? A + (long)(m0 + am) * sa_m + (long)(k0 + ak) * sa_k : A, in);
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int e = tid + i * 256;
-      const int bn = b_n_fast ? (e & 63) : (e >> 4), bk = b_n_fast ? (e >> 6) : (e & 15);
-      const bool in = (n0 + bn < N && k0 + bk < Kd);
-      async_copy8(&Bs[buf][bk][bn ^ ((bk & 3) << 2)], in ? B + (long)(k0 + bk) * sb_k + (long)(n0 + bn) * sb_n : B, in);
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
+  const int n_slices = g.Kd / kBK;
+  const double* a_src = operand_start<BM, AK>(g.A, g.lda, m0, 0);
+  const double* b_src = operand_start<kBN, BK>(g.B, g.ldb, n0, 0);
+  const long a_step = AK ? kBK : kBK * g.lda, b_step = BK ? kBK : kBK * g.ldb;
+  const int m_valid = g.M - m0;
+  auto fetch_slice = [&](int slice) {
+    const int buf = slice % kGemmRing;
+    fetch_operand<BM, AK>(As + buf * (BM * kBK), a_src + slice * a_step, g.lda, m_valid);
+    fetch_operand<kBN, BK>(Bs + buf * (kBN * kBK), b_src + slice * b_step, g.ldb, kBN);
   };
-  double acc[MT][4][2] = {};
-  if (k_begin < k_end) fetch_slice(0, k_begin);
-  int buf = 0;
-  for (int k0 = k_begin; k0 < k_end; k0 += kBK, buf ^= 1) {
-    if (k0 + kBK < k_end) {
-      fetch_slice(buf ^ 1, k0 + kBK);
-      asm volatile("cp.async.wait_group 1;" ::: "memory");
-    } else {
-      asm volatile("cp.async.wait_group 0;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < kGemmRing - 1; ++i) {
+    if (i < n_slices) fetch_slice(i);
+    async_commit();
+  }
+  // Accumulator layout: rows fr, columns 2 fk and 2 fk + 1 of each 8 x 8 tile.  C = alpha (A B + (beta / alpha) C), alpha =
+  // +-1: the accumulators start from C, whose loads run under the first slices' copies.
+  const bool rows_valid = m0 + wm < g.M;   // M is a multiple of 64: a warp's rows lie on one side of it
+  double* const C = g.C + static_cast<long>(m0 + wm + fr) * g.ldc + n0 + wn + 2 * fk;
+  const bool pairs = (reinterpret_cast<uintptr_t>(g.C) & 15) == 0;   // a caller's statistic may be 8-byte aligned only
+  double acc[MT][4][2];
+#pragma unroll
+  for (int i = 0; i < MT; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const double* c = C + static_cast<long>(8 * i) * g.ldc + 8 * j;
+      double2 v = make_double2(0.0, 0.0);
+      if (g.beta != 0.0 && rows_valid) v = pairs ? *reinterpret_cast<const double2*>(c) : make_double2(c[0], c[1]);
+      acc[i][j][0] = g.alpha * v.x;   // beta is 0 or 1, alpha is its own inverse
+      acc[i][j][1] = g.alpha * v.y;
     }
-    __syncthreads();
+  for (int s = 0; s < n_slices; ++s) {
+    async_wait<kGemmRing - 2>();
+    __syncthreads();   // slice s is complete, and everyone is done with the slice whose place the next one takes
+    if (s + kGemmRing - 1 < n_slices) fetch_slice(s + kGemmRing - 1);
+    async_commit();
+    const double* as = As + (s % kGemmRing) * (BM * kBK);
+    const double* bs = Bs + (s % kGemmRing) * (kBN * kBK);
 #pragma unroll
     for (int k = 0; k < kBK; k += 4) {
       // FP64 tensor-core step (8 x 8 x 4): this lane holds A[row fr][k fk] and B[k fk][column fr] of each tile
       double a[MT], b[4];
 #pragma unroll
-      for (int i = 0; i < MT; ++i) a[i] = As[buf][k + fk][(wm + 8 * i + fr) ^ (fk << 2)];
+      for (int i = 0; i < MT; ++i) a[i] = as[slice_at<BM, AK>(k + fk, wm + 8 * i + fr)];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = Bs[buf][k + fk][(wn + 8 * j + fr) ^ (fk << 2)];
+      for (int j = 0; j < 4; ++j) b[j] = bs[slice_at<kBN, BK>(k + fk, wn + 8 * j + fr)];
 #pragma unroll
       for (int i = 0; i < MT; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) dmma_8x8x4(acc[i][j], a[i], b[j]);
     }
-    __syncthreads();  // everyone is done with this slice before the next fetch overwrites it
   }
-  // Accumulator layout: rows fr, columns 2 fk and 2 fk + 1 of each 8 x 8 tile.  Two passes over the outputs, all
-  // loads of C before the first store: with run-time strides the compiler cannot tell that the addresses differ, and
-  // a load placed after a store would wait for it, one memory round trip each.
-  if (beta != 0.0) {
-#pragma unroll
-    for (int i = 0; i < MT; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-          const int m = m0 + wm + 8 * i + fr, n = n0 + wn + 8 * j + 2 * fk + c;
-          const double v = (m < M && n < N) ? C[(long)m * sc_m + (long)n * sc_n] : 0.0;
-          acc[i][j][c] = fma(alpha, acc[i][j][c], beta * v);
-        }
-  } else {
-#pragma unroll
-    for (int i = 0; i < MT; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) acc[i][j][0] *= alpha, acc[i][j][1] *= alpha;
-  }
+  if (!rows_valid) return;
 #pragma unroll
   for (int i = 0; i < MT; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
-#pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        const int m = m0 + wm + 8 * i + fr, n = n0 + wn + 8 * j + 2 * fk + c;
-        if (m < M && n < N) C[(long)m * sc_m + (long)n * sc_n] = acc[i][j][c];
+    for (int j = 0; j < 4; ++j) {
+      double* c = C + static_cast<long>(8 * i) * g.ldc + 8 * j;
+      const double c0 = g.alpha * acc[i][j][0], c1 = g.alpha * acc[i][j][1];
+      if (pairs) {
+        *reinterpret_cast<double2*>(c) = make_double2(c0, c1);
+      } else {
+        c[0] = c0;
+        c[1] = c1;
       }
-}
-
-__global__ void bf16_to_f64_kernel(const uint16_t* __restrict__ in, double* __restrict__ out, long n) {
-  const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) out[i] = (double)__uint_as_float((uint32_t)in[i] << 16);
-}
-
-// Dead input channels (H_kk = 0) get H_kk = 1, and the mean of the diagonal after that fix goes to *mean_out.
-// One block; the sum runs in a fixed order (thread-strided partial sums, then a tree), so it is deterministic.
-__global__ void gptq_diag_mean_kernel(double* __restrict__ H, int K, unsigned char* __restrict__ dead,
-                                      double* __restrict__ mean_out) {
-  __shared__ double part[256];
-  double s = 0.0;
-  for (int k = threadIdx.x; k < K; k += 256) {
-    double d = H[(long)k * K + k];
-    const bool is_dead = (d == 0.0);
-    if (is_dead) {
-      d = 1.0;
-      H[(long)k * K + k] = 1.0;
     }
-    dead[k] = is_dead ? 1 : 0;
-    s += d;
+}
+
+// BF16 -> FP64, two values per thread; values from `n` on (the rows that pad a batch of tokens to a whole slice) are zeros.
+__global__ void bf16_to_f64_kernel(const uint16_t* __restrict__ in, double2* __restrict__ out, long n, long n_padded) {
+  const long i = 2 * ((long)blockIdx.x * blockDim.x + threadIdx.x);
+  if (i >= n_padded) return;
+  const uint32_t lo = i < n ? in[i] : 0u, hi = i + 1 < n ? in[i + 1] : 0u;
+  out[i >> 1] = make_double2((double)__uint_as_float(lo << 16), (double)__uint_as_float(hi << 16));
+}
+
+// Dead input channels (H_kk = 0) count as H_kk = 1; percdamp times the mean of the diagonal after that fix goes to *damp.
+// One block; the sum runs in a fixed order (thread-strided partial sums, then a tree), so it is deterministic.
+__global__ void gptq_diag_kernel(const double* __restrict__ H, int K, double percdamp, unsigned char* __restrict__ dead,
+                                 double* __restrict__ damp) {
+  __shared__ double part[1024];
+  double s = 0.0;
+  for (int k = threadIdx.x; k < K; k += 1024) {
+    const double d = H[(long)k * K + k];
+    dead[k] = d == 0.0 ? 1 : 0;
+    s += d == 0.0 ? 1.0 : d;
   }
   part[threadIdx.x] = s;
   __syncthreads();
-  for (int w = 128; w > 0; w >>= 1) {
+  for (int w = 512; w > 0; w >>= 1) {
     if (threadIdx.x < w) part[threadIdx.x] += part[threadIdx.x + w];
     __syncthreads();
   }
-  if (threadIdx.x == 0) *mean_out = part[0] / (double)K;
-}
-
-__global__ void gptq_damp_kernel(double* __restrict__ H, int K, const double* __restrict__ mean, double percdamp) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k < K) H[(long)k * K + k] += percdamp * *mean;
-}
-
-// W = FP64(R) with the rows of dead input channels zeroed.
-__global__ void gptq_init_w_kernel(const float* __restrict__ R, const unsigned char* __restrict__ dead,
-                                   double* __restrict__ W, int K, int N) {
-  const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < (long)K * N) W[i] = dead[i / N] ? 0.0 : (double)R[i];
+  if (threadIdx.x == 0) *damp = percdamp * (part[0] / (double)K);
 }
 
 // ---------------------------------------------------------------------------------------------------------
 // H = V V^T, V upper triangular, from the last block to the first (A holds H's upper triangle and ends as V).
 // ---------------------------------------------------------------------------------------------------------
 
-// The 64 x 64 diagonal block at j0, whose trailing updates are already applied: column 63 down to column 0, one
-// barrier per column.  Sixteen threads share a row.  At column j every thread forms 1 / sqrt(pivot) itself, scales
-// the entries of column j it needs on the fly (they stay unscaled in shared memory; the scaled column goes straight
-// to global memory, nobody reads it again here) and updates its part of the columns to the left, so reads (column j)
-// and writes (columns < j) of one step never meet.  A pivot that is not positive raises *not_pd.
-constexpr int kDiagParts = 16;  // threads per row (4, 8 and 16 measure within 1 % of one another per layer)
-constexpr int kDiagThreads = kDiagParts * kNb;
-__global__ void __launch_bounds__(kDiagThreads) chol_diag_kernel(double* __restrict__ A, long ld, int j0, int* not_pd) {
-  __shared__ double S[kNb][kNb + 1];
-  const int t = threadIdx.x & (kNb - 1), part = threadIdx.x >> 6;
-  for (int r = part; r < kNb; r += kDiagParts) S[r][t] = A[(long)(j0 + r) * ld + j0 + t];
+// One 64-column step: the diagonal block at j0, whose trailing updates are already applied, is factored, and the 64-row
+// strip of the panel above it that belongs to this block of threads becomes the solution of x D^T = row (D the factored
+// block), both in one elimination from the last column to the first: the strip's rows take the same column operations as
+// the diagonal block's.  Every block factors the diagonal block for itself: that adds nothing to the chain of steps, which
+// is what this kernel is bound by.  The strips of V stay in A for the factorization's own products; L gets block and strips
+// with every column divided by its diagonal element, which is what the sweep reads.  The diagonal (dead channels, damping)
+// is completed on the way in.  Entries below the diagonal are never used for a result (H_in's lower triangle is not
+// defined).
+// Eight columns at a time: each of 128 threads factors the 8 x 8 corner for itself in registers (a chain of eight reciprocal
+// square roots) and solves its own row against it; then the columns still to come take the eight as 8 x 8 x 4 FP64
+// tensor-core steps, warp w on the row tiles w of block and strip.  Two barriers per eight columns, and a loop body small
+// enough for the instruction cache: column by column, 64 steps unrolled took 24 us per launch, rolled with predicates 55,
+// in shared memory 39 + 16 in two kernels; this 18.6 (K = 5120).
+constexpr int kCholThreads = 256, kCholSub = 8;
+constexpr int kCholPitch = kNb + 2, kCholFPitch = 12;
+constexpr size_t kCholSmemBytes = 2 * kNb * (kCholPitch + kCholFPitch) * sizeof(double);
+__global__ void __launch_bounds__(kCholThreads) chol_step_kernel(double* __restrict__ A, double* __restrict__ L, long ld,
+                                                                 int j0, const unsigned char* __restrict__ dead,
+                                                                 const double* __restrict__ damp, int* not_pd) {
+  extern __shared__ __align__(16) double chol_smem[];
+  double(*S)[kCholPitch] = reinterpret_cast<double(*)[kCholPitch]>(chol_smem);   // rows 0..63 diagonal block, 64..127 strip
+  double(*F)[kCholFPitch] = reinterpret_cast<double(*)[kCholFPitch]>(chol_smem + 2 * kNb * kCholPitch);   // eight finished columns
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int fr = lane >> 2, fk = lane & 3;
+  const long strip0 = (long)blockIdx.x * kNb;
+  const bool has_strip = strip0 < j0;                       // the one block of the last step (j0 = 0) has none
+  for (int i = t >> 5; i < kNb; i += kCholThreads / 32) {
+    async_copy16(&S[i][2 * lane], A + (long)(j0 + i) * ld + j0 + 2 * lane, true);
+    async_copy16(&S[kNb + i][2 * lane], has_strip ? A + (strip0 + i) * ld + j0 + 2 * lane : A, has_strip);
+  }
+  async_commit();
+  const double on_diagonal = t < kNb ? *damp + (dead[j0 + t] ? 1.0 : 0.0) : 0.0;
+  async_wait<0>();
   __syncthreads();
-  for (int j = kNb - 1; j >= 0; --j) {
-    const double d = S[j][j];
-    const double inv = rsqrt(d), root = d * inv;  // one short chain per column instead of a root and a division
-    if (threadIdx.x == j) {
-      if (!(d > 0.0)) *not_pd = 1;
-      A[(long)(j0 + j) * ld + j0 + j] = root;
+  if (t < kNb) S[t][t] += on_diagonal;
+  __syncthreads();
+#pragma unroll 1
+  for (int kb = kNb / kCholSub - 1; kb >= 0; --kb) {
+    const int c0 = kCholSub * kb;
+    if (t < 2 * kNb) {
+      double a[kCholSub][kCholSub], inv[kCholSub];   // upper triangle of the corner
+#pragma unroll
+      for (int i = 0; i < kCholSub; ++i)
+#pragma unroll
+        for (int j = i & ~1; j < kCholSub; j += 2) {
+          const double2 v = *reinterpret_cast<const double2*>(&S[c0 + i][c0 + j]);
+          a[i][j] = v.x;   // (an entry below the diagonal in the first pair of an odd row: not used)
+          a[i][j + 1] = v.y;
+        }
+#pragma unroll
+      for (int j = kCholSub - 1; j >= 0; --j) {
+        if (t == 0 && !(a[j][j] > 0.0)) *not_pd = 1;
+        inv[j] = rsqrt(a[j][j]);
+#pragma unroll
+        for (int i = 0; i < j; ++i) a[i][j] *= inv[j];
+#pragma unroll
+        for (int i = 0; i < j; ++i)
+#pragma unroll
+          for (int m = i; m < j; ++m) a[i][m] = fma(-a[i][j], a[m][j], a[i][m]);
+      }
+      double x[kCholSub];
+#pragma unroll
+      for (int j = 0; j < kCholSub; j += 2) {
+        const double2 v = *reinterpret_cast<const double2*>(&S[t][c0 + j]);
+        x[j] = v.x;
+        x[j + 1] = v.y;
+      }
+#pragma unroll
+      for (int j = kCholSub - 1; j >= 0; --j) {
+        x[j] *= inv[j];
+#pragma unroll
+        for (int m = 0; m < j; ++m) x[m] = fma(-x[j], a[m][j], x[m]);
+      }
+#pragma unroll
+      for (int j = 0; j < kCholSub; j += 2) {
+        const double2 v = make_double2(x[j], x[j + 1]);
+        *reinterpret_cast<double2*>(&F[t][j]) = v;
+        const double2 l = make_double2(x[j] * inv[j], x[j + 1] * inv[j + 1]);
+        if (t < kNb ? blockIdx.x == 0 : has_strip)
+          *reinterpret_cast<double2*>(L + (t < kNb ? j0 + t : strip0 + t - kNb) * ld + j0 + c0 + j) = l;
+      }
     }
-    if (t < j) {
-      const double f = S[t][j] * inv;
-      if (part == 0) A[(long)(j0 + t) * ld + j0 + j] = f;
-      for (int c = t + part; c < j; c += kDiagParts) S[t][c] = fma(-f, S[c][j] * inv, S[t][c]);
+    __syncthreads();
+    if (t < 2 * kNb) {   // after the barrier: the rows of the corner were still being read
+#pragma unroll
+      for (int j = 0; j < kCholSub; j += 2)
+        *reinterpret_cast<double2*>(&S[t][c0 + j]) = *reinterpret_cast<const double2*>(&F[t][j]);
+    }
+#pragma unroll
+    for (int part = 0; part < 2; ++part) {   // strip, diagonal block (its tiles on and above the diagonal)
+      const int row = 8 * warp + (part == 0 ? kNb : 0) + fr;
+      double f[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) f[h] = -F[row][4 * h + fk];
+#pragma unroll 1
+      for (int ct = part == 0 ? 0 : warp; ct < kb; ++ct) {
+        double2* at = reinterpret_cast<double2*>(&S[row][8 * ct + 2 * fk]);
+        double c[2] = {at->x, at->y};
+#pragma unroll
+        for (int h = 0; h < 2; ++h) dmma_8x8x4(c, f[h], F[8 * ct + fr][4 * h + fk]);
+        *at = make_double2(c[0], c[1]);
+      }
     }
     __syncthreads();
   }
-  // below the diagonal: zeros (the triangular inverse reads the whole block)
-  for (int r = part; r < kNb; r += kDiagParts)
-    if (t < r) A[(long)(j0 + r) * ld + j0 + t] = 0.0;
+  if (has_strip)
+    for (int i = t >> 5; i < kNb; i += kCholThreads / 32)
+      *reinterpret_cast<double2*>(A + (strip0 + i) * ld + j0 + 2 * lane) = *reinterpret_cast<const double2*>(&S[kNb + i][2 * lane]);
 }
 
-// The panel above the diagonal block: each row x of A[0:j0, j0:j0+64] becomes the solution of x D^T = row, D the
-// factored diagonal block.  One thread per row, the row in registers.
-__global__ void __launch_bounds__(kNb) chol_panel_kernel(double* __restrict__ A, long ld, int j0) {
+// Inverses of L's 64 x 64 diagonal blocks (unit upper triangular; nothing but the entries above the diagonal is read), one
+// block of threads each: G [K / 64][64][64].  Thread c solves L x = e_c.
+__global__ void __launch_bounds__(kNb) unit_inverse_kernel(const double* __restrict__ L, double* __restrict__ G, long ld) {
   __shared__ double D[kNb][kNb + 1];
-  __shared__ double rD[kNb];  // reciprocal diagonal: a product per column instead of a division in the serial chain
-  const int t = threadIdx.x;
-  for (int r = 0; r < kNb; ++r) D[r][t] = A[(long)(j0 + r) * ld + j0 + t];
-  rD[t] = 1.0 / A[(long)(j0 + t) * ld + j0 + t];
-  __syncthreads();
-  const int row = blockIdx.x * kNb + t;
-  if (row >= j0) return;
-  double* p = A + (long)row * ld + j0;
-  double b[kNb];
-#pragma unroll
-  for (int c = 0; c < kNb; ++c) b[c] = p[c];
-#pragma unroll
-  for (int c = kNb - 1; c >= 0; --c) {
-    b[c] = b[c] * rD[c];
-#pragma unroll
-    for (int c2 = 0; c2 < c; ++c2) b[c2] = fma(-b[c], D[c2][c], b[c2]);
-  }
-#pragma unroll
-  for (int c = 0; c < kNb; ++c) p[c] = b[c];
-}
-
-// ---------------------------------------------------------------------------------------------------------
-// U = V^-1 (both upper triangular), block row by block row from the bottom.
-// ---------------------------------------------------------------------------------------------------------
-
-// Inverse of the 64 x 64 diagonal blocks of V from row `first` on (one block of threads each) into the same place of
-// U: thread c solves D x = e_c.
-__global__ void __launch_bounds__(kNb) triinv_diag_kernel(const double* __restrict__ V, double* __restrict__ U,
-                                                          long ld, int first) {
-  __shared__ double D[kNb][kNb + 1];
-  const int t = threadIdx.x, i0 = first + blockIdx.x * kNb;
-  for (int r = 0; r < kNb; ++r) D[r][t] = V[(long)(i0 + r) * ld + i0 + t];
+  const int t = threadIdx.x, i0 = blockIdx.x * kNb;
+  for (int r = 0; r < kNb; ++r) D[r][t] = L[(long)(i0 + r) * ld + i0 + t];
   __syncthreads();
   double b[kNb];
 #pragma unroll
   for (int r = 0; r < kNb; ++r) b[r] = (r == t) ? 1.0 : 0.0;
 #pragma unroll
-  for (int k = kNb - 1; k >= 0; --k) {
-    b[k] = b[k] / D[k][k];
+  for (int k = kNb - 1; k >= 0; --k)
 #pragma unroll
     for (int r = 0; r < k; ++r) b[r] = fma(-D[r][k], b[k], b[r]);
-  }
 #pragma unroll
-  for (int r = 0; r < kNb; ++r) U[(long)(i0 + r) * ld + i0 + t] = b[r];
+  for (int r = 0; r < kNb; ++r) G[(long)(i0 + r) * kNb + t] = b[r];
 }
 
 // ---------------------------------------------------------------------------------------------------------
-// The sweep over one group of 64 input channels starting at k0 (Algorithm 1's inner loop).
-// scale = FP32(max |w| / 7) over the group as it stands on entry; per channel code = clamp(round-half-even(w /
-// scale), -8, 7) (0 for an all-zero group), err = (w - code * scale) / U_kk, later channels of the group -= err *
-// U_kj.  Err [64, N] keeps the scaled errors for the update of the groups still to come.
-// Two neighbouring lanes share an output channel: the even lane keeps the group's even input channels in registers,
-// the odd lane the odd ones.  At step k both get w_k from its owner by a shuffle and compute code and error alike
-// (same operations, same results), and each updates its own later channels: half the multiply-adds and half the
-// unrolled code per thread.
-// ---------------------------------------------------------------------------------------------------------
-// MX: the same sweep on the MXFP4 grid of the MX variant (OCP MX v1.0): one E8M0 exponent per 32 input channels,
+// The sweep over one lazy batch of up to 256 input channels starting at b0 (Algorithm 1's inner loops), for 32 output
+// channels per block; output channels are independent of one another.
+// scale = FP32(max |w| / 7) over a group of 64 input channels as it stands when the sweep enters it; per channel code =
+// clamp(round-half-even(w / scale), -8, 7) (0 for an all-zero group), z = original weight - code * scale, later channels +=
+// z * L_kj with L = V with its columns divided by the diagonal.  Z [256, ldw] keeps the z for the update of the channels after
+// the batch; T holds what the batches before have added to this one's channels (nothing in the first batch).
+// MX: the same on the MXFP4 grid of the MX variant (OCP MX v1.0): one E8M0 exponent per 32 input channels,
 // floor(log2 max|w|) - 2 over the block as it stands when the sweep enters it, and E2M1 elements {0, 0.5, 1, 1.5, 2,
 // 3, 4, 6} * 2^e, nearest with ties to the even code, saturating at 6, sign bit from the compensated weight.
-constexpr int kGroupCols = 32;  // output channels per block of 64 threads
+//
+// What has been added to the batch's weights stays in shared memory (64 KiB of FP64), and the channels are taken eight channels at a time.  Warp 0 holds the
+// eight of its 32 output channels (one per lane) in registers and walks them one after the other -- the chain that
+// bounds the sweep -- after applying the previous eight's z to them itself; meanwhile the other warps apply the
+// previous z to the channels further on, as 8 x 8 x 4 FP64 tensor-core steps.  One barrier per eight channels; where
+// a group begins, everyone finishes the update first and all warps take part in the product with G and the maxima.  88 us
+// per 256 channels at N = 5120; one launch per 64 channels with the weights in registers and a rank-64 product after it
+// took 38 + 15 us per 64.
+// ---------------------------------------------------------------------------------------------------------
+constexpr int kSweepCols = 32, kSub = 8, kSweepThreads = 256;
+struct SweepSmem {
+  double t[kLazy * kSweepCols];          // sum of L_kj z_k over the channels k done so far; element (r, c) at r * 32 + (c ^ 8 (r & 1))
+  double u[2][kSub][kLazy];              // eight rows of L over the batch's columns, column c at c ^ 4 (row & 3)
+  double ud[4][kSub][2 * kSub];          // eight rows of L, their own eight columns and the next eight
+  double z[2][kSub][kSweepCols];         // column c at c ^ 4 (row & 3)
+  double amax[kSweepThreads / 32][kSweepCols];
+  unsigned char dead[kLazy];
+};
+__device__ __forceinline__ int sweep_t(int r, int c) { return r * kSweepCols + (c ^ ((r & 1) << 3)); }
+
+// INT4: the code of w at scale s (inv = 1 / s, safe = s (1/2 - 1e-9)).  The product with the reciprocal decides the code
+// wherever the remainder is clearly below half a step; elsewhere (ties, clipping, s == 0) the true division does.
+__device__ __forceinline__ double quantize_int4(double w, double s, double inv, double safe) {
+  const double t = w * inv;
+  double q = (t + 6755399441055744.0) - 6755399441055744.0;   // 1.5 * 2^52: round half to even
+  q = t > 7.0 ? 7.0 : (t < -8.0 ? -8.0 : q);
+  if (!(fabs(fma(-q, s, w)) <= safe)) q = s > 0.0 ? fmin(fmax(rint(w / s), -8.0), 7.0) : 0.0;
+  return q;
+}
+
 template <bool MX>
-__global__ void __launch_bounds__(2 * kGroupCols) gptq_group_kernel(const double* __restrict__ W, int N,
-                                                                    const double* __restrict__ U, long ldu, int k0,
-                                                                    void* __restrict__ codes_out,
-                                                                    void* __restrict__ scales_out,
-                                                                    double* __restrict__ Err) {
-  __shared__ double D[kNb][kNb + 1];
-  __shared__ double rD[kNb];  // 1 / U_kk: the error is scaled by a product, which keeps one division out of the
-                              // chain from one input channel to the next (the code is still decided by w / s)
-  const int t = threadIdx.x;
-  for (int r = 0; r < kNb; ++r) D[r][t] = U[(long)(k0 + r) * ldu + k0 + t];
-  rD[t] = 1.0 / U[(long)(k0 + t) * ldu + k0 + t];
-  __syncthreads();
-  const int lane = t & 31, p = t & 1;
-  const int col = blockIdx.x * kGroupCols + (t >> 1);
-  const bool valid = col < N;           // both lanes of a pair agree; nobody leaves before the last shuffle
-  const int n = valid ? col : N - 1;
-  double w[kNb / 2];                    // input channels 2 i + p
+__global__ void __launch_bounds__(kSweepThreads, 2) gptq_sweep_kernel(const float* __restrict__ R,
+                                                                      const unsigned char* __restrict__ dead,
+                                                                      const double* __restrict__ T, int ldw, int N,
+                                                                      const double* __restrict__ L, long ldl,
+                                                                      const double* __restrict__ G, int b0,
+                                                                      int channels, void* __restrict__ codes_out,
+                                                                      void* __restrict__ scales_out,
+                                                                      double* __restrict__ Z) {
+  extern __shared__ __align__(16) unsigned char sweep_smem[];
+  SweepSmem& sm = *reinterpret_cast<SweepSmem*>(sweep_smem);
+  constexpr int kGroup = MX ? 32 : 64, kGroupSubs = kGroup / kSub;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int n0 = blockIdx.x * kSweepCols, n = n0 + lane;
+  const int fr = lane >> 2, fk = lane & 3;
+  const int subs = channels / kSub;
+  const double* const Lb = L + (long)b0 * ldl + b0;   // the batch's own corner of L
+
+  // Eight rows of L from the block after their own on, by the `count` threads from `first` on.
+  auto fetch_u = [&](int sub, int first, int count) {
+    const int c0 = kSub * (sub + 1), pairs = (channels - c0) / 2;
+    for (int i = tid - first; i < kSub * pairs; i += count) {
+      const int k = i / pairs, c = c0 + 2 * (i - k * pairs);
+      async_copy16(&sm.u[sub & 1][k][c ^ ((k & 3) << 2)], Lb + (long)(kSub * sub + k) * ldl + c, true);
+    }
+  };
+  auto fetch_ud = [&](int sub) {   // by one warp
+    if (sub >= subs) return;
 #pragma unroll
-  for (int i = 0; i < kNb / 2; ++i) w[i] = W[(long)(k0 + 2 * i + p) * N + n];
-  double s = 0.0, inv_s = 0.0;          // INT4: the group's scale.  MX: 2^e of the running block and its reciprocal
-  if constexpr (!MX) {
-    double amax = 0.0;
-#pragma unroll
-    for (int i = 0; i < kNb / 2; ++i) amax = fmax(amax, fabs(w[i]));
-    amax = fmax(amax, __shfl_xor_sync(0xffffffffu, amax, 1));
-    const float s32 = (float)(amax / 7.0);  // FP64 quotient rounded once to FP32
-    if (valid && p == 0) static_cast<float*>(scales_out)[(long)(k0 / kNb) * N + n] = s32;
-    s = (double)s32;
+    for (int i = 0; i < 2; ++i) {
+      const int k = (lane >> 3) + 4 * i, c = 2 * (lane & 7);
+      if (kSub * sub + c < channels) async_copy16(&sm.ud[sub & 3][k][c], Lb + (long)(kSub * sub + k) * ldl + kSub * sub + c, true);
+    }
+  };
+  // The original weight of channel b0 + r in output channel c; live() afterwards makes a dead channel's 0.  (Two steps, so
+  // that a load made ahead of its use does not wait for the flag.)
+  auto original = [&](int r, int c) { return c < N ? __ldg(R + (long)(b0 + r) * N + c) : 0.0f; };
+  auto live = [&](int r, float w) { return sm.dead[r] ? 0.0f : w; };
+  for (int i = tid; i < channels * (kSweepCols / 2); i += kSweepThreads) {
+    const int r = i / (kSweepCols / 2), c = 2 * (i % (kSweepCols / 2));
+    async_copy16(&sm.t[sweep_t(r, c)], b0 > 0 ? T + (long)(b0 + r) * ldw + n0 + c : T, b0 > 0);   // zeros in the first batch
   }
+  if (warp == 0) {
+    fetch_ud(0);
+    fetch_ud(1);
+  }
+  async_commit();
+  if (tid < channels) sm.dead[tid] = dead[b0 + tid];
+  async_wait<0>();
+  __syncthreads();
+
+  // Row blocks first, first + step, ... += L^T z of the eight channels `sub`.
+  auto apply = [&](int sub, int first, int step) {
+    double b[2][4];
+    const double(*z)[kSweepCols] = sm.z[sub & 1];
+    const double(*u)[kLazy] = sm.u[sub & 1];
 #pragma unroll
-  for (int k = 0; k < kNb; ++k) {
-    const int i = k >> 1;
-    if constexpr (MX) {
-      if ((k & 31) == 0) {  // entering a block of 32 input channels: its exponent from the weights as they stand
-        double amax = 0.0;
+    for (int h = 0; h < 2; ++h)
 #pragma unroll
-        for (int i2 = 0; i2 < 16; ++i2) amax = fmax(amax, fabs(w[i + i2]));
-        amax = fmax(amax, __shfl_xor_sync(0xffffffffu, amax, 1));
-        int e = amax > 0.0 ? ilogb(amax) - 2 : -127;
-        e = max(-127, min(125, e));
-        s = scalbn(1.0, e);
-        inv_s = scalbn(1.0, -e);
-        if (valid && p == 0) static_cast<uint8_t*>(scales_out)[(long)((k0 + k) / 32) * N + n] = (uint8_t)(e + 127);
+      for (int j = 0; j < 4; ++j) b[h][j] = z[4 * h + fk][(8 * j + fr) ^ (fk << 2)];
+    for (int rb = first; rb < subs; rb += step) {
+      double a[2], c[4][2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) a[h] = u[4 * h + fk][(kSub * rb + fr) ^ (fk << 2)];
+      double2* at[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        at[j] = reinterpret_cast<double2*>(&sm.t[sweep_t(kSub * rb + fr, 8 * j + 2 * fk)]);
+        c[j][0] = at[j]->x, c[j][1] = at[j]->y;
       }
-    }
-    const double wk = __shfl_sync(0xffffffffu, w[i], (lane & ~1) | (k & 1));
-    double deq;
-    int code;
-    if constexpr (MX) {
-      const double v = fmin(fabs(wk) * inv_s, 6.0);  // exact: the scale is a power of two
-      // one comparison per midpoint between neighbouring magnitudes, strict where the lower neighbour is the even code
-      const int idx = (v > 0.25) + (v >= 0.75) + (v > 1.25) + (v >= 1.75) + (v > 2.5) + (v >= 3.5) + (v > 5.0);
-      const double mag = idx < 4 ? 0.5 * idx : (idx < 6 ? idx - 2.0 : 2.0 * idx - 8.0);
-      deq = (wk < 0.0 ? -mag : mag) * s;
-      code = idx + (wk < 0.0 ? 8 : 0);
-    } else {
-      double q = 0.0;
-      if (s > 0.0) q = fmin(fmax(rint(wk / s), -8.0), 7.0);
-      deq = q * s;
-      code = (int)q;
-    }
-    const double e = (wk - deq) * rD[k];
-    if (valid && p == (k & 1)) {
-      if constexpr (MX) static_cast<uint8_t*>(codes_out)[(long)(k0 + k) * N + n] = (uint8_t)code;
-      else static_cast<int8_t*>(codes_out)[(long)(k0 + k) * N + n] = (int8_t)code;
-      Err[(long)k * N + n] = e;
-    }
-    if ((k & 1) == 0 && p == 1) w[i] -= e * D[k][k + 1];  // channel k + 1 lives in the odd lane
 #pragma unroll
-    for (int i2 = i + 1; i2 < kNb / 2; ++i2) w[i2] -= e * D[k][2 * i2 + p];
+      for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) dmma_8x8x4(c[j], a[h], b[h][j]);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) *at[j] = make_double2(c[j][0], c[j][1]);
+    }
+  };
+
+  double s = 0.0, inv = 0.0, safe = 0.0;   // warp 0: the lane's running scale
+  double z[kSub] = {};                     // warp 0: z of the previous eight channels
+  float next_w0[kSub];                     // warp 0: original weights of the next eight, on their way
+  if (warp == 0) {
+#pragma unroll
+    for (int i = 0; i < kSub; ++i) next_w0[i] = original(i, n);
+  }
+  for (int sub = 0; sub < subs; ++sub) {
+    const bool entry = sub % kGroupSubs == 0;
+    if (entry) {
+      // The scale's weights: warp w forms eight rows of W + G^T t (G = inverse of the group's diagonal block of L).
+      constexpr int kSteps = kGroup / 4;
+      const int r0 = kSub * sub, in_block = r0 & (kNb - 1);
+      const bool has_rows = warp < kGroupSubs;
+      double g[kSteps];
+      float w0[4][2];
+      if (has_rows) {
+#pragma unroll
+        for (int k = 0; k < kSteps; ++k)
+          g[k] = G[(long)(b0 + r0 + 4 * k + fk) * kNb + in_block + 8 * warp + fr];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+          for (int c = 0; c < 2; ++c) w0[j][c] = original(r0 + 8 * warp + fr, n0 + 8 * j + 2 * fk + c);
+      }
+      if (sub > 0) {
+        apply(sub - 1, sub + warp, kSweepThreads / 32);
+        __syncthreads();
+      }
+      if (has_rows) {
+        double y[4][2];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) y[j][0] = live(r0 + 8 * warp + fr, w0[j][0]), y[j][1] = live(r0 + 8 * warp + fr, w0[j][1]);
+#pragma unroll
+        for (int k = 0; k < kSteps; ++k)
+          if (k < 2 * (warp + 1)) {   // G is upper triangular
+#pragma unroll
+            for (int j = 0; j < 4; ++j) dmma_8x8x4(y[j], g[k], sm.t[sweep_t(r0 + 4 * k + fk, 8 * j + fr)]);
+          }
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            double m = fabs(y[j][c]);
+#pragma unroll
+            for (int o = 4; o < 32; o *= 2) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+            if (fr == 0) sm.amax[warp][8 * j + 2 * fk + c] = m;
+          }
+      }
+      __syncthreads();
+    }
+    if (warp == 0) {
+      fetch_ud(sub + 2);
+      async_commit();
+      if (entry) {
+        double m = sm.amax[0][lane];
+#pragma unroll
+        for (int i = 1; i < kGroupSubs; ++i) m = fmax(m, sm.amax[i][lane]);
+        const long at = (long)((b0 + kSub * sub) / kGroup) * N + n;
+        if constexpr (MX) {
+          int x = m > 0.0 ? ilogb(m) - 2 : -127;
+          x = max(-127, min(125, x));
+          s = scalbn(1.0, x);
+          inv = scalbn(1.0, -x);
+          if (n < N) static_cast<uint8_t*>(scales_out)[at] = (uint8_t)(x + 127);
+        } else {
+          const float s32 = (float)(m / 7.0);  // FP64 quotient rounded once to FP32
+          if (n < N) static_cast<float*>(scales_out)[at] = s32;
+          s = (double)s32;
+          inv = s > 0.0 ? 1.0 / s : 0.0;
+          safe = s * (0.5 - 1e-9);
+        }
+      }
+      double w[kSub];
+      float w0[kSub];
+#pragma unroll
+      for (int i = 0; i < kSub; ++i) {
+        w0[i] = live(kSub * sub + i, next_w0[i]);
+        w[i] = (double)w0[i] + sm.t[sweep_t(kSub * sub + i, lane)];
+      }
+      if (sub + 1 < subs) {
+#pragma unroll
+        for (int i = 0; i < kSub; ++i) next_w0[i] = original(kSub * (sub + 1) + i, n);
+      }
+      if (!entry) {   // the previous eight's z, which the other warps apply further on
+#pragma unroll
+        for (int k = 0; k < kSub; ++k)
+#pragma unroll
+          for (int i = 0; i < kSub; ++i) w[i] = fma(z[k], sm.ud[(sub - 1) & 3][k][kSub + i], w[i]);
+      }
+      const double(*ud)[2 * kSub] = sm.ud[sub & 3];
+#pragma unroll
+      for (int k = 0; k < kSub; ++k) {
+        int code;
+        if constexpr (MX) {
+          const double v = fmin(fabs(w[k]) * inv, 6.0);  // exact: the scale is a power of two
+          // one comparison per midpoint between neighbouring magnitudes, strict where the lower neighbour is the even code
+          const int idx = (v > 0.25) + (v >= 0.75) + (v > 1.25) + (v >= 1.75) + (v > 2.5) + (v >= 3.5) + (v > 5.0);
+          const double twice = __hiloint2double(0x43300000, (0xC8643210u >> (4 * idx)) & 15u) - 4503599627370496.0;
+          z[k] = fma(w[k] < 0.0 ? 0.5 * twice : -0.5 * twice, s, (double)w0[k]);
+          code = idx + (w[k] < 0.0 ? 8 : 0);
+        } else {
+          const double q = quantize_int4(w[k], s, inv, safe);
+          z[k] = fma(-q, s, (double)w0[k]);
+          code = (int)q;
+        }
+#pragma unroll
+        for (int i = k + 1; i < kSub; ++i) w[i] = fma(z[k], ud[k][i], w[i]);
+        const int row = b0 + kSub * sub + k;
+        if (n < N) {
+          if constexpr (MX) static_cast<uint8_t*>(codes_out)[(long)row * N + n] = (uint8_t)code;
+          else static_cast<int8_t*>(codes_out)[(long)row * N + n] = (int8_t)code;
+        }
+        sm.z[sub & 1][k][lane ^ ((k & 3) << 2)] = z[k];
+        Z[(long)(kSub * sub + k) * ldw + n] = z[k];
+      }
+      async_wait<0>();
+    } else {
+      fetch_u(sub, 32, kSweepThreads - 32);
+      async_commit();
+      if (!entry) apply(sub - 1, sub + warp, kSweepThreads / 32 - 1);
+      async_wait<0>();
+    }
+    __syncthreads();
   }
 }
 
 // The temporaries of one call, carved out of one workspace (256-byte aligned pieces).
 struct Workspace {
-  double *H, *U, *Xd, *W, *Err, *T, *mean;
+  double *H, *L, *G, *Xd, *T, *Z, *damp;
   unsigned char* dead;
   int* not_pd;
+  int ldw;
   size_t bytes;
+  static size_t padded_tokens(int M_cal) { return ((size_t)M_cal + kBK - 1) / kBK * kBK; }   // whole slices of the product
   Workspace(unsigned char* base, int K, int N, int M_cal) {
     size_t off = 0;
     auto take = [&](size_t n) {
@@ -377,32 +612,17 @@ struct Workspace {
       return p;
     };
     const size_t kk = (size_t)K * K * sizeof(double);
+    G = reinterpret_cast<double*>(take((size_t)K * kNb * sizeof(double)));
+    ldw = (N + kNb - 1) / kNb * kNb;   // rows of T and Z padded to whole tiles
     H = reinterpret_cast<double*>(take(kk));
-    U = reinterpret_cast<double*>(take(kk));
-    W = reinterpret_cast<double*>(take((size_t)K * N * sizeof(double)));
-    Err = reinterpret_cast<double*>(take((size_t)2 * kLazy * N * sizeof(double)));  // two error batches
-    T = reinterpret_cast<double*>(take((size_t)kBand * K * sizeof(double)));
-    Xd = reinterpret_cast<double*>(take((size_t)M_cal * K * sizeof(double)));
-    mean = reinterpret_cast<double*>(take(sizeof(double)));
+    L = reinterpret_cast<double*>(take(kk));
+    T = reinterpret_cast<double*>(take((size_t)K * ldw * sizeof(double)));
+    Z = reinterpret_cast<double*>(take((size_t)kLazy * ldw * sizeof(double)));
+    Xd = reinterpret_cast<double*>(take(padded_tokens(M_cal) * K * sizeof(double)));
+    damp = reinterpret_cast<double*>(take(sizeof(double)));
     dead = take((size_t)K);
     not_pd = reinterpret_cast<int*>(take(sizeof(int)));
     bytes = off;
-  }
-};
-
-// The second stream of a call and the two events that order it against the caller's stream.
-struct SideStream {
-  cudaStream_t stream = nullptr;
-  cudaEvent_t ev_main = nullptr, ev_side = nullptr;
-  bool create() {
-    return cudaStreamCreateWithFlags(&stream, cudaStreamNonBlocking) == cudaSuccess &&
-           cudaEventCreateWithFlags(&ev_main, cudaEventDisableTiming) == cudaSuccess &&
-           cudaEventCreateWithFlags(&ev_side, cudaEventDisableTiming) == cudaSuccess;
-  }
-  ~SideStream() {
-    if (ev_main) cudaEventDestroy(ev_main);
-    if (ev_side) cudaEventDestroy(ev_side);
-    if (stream) cudaStreamDestroy(stream);
   }
 };
 
@@ -411,18 +631,32 @@ struct OwnedAllocation {
   ~OwnedAllocation() { cudaFree(p); }
 };
 
-void dgemm(cudaStream_t st, int M, int N, int Kd, const double* A, long sa_m, long sa_k, const double* B, long sb_k,
-           long sb_n, double* C, long sc_m, long sc_n, double alpha, double beta, int flags = 0) {
-  if (M <= 0 || N <= 0) return;
-  if (M > 64) {
-    dim3 grid((N + kBN - 1) / kBN, (M + 127) / 128);
-    dgemm_kernel<8><<<grid, 256, 0, st>>>(M, N, Kd, A, sa_m, sa_k, B, sb_k, sb_n, C, sc_m, sc_n, alpha, beta, flags);
-  } else {
-    dim3 grid((N + kBN - 1) / kBN, 1);
-    dgemm_kernel<4><<<grid, 256, 0, st>>>(M, N, Kd, A, sa_m, sa_k, B, sb_k, sb_n, C, sc_m, sc_n, alpha, beta, flags);
-  }
+template <int BM, bool AK, bool BK>
+void launch_dgemm(cudaStream_t st, const GemmArgs& g) {
+  static_assert(dgemm_smem_bytes(BM) <= 113 * 1024, "two blocks per SM");
+  const dim3 grid(g.N / kBN, (g.M + BM - 1) / BM);
+  dgemm_kernel<BM, AK, BK><<<grid, 256, dgemm_smem_bytes(BM), st>>>(g);
 }
-
+// 128-row tiles where they fill the SMs; 64-row tiles (twice the blocks, 4/3 of the operand traffic) where they would not.
+template <bool AK, bool BK>
+void dgemm(cudaStream_t st, const GemmArgs& g) {
+  if (g.M <= 0 || g.N <= 0 || g.Kd <= 0) return;
+  const long blocks = (long)(g.N / kBN) * ((g.M + 127) / 128);
+  if (g.M > 64 && blocks >= 148) launch_dgemm<128, AK, BK>(st, g);
+  else launch_dgemm<64, AK, BK>(st, g);
+}
+template <bool AK, bool BK>
+bool prepare_dgemm() {
+  return cudaFuncSetAttribute(dgemm_kernel<128, AK, BK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dgemm_smem_bytes(128)) == cudaSuccess &&
+         cudaFuncSetAttribute(dgemm_kernel<64, AK, BK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dgemm_smem_bytes(64)) == cudaSuccess;
+}
+// Shared-memory limits of this file's kernels on the current device.
+bool prepare_kernels() {
+  return prepare_dgemm<false, false>() && prepare_dgemm<true, true>() &&
+         cudaFuncSetAttribute(chol_step_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCholSmemBytes) == cudaSuccess &&
+         cudaFuncSetAttribute(gptq_sweep_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SweepSmem)) == cudaSuccess &&
+         cudaFuncSetAttribute(gptq_sweep_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SweepSmem)) == cudaSuccess;
+}
 
 bool gptq_shape_ok(int K, int N, int M_cal) {
   return K > 0 && N > 0 && K % kNb == 0 && K <= 16384 && N <= 65536 && M_cal >= 0 && M_cal <= (1 << 20);
@@ -437,6 +671,13 @@ extern "C" size_t w4a4_gptq_workspace_bytes(int K, int N, int M_cal) {
 
 namespace {
 
+// H (upper tiles) = beta H + X^T X, X [rows, K] in FP64, rows a multiple of kBK.
+void statistic(cudaStream_t st, const double* X, int rows, int K, double* H, double beta) {
+  GemmArgs g{K, K, rows, X, K, X, K, H, K, 1.0, beta};
+  g.upper_out = true;
+  dgemm<false, false>(st, g);
+}
+
 w4a4_status_t gptq_run(bool mx, int device, const float* R, const uint16_t* Xhat, int M_cal, const double* H_in, int K,
                        int N, double percdamp, void* codes, void* scales, void* workspace, size_t workspace_bytes,
                        void* stream) {
@@ -450,9 +691,9 @@ w4a4_status_t gptq_run(bool mx, int device, const float* R, const uint16_t* Xhat
   if (workspace != nullptr && (workspace_bytes < need || (reinterpret_cast<uintptr_t>(workspace) & 255) != 0))
     return W4A4_ERR_INVALID_ARG;
   if (cudaSetDevice(device) != cudaSuccess) return W4A4_ERR_CUDA;
-  cudaDeviceProp prop;
-  if (cudaGetDeviceProperties(&prop, device) != cudaSuccess) return W4A4_ERR_CUDA;
-  if (prop.major != 10) return W4A4_ERR_ARCH;
+  int major = 0;   // (one attribute: the whole property record takes the driver milliseconds)
+  if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, device) != cudaSuccess) return W4A4_ERR_CUDA;
+  if (major != 10) return W4A4_ERR_ARCH;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
 
   OwnedAllocation own;
@@ -464,107 +705,57 @@ w4a4_status_t gptq_run(bool mx, int device, const float* R, const uint16_t* Xhat
     workspace = own.p;
   }
   const Workspace d(static_cast<unsigned char*>(workspace), K, N, M_cal);
-  SideStream side;
-  if (!side.create()) {
+  if (!prepare_kernels()) {
     cudaGetLastError();
     return W4A4_ERR_CUDA;
   }
   const size_t kk = (size_t)K * K * sizeof(double);
   cudaMemsetAsync(d.not_pd, 0, sizeof(int), st);
-  cudaMemsetAsync(d.U, 0, kk, st);
 
   // 1. H, its dead channels and damping.
   if (Xhat != nullptr) {
-    const long n = (long)M_cal * K;
-    bf16_to_f64_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(Xhat, d.Xd, n);
-    cudaMemsetAsync(d.H, 0, kk, st);
-    dgemm(st, K, K, M_cal, d.Xd, 1, K, d.Xd, K, 1, d.H, K, 1, 1.0, 0.0, kUpperOut);
+    const long n = (long)M_cal * K, padded = (long)Workspace::padded_tokens(M_cal) * K;
+    bf16_to_f64_kernel<<<(unsigned)((padded / 2 + 255) / 256), 256, 0, st>>>(Xhat, reinterpret_cast<double2*>(d.Xd), n, padded);
+    statistic(st, d.Xd, (int)(padded / K), K, d.H, 0.0);
   } else {
     cudaMemcpyAsync(d.H, H_in, kk, cudaMemcpyDeviceToDevice, st);
   }
-  gptq_diag_mean_kernel<<<1, 256, 0, st>>>(d.H, K, d.dead, d.mean);
-  gptq_damp_kernel<<<(K + 255) / 256, 256, 0, st>>>(d.H, K, d.mean, percdamp);
-  {
-    const long n = (long)K * N;
-    gptq_init_w_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(R, d.dead, d.W, K, N);
-  }
+  gptq_diag_kernel<<<1, 1024, 0, st>>>(d.H, K, percdamp, d.dead, d.damp);
 
-  // 2. H = V V^T in place (main stream) and U = V^-1 (side stream), band by band from the last channels.
-  // Factorization: inside a band of kBand columns every 64-column block is factored, solved against all rows above
-  // it and applied to the band's columns still to come; the columns to the left of the band then take the whole
-  // band's panels in one product that is kBand deep.  Rows lo..hi of V are final once the band's blocks are done (the
-  // product that follows only touches rows and columns below lo), so the side stream inverts that band meanwhile:
-  // the diagonal part block by block (U[i, rest] = -inv(V_ii) (V[i, rest] U[rest, rest]), 64-row products), the
-  // part to the right of it in two products that are kBand rows high.  The factorization's chain of small kernels
-  // and the inverse's large products overlap.
-  cudaEventRecord(side.ev_main, st);  // U is zeroed
-  cudaStreamWaitEvent(side.stream, side.ev_main, 0);
+  // 2. H = V V^T, band by band from the last channels: inside a band of kBand columns every 64-column block is factored,
+  // solved against all rows above it and applied to the band's columns still to come; the columns to the left of the band
+  // then take the whole band's panels in one product that is kBand deep.
   for (int hi = K; hi > 0;) {
     const int lo = hi - kBand > 0 ? hi - kBand : 0;
     for (int j0 = hi - kNb; j0 >= lo; j0 -= kNb) {
-      chol_diag_kernel<<<1, kDiagThreads, 0, st>>>(d.H, K, j0, d.not_pd);
-      if (j0 == 0) break;
-      chol_panel_kernel<<<(j0 + kNb - 1) / kNb, kNb, 0, st>>>(d.H, K, j0);
+      chol_step_kernel<<<j0 > 0 ? j0 / kNb : 1, kCholThreads, kCholSmemBytes, st>>>(d.H, d.L, K, j0, d.dead, d.damp, d.not_pd);
       // H[0:j0, lo:j0] -= P P[lo:j0]^T, P = the panel just solved
-      dgemm(st, j0, j0 - lo, kNb, d.H + j0, K, 1, d.H + (long)lo * K + j0, 1, K, d.H + lo, K, 1, -1.0, 1.0);
+      GemmArgs g{j0, j0 - lo, kNb, d.H + j0, K, d.H + (long)lo * K + j0, K, d.H + lo, K, -1.0, 1.0};
+      g.upper_out = true;
+      g.diag_shift = lo;
+      dgemm<true, true>(st, g);
     }
-    cudaEventRecord(side.ev_main, st);
-    // H[0:lo, 0:lo] -= P P^T over the band's panels (upper triangle only)
-    dgemm(st, lo, lo, hi - lo, d.H + lo, K, 1, d.H + lo, 1, K, d.H, K, 1, -1.0, 1.0, kUpperOut);
-
-    cudaStream_t s2 = side.stream;
-    cudaStreamWaitEvent(s2, side.ev_main, 0);
-    triinv_diag_kernel<<<(hi - lo) / kNb, kNb, 0, s2>>>(d.H, d.U, K, lo);
-    for (int i0 = hi - 2 * kNb; i0 >= lo; i0 -= kNb) {
-      const int r0 = i0 + kNb, rest = hi - r0;
-      dgemm(s2, kNb, rest, rest, d.H + (long)i0 * K + r0, K, 1, d.U + (long)r0 * K + r0, K, 1, d.T, K, 1, 1.0, 0.0,
-            kBUpper);
-      dgemm(s2, kNb, rest, kNb, d.U + (long)i0 * K + i0, K, 1, d.T, K, 1, d.U + (long)i0 * K + r0, K, 1, -1.0, 0.0);
-    }
-    const int band = hi - lo, right = K - hi;
-    if (right > 0) {
-      dgemm(s2, band, right, right, d.H + (long)lo * K + hi, K, 1, d.U + (long)hi * K + hi, K, 1, d.T, K, 1, 1.0, 0.0,
-            kBUpper);
-      dgemm(s2, band, right, band, d.U + (long)lo * K + lo, K, 1, d.T, K, 1, d.U + (long)lo * K + hi, K, 1, -1.0, 0.0,
-            kAUpper);
-    }
+    // H[0:lo, 0:lo] -= P P^T over the band's panels
+    GemmArgs far{lo, lo, hi - lo, d.H + lo, K, d.H + lo, K, d.H, K, -1.0, 1.0};
+    far.upper_out = true;
+    dgemm<true, true>(st, far);
     hi = lo;
   }
-  cudaEventRecord(side.ev_side, side.stream);
-  cudaStreamWaitEvent(st, side.ev_side, 0);  // U is complete
 
-  // 3. The sweep, group by group.  Inside a lazy batch of kLazy input channels each group's scaled errors update the
-  // batch's groups still to come.  The channels after the batch take the whole batch in one product, W[later] -=
-  // U[batch, later]^T Err, split in two: the next batch's channels on the main stream, the rest on the side stream
-  // while the next batch is swept.  Both touch the same rows as the next batch's own products, so each main-stream
-  // product first waits for the side stream's previous one; the error batches alternate between two buffers.
-  int batch = 0;
-  for (int b0 = 0; b0 < K; b0 += kLazy, ++batch) {
+  // 3. The sweep, one lazy batch of kLazy input channels per launch, and after each T[later] += L[batch, later]^T Z.
+  unit_inverse_kernel<<<K / kNb, kNb, 0, st>>>(d.L, d.G, K);
+  const int ldw = d.ldw;
+  for (int b0 = 0; b0 < K; b0 += kLazy) {
     const int b1 = b0 + kLazy < K ? b0 + kLazy : K;
-    double* err_batch = d.Err + (long)(batch & 1) * kLazy * N;
-    for (int k0 = b0; k0 < b1; k0 += kNb) {
-      double* err = err_batch + (long)(k0 - b0) * N;
-      const dim3 grid((N + kGroupCols - 1) / kGroupCols);
-      if (mx) gptq_group_kernel<true><<<grid, 2 * kGroupCols, 0, st>>>(d.W, N, d.U, K, k0, codes, scales, err);
-      else gptq_group_kernel<false><<<grid, 2 * kGroupCols, 0, st>>>(d.W, N, d.U, K, k0, codes, scales, err);
-      const int r0 = k0 + kNb;
-      dgemm(st, b1 - r0, N, kNb, d.U + (long)k0 * K + r0, 1, K, err, N, 1, d.W + (long)r0 * N, N, 1, -1.0, 1.0);
-    }
-    if (b1 == K) break;
-    const int b2 = b1 + kLazy < K ? b1 + kLazy : K;  // end of the next batch
-    cudaStreamWaitEvent(st, side.ev_side, 0);        // the side stream's product of the batch before
-    dgemm(st, b2 - b1, N, b1 - b0, d.U + (long)b0 * K + b1, 1, K, err_batch, N, 1, d.W + (long)b1 * N, N, 1, -1.0, 1.0);
-    cudaEventRecord(side.ev_main, st);
-    cudaStreamWaitEvent(side.stream, side.ev_main, 0);
-    dgemm(side.stream, K - b2, N, b1 - b0, d.U + (long)b0 * K + b2, 1, K, err_batch, N, 1, d.W + (long)b2 * N, N, 1,
-          -1.0, 1.0);
-    cudaEventRecord(side.ev_side, side.stream);
+    const unsigned blocks = (unsigned)(ldw / kSweepCols);
+    if (mx) gptq_sweep_kernel<true><<<blocks, kSweepThreads, sizeof(SweepSmem), st>>>(R, d.dead, d.T, ldw, N, d.L, K, d.G, b0, b1 - b0, codes, scales, d.Z);
+    else gptq_sweep_kernel<false><<<blocks, kSweepThreads, sizeof(SweepSmem), st>>>(R, d.dead, d.T, ldw, N, d.L, K, d.G, b0, b1 - b0, codes, scales, d.Z);
+    dgemm<false, false>(st, {K - b1, ldw, b1 - b0, d.L + (long)b0 * K + b1, K, d.Z, ldw, d.T + (long)b1 * ldw, ldw, 1.0, b0 > 0 ? 1.0 : 0.0});
   }
-  cudaStreamWaitEvent(st, side.ev_side, 0);
 
   int not_pd = 0;
   if (cudaMemcpyAsync(&not_pd, d.not_pd, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-      cudaStreamSynchronize(st) != cudaSuccess || cudaStreamSynchronize(side.stream) != cudaSuccess ||
+      cudaStreamSynchronize(st) != cudaSuccess ||
       cudaGetLastError() != cudaSuccess)
     return W4A4_ERR_CUDA;
   return not_pd ? W4A4_ERR_INVALID_ARG : W4A4_OK;
@@ -577,23 +768,24 @@ extern "C" w4a4_status_t w4a4_gptq_accumulate(int device, const uint16_t* Xhat, 
   if (Xhat == nullptr || H == nullptr) return W4A4_ERR_INVALID_ARG;
   if (!gptq_shape_ok(K, 1, M_cal) || M_cal <= 0) return W4A4_ERR_SHAPE;
   if (cudaSetDevice(device) != cudaSuccess) return W4A4_ERR_CUDA;
-  cudaDeviceProp prop;
-  if (cudaGetDeviceProperties(&prop, device) != cudaSuccess) return W4A4_ERR_CUDA;
-  if (prop.major != 10) return W4A4_ERR_ARCH;
+  int major = 0;   // (one attribute: the whole property record takes the driver milliseconds)
+  if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, device) != cudaSuccess) return W4A4_ERR_CUDA;
+  if (major != 10) return W4A4_ERR_ARCH;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   constexpr int kChunkRows = 4096;  // tokens converted to FP64 at a time
   const int chunk = M_cal < kChunkRows ? M_cal : kChunkRows;
   OwnedAllocation xd;
-  if (cudaMalloc(&xd.p, (size_t)chunk * K * sizeof(double)) != cudaSuccess) {
+  if (cudaMalloc(&xd.p, Workspace::padded_tokens(chunk) * K * sizeof(double)) != cudaSuccess) {
     cudaGetLastError();
     return W4A4_ERR_ALLOC;
   }
+  if (!prepare_kernels()) return W4A4_ERR_CUDA;
   double* Xd = static_cast<double*>(xd.p);
   for (int m0 = 0; m0 < M_cal; m0 += chunk) {
     const int rows = M_cal - m0 < chunk ? M_cal - m0 : chunk;
-    const long n = (long)rows * K;
-    bf16_to_f64_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(Xhat + (size_t)m0 * K, Xd, n);
-    dgemm(st, K, K, rows, Xd, 1, K, Xd, K, 1, H, K, 1, 1.0, 1.0, kUpperOut);
+    const long n = (long)rows * K, padded = (long)Workspace::padded_tokens(rows) * K;
+    bf16_to_f64_kernel<<<(unsigned)((padded / 2 + 255) / 256), 256, 0, st>>>(Xhat + (size_t)m0 * K, reinterpret_cast<double2*>(Xd), n, padded);
+    statistic(st, Xd, (int)(padded / K), K, H, 1.0);
   }
   if (cudaStreamSynchronize(st) != cudaSuccess || cudaGetLastError() != cudaSuccess) return W4A4_ERR_CUDA;
   return W4A4_OK;

@@ -275,3 +275,26 @@ def test_statistic_accumulated_over_batches():
     R64 = R.double().numpy()
     q_ref, s_ref = oracle.gptq_quantize(R64, H_ref)
     compare(R64, H_ref, codes.cpu().numpy(), scales.cpu().numpy(), q_ref, s_ref, max_bad_columns=1)
+
+
+@pytest.mark.parametrize("K,N,M_cal,mx,offset", [
+    (64, 1, 1, True, 0),           # one group, one output channel, one token (padded to a slice of the product)
+    (192, 63, 17, False, 1),       # a band and a lazy batch of their own size; statistic on an 8-byte boundary
+    (576, 65, 33, True, 1),        # one 64-column block past a band, one output channel past a tile
+    (832, 129, 15, False, 0),
+])
+def test_tile_edges(K, N, M_cal, mx, offset):
+    # Against the oracle on the statistic that the library accumulates (compared itself: FP64 sums of M_cal products).
+    import paper_2605_27003_b200 as w4
+    R, x = gen.make_gptq_inputs(K, N, M_cal, seed=K + N)
+    H = torch.zeros(K * K + 1, dtype=torch.float64, device=DEV)[offset:offset + K * K].view(K, K)
+    w4.w4a4_gptq_accumulate(x.to(DEV), H)
+    H_ref = oracle.gptq_hessian(bits(x))
+    iu = np.triu_indices(K)
+    assert np.abs(H.cpu().numpy()[iu] - H_ref[iu]).max() <= M_cal * 2.0 ** -52 * np.abs(H_ref).max()
+    codes = torch.empty((K, N), dtype=torch.uint8 if mx else torch.int8, device=DEV)
+    scales = torch.empty((K // (32 if mx else 64), N), dtype=torch.uint8 if mx else torch.float32, device=DEV)
+    (w4.w4a4_mx_gptq_quantize if mx else w4.w4a4_gptq_quantize)(R.to(DEV), codes, scales, H=H, percdamp=0.05)
+    q_ref, s_ref = (oracle.gptq_quantize_mx if mx else oracle.gptq_quantize)(R.double().numpy(), H_ref, percdamp=0.05)
+    bad = (codes.cpu().numpy() != q_ref).any(axis=0) | (scales.cpu().numpy() != s_ref).any(axis=0)
+    assert bad.sum() <= max(1, N // 200), f"{bad.sum()} output channels differ"
