@@ -51,6 +51,10 @@
 // Tile order: column tiles are walked in super-columns (GemmParams::order, all row blocks of a
 // super-column before the next) sized so that the weight bytes a wave of CTAs touches stay in L2; with the plain
 // row-major order the 71 MB weight image of the FFN shapes streamed from DRAM once per 1.4 row blocks.
+// Split K (SPLIT instantiation): where the tiles alone leave most SMs idle, the CTAs of a thread-block cluster share one
+// tile, each over its part of the operand stages (the first one with the low-rank product).  Their FP32 partial tiles meet
+// in shared memory (the operand ring's, idle by then), and every CTA adds its share of them over distributed shared
+// memory in split order, so results do not depend on timing.  One tile per CTA, no loop.
 // Every role loops warp-uniformly (waits are voted, only the TMA / tcgen05 instructions are predicated on one elected
 // lane), which keeps ring positions, addresses and descriptors in uniform registers.  All waits are bounded
 // (pipeline.cuh).  Finally + bias -> optional GELU -> BF16, or the squared error against a reference (clip search).
@@ -230,7 +234,7 @@ __global__ void sop_weight_kernel(const float* __restrict__ wscale, uint4* __res
   out[image * 256 + (g & 1) * 128 + ((n & 127) >> 3) * 8 + (n & 7)] = (g & 1) ? make_uint4(0u, 0u, w, w) : make_uint4(w, w, 0u, 0u);
 }
 
-template <bool DEBUG>
+template <bool DEBUG, bool SPLIT>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                  const __grid_constant__ CUtensorMap tmT, const __grid_constant__ CUtensorMap tmL2,
@@ -253,8 +257,14 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;  // provably warp-uniform
   const int G = p.K >> 6;
   const int n_int_stages = (G + 1) >> 1;
-  const int n_lr_stages = p.r > 0 ? (2 * p.r + 63) / 64 : 0;
+  const int n_lr_stages = p.r > 0 && (!SPLIT || cluster_ctarank() == 0) ? (2 * p.r + 63) / 64 : 0;
   const int num_tiles = p.tiles_m * p.tiles_n;
+  // This CTA's tiles and operand stages (all of them unless K is split).
+  const int split = SPLIT ? static_cast<int>(cluster_ctarank()) : 0;
+  const int first_tile = SPLIT ? blockIdx.x / p.splits : blockIdx.x, tile_step = SPLIT ? num_tiles : gridDim.x;
+  const int st_begin = SPLIT ? n_int_stages * split / p.splits : 0;
+  const int st_end = SPLIT ? n_int_stages * (split + 1) / p.splits : n_int_stages;
+  const int g_begin = SPLIT ? 2 * st_begin : 0, g_end = SPLIT ? min(G, 2 * st_end) : G;
   const WaitEnv env{p.err, s_abort, p.wait_limit_ns};
 
   if (threadIdx.x == 0) {
@@ -304,11 +314,11 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       Ring<kGemmStages> op;
       bool ok = true;
       int stage_no = 0;
-      for (int tile = blockIdx.x; ok && tile < num_tiles; tile += gridDim.x) {
+      for (int tile = first_tile; ok && tile < num_tiles; tile += tile_step) {
         int tm, tn;
         tile_coords(tile, p.order, tm, tn);
         const int m0 = tm * kBM, n0 = tn * kBN;
-        for (int st = 0; st < n_lr_stages + n_int_stages; ++st) {
+        for (int st = 0; st < n_lr_stages + st_end - st_begin; ++st) {
           ok = __all_sync(0xffffffffu, bounded_wait<64>(bar_op_empty + 8 * op.slot, op.parity ^ 1u, env, kErrProducerWait));
           if (!ok) break;
           if (DEBUG) {
@@ -328,7 +338,7 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
               tma_load_2d(dst + kOpATile, &tmL2, full, st * 64, n0);
             }
           } else if (issuer) {
-            const int ks = st - n_lr_stages;
+            const int ks = st - n_lr_stages + st_begin;
             const uint32_t sop = dst + kOpATile + kOpBTile;
             mbar_arrive_expect_tx(full, kStageBytes);
             tma_load_2d(dst, &tmA, full, ks * kBK, m0);
@@ -352,7 +362,7 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       Ring<kGemmStages> op;
       Ring<kTmemSlots> tm;
       bool ok = true;
-      for (int tile = blockIdx.x; ok && tile < num_tiles; tile += gridDim.x) {
+      for (int tile = first_tile; ok && tile < num_tiles; tile += tile_step) {
         if (n_lr_stages > 0) {
           ok = __all_sync(0xffffffffu, bounded_wait<0, 1>(bar_tmem_empty + 8 * tm.slot, tm.parity ^ 1u, env, kErrMmaWait));
           if (ok) tc_fence_after_sync();
@@ -374,7 +384,7 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           if (!ok) break;
           if (issuer) umma_commit(full_bar);
         }
-        for (int st = 0; ok && st < n_int_stages; ++st) {
+        for (int st = st_begin; ok && st < st_end; ++st) {
           ok = __all_sync(0xffffffffu, bounded_wait<0, 1>(bar_op_full + 8 * op.slot, op.parity, env, kErrMmaWait));
           if (!ok) break;
           const uint32_t a = smem_base + op.slot * kStageBytes, b = a + kOpATile;
@@ -410,7 +420,7 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       Ring<kGemmStages> op;
       Ring<kTmemSlots> tm;
       bool ok = true;
-      for (int tile = blockIdx.x; ok && tile < num_tiles; tile += gridDim.x) {
+      for (int tile = first_tile; ok && tile < num_tiles; tile += tile_step) {
         if (n_lr_stages > 0) {
           ok = __all_sync(0xffffffffu, bounded_wait<0, 1>(bar_tmem_empty + 8 * tm.slot, tm.parity ^ 1u, env, kErrMmaWait));
           if (!ok) break;
@@ -425,7 +435,7 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           }
           if (!ok) break;
         }
-        for (int st = 0; ok && st < n_int_stages; ++st) {
+        for (int st = st_begin; ok && st < st_end; ++st) {
           ok = __all_sync(0xffffffffu, bounded_wait<0, 1>(bar_op_full + 8 * op.slot, op.parity, env, kErrMmaWait));
           if (!ok) break;
           const uint32_t sa = smem_base + op.slot * kStageBytes + kOpATile + kOpBTile, sb = sa + kSopATile;
@@ -462,7 +472,7 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       const uint32_t out_tile = out_base + kOutTile * ew;
       SlotUse use;
       bool ok = true;
-      for (int tile = blockIdx.x; ok && tile < num_tiles; tile += gridDim.x) {
+      for (int tile = first_tile; ok && tile < num_tiles; tile += tile_step) {
         int tm_e, tn_e;
         tile_coords(tile, p.order, tm_e, tn_e);
         const int m0 = tm_e * kBM, n0 = tn_e * kBN;
@@ -493,7 +503,7 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 #pragma unroll
           for (int j = 0; j < 16; ++j) acc[j] = make_float2(0.0f, 0.0f);
         }
-        for (int g = 0; g < G; ++g) {
+        for (int g = g_begin; g < g_end; ++g) {
           const uint32_t t = t_lane + use.slot() * 2 * kBN;
           uint32_t pv[16], sv[16];
           if (!__all_sync(0xffffffffu, wait_then_ld16(bar_tmem_full + 8 * use.slot(), use.parity(), t, pv) != 0)) {
@@ -523,6 +533,16 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           fma_fragment<DEBUG>(pv, sv, acc + 8, DEBUG && d0 ? d0 + 16 : nullptr);
         }
         if (!ok) break;
+        if constexpr (SPLIT) {
+          // Partial tile: 512-byte rows of FP32, 16-byte chunk c at c ^ (row % 8): conflict free for both sides.
+          const int row = 32 * quarter + lane;
+#pragma unroll
+          for (int c = 0; c < 8; ++c)
+            sts_u32x4(smem_base + 512 * row + 16 * ((8 * colblk + c) ^ (row & 7)),
+                      make_uint4(__float_as_uint(acc[2 * c].x), __float_as_uint(acc[2 * c].y), __float_as_uint(acc[2 * c + 1].x),
+                                 __float_as_uint(acc[2 * c + 1].y)));
+          break;
+        }
         // The tile's end: bias, activation, BF16, then through shared memory so that a warp's 16-byte accesses to Y (or to
         // the reference) cover eight rows x 64 bytes instead of 32 rows x 16.
         __syncwarp();
@@ -582,6 +602,44 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     }
   }
 
+  if constexpr (SPLIT) {
+    cluster_sync_all();   // all partial tiles are written
+    if (live && warp >= kEpiWarp0 && !*s_abort) {
+      int tm_e, tn_e;
+      tile_coords(first_tile, p.order, tm_e, tn_e);
+      float sq = 0.0f;
+      // A warp takes one row at a time, a lane four channels.
+      for (int row = 16 * split + warp - kEpiWarp0; row < kBM; row += 16 * p.splits) {
+        if (tm_e * kBM + row >= p.M) break;
+        const uint32_t at = smem_base + 512 * row + 16 * (lane ^ (row & 7));
+        float4 y = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        for (int i = 0; i < p.splits; ++i) {
+          const float4 v = ld_cluster_f32x4(map_to_cta(at, i));
+          y.x += v.x, y.y += v.y, y.z += v.z, y.w += v.w;
+        }
+        const int ch = tn_e * kBN + 4 * lane;
+        const float4 b = p.bias ? __ldg(reinterpret_cast<const float4*>(p.bias + ch)) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        y.x += b.x, y.y += b.y, y.z += b.z, y.w += b.w;
+        if (p.act != 0)
+          y = make_float4(apply_activation(y.x, p.act), apply_activation(y.y, p.act), apply_activation(y.z, p.act), apply_activation(y.w, p.act));
+        const uint2 o = make_uint2(bf16x2_bits(make_float2(y.x, y.y)), bf16x2_bits(make_float2(y.z, y.w)));
+        const size_t dst = static_cast<size_t>(tm_e * kBM + row) * p.N + ch;
+        if (p.yref == nullptr) {
+          *reinterpret_cast<uint2*>(p.Y + dst) = o;
+        } else {
+          const uint2 ref = __ldg(reinterpret_cast<const uint2*>(p.yref + dst));
+          sq = sq_diff_bf16x2(ref.x, o.x, sq);
+          sq = sq_diff_bf16x2(ref.y, o.y, sq);
+        }
+      }
+      if (p.yref != nullptr) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+        if (lane == 0) atomicAdd(p.sq_err, static_cast<double>(sq));
+      }
+    }
+    cluster_sync_all();   // nobody leaves while its shared memory is still being read
+  }
   // ---------------------------------------------------------------------- common tail
   tc_fence_before_sync();
   __syncthreads();

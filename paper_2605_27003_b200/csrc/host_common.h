@@ -34,6 +34,7 @@ struct w4a4_ctx {
   size_t bytes = 0;
   int num_sms = 0;
   size_t l2_bytes = 0;        // size of the device's L2 (sizes the GEMM's tile order)
+  int gemm_clusters[9] = {};  // clusters of that many CTAs of the INT4 GEMM that run at a time (index 2 .. 8)
   int debug_sc_tiles = 0;     // test hook: forced super-column width of the GEMM's tile order (0: automatic)
   EncodeTiledFn encode = nullptr;
   // Host-buffer forward (w4a4_linear_forward_host): staging buffers, copy streams and events.
@@ -94,6 +95,15 @@ struct OverlappedLaunch {
   }
   OverlappedLaunch(const OverlappedLaunch&) = delete;
 };
+
+constexpr int kMaxGemmSplits = 8;   // the portable cluster size
+// CTAs that share the K of one output tile: as many as still run all tiles at once, if each keeps `min_stages` of the tile's
+// operand stages.  `clusters[s]`: clusters of s CTAs that fit the device at a time (a cluster stays within one GPC).
+inline int gemm_k_splits(int tiles, int stages, int min_stages, const int* clusters) {
+  for (int s = kMaxGemmSplits; s > 1; --s)
+    if (tiles <= clusters[s] && stages / s >= min_stages) return s;
+  return 1;
+}
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 

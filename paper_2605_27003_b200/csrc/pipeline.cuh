@@ -147,6 +147,7 @@ struct GemmParams {
   int M, N, K, r;
   int tiles_m, tiles_n;
   TileOrder order;
+  int splits;           // CTAs of a cluster that share a tile's K (1: K is not split)
   int* err;
   uint64_t wait_limit_ns;
   int32_t* dbg_P;       // debug tap: [kBM, G, kBN] or nullptr

@@ -196,6 +196,11 @@ __device__ __forceinline__ float2 ld_cluster_f32x2(uint32_t cluster_addr) {
   asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(cluster_addr) : "memory");
   return v;
 }
+__device__ __forceinline__ float4 ld_cluster_f32x4(uint32_t cluster_addr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(cluster_addr) : "memory");
+  return v;
+}
 // Relaxed on purpose: the arrive only hands TMEM columns back (tcgen05.wait::ld has completed the reads, the
 // tcgen05 fence orders them); a release at cluster scope would also wait for the warp's earlier global stores
 // (the previous tile's outputs) to become visible, which cost about 1200 clocks per tile.

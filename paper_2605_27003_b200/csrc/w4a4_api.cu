@@ -288,10 +288,14 @@ w4a4_status_t launch_gemm(w4a4_handle_t h, int M, int expert_id, void* Y, cudaSt
   const dim3 grid(num_tiles < ctx->num_sms ? num_tiles : ctx->num_sms), block(kGemmThreads);
   const CUtensorMap& tmT = h->r > 0 ? h->tmT : h->tmA;   // unused when r == 0
   const CUtensorMap& tmL2 = h->r > 0 ? e.tmL2 : h->tmB;
-  const OverlappedLaunch l(grid, block, kGemmSmemBytes, stream);
+  // Few tiles: clusters of CTAs share a tile's K.  Four stages (eight groups) per CTA at least: the cluster's two barriers and
+  // the exchange cost about as much as six groups.
+  p.splits = stall_stage >= 0 ? 1 : gemm_k_splits(num_tiles, (h->K / 64 + 1) / 2, 4, ctx->gemm_clusters);
+  const OverlappedLaunch l(p.splits > 1 ? dim3(num_tiles * p.splits) : grid, block, kGemmSmemBytes, stream, dim3(p.splits));
   cudaError_t le;
-  if (dbg_P || stall_stage >= 0) le = cudaLaunchKernelEx(&l.cfg, gemm_w4a4_kernel<true>, h->tmA, h->tmB, tmT, tmL2, h->tmSopA, e.tmSopB, p);
-  else le = cudaLaunchKernelEx(&l.cfg, gemm_w4a4_kernel<false>, h->tmA, h->tmB, tmT, tmL2, h->tmSopA, e.tmSopB, p);
+  auto launch = [&](auto* kernel) { return cudaLaunchKernelEx(&l.cfg, kernel, h->tmA, h->tmB, tmT, tmL2, h->tmSopA, e.tmSopB, p); };
+  if (dbg_P || stall_stage >= 0) le = p.splits > 1 ? launch(gemm_w4a4_kernel<true, true>) : launch(gemm_w4a4_kernel<true, false>);
+  else le = p.splits > 1 ? launch(gemm_w4a4_kernel<false, true>) : launch(gemm_w4a4_kernel<false, false>);
   if (le != cudaSuccess) cudaGetLastError();
   return le == cudaSuccess ? W4A4_OK : W4A4_ERR_CUDA;
 }
@@ -374,13 +378,22 @@ w4a4_status_t w4a4_ctx_create(int device, int max_M, int max_K, int max_r, w4a4_
                          static_cast<int>(quantize_smem_bytes(64)));
     cudaFuncSetAttribute(quantize_kernel<96, quantize_warps(96), kCodesE4M3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          static_cast<int>(quantize_smem_bytes(96)));
-    const cudaError_t e1 = cudaFuncSetAttribute(gemm_w4a4_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmemBytes);
-    const cudaError_t e2 = cudaFuncSetAttribute(gemm_w4a4_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmemBytes);
-    // The kernel redistributes its launch's registers: it must have been compiled with as many as it hands out.
-    cudaFuncAttributes a1, a2;
-    const bool regs_ok = cudaFuncGetAttributes(&a1, gemm_w4a4_kernel<false>) == cudaSuccess && a1.numRegs == kGemmRegs &&
-                         cudaFuncGetAttributes(&a2, gemm_w4a4_kernel<true>) == cudaSuccess && a2.numRegs == kGemmRegs;
-    if (e1 != cudaSuccess || e2 != cudaSuccess || !regs_ok) {
+    // The GEMM redistributes its launch's registers: it must have been compiled with as many as it hands out.
+    auto prepare_gemm = [](auto* kernel) {
+      cudaFuncAttributes a;
+      return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmemBytes) == cudaSuccess &&
+             cudaFuncGetAttributes(&a, kernel) == cudaSuccess && a.numRegs == kGemmRegs;
+    };
+    const bool gemm_ok = prepare_gemm(gemm_w4a4_kernel<false, false>) && prepare_gemm(gemm_w4a4_kernel<true, false>) &&
+                         prepare_gemm(gemm_w4a4_kernel<false, true>) && prepare_gemm(gemm_w4a4_kernel<true, true>);
+    for (int s = 2; s <= kMaxGemmSplits; ++s) {
+      const OverlappedLaunch l(dim3(s), dim3(kGemmThreads), kGemmSmemBytes, nullptr, dim3(s));
+      if (cudaOccupancyMaxActiveClusters(&ctx->gemm_clusters[s], gemm_w4a4_kernel<false, true>, &l.cfg) != cudaSuccess) {
+        cudaGetLastError();
+        ctx->gemm_clusters[s] = 0;
+      }
+    }
+    if (!gemm_ok) {
       cudaGetLastError();
       st = W4A4_ERR_CUDA;
     }

@@ -414,3 +414,40 @@ def test_qkv_packed_as_one_layer_shares_one_activation_pass(M, K, N, r):
     bound = 2.0 ** -7 * np.abs(Y64) + 1e-3 * np.sqrt(np.mean(Y64 ** 2))
     assert np.all(np.abs(Yp - Y64) <= bound) and np.all(np.abs(Ys - Y64) <= bound)
     assert np.mean(Yp == Ys) > 0.9                 # nearly always the same BF16 value
+
+
+@pytest.mark.parametrize("M,K,N,r", [
+    (1, 1024, 128, 16),      # one token, one tile, eight operand stages: two CTAs share it
+    (129, 4160, 256, 0),     # 65 groups: the last stage holds one; two row blocks, the second with one row
+    (100, 2048, 640, 96),    # three low-rank stages, all with the first CTA of the cluster
+    (300, 1984, 384, 64),    # 31 groups, rows past M in the last row block
+])
+def test_tiles_shared_by_a_cluster(M, K, N, r):
+    # Few output tiles: the CTAs of a cluster split K.  Output and the partial sums of the last tile against the oracle.
+    idx = gen.outlier_channels(K, 0, 5, count=4)
+    x = gen.make_activations(M, K, outlier_idx=idx, outlier_gain=40.0, seed=M)
+    layer = gen.make_layer_direct(K, N, r, seed=K)
+    clip = torch.full((1, 1, 1), 0.85, dtype=torch.float32)
+    bm, bn = w4.w4a4_tile_shape()
+    run_case(x, [layer], clip, 0, 0, check_partials_tiles=[((M - 1) // bm * bm, N - bn)])
+
+
+def test_shared_tiles_in_the_clip_search():
+    # The squared error of a cluster's tile: against the forward's own output, summed in FP64.  Both round to BF16 alike;
+    # the library sums FP32 within a warp (128 terms per row: 128 * 2^-24).
+    M, K, N, r = 130, 1088, 256, 32
+    x = gen.make_activations(M, K, seed=3).to(DEV)
+    layer = gen.make_layer_direct(K, N, r, seed=4)
+    ctx = w4.Context(0, M, K, r)
+    L = w4.Layer(ctx, [layer.to(DEV)], num_bins=1)
+    yref = gen.reference_output(x.cpu(), layer).to(DEV)
+    table = torch.full((1, 1, 1), 1.0, device=DEV)
+    cands = [0.7, 1.0]
+    _, errs = w4.w4a4_clip_search(L.ptr, [x], [yref], M, 0, 0, cands, table)
+    for c, e in zip(cands, errs):
+        table.fill_(c)
+        y = L.forward(x, 0, 0, table)
+        ref = (yref.double() - y.double()).pow(2).sum().item()
+        assert abs(e - ref) <= 128 * 2.0 ** -24 * ref
+    L.close()
+    ctx.close()
