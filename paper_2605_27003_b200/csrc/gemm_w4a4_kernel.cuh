@@ -202,18 +202,6 @@ __device__ __forceinline__ void fma_fragment(const uint32_t (&pv)[16], const uin
   }
 }
 
-__device__ __forceinline__ uint32_t bf16x2_bits(float2 v) {
-  const __nv_bfloat162 b = __floats2bfloat162_rn(v.x, v.y);
-  return *reinterpret_cast<const uint32_t*>(&b);
-}
-
-// acc + (a0 - b0)^2 + (a1 - b1)^2 for two pairs of BF16 values.
-__device__ __forceinline__ float sq_diff_bf16x2(uint32_t a, uint32_t b, float acc) {
-  const float d0 = __uint_as_float(a << 16) - __uint_as_float(b << 16);
-  const float d1 = __uint_as_float(a & 0xffff0000u) - __uint_as_float(b & 0xffff0000u);
-  return fmaf(d1, d1, fmaf(d0, d0, acc));
-}
-
 // One scale as two BF16 pieces: s = h + m up to 2^-16 relative.
 __device__ __forceinline__ uint32_t scale_pieces(float s) {
   const __nv_bfloat16 h = __float2bfloat16_rn(s);

@@ -35,6 +35,7 @@ struct w4a4_ctx {
   int num_sms = 0;
   size_t l2_bytes = 0;        // size of the device's L2 (sizes the GEMM's tile order)
   int gemm_clusters[9] = {};  // clusters of that many CTAs of the INT4 GEMM that run at a time (index 2 .. 8)
+  int mx_gemm_clusters[9] = {};   // the same for the MXFP4 variant's single-CTA GEMM
   int debug_sc_tiles = 0;     // test hook: forced super-column width of the GEMM's tile order (0: automatic)
   EncodeTiledFn encode = nullptr;
   // Host-buffer forward (w4a4_linear_forward_host): staging buffers, copy streams and events.
@@ -103,6 +104,17 @@ inline int gemm_k_splits(int tiles, int stages, int min_stages, const int* clust
   for (int s = kMaxGemmSplits; s > 1; --s)
     if (tiles <= clusters[s] && stages / s >= min_stages) return s;
   return 1;
+}
+
+template <typename Kernel>
+void count_clusters(int* clusters, Kernel* kernel, int threads, size_t smem) {
+  for (int s = 2; s <= kMaxGemmSplits; ++s) {
+    const OverlappedLaunch l(dim3(s), dim3(threads), smem, nullptr, dim3(s));
+    if (cudaOccupancyMaxActiveClusters(&clusters[s], kernel, &l.cfg) != cudaSuccess) {
+      cudaGetLastError();
+      clusters[s] = 0;
+    }
+  }
 }
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }

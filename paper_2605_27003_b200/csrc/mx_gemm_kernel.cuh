@@ -30,6 +30,11 @@
 //               for the epilogue to drain it before the next tile: sixteen warps pull the whole accumulator into
 //               registers at once and hand it back before they convert and store.
 //
+// Split K (mx_gemm_kernel<true>): where the tiles alone leave most SMs idle, the CTAs of a thread-block cluster share one
+// tile, each over its part of the K stages (the first one with the low-rank product).  Their FP32 accumulators meet in
+// shared memory (the operand ring's, idle by then), and every CTA adds its share of them over distributed shared memory in
+// split order.  One tile per CTA, no loop.
+//
 // Every wait is bounded (pipeline.cuh).
 #pragma once
 
@@ -70,6 +75,7 @@ struct MxGemmParams {
   const uint16_t* yref;  // [M, N] BF16 or nullptr
   double* sq_err;
   int act;              // output activation: 0 none, 1 GELU (tanh form)
+  int splits;           // mx_gemm_kernel: CTAs of a cluster that share a tile's K (1: K is not split)
   int run;              // CTA-pair kernel: consecutive column tiles of a row pair that one cluster takes at a time
 };
 
@@ -114,6 +120,7 @@ __device__ __forceinline__ void bulk_load(uint32_t dst_smem, const void* src, ui
                : "memory");
 }
 
+template <bool SPLIT>
 __global__ void __launch_bounds__(kMxThreads, 1)
 mx_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmT, const __grid_constant__ CUtensorMap tmL2, const MxGemmParams p) {
@@ -130,8 +137,12 @@ mx_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   volatile int* s_abort = reinterpret_cast<volatile int*>(smem + misc_off + 4);
 
   const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;  // provably warp-uniform
-  const int n_k_stages = p.K / kMxBK;
-  const int n_lr_stages = p.r > 0 ? (2 * p.r + 63) / 64 : 0;
+  // This CTA's K stages and tiles (all of them unless K is split).
+  const int split = SPLIT ? static_cast<int>(cluster_ctarank()) : 0;
+  const int ks_begin = SPLIT ? p.K / kMxBK * split / p.splits : 0;
+  const int n_k_stages = (SPLIT ? p.K / kMxBK * (split + 1) / p.splits : p.K / kMxBK) - ks_begin;
+  const int n_lr_stages = p.r > 0 && split == 0 ? (2 * p.r + 63) / 64 : 0;
+  const int first_tile = SPLIT ? blockIdx.x / p.splits : blockIdx.x, tile_step = SPLIT ? p.tiles_m * p.tiles_n : gridDim.x;
   const int atoms_k = p.K / 128;
   const int num_tiles = p.tiles_m * p.tiles_n;
   const WaitEnv env{p.err, s_abort, kWaitLimitNs};
@@ -171,7 +182,7 @@ mx_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const bool issuer = elect_one_lane();
     Ring<kMxStages> rg;
     bool ok = true;
-    for (int tile = blockIdx.x; ok && tile < num_tiles; tile += gridDim.x) {
+    for (int tile = first_tile; ok && tile < num_tiles; tile += tile_step) {
       const int tm = tile / p.tiles_n, tn = tile % p.tiles_n;
       const int m0 = tm * kBM, n0 = tn * kMxBN;
       const bool upper = n0 + 128 < p.N;  // does the tile's second 128-column half exist?
@@ -187,7 +198,7 @@ mx_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             tma_load_2d(dst + kMxATile, &tmL2, full, st * 64, n0);  // rows past N arrive as zeros
           }
         } else if (issuer) {
-          const int ks = st - n_lr_stages;
+          const int ks = ks_begin + st - n_lr_stages;
           const uint32_t sf = dst + kMxATile + kMxBTile;
           mbar_arrive_expect_tx(full, kMxATile + kMxBTile + (upper ? 3u : 2u) * kMxSfTile);
           tma_load_2d(dst, &tmA, full, ks * 128, m0);
@@ -207,7 +218,7 @@ mx_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     Ring<kMxStages> rg;
     Ring<1> ab;
     bool ok = true;
-    for (int tile = blockIdx.x; ok && tile < num_tiles; tile += gridDim.x) {
+    for (int tile = first_tile; ok && tile < num_tiles; tile += tile_step) {
       ok = __all_sync(0xffffffffu, bounded_wait<64>(bar_acc_empty, ab.parity ^ 1u, env, kErrMmaWait));
       if (!ok) break;
       tc_fence_after_sync();
@@ -257,7 +268,7 @@ mx_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const int quarter = ew & 3, colblk = ew >> 2;
     Ring<1> ab;
     bool ok = true;
-    for (int tile = blockIdx.x; ok && tile < num_tiles; tile += gridDim.x) {
+    for (int tile = first_tile; ok && tile < num_tiles; tile += tile_step) {
       const int m0 = (tile / p.tiles_n) * kBM, n0 = (tile % p.tiles_n) * kMxBN;
       const int row = m0 + 32 * quarter + lane;
       ok = bounded_wait(bar_acc_full, ab.parity, env, kErrEpilogueWait);
@@ -271,6 +282,15 @@ mx_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       tc_fence_before_sync();
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_acc_empty);
+      if constexpr (SPLIT) {
+        // Partial tile: 1024-byte rows of FP32, 16-byte chunk c at c ^ (row % 8): conflict free for both sides.
+        const int r = 32 * quarter + lane;
+#pragma unroll
+        for (int c = 0; c < 16; ++c)
+          sts_u32x4(smem_base + 1024 * r + 16 * ((16 * colblk + c) ^ (r & 7)),
+                    make_uint4(v[c >> 2][4 * (c & 3)], v[c >> 2][4 * (c & 3) + 1], v[c >> 2][4 * (c & 3) + 2], v[c >> 2][4 * (c & 3) + 3]));
+        break;
+      }
       const int ch0 = n0 + 64 * colblk;
       if (p.yref != nullptr) {
         // Eq. 10's objective over this thread's 64 outputs, Y_hat rounded to BF16 as the forward stores it.
@@ -329,6 +349,44 @@ mx_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     }
   }
 
+  if constexpr (SPLIT) {
+    cluster_sync_all();   // all partial tiles are written
+    if (live && warp >= kMxEpiWarp0 && !*s_abort) {
+      const int m0 = (first_tile / p.tiles_n) * kBM, n0 = (first_tile % p.tiles_n) * kMxBN;
+      float sq = 0.0f;
+      // A warp takes 128 channels of a row at a time, a lane four of them.
+      for (int i = 16 * split + warp - kMxEpiWarp0; i < 2 * kBM; i += 16 * p.splits) {
+        const int row = i >> 1, ch = n0 + 128 * (i & 1) + 4 * lane;
+        if (m0 + row >= p.M) break;
+        if (ch >= p.N) continue;
+        const uint32_t at = smem_base + 1024 * row + 16 * ((32 * (i & 1) + lane) ^ (row & 7));
+        float4 y = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        for (int c = 0; c < p.splits; ++c) {
+          const float4 a = ld_cluster_f32x4(map_to_cta(at, c));
+          y.x += a.x, y.y += a.y, y.z += a.z, y.w += a.w;
+        }
+        const float4 b = p.bias ? __ldg(reinterpret_cast<const float4*>(p.bias + ch)) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        y.x += b.x, y.y += b.y, y.z += b.z, y.w += b.w;
+        if (p.act != 0)
+          y = make_float4(apply_activation(y.x, p.act), apply_activation(y.y, p.act), apply_activation(y.z, p.act), apply_activation(y.w, p.act));
+        const uint2 o = make_uint2(bf16x2_bits(make_float2(y.x, y.y)), bf16x2_bits(make_float2(y.z, y.w)));
+        const size_t dst = static_cast<size_t>(m0 + row) * p.N + ch;
+        if (p.yref == nullptr) {
+          *reinterpret_cast<uint2*>(p.Y + dst) = o;
+        } else {
+          const uint2 ref = __ldg(reinterpret_cast<const uint2*>(p.yref + dst));
+          sq = sq_diff_bf16x2(ref.x, o.x, sq);
+          sq = sq_diff_bf16x2(ref.y, o.y, sq);
+        }
+      }
+      if (p.yref != nullptr) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+        if (lane == 0) atomicAdd(p.sq_err, static_cast<double>(sq));
+      }
+    }
+    cluster_sync_all();   // nobody leaves while its shared memory is still being read
+  }
   // ---------------------------------------------------------------------- common tail
   tc_fence_before_sync();
   __syncthreads();

@@ -386,13 +386,7 @@ w4a4_status_t w4a4_ctx_create(int device, int max_M, int max_K, int max_r, w4a4_
     };
     const bool gemm_ok = prepare_gemm(gemm_w4a4_kernel<false, false>) && prepare_gemm(gemm_w4a4_kernel<true, false>) &&
                          prepare_gemm(gemm_w4a4_kernel<false, true>) && prepare_gemm(gemm_w4a4_kernel<true, true>);
-    for (int s = 2; s <= kMaxGemmSplits; ++s) {
-      const OverlappedLaunch l(dim3(s), dim3(kGemmThreads), kGemmSmemBytes, nullptr, dim3(s));
-      if (cudaOccupancyMaxActiveClusters(&ctx->gemm_clusters[s], gemm_w4a4_kernel<false, true>, &l.cfg) != cudaSuccess) {
-        cudaGetLastError();
-        ctx->gemm_clusters[s] = 0;
-      }
-    }
+    count_clusters(ctx->gemm_clusters, gemm_w4a4_kernel<false, true>, kGemmThreads, kGemmSmemBytes);
     if (!gemm_ok) {
       cudaGetLastError();
       st = W4A4_ERR_CUDA;

@@ -116,6 +116,17 @@ w4a4_status_t mx_launch_gemm(w4a4_mx_handle_t h, int M, int expert_id, void* Y, 
   const CUtensorMap& tmSFA = second_ws ? h->tmSFA2 : h->tmSFA;
   const CUtensorMap& tmT = h->r > 0 ? (second_ws ? h->tmT2 : h->tmT) : tmA;  // unused when r == 0
   const CUtensorMap& tmL2 = h->r > 0 ? e.tmL2 : e.tmB;
+  // Few tiles: clusters of single CTAs share a tile's K, at least three 256-deep stages each (a CTA pair per tile would leave
+  // half of the SMs or more without work).
+  p.splits = next ? 1 : gemm_k_splits(num_tiles, h->K / kMxBK, 3, ctx->mx_gemm_clusters);
+  if (p.splits > 1) {
+    const OverlappedLaunch l(dim3(num_tiles * p.splits), block, kMxSmemBytes, stream, dim3(p.splits));
+    if (cudaLaunchKernelEx(&l.cfg, mx_gemm_kernel<true>, tmA, e.tmB, tmT, tmL2, p) != cudaSuccess) {
+      cudaGetLastError();
+      return W4A4_ERR_CUDA;
+    }
+    return W4A4_OK;
+  }
   // CTA pairs (cta_group::2) need at least two row tiles and an even number of CTAs.
   if (p.tiles_m >= 2 && ctx->num_sms >= 2) {
     const int runs = ((p.tiles_m + 1) / 2) * ((p.tiles_n + p.run - 1) / p.run);
@@ -145,7 +156,7 @@ w4a4_status_t mx_launch_gemm(w4a4_mx_handle_t h, int M, int expert_id, void* Y, 
   }
   if (next) return W4A4_ERR_SHAPE;   // the fused form runs on CTA pairs only
   const OverlappedLaunch l(grid, block, kMxSmemBytes, stream);
-  if (cudaLaunchKernelEx(&l.cfg, mx_gemm_kernel, tmA, e.tmB, tmT, tmL2, p) != cudaSuccess) {
+  if (cudaLaunchKernelEx(&l.cfg, mx_gemm_kernel<false>, tmA, e.tmB, tmT, tmL2, p) != cudaSuccess) {
     cudaGetLastError();
     return W4A4_ERR_CUDA;
   }
@@ -206,8 +217,11 @@ w4a4_status_t w4a4_mx_pack_weights(w4a4_ctx_t ctx, const w4a4_mx_weight_desc_t* 
     const size_t nb = mx_sfa_bytes(ctx->max_M, ctx->max_K);
     st = dev_alloc(&ctx->mx_sfa, nb, &ctx->bytes);
     if (st == W4A4_OK && cudaMemset(ctx->mx_sfa, 0, nb) != cudaSuccess) st = W4A4_ERR_CUDA;
-    if (st == W4A4_OK)
-      cudaFuncSetAttribute(mx_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kMxSmemBytes));
+    if (st == W4A4_OK) {
+      cudaFuncSetAttribute(mx_gemm_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kMxSmemBytes));
+      cudaFuncSetAttribute(mx_gemm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kMxSmemBytes));
+      count_clusters(ctx->mx_gemm_clusters, mx_gemm_kernel<true>, kMxThreads, kMxSmemBytes);
+    }
     if (st == W4A4_OK)
       cudaFuncSetAttribute(mx_gemm2_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kMx2SmemBytes));
     if (st == W4A4_OK)

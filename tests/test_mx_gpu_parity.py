@@ -139,3 +139,13 @@ def test_mx_full_size_sampled_rows(name):
     rows = sorted({0, 127, 128, 255, 256, last - 1, last, M - 1, *rng.choice(M, 256, replace=False).tolist()})
     clip = gen.make_clip_table(1, 1, 8, [(0.6, 1.0)], seed=6)
     run_mx_case(x, [layer], clip, 0, 2, rows=rows)
+
+
+@pytest.mark.parametrize("M,K,N,r", [
+    (1, 1536, 128, 16),      # one token, half a column tile, six K stages: two CTAs share it
+    (100, 4864, 384, 0),     # 19 stages over six CTAs, the last column tile half outside
+    (257, 2048, 512, 64),    # three row blocks, the last with one row; two low-rank stages, with the first CTA of a cluster
+])
+def test_mx_tiles_shared_by_a_cluster(M, K, N, r):
+    x = gen.make_activations(M, K, outlier_idx=gen.outlier_channels(K, 0.02, 4), outlier_gain=50.0, seed=M)
+    run_mx_case(x, [gen.make_layer_mx_direct(K, N, r, seed=K)], torch.full((1, 1, 1), 0.85), 0, 0, max_M=M + 5)
