@@ -165,7 +165,7 @@ void w4a4_tile_shape(int* tile_m, int* tile_n);
  * synchronisation of cudaMalloc is not acceptable cannot create a context or a handle.  This call needs
  * neither: it computes Xh = X / lambda, the per-(token, 64-channel group) scales and the 4-bit codes
  * (Eq. 3-5, 8-9; no low-rank branch) with its scratch held in a fixed array inside the library image
- * (about 2.3 MiB of device memory on every GPU that loads the library, for the life of the process).
+ * (64 KiB of device memory on every GPU that loads the library, for the life of the process).
  *   X       device BF16 [M, K] row-major, 16-byte aligned          lambda  device FP32 [K], > 0
  *   clip_table / clip_index   device FP32 table and the index of the ratio to use (read on the device)
  *   codes   device int8 [M, K], one code per byte in [-8, 7]       scales  device FP32 [M, K/64]

@@ -34,7 +34,7 @@ struct w4a4_ctx {
   size_t bytes = 0;
   int num_sms = 0;
   size_t l2_bytes = 0;        // size of the device's L2 (sizes the GEMM's tile order)
-  int gemm_clusters[9] = {};  // clusters of that many CTAs of the INT4 GEMM that run at a time (index 2 .. 8)
+  int gemm_clusters[9] = {};  // clusters of that many CTAs of the INT4 GEMM (one per SM) that run at a time (index 2 .. 8)
   int mx_gemm_clusters[9] = {};   // the same for the MXFP4 variant's single-CTA GEMM
   int debug_sc_tiles = 0;     // test hook: forced super-column width of the GEMM's tile order (0: automatic)
   EncodeTiledFn encode = nullptr;

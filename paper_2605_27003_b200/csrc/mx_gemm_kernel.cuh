@@ -933,14 +933,6 @@ mx_gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
   }
 }
 
-// Weight pack kernels of the MXFP4 variant (run once per layer).
-// L1 [K, r] BF16 -> L1 transposed [r, K]: the K-major B operand of the fused producer's T MMA.
-__global__ void mx_transpose_l1_kernel(const uint16_t* __restrict__ l1, uint16_t* __restrict__ out, int K, int r) {
-  const size_t idx = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (idx >= static_cast<size_t>(K) * r) return;
-  const int k = static_cast<int>(idx / r), c = static_cast<int>(idx % r);
-  out[static_cast<size_t>(c) * K + k] = l1[idx];
-}
 // codes [K, N] (one E2M1 code per byte) -> [N, K/2], two codes per byte, even K in the low nibble.
 __global__ void mx_pack_weight_kernel(const uint8_t* __restrict__ codes, uint8_t* __restrict__ out, int K, int N,
                                       int* __restrict__ bad) {

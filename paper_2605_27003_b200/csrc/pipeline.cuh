@@ -185,7 +185,7 @@ __device__ __forceinline__ void drain_after_abort(volatile int* s_abort) {
 // Exercises the give-up path of bounded_wait without any pipeline around it: one warp waits for a phase of an
 // mbarrier that nobody ever completes.  No copy, tensor-core operation or TMEM allocation is involved, so there is
 // nothing to drain: after limit_ns the wait records kErrProbeWait in *err and the kernel returns normally.
-__global__ void wait_probe_kernel(int* err, uint64_t limit_ns) {
+static __global__ void wait_probe_kernel(int* err, uint64_t limit_ns) {
   __shared__ __align__(8) uint64_t bar;
   __shared__ int s_abort;
   if (threadIdx.x == 0) {

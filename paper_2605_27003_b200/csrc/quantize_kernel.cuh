@@ -1,45 +1,45 @@
 // Kernel 1: fused smoothing + per-(token, 64-channel group) 4-bit quantization + code output
-// + low-rank down-projection, one streaming pass over the BF16 activations (HBM bound).
+// + low-rank down-projection, one streaming pass over the BF16 activations (HBM bound by design).
 //
 //   Eq. 5      xh = f32(x) * (1/lambda)                      one FP32 multiply per element
-//   Eq. 8      a  = max |xh| over the 64-channel group       quad shuffles
-//   Eq. 9 / 4  s  = (rho * a) / 7 ,  is = 1 / s              IEEE divides, once per (row, group)
-//   Eq. 3      q  = clip(rint(xh * is), -8, 7)               rounding by the 1.5*2^23 magic add (ties to even)
-//   Eq. 7      T  = bf16(xh) L1                              mma.sync m16n8k16 BF16, FP32 accumulate
+//   Eq. 8      a  = max |xh| over the 64-channel group       shuffles among the eight lanes of a row
+//   Eq. 9 / 4  s  = (rho * a) / 7 ,  is = 1 / s              correctly rounded, once per (row, group)
+//   Eq. 3      q  = clip(rint(xh * is), -8, 7)               ties to even, by an addition that leaves no fraction bits
+//   Eq. 7      T  = bf16(xh) L1                              tcgen05.mma kind::f16, accumulated in TMEM over all of K
 //
-// Work split: a CTA of kQuantWarps warps owns 16 consecutive token rows per warp; all warps walk the K groups
-// together, so the group's L1 fragments and smoothing factors are staged once per CTA.  Inside a warp,
-// lane = 4*i + j owns rows i and i+8 and, within the group, channels
-//      32*(j/2) + 8*(j%2) + [0,8)     and the same + 16,
-// which is exactly the pair of 8-channel runs that fill two whole 32-bit words of the packed layout
-// below, so no lane exchange is needed to pack.  The tensor-core K order is free (a dot product does
-// not care about order), so the lane's 16 channels are used as-is as A-fragment slots and the L1
-// fragments are laid out at pack time to match (see l1_fragment_channel()).
+// Work split.  A CTA of up to eight element-wise warps owns 4 STEPS rows per warp and walks the K groups; a lane holds 8
+// consecutive channels (16 bytes) of one row per step, eight lanes a group.  The activations come by cp.async into a ring of
+// shared memory in which every lane reads back only what it copied itself.  bf16(xh) goes into a K-major 128-byte-swizzled
+// tile, from which one more warp issues four tcgen05.mma per group (M = 128, N = r, K = 16 each; the rows past the CTA's own
+// read whatever lies behind the tile and only touch accumulator rows that nobody reads) against the group's r x 64 tile
+// of L1, which it fetches by TMA into a ring of its own.
+// The bound is instruction issue: 101 (MXFP4) to 115 instructions per 8 values and lane at r = 32, 57 to 65 % of the issue slots
+// of two CTAs per SM, DRAM at about 70 %.  So the loop's addresses are kept in registers (derived anew in every pass they
+// cost 15 of those instructions: 127 -> 94 us at 32760 x 5120 MXFP4) and the rare cases of the scale arithmetic have a branch
+// of their own.  The predecessor held 16 rows of a warp in mma.sync fragments, with r accumulators per row in registers.
+// 32760 x 5120, INT4 | MXFP4: r = 0 120 -> 100 | 93 -> 79 us, r = 32 148 -> 113 | 122 -> 92, r = 64 192 -> 120 | 158 -> 100, r = 96
+// 278 -> 140 (INT4); 32760 x 13824, r = 32 389 -> 290 | 320 -> 233.  (335 MB in and 168 | 89 MB out take 76 | 64 us.)
 //
-// K split (gridDim.y > 1): with few token rows there are too few 16-row warps to fill the machine, so the K groups
-// are divided among gridDim.y CTAs per row block, which form one thread-block cluster.  Codes and scales of different
-// groups are independent; the partial sums of T stay in each CTA's shared memory, and after a cluster barrier every CTA
-// adds its share of them over distributed shared memory, in split order, and writes the BF16 high | low pair.  (A
-// reduction kernel over a global scratch cost a dependent launch.)
+// K split (gridDim.y > 1): with few token rows there are too few row blocks to fill the machine, so the K groups are divided
+// among gridDim.y CTAs per row block, which form one thread-block cluster when there is a low-rank branch.  Codes and scales
+// of different groups are independent; of T every CTA adds up a share of the rows, for which the others push their partial
+// sums into its shared memory (st.async on an mbarrier there) and which it adds in split order.  Pulled over distributed
+// shared memory between two cluster barriers instead, the end of the kernel took 5000 clocks, pushed about 2000.
+// 100 x 5120, r = 32 12.9 -> 5.4 us INT4, 9.0 -> 5.1 MXFP4; 700 x 8192, r = 64 22.6 -> 11.6 | 15.9 -> 10.6.
 //
 // Weight expansion (ExpandJob): the CTAs past the row blocks turn the layer's 4-bit weights into the byte image the
 // INT4 GEMM reads.  It is independent of the activations, so it shares their launch instead of being a kernel between
-// two dependent ones; at the large sizes its traffic hides behind the activation CTAs.  Both together, per forward: 256 x
-// 512 -> 512 20.5 -> 14.3 us (four launches -> two), 1560 x 5120 -> 5120 at rank 64 112 -> 105 us.
+// two dependent ones; at the large sizes its traffic hides behind the activation CTAs.
 //
 // Code output, three formats (template parameter FORMAT):
 //   kCodesE4M3    one E4M3 byte per code, row-major [M, K]: the tensor-core operand of kernel 2 as it is
 //                 (fp8_codes.cuh), fetched by TMA straight into the swizzled operand tile;
-//   kCodesPacked  nibble-packed INT4, half the bytes, for callers that want the compact form;
+//   kCodesInt8    one two's complement byte per code, row-major [M, K], and scales [M, K/64], for callers of
+//                 w4a4_quantize_noalloc;
 //   kCodesMxfp4   the MXFP4 variant of the layer (OCP MX v1.0: E2M1 elements, one E8M0 scale per 32 channels,
 //                 shared exponent floor(log2(rho * block maximum)) - 2): two codes per byte, row-major
 //                 [M, K/2], and the scale bytes in the 512-byte atoms the block-scaled tensor-core
 //                 instruction wants in TMEM (see mx_gemm_kernel.cuh).
-// Packed activation layout: per row, per 32 consecutive channels
-// [32c, 32c+32) one 16-byte chunk of four 32-bit words; word w, byte b holds channel 32c + 4w + b in
-// its LOW nibble and channel 32c + 16 + 4w + b in its HIGH nibble (two's complement nibbles).  With
-// that interleave `word & 0x0F0F0F0F` and `(word >> 4) & 0x0F0F0F0F` are each four K-contiguous codes,
-// one per byte.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -47,33 +47,32 @@
 #include <stdint.h>
 
 #include "fp8_codes.cuh"
+#include "pipeline.cuh"
 #include "ptx.cuh"
 
 namespace w4a4 {
 
-constexpr int kCodesPacked = 0, kCodesE4M3 = 1, kCodesMxfp4 = 2;
-constexpr int kQuantRows = 16;      // token rows per CTA
-// Warps per CTA (16 rows each).  Small CTAs spread evenly over the 148 SMs; the widest rank shares its
-// larger L1 fragments among more warps.
-constexpr int quantize_warps(int R) { return R >= 64 ? 4 : 2; }
-constexpr int kStages = 3;          // depth of the cp.async rings (groups in flight = kStages - 1)
+constexpr int kCodesInt8 = 0, kCodesE4M3 = 1, kCodesMxfp4 = 2;
+constexpr int kQuantWarps = 8;                               // element-wise warps at most
+constexpr int quantize_rows(int steps, int warps = kQuantWarps) { return 4 * warps * steps; }
+constexpr int quantize_threads(int R, int warps = kQuantWarps) { return 32 * (warps + (R > 0 ? 1 : 0)); }
+constexpr int kL1Stages = 3, kXhBuffers = 2;
+constexpr uint32_t xh_tile_bytes(int steps, int warps) { return quantize_rows(steps, warps) * 128u; }   // rows x 64 channels in BF16
 
-// Dynamic shared memory of quantize_kernel<R>: activation rings, smoothing-factor ring, L1 fragment ring.
-constexpr size_t quantize_smem_bytes(int R) {
-  return static_cast<size_t>(quantize_warps(R)) * kStages * 4 * 32 * 16 + kStages * 64 * 4 +
-         static_cast<size_t>(kStages) * (4 * (R / 8) * 32 * 8);
+// One stage of the activation ring: what the element-wise warps read for one group, 16 bytes per lane and step and the
+// group's 64 reciprocals once per warp.
+constexpr uint32_t x_stage_bytes(int steps, int warps) { return warps * (steps * 512u + 256u); }
+constexpr int kXStages(int R, int steps) { return steps == 2 ? (R >= 96 ? 3 : 4) : (R == 0 ? 5 : (R <= 64 ? 3 : 2)); }
+
+// Dynamic shared memory: alignment slack, L1 ring, x_hat tiles, activation ring (and what the 128-row operand reads behind
+// the last x_hat tile), and in a K-split launch this CTA's share of all partial sums of T.
+constexpr uint32_t x_ring_bytes(int R, int steps, int warps) {
+  const uint32_t ring = kXStages(R, steps) * x_stage_bytes(steps, warps), behind = 128 * 128 - xh_tile_bytes(steps, warps);
+  return R == 0 || ring > behind ? ring : behind;
 }
-
-// Channel (within its 64-group) that lane-in-quad j holds as its e-th element, e in [0,16).
-__host__ __device__ constexpr int l1_fragment_channel(int j, int e) {
-  return 32 * (j >> 1) + 8 * (j & 1) + (e < 8 ? e : e + 8);
-}
-
-__device__ __forceinline__ void mma_bf16_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+constexpr size_t quantize_smem_bytes(int R, int steps, int warps, int splits) {
+  return (R == 0 ? 0 : 1024 + kL1Stages * R * 128 + kXhBuffers * xh_tile_bytes(steps, warps)) + x_ring_bytes(R, steps, warps) +
+         (splits > 1 ? (quantize_rows(steps, warps) + splits) * R * 4 : 0);
 }
 
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
@@ -81,13 +80,13 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   return *reinterpret_cast<uint32_t*>(&v);
 }
 
-__device__ __forceinline__ uint4 ldg_stream_v4(const void* p) {
-  uint4 v;
-  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
-               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-               : "l"(p));
-  return v;
+// 16 bytes global -> shared, past L1; one commit group per activation stage.
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 // Smooth 8 BF16 values (one 16-byte load) with 8 reciprocals.
 __device__ __forceinline__ void smooth8(const uint4& raw, const float4& r0, const float4& r1, float* xh) {
@@ -98,84 +97,104 @@ __device__ __forceinline__ void smooth8(const uint4& raw, const float4& r0, cons
   xh[0] = a.x; xh[1] = a.y; xh[2] = b.x; xh[3] = b.y; xh[4] = c.x; xh[5] = c.y; xh[6] = d.x; xh[7] = d.y;
 }
 
-// Group absolute maximum of the lane's 16 smoothed values, combined over the quad (= 64 channels).
-__device__ __forceinline__ float quad_absmax16(const float* xh) {
-  float a0 = fmaxf(fabsf(xh[0]), fabsf(xh[1])), a1 = fmaxf(fabsf(xh[2]), fabsf(xh[3]));
+// max |v| over a lane's 8 values, with three-input maxima.  PROPAGATE: NaN if any of them is NaN (else NaNs are ignored).
+template <bool PROPAGATE>
+__device__ __forceinline__ float max3_abs(float a, float b, float c) {
+  float d;
+  if constexpr (PROPAGATE) asm("max.NaN.abs.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  else asm("max.abs.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+template <bool PROPAGATE>
+__device__ __forceinline__ float absmax8(const float* xh) {
+  const float a = max3_abs<PROPAGATE>(xh[0], xh[1], xh[2]), b = max3_abs<PROPAGATE>(xh[3], xh[4], xh[5]);
+  return max3_abs<PROPAGATE>(max3_abs<PROPAGATE>(a, xh[6], xh[7]), b, b);
+}
+// ... and over the 2^n neighbouring lanes below LANES.
+template <int LANES, bool PROPAGATE>
+__device__ __forceinline__ float absmax_lanes(float a) {
 #pragma unroll
-  for (int e = 4; e < 16; e += 2) {
-    a0 = fmaxf(a0, fabsf(xh[e]));
-    a1 = fmaxf(a1, fabsf(xh[e + 1]));
+  for (int o = 1; o < LANES; o *= 2) {
+    const float b = __shfl_xor_sync(0xffffffffu, a, o);
+    if constexpr (PROPAGATE) asm("max.NaN.f32 %0, %1, %2;" : "=f"(a) : "f"(a), "f"(b));
+    else a = fmaxf(a, b);
   }
-  float a = fmaxf(a0, a1);
-  a = fmaxf(a, __shfl_xor_sync(0xffffffffu, a, 1));
-  a = fmaxf(a, __shfl_xor_sync(0xffffffffu, a, 2));
   return a;
 }
 
-// Eq. 8-9 / Eq. 4: s = (rho * a) / 7 and its reciprocal, both correctly rounded (IEEE); a == 0 -> 0, 0.
-__device__ __forceinline__ void group_scale(float rho, float a, float& s, float& is) {
-  s = 0.0f;
-  is = 0.0f;
-  if (a > 0.0f) {
-    s = __fdiv_rn(__fmul_rn(rho, a), 7.0f);
-    is = __frcp_rn(s);  // == 1.0f / s, round to nearest
-  }
+// Eq. 8-9 / Eq. 4: s = x / 7 with x = rho * a, and is = 1 / s, both correctly rounded (IEEE); a == 0 -> 0, 0.
+__device__ __forceinline__ void group_scale(float x, float& s, float& is) {
+  s = x > 0.0f ? __fdiv_rn(x, 7.0f) : 0.0f;
+  is = s > 0.0f ? __frcp_rn(s) : 0.0f;
+}
+// The same for kOrdinaryMin <= x <= kOrdinaryMax, where nothing under- or overflows: an approximation corrected by its exact
+// remainder (Markstein, IBM J. Res. Dev. 34, 1990) is the correctly rounded quotient; compared with the two functions above
+// for every significand.  9 instructions instead of 27.
+constexpr float kOrdinaryMin = 1e-30f, kOrdinaryMax = 1e30f;
+__device__ __forceinline__ void group_scale_ordinary(float x, float& s, float& is) {
+  const float seventh = 0.142857142857142857f;
+  const float q = __fmul_rn(x, seventh);
+  s = __fmaf_rn(__fmaf_rn(-7.0f, q, x), seventh, q);
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(s));
+  is = __fmaf_rn(__fmaf_rn(-s, y, 1.0f), y, y);
 }
 
-// Eq. 3 for the lane's 16 smoothed values of one row: code + 8 in [0, 15].
-__device__ __forceinline__ void quantize16_offset(const float* xh, float is, uint32_t (&u)[16]) {
-  // (float bits of z + 1.5*2^23 + 8) - bits(1.5*2^23), clamped.
+// Eq. 3 for a lane's 8 smoothed values: z = xh * is rounded to FP32, then to the nearest integer with ties to even, then
+// clamped to [-8, 7].  The result is the code + 8, two to a word.
+__device__ __forceinline__ void quantize8(const float* xh, float is, uint32_t* u) {
 #pragma unroll
-  for (int e = 0; e < 16; ++e) {
-    const float f = __fadd_rn(__fmul_rn(xh[e], is), 12582920.0f);
-    u[e] = static_cast<uint32_t>(__viaddmin_s32_relu(__float_as_int(f), -0x4B400000, 15));
+  for (int e = 0; e < 8; e += 2) {
+    const int a = min(max(__float2int_rn(__fmul_rn(xh[e], is)), -8), 7) + 8, b = min(max(__float2int_rn(__fmul_rn(xh[e + 1], is)), -8), 7) + 8;
+    u[e >> 1] = static_cast<uint32_t>(a | (b << 16));
   }
+}
+// The same where |z| < 2^15 and z is a number (ordinary scale, rho >= kRhoOrdinary: |z| <= 7 / rho): adding 1.5 * 2^23 rounds to the
+// nearest even integer and leaves it in the low half-word, and one 16x2 add-min-relu clamps two of them.  16 instructions for
+// 8 values, none of them on the conversion unit, whose 8 conversions to integer would take 64 cycles.  `one` is 1 and unknown to
+// the compiler: a packed product and a packed sum, even in PTX with .rn, became one FMA that skips the first rounding.
+constexpr float kRhoOrdinary = 0x1p-10f;
+__device__ __forceinline__ void quantize8_ordinary(const float* xh, float is, float one, uint32_t* u) {
+#pragma unroll
+  for (int e = 0; e < 8; e += 2) {
+    const float2 z = __fmul2_rn(make_float2(xh[e], xh[e + 1]), make_float2(is, is));
+    const float2 m = __ffma2_rn(z, make_float2(one, one), make_float2(12582912.0f, 12582912.0f));
+    u[e >> 1] = __viaddmin_s16x2_relu(__byte_perm(__float_as_uint(m.x), __float_as_uint(m.y), 0x5410), 0x00080008u, 0x000f000fu);
+  }
+}
+// Codes + 8, two to a word -> E4M3 bytes.  A half-word 0 .. 15 read as FP16 is u 2^-24: two exact FP16 steps make it u - 8,
+// and the conversion is exact too.
+__device__ __forceinline__ uint2 e4m3_of_codes(const uint32_t* u) {
+  uint16_t b[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    uint32_t h;
+    asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(h) : "r"(u[i]), "r"(0x78007800u), "r"(0xa400a400u));   // u 2^-24 2^15 - 2^-6
+    asm("mul.rn.f16x2 %0, %1, %2;" : "=r"(h) : "r"(h), "r"(0x60006000u));                           // * 2^9
+    asm("cvt.rn.satfinite.e4m3x2.f16x2 %0, %1;" : "=h"(b[i]) : "r"(h));
+  }
+  uint2 w;
+  asm("mov.b32 %0, {%1, %2};" : "=r"(w.x) : "h"(b[0]), "h"(b[1]));
+  asm("mov.b32 %0, {%1, %2};" : "=r"(w.y) : "h"(b[2]), "h"(b[3]));
+  return w;
+}
+// ... -> two's complement bytes.
+__device__ __forceinline__ uint2 int8_of_codes(const uint32_t* u) {
+  uint2 w;
+  w.x = ((__byte_perm(u[0], u[1], 0x6420) | 0x80808080u) - 0x08080808u) ^ 0x80808080u;
+  w.y = ((__byte_perm(u[2], u[3], 0x6420) | 0x80808080u) - 0x08080808u) ^ 0x80808080u;
+  return w;
 }
 
-// Quantize the lane's 16 values and return them as E4M3 bytes: .x/.y = elements 0..7 (channels coff .. +7),
-// .z/.w = elements 8..15 (channels coff + 16 .. +23).
-__device__ __forceinline__ uint4 quantize16_bytes(const float* xh, float is) {
-  // Eq. 3: z = xh * is rounded to FP32, then to the nearest integer with ties to even (cvt.rni), then clamped to
-  // [-8, 7]: cvt.pack.sat.s4 saturates two integers to 4 bits and shifts them in under the nibbles packed so far,
-  // so the eight codes of a word take four instructions, element 0 in the lowest nibble.
-  uint32_t n[2];
-#pragma unroll
-  for (int hh = 0; hh < 2; ++hh) {
-    int v[8];
-#pragma unroll
-    for (int e = 0; e < 8; e += 2) {
-      const float2 z = __fmul2_rn(make_float2(xh[8 * hh + e], xh[8 * hh + e + 1]), make_float2(is, is));
-      v[e] = __float2int_rn(z.x);
-      v[e + 1] = __float2int_rn(z.y);
-    }
-    uint32_t w;
-    asm("cvt.pack.sat.s4.s32.b32 %0, %1, %2, %3;" : "=r"(w) : "r"(v[7]), "r"(v[6]), "r"(0));
-    asm("cvt.pack.sat.s4.s32.b32 %0, %1, %2, %3;" : "=r"(w) : "r"(v[5]), "r"(v[4]), "r"(w));
-    asm("cvt.pack.sat.s4.s32.b32 %0, %1, %2, %3;" : "=r"(w) : "r"(v[3]), "r"(v[2]), "r"(w));
-    asm("cvt.pack.sat.s4.s32.b32 %0, %1, %2, %3;" : "=r"(w) : "r"(v[1]), "r"(v[0]), "r"(w));
-    n[hh] = w ^ 0x88888888u;   // two's complement nibbles -> code + 8, the index the byte lookup takes
-  }
-  return make_uint4(e4m3_of_offset_nibbles4(n[0]), e4m3_of_offset_nibbles4(n[0] >> 16), e4m3_of_offset_nibbles4(n[1]),
-                    e4m3_of_offset_nibbles4(n[1] >> 16));
+// Where channel c of a group stands in the K order of T's operands: an MMA step of 16 takes four channels from each of four
+// runs of 8.  Any order gives a dot product; with this one T keeps the bits that its mma.sync predecessor gave it, and with
+// them the 4-bit codes of the fused FFN's hidden activations (another order moved its outputs by 4.5e-4 instead of 1.8e-5).
+__host__ __device__ constexpr uint32_t xh_position(uint32_t c) {
+  return (c >> 4 & 1) * 32 + (c >> 2 & 1) * 16 + (c >> 5) * 8 + (c >> 3 & 1) * 4 + (c & 3);
 }
 
-// Quantize the lane's 16 smoothed values of one row (Eq. 3) and return its two packed words.
-__device__ __forceinline__ uint2 quantize16(const float* xh, float is) {
-  uint32_t u[16];
-  quantize16_offset(xh, is, u);
-  // One shift-add per code places its nibble: word w, byte b = low nibble u[4w+b], high nibble u[8+4w+b].
-  uint32_t w0 = u[0], w1 = u[4];
-#pragma unroll
-  for (int b = 0; b < 4; ++b) {
-    if (b > 0) {
-      w0 += u[b] << (8 * b);
-      w1 += u[4 + b] << (8 * b);
-    }
-    w0 += u[8 + b] << (8 * b + 4);
-    w1 += u[12 + b] << (8 * b + 4);
-  }
-  return make_uint2(w0 ^ 0x88888888u, w1 ^ 0x88888888u);  // offset-binary -> two's complement nibbles
-}
+// Keeps an address that the loop needs from being derived again in every pass.
+__device__ __forceinline__ void keep_in_register(uint32_t& v) { asm volatile("" : "+r"(v)); }
 
 // Two neighbouring entries of a row of T as BF16 high parts (columns c, c + 1 of the row) and the BF16 rounding of the
 // remainders (columns R + c, R + c + 1).
@@ -201,35 +220,12 @@ __device__ __forceinline__ uint32_t e2m1x8(const float* v) {
   return r;
 }
 
-// MXFP4 conversion of the lane's 16 values of one row; they all lie in one 32-channel block, whose other half the
-// neighbouring lane holds.  Returns the E8M0 exponent byte; packed codes in lo (elements 0..7) and hi (8..15).
-__device__ __forceinline__ uint32_t mxfp4_block16(const float* xh, float rho, uint32_t& lo, uint32_t& hi) {
-  float a0 = fmaxf(fabsf(xh[0]), fabsf(xh[1])), a1 = fmaxf(fabsf(xh[2]), fabsf(xh[3]));
-#pragma unroll
-  for (int e = 4; e < 16; e += 2) {
-    a0 = fmaxf(a0, fabsf(xh[e]));
-    a1 = fmaxf(a1, fabsf(xh[e + 1]));
-  }
-  float a = fmaxf(a0, a1);
-  a = fmaxf(a, __shfl_xor_sync(0xffffffffu, a, 1));
-  const uint32_t field = (__float_as_uint(__fmul_rn(rho, a)) >> 23) & 0xffu;   // exponent of the clip threshold (Eq. 8)
-  const uint32_t ex = field > 2u ? field - 2u : 0u;                            // minus the exponent of E2M1's top binade
-  const float inv = __uint_as_float((254u - ex) << 23);                        // 2^(127 - ex): exact scaling
-  float v[16];
-#pragma unroll
-  for (int e = 0; e < 16; ++e) v[e] = __fmul_rn(xh[e], inv);
-  lo = e2m1x8(v);
-  hi = e2m1x8(v + 8);
-  return ex;
-}
-
 // The token side of the GEMM's scale MMA for one (row, group): the scale as two BF16 pieces, s = h + m up to 2^-16
 // relative, laid out [h, h, m, m] against the channel side's [w1, w2, w1, w2].
 __device__ __forceinline__ uint2 sop_slots_activation(float s) {
-  const __nv_bfloat16 h = __float2bfloat16_rn(s);
-  const __nv_bfloat16 m = __float2bfloat16_rn(s - __bfloat162float(h));
-  const uint32_t hb = __bfloat16_as_ushort(h), mb = __bfloat16_as_ushort(m);
-  return make_uint2(hb | (hb << 16), mb | (mb << 16));
+  const uint32_t h = pack_bf16x2(s, s);   // the packed conversion stays off the conversion unit
+  const float m = s - __uint_as_float(h << 16);
+  return make_uint2(h, pack_bf16x2(m, m));
 }
 
 // Weight codes at rest -> the E4M3 byte image the INT4 GEMM reads: [N, K/2] packed as code + 8 (byte j of a row holds
@@ -247,245 +243,402 @@ __device__ __forceinline__ void expand_chunk(const uint4& w, uint4* out) {
   out[1] = make_uint4(e4m3_of_offset_nibbles4(w.z), e4m3_of_offset_nibbles4(w.z >> 16), e4m3_of_offset_nibbles4(w.w),
                       e4m3_of_offset_nibbles4(w.w >> 16));
 }
-constexpr int kExpandUnroll = 4;   // 16-byte loads a thread keeps in flight
+constexpr int kExpandUnroll = 4;   // 16-byte loads a thread keeps in flight, in batches: the next one is on its way while one is turned
 // `index` / `count`: this thread among all threads that share the job.
 __device__ __forceinline__ void expand_weights(const ExpandJob& job, uint32_t index, uint32_t count) {
-  for (uint32_t i = index; i < job.chunks; i += kExpandUnroll * count) {
-    uint4 w[kExpandUnroll];
+  uint4 w[kExpandUnroll];
+  auto load = [&](uint32_t i) {
 #pragma unroll
     for (int j = 0; j < kExpandUnroll; ++j)
       if (i + j * count < job.chunks) w[j] = __ldg(job.packed + i + j * count);
+  };
+  load(index);
+  for (uint32_t i = index; i < job.chunks; i += kExpandUnroll * count) {
+    uint4 now[kExpandUnroll];
+#pragma unroll
+    for (int j = 0; j < kExpandUnroll; ++j) now[j] = w[j];
+    load(i + kExpandUnroll * count);
 #pragma unroll
     for (int j = 0; j < kExpandUnroll; ++j)
-      if (i + j * count < job.chunks) expand_chunk(w[j], job.out + 2 * static_cast<size_t>(i + j * count));
+      if (i + j * count < job.chunks) expand_chunk(now[j], job.out + 2 * static_cast<size_t>(i + j * count));
   }
+}
+// CTAs for a job: up to four batches each where that still leaves two CTAs per SM.
+inline int expand_ctas(uint32_t chunks, int threads, int sms) {
+  const uint32_t batches = (chunks + kExpandUnroll * threads - 1) / (kExpandUnroll * threads);
+  const uint32_t each = batches / (2 * sms);
+  return static_cast<int>(each <= 1 ? batches : (batches + (each < 4 ? each : 4) - 1) / (each < 4 ? each : 4));
 }
 // The same as a kernel of its own, for the GEMM without an activation pass in front of it.
 static __global__ void expand_weight_kernel(const ExpandJob job) {
   expand_weights(job, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
 }
 
-template <int R, int WARPS, int FORMAT>
-// Sixteen resident warps per SM (at most 128 registers) at every rank, so that the 2048 warps of row blocks of the
-// DiT shapes fit one wave: at 130-160 registers the wide ranks ran 1.15 waves.
-__global__ void __launch_bounds__(32 * WARPS, 16 / WARPS)
-quantize_kernel(const uint16_t* __restrict__ X, int M, int K, const float* __restrict__ rlam,
-                const float* __restrict__ clip_table, int clip_index, const uint2* __restrict__ l1frag,
-                uint8_t* __restrict__ codes, float* __restrict__ scales, int scales_ld,
-                uint16_t* __restrict__ t_hilo, uint2* __restrict__ a_sop, const ExpandJob expand) {
-  grid_dependency_wait();
-  if (blockIdx.x >= expand.first_cta) {   // whole clusters: the cluster spans gridDim.y, never blockIdx.x
-    const uint32_t cta = (blockIdx.x - expand.first_cta) * gridDim.y + blockIdx.y;
-    expand_weights(expand, cta * (32 * WARPS) + threadIdx.x, (gridDim.x - expand.first_cta) * gridDim.y * (32 * WARPS));
+struct QuantizeParams {
+  const uint16_t* X;        // [M, K] BF16
+  int M, K;
+  const float* rlam;        // [K] reciprocal smoothing factors
+  const float* clip_table;
+  int clip_index;
+  uint8_t* codes;
+  float* scales;            // kCodesE4M3: FP32 [K/64, scales_ld] or nullptr; kCodesInt8: [M, K/64]; kCodesMxfp4: scale atoms
+  int scales_ld;            // kCodesE4M3: pitch; kCodesMxfp4: atoms per row block
+  uint16_t* t_hilo;         // [M, 2R]
+  uint2* a_sop;             // kCodesE4M3: token-side scale operands of the GEMM
+  ExpandJob expand;
+  int* err;                 // error word of the bounded waits (R > 0)
+  float one = 1.0f;         // see quantize8_ordinary
+};
+
+// MINB CTAs per SM: the register budget.
+template <int R, int FORMAT, int STEPS, int MINB>
+__global__ void __launch_bounds__(quantize_threads(R), MINB)
+quantize_kernel(const __grid_constant__ CUtensorMap tmL1, const QuantizeParams p) {
+  const int warps = static_cast<int>(blockDim.x >> 5) - (R > 0 ? 1 : 0), cta_rows = quantize_rows(STEPS, warps);
+  const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+  if (blockIdx.x >= p.expand.first_cta) {   // whole clusters: the cluster spans gridDim.y, never blockIdx.x
+    grid_dependency_wait();
+    grid_dependency_launch();
+    const uint32_t cta = (blockIdx.x - p.expand.first_cta) * gridDim.y + blockIdx.y;
+    expand_weights(p.expand, cta * blockDim.x + threadIdx.x, (gridDim.x - p.expand.first_cta) * gridDim.y * blockDim.x);
     return;
   }
-  constexpr int NT = R / 8;                          // n-tiles of the m16n8k16 MMA
-  constexpr int kFragBytes = 4 * NT * 32 * 8;        // L1 fragments of one group (4 KiB at r = 32)
-  constexpr int kFragChunks = kFragBytes / 16;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int qi = lane >> 2, qj = lane & 3;
-  const int G = K >> 6;
-  const int row0 = (blockIdx.x * WARPS + warp) * kQuantRows;
-  const int rowA = row0 + qi, rowB = rowA + 8;
-  const bool okA = rowA < M, okB = rowB < M;
-  const float rho = __ldg(clip_table + clip_index);
-  const int coff = 32 * (qj >> 1) + 8 * (qj & 1);  // lane's first channel inside a group
+  // This CTA's share of the groups (all of them unless the launch splits K).
+  const int G = p.K >> 6;
+  const int g_per_split = (G + gridDim.y - 1) / gridDim.y;
+  const int g_begin = min(G, static_cast<int>(blockIdx.y) * g_per_split), g_end = min(G, g_begin + g_per_split);
+  const int row0 = blockIdx.x * cta_rows;
 
-  const uint16_t* xa = X + static_cast<size_t>(okA ? rowA : 0) * K + coff;
-  const uint16_t* xb = X + static_cast<size_t>(okB ? rowB : 0) * K + coff;
-
-  float acc[NT > 0 ? NT : 1][4];
-#pragma unroll
-  for (int nt = 0; nt < (NT > 0 ? NT : 1); ++nt) acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.0f;
-
-  // Everything a group needs is streamed through shared-memory rings with cp.async, kStages - 1 groups
-  // ahead of the one being processed:
-  //   xring   per warp: the 16 rows x 64 channels of activations (2 KiB); every lane reads back only the
-  //           4 x 16 bytes it requested itself ([piece][lane] layout, conflict free, no barrier needed);
-  //   fring   per CTA: the group's L1 fragments, shared by the CTA's warps (they all walk the same groups,
-  //           each on its own 16 rows), so L1 crosses L2 once per 64 rows instead of once per 16;
-  //   lring   per CTA: the group's 64 reciprocal smoothing factors.
-  extern __shared__ __align__(16) uint8_t quant_smem[];
-  typedef uint4 (*XRing)[kStages][4][32];
-  typedef uint4 (*FRing)[kFragChunks > 0 ? kFragChunks : 1];
-  typedef float (*LRing)[64];
-  XRing xring = reinterpret_cast<XRing>(quant_smem);
-  LRing lring = reinterpret_cast<LRing>(quant_smem + WARPS * kStages * 4 * 32 * 16);
-  FRing fring = reinterpret_cast<FRing>(quant_smem + WARPS * kStages * 4 * 32 * 16 + kStages * 64 * 4);
-  const uint32_t xring0 = static_cast<uint32_t>(__cvta_generic_to_shared(&xring[warp][0][0][lane]));
-  auto issue = [&](int gg, int stage) {
-    const uint32_t dst = xring0 + stage * (4 * 32 * 16);
-    const uint32_t szA = okA ? 16u : 0u, szB = okB ? 16u : 0u;  // rows past M are zero-filled
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(xa + 64 * gg), "r"(szA) : "memory");
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst + 512), "l"(xa + 64 * gg + 16), "r"(szA) : "memory");
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst + 1024), "l"(xb + 64 * gg), "r"(szB) : "memory");
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst + 1536), "l"(xb + 64 * gg + 16), "r"(szB) : "memory");
-    if constexpr (NT > 0) {
-      const uint4* src = reinterpret_cast<const uint4*>(l1frag) + static_cast<size_t>(gg) * kFragChunks;
-      for (int c = threadIdx.x; c < kFragChunks; c += (32 * WARPS)) {
-        const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(&fring[stage][c]));
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src + c) : "memory");
-      }
-    }
-    if (threadIdx.x < 16) {
-      const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(&lring[stage][4 * threadIdx.x]));
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(rlam + 64 * gg + 4 * threadIdx.x) : "memory");
+  extern __shared__ uint8_t quant_smem[];
+  __shared__ __align__(8) uint64_t s_bars[kL1Stages + 2 * kXhBuffers + 2];
+  __shared__ uint32_t s_tmem;
+  __shared__ int s_abort_word;
+  constexpr uint32_t kTmemCols = R <= 32 ? 32 : (R <= 64 ? 64 : 128);
+  const uint32_t ring = R > 0 ? (smem_u32(quant_smem) + 1023u) & ~1023u : smem_u32(quant_smem);
+  const uint32_t xh0 = ring + kL1Stages * R * 128, xh_tile = xh_tile_bytes(STEPS, warps);
+  const uint32_t x_ring = R > 0 ? xh0 + kXhBuffers * xh_tile : ring;
+  const uint32_t bar_l1 = smem_u32(s_bars), bar_xh_full = bar_l1 + 8 * kL1Stages, bar_xh_empty = bar_xh_full + 8 * kXhBuffers,
+                 bar_t = bar_xh_empty + 8 * kXhBuffers, bar_push = bar_t + 8;
+  // K split: CTA c of the cluster adds up rows [c rows_each, (c + 1) rows_each) of the tile; the others push their partial
+  // sums of those rows into its shared memory.
+  const uint32_t pushed = x_ring + x_ring_bytes(R, STEPS, warps);
+  const int rows = min(cta_rows, p.M - row0), rows_each = (rows + gridDim.y - 1) / gridDim.y;
+  const int rows_mine = max(0, min(rows_each, rows - static_cast<int>(blockIdx.y) * rows_each));
+  uint32_t tmem = 0;
+  const WaitEnv env{p.err, &s_abort_word, kWaitLimitNs};
+  auto load_l1 = [&](int it) {   // by one lane
+    const uint32_t bar = bar_l1 + 8 * (it % kL1Stages);
+    mbar_arrive_expect_tx(bar, R * 128);
+    tma_load_2d(ring + (it % kL1Stages) * (R * 128), &tmL1, bar, 64 * (g_begin + it), 0);
+  };
+  auto join_setup = [&] {   // barriers and TMEM are there; a cluster's CTAs have all started (the wait comes before the pushes)
+    if constexpr (R > 0) {
+      __syncthreads();
+      tc_fence_after_sync();
+      tmem = __shfl_sync(0xffffffffu, s_tmem, 0);
+      if (gridDim.y > 1) cluster_arrive();
     }
   };
-  // This CTA's share of the groups (all of them unless the launch splits K).
-  const int g_per_split = (G + gridDim.y - 1) / gridDim.y;
-  const int g_begin = blockIdx.y * g_per_split;
-  const int g_end = min(G, g_begin + g_per_split);
+
+  if (R > 0 && warp == warps) {
+    // ------------------------------------------------------------------ L1 producer and MMA issuer (one lane issues)
+    constexpr uint32_t idesc = umma_idesc(1, 1, 128, R > 0 ? R : 16);
+    const bool issuer = elect_one_lane();
+    const int n = g_end - g_begin;
+    bool ok = true;
+    if (issuer) {
+      for (int i = 0; i < kL1Stages; ++i) mbar_init(bar_l1 + 8 * i, 1);
+      for (int i = 0; i < kXhBuffers; ++i) {
+        mbar_init(bar_xh_full + 8 * i, warps);
+        mbar_init(bar_xh_empty + 8 * i, 1);
+      }
+      mbar_init(bar_t, 1);
+      mbar_init(bar_push, 1);
+      mbar_fence_init();
+      fence_proxy_async_smem();
+      s_abort_word = 0;
+      // constants of the layer: no need to wait for the kernel before this one
+      for (int it = 0; it < kL1Stages - 1 && it < n; ++it) load_l1(it);
+      if (gridDim.y > 1 && rows_mine > 0) mbar_arrive_expect_tx(bar_push, gridDim.y * rows_mine * (R * 4));
+    }
+    __syncwarp();
+    tmem_alloc(smem_u32(&s_tmem), kTmemCols);
+    tmem_relinquish();
+    tc_fence_before_sync();
+    join_setup();
+    grid_dependency_wait();
+    for (int it = 0; ok && it < n; ++it) {
+      const int b = it % kXhBuffers;
+      // the tile of the group after next goes where the previous group's was, once its MMAs are done
+      if (it > 0)
+        ok = __all_sync(0xffffffffu, bounded_wait<0, 5>(bar_xh_empty + 8 * ((it - 1) % kXhBuffers), ((it - 1) / kXhBuffers) & 1u, env, kErrMmaWait));
+      if (!ok) break;
+      if (issuer && it + kL1Stages - 1 < n) load_l1(it + kL1Stages - 1);
+      ok = __all_sync(0xffffffffu, bounded_wait<0, 5>(bar_l1 + 8 * (it % kL1Stages), (it / kL1Stages) & 1u, env, kErrMmaWait)) &&
+           __all_sync(0xffffffffu, bounded_wait<0, 5>(bar_xh_full + 8 * b, (it / kXhBuffers) & 1u, env, kErrMmaWait));
+      if (!ok) break;
+      tc_fence_after_sync();
+      if (issuer) {
+        const uint32_t a = xh0 + b * xh_tile, l1 = ring + (it % kL1Stages) * (R * 128);
 #pragma unroll
-  for (int d = 0; d < kStages - 1; ++d) {
-    if (g_begin + d < g_end) issue(g_begin + d, d);
-    asm volatile("cp.async.commit_group;" ::: "memory");
+        for (int kk = 0; kk < 4; ++kk)
+          umma_f16(tmem, umma_desc_k_sw128(a, 32 * kk), umma_desc_k_sw128(l1, 32 * kk), idesc, it > 0 || kk > 0 ? 1u : 0u);
+        umma_commit(bar_xh_empty + 8 * b);
+        if (it + 1 == n) umma_commit(bar_t);
+      }
+      __syncwarp();
+    }
+  } else {
+    // ------------------------------------------------------------------ element-wise warps
+    grid_dependency_wait();
+    const int j = lane & 7;                                     // this lane's channels: 8 j .. 8 j + 7 of the group
+    const int tile_row = warp * (4 * STEPS) + (lane >> 4) + 2 * (lane >> 3 & 1);   // and rows: + 4 per step
+    const float rho = __ldg(p.clip_table + p.clip_index);
+    const float x_min = rho >= kRhoOrdinary ? kOrdinaryMin : kOrdinaryMax * 2.0f;   // below it the general path is taken
+    // 32-bit byte offsets from the CTA's first row (at most 128 rows of 16384 channels and a margin): half the address
+    // arithmetic of 64-bit pointers.
+    const uint8_t* const x_base = reinterpret_cast<const uint8_t*>(p.X + static_cast<size_t>(row0) * p.K);
+    const uint8_t* const rl_base = reinterpret_cast<const uint8_t*>(p.rlam);
+    constexpr uint32_t kCodeBits = FORMAT == kCodesMxfp4 ? 4 : 8;
+    uint8_t* const code_base = p.codes + static_cast<size_t>(row0) * (p.K / 8 * kCodeBits);
+    uint32_t x_off[STEPS], code_off[STEPS], xh_off[STEPS], scale_off[STEPS];
+    bool row_ok[STEPS];
+    // Where the scales of row0's 128-row block and of the next one begin: operand images, or atoms.
+    const uint32_t block_pitch = FORMAT == kCodesMxfp4 ? p.scales_ld * 512u : ((G + 1) >> 1) * 2048u;
+    uint8_t* const scale_base = reinterpret_cast<uint8_t*>(FORMAT == kCodesMxfp4 ? reinterpret_cast<void*>(p.scales) : p.a_sop) +
+                                static_cast<size_t>(row0 >> 7) * block_pitch;
+#pragma unroll
+    for (int s = 0; s < STEPS; ++s) {   // rows past M read the last one and store nothing
+      const int r = tile_row + 4 * s;
+      row_ok[s] = r < rows;
+      x_off[s] = static_cast<uint32_t>(min(r, rows - 1)) * p.K * 2 + 16 * j;
+      code_off[s] = static_cast<uint32_t>(r) * (p.K / 8 * kCodeBits) + kCodeBits * j;
+      xh_off[s] = xh0 + 128 * r + (xh_position(8 * j) * 2u ^ 16u * (r & 7));
+      if constexpr (FORMAT == kCodesMxfp4) {
+        // per 128-row block and per 4 scale blocks (128 channels) one 512-byte atom,
+        // byte (row % 32) * 16 + (row % 128 / 32) * 4 + (scale block % 4)
+        const int row = row0 + r;
+        scale_off[s] = ((row >> 7) - (row0 >> 7)) * block_pitch + (row & 31) * 16 + ((row & 127) >> 5) * 4 + (j >> 2);
+      } else {
+        // The scale as four BF16 slots of the operand from which the GEMM's tensor core forms sx * sw: 2 KiB shared-memory
+        // images per (128 rows, 2 groups), [8-row group][8 rows][group parity][8 bytes].  One lane per two steps (below).
+        const int row = row0 + r + (STEPS > 1 ? 4 * (j & 1) : 0);
+        scale_off[s] = ((row >> 7) - (row0 >> 7)) * block_pitch + ((row & 127) >> 3) * 128 + (row & 7) * 16;
+      }
+      keep_in_register(x_off[s]), keep_in_register(code_off[s]), keep_in_register(xh_off[s]), keep_in_register(scale_off[s]);
+    }
+    // A lane copies what it reads itself, and one lane in two 16 bytes of its warp's reciprocals, so a stage needs no
+    // barrier beyond its own commit group and a __syncwarp.
+    constexpr int kStages = kXStages(R, STEPS);
+    const uint32_t stage_bytes = x_stage_bytes(STEPS, warps);
+    const uint32_t my_x = x_ring + warp * (STEPS * 512u) + 16u * lane, my_rl = x_ring + warps * (STEPS * 512u) + 256u * warp;
+    auto load = [&](int g, uint32_t slot) {
+      if (g < g_end) {
+#pragma unroll
+        for (int s = 0; s < STEPS; ++s) cp_async16(my_x + slot + 512 * s, x_base + (x_off[s] + 128u * g));
+        if (lane < 16) cp_async16(my_rl + slot + 16 * lane, rl_base + (256u * g + 16u * lane));
+      }
+      cp_async_commit();
+    };
+#pragma unroll
+    for (int i = 0; i < kStages - 1; ++i) load(g_begin + i, stage_bytes * i);
+    join_setup();   // its microsecond passes beside the first loads
+    uint32_t slot = 0, slot_before = stage_bytes * (kStages - 1);   // this group's and the previous group's
+    bool ok = true;
+    for (int g = g_begin; g < g_end; ++g) {
+      float xh[STEPS][8];
+      cp_async_wait<kStages - 2>();
+      __syncwarp();
+      load(g + kStages - 1, slot_before);
+      {
+        const float4 rl0 = lds_f32x4(my_rl + slot + 32 * j), rl1 = lds_f32x4(my_rl + slot + 32 * j + 16);
+#pragma unroll
+        for (int s = 0; s < STEPS; ++s) smooth8(lds_u32x4(my_x + slot + 512 * s), rl0, rl1, xh[s]);
+      }
+      slot_before = slot;
+      slot = slot + stage_bytes == kStages * stage_bytes ? 0u : slot + stage_bytes;
+      if constexpr (R > 0) {
+        const int it = g - g_begin, b = it % kXhBuffers;
+        ok = __all_sync(0xffffffffu, bounded_wait<0, 6>(bar_xh_empty + 8 * b, ((it / kXhBuffers) & 1u) ^ 1u, env, kErrEpilogueWait));
+        if (!ok) break;
+#pragma unroll
+        for (int s = 0; s < STEPS; ++s) {
+          uint4 v;
+          v.x = pack_bf16x2(xh[s][0], xh[s][1]), v.y = pack_bf16x2(xh[s][2], xh[s][3]);
+          v.z = pack_bf16x2(xh[s][4], xh[s][5]), v.w = pack_bf16x2(xh[s][6], xh[s][7]);
+          sts_u32x2(xh_off[s] + b * xh_tile, v.x, v.y);
+          sts_u32x2((xh_off[s] ^ 32u) + b * xh_tile, v.z, v.w);
+        }
+      }
+      // After the scale chain, so that the fence finds its stores done.
+      auto publish_xh = [&] {
+        if constexpr (R > 0) {
+          fence_proxy_async_smem();
+          __syncwarp();
+          mbar_arrive_if(lane == 0 ? 1u : 0u, bar_xh_full + 8 * ((g - g_begin) % kXhBuffers));
+        }
+      };
+      if constexpr (FORMAT == kCodesMxfp4) {
+        float a[STEPS];
+#pragma unroll
+        for (int s = 0; s < STEPS; ++s) a[s] = absmax_lanes<4, false>(absmax8<false>(xh[s]));
+        publish_xh();
+#pragma unroll
+        for (int s = 0; s < STEPS; ++s) {
+          const uint32_t field = (__float_as_uint(__fmul_rn(rho, a[s])) >> 23) & 0xffu;   // exponent of the clip threshold (Eq. 8)
+          const uint32_t ex = field > 2u ? field - 2u : 0u;                            // minus the exponent of E2M1's top binade
+          const float inv = __uint_as_float((254u - ex) << 23);                        // 2^(127 - ex): exact scaling
+          float v[8];
+#pragma unroll
+          for (int e = 0; e < 8; e += 2) {
+            const float2 z = __fmul2_rn(make_float2(xh[s][e], xh[s][e + 1]), make_float2(inv, inv));
+            v[e] = z.x;
+            v[e + 1] = z.y;
+          }
+          const uint32_t w = e2m1x8(v);
+          if (row_ok[s]) {
+            *reinterpret_cast<uint32_t*>(code_base + (code_off[s] + 32u * g)) = w;
+            if ((j & 3) == 0) scale_base[scale_off[s] + ((g >> 1) * 512u + (g & 1) * 2u)] = static_cast<uint8_t>(ex);
+          }
+        }
+      } else {
+        // Two steps share the scale arithmetic: even lanes derive the first row's, odd lanes the second's.
+        float s_mine[STEPS], is_mine[STEPS], is[STEPS];
+        bool ordinary = true;
+        uint32_t u[STEPS][4];
+        {
+          float a[STEPS];
+#pragma unroll
+          for (int s = 0; s < STEPS; ++s) a[s] = absmax_lanes<8, true>(absmax8<true>(xh[s]));
+#pragma unroll
+          for (int s = 0; s < STEPS; s += 2) {
+            const float x = __fmul_rn(rho, STEPS > 1 && (j & 1) ? a[s + 1 < STEPS ? s + 1 : s] : a[s]);
+            ordinary = ordinary && x >= x_min && x <= kOrdinaryMax;
+            group_scale_ordinary(x, s_mine[s], is_mine[s]);
+          }
+        }
+        publish_xh();
+        auto share = [&] {
+#pragma unroll
+          for (int s = 0; s < STEPS; s += 2) {
+            is[s] = is_mine[s];
+            if constexpr (STEPS > 1) {
+              const float is_other = __shfl_xor_sync(0xffffffffu, is_mine[s], 1);
+              is[s] = (j & 1) ? is_other : is_mine[s];
+              is[s + 1] = (j & 1) ? is_mine[s] : is_other;
+            }
+          }
+        };
+        if (__all_sync(0xffffffffu, ordinary)) {
+          share();
+#pragma unroll
+          for (int s = 0; s < STEPS; ++s) quantize8_ordinary(xh[s], is[s], p.one, u[s]);
+        } else {   // an empty group, or magnitudes at the ends of FP32's range, or no numbers at all
+          float a[STEPS];
+#pragma unroll
+          for (int s = 0; s < STEPS; ++s) a[s] = absmax_lanes<8, false>(absmax8<false>(xh[s]));
+#pragma unroll
+          for (int s = 0; s < STEPS; s += 2)
+            group_scale(__fmul_rn(rho, STEPS > 1 && (j & 1) ? a[s + 1 < STEPS ? s + 1 : s] : a[s]), s_mine[s], is_mine[s]);
+          share();
+#pragma unroll
+          for (int s = 0; s < STEPS; ++s) quantize8(xh[s], is[s], u[s]);
+        }
+#pragma unroll
+        for (int s = 0; s < STEPS; ++s) {
+          const uint2 w = FORMAT == kCodesE4M3 ? e4m3_of_codes(u[s]) : int8_of_codes(u[s]);
+          uint8_t* const dst = code_base + (code_off[s] + 64u * g);
+          if (FORMAT == kCodesInt8 && (reinterpret_cast<uintptr_t>(p.codes) & 7) != 0) {   // a caller's buffer on any boundary
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+              if (row_ok[s]) dst[e] = static_cast<uint8_t>((e < 4 ? w.x : w.y) >> (8 * (e & 3)));
+          } else if (row_ok[s]) {
+            *reinterpret_cast<uint2*>(dst) = w;
+          }
+        }
+#pragma unroll
+        for (int s = 0; s < STEPS; s += 2) {
+          if (j < (STEPS > 1 ? 2 : 1) && (STEPS > 1 && j == 1 ? row_ok[s + 1 < STEPS ? s + 1 : s] : row_ok[s])) {
+            const float sc = s_mine[s];
+            const size_t row = row0 + tile_row + 4 * s + (STEPS > 1 ? 4 * j : 0);
+            if constexpr (FORMAT == kCodesInt8) {
+              p.scales[row * G + g] = sc;
+            } else {
+              *reinterpret_cast<uint2*>(scale_base + (scale_off[s] + ((g >> 1) * 2048u + (g & 1) * 8u))) = sop_slots_activation(sc);
+              if (p.scales != nullptr) p.scales[static_cast<size_t>(g) * p.scales_ld + row] = sc;   // for the parity tap
+            }
+          }
+        }
+      }
+    }
+    cp_async_wait<0>();
+    // The GEMM's CTAs may come in now, as room allows.  (The GEMM itself lets nobody in before its end: the next forward's
+    // activation CTAs then sat beside it, 78 -> 84 us at 1560 x 5120 -> 13824 MXFP4.)
+    grid_dependency_launch();
+    if constexpr (R > 0) {
+      // T: TMEM lane = row of the tile; warp w reads lanes 32 w .. 32 w + 31.
+      if (32 * warp < cta_rows && warp < 4) {
+        const bool any = g_begin < g_end;
+        if (gridDim.y > 1) cluster_wait();
+        if (ok && any) ok = __all_sync(0xffffffffu, bounded_wait<0, 6>(bar_t, 0u, env, kErrEpilogueWait));
+        tc_fence_after_sync();
+        const int r = 32 * warp + lane, row = row0 + r;
+#pragma unroll
+        for (int c = 0; c < R; c += 16) {
+          uint32_t v[16];
+          if (any) {
+            tmem_ld_32x32b_x16(tmem + (static_cast<uint32_t>(32 * warp) << 16) + c, v);
+            tmem_wait_ld();
+          } else {
+#pragma unroll
+            for (int e = 0; e < 16; ++e) v[e] = 0u;
+          }
+          if (gridDim.y == 1) {
+            if (ok && r < rows) {
+#pragma unroll
+              for (int e = 0; e < 16; e += 2)
+                store_t_pair(p.t_hilo + static_cast<size_t>(row) * (2 * R), R, c + e, __uint_as_float(v[e]), __uint_as_float(v[e + 1]));
+            }
+          } else if (ok && r < rows) {
+            const uint32_t owner = r / rows_each, at = pushed + ((blockIdx.y * rows_each + r - owner * rows_each) * R + c) * 4;
+            const uint32_t to = map_to_cta(at, owner), bar = map_to_cta(bar_push, owner);
+#pragma unroll
+            for (int e = 0; e < 16; e += 4) st_async_u32x4(to + 4 * e, make_uint4(v[e], v[e + 1], v[e + 2], v[e + 3]), bar);
+          }
+        }
+        tc_fence_before_sync();
+      }
+    }
   }
-  int stage = 0;
-  for (int g = g_begin; g < g_end; ++g) {
-    // This thread's copies for group g have landed; after the barrier so have everyone's, and every warp
-    // has finished group g - 1, whose ring slot the prefetch below overwrites.
-    asm volatile("cp.async.wait_group %0;" ::"n"(kStages - 2) : "memory");
+  if constexpr (R > 0) {
+    if (gridDim.y > 1) {
+      if (!(warp < 4 && 32 * warp < cta_rows)) cluster_wait();
+      cluster_arrive();
+      if (warp < warps && rows_mine > 0 &&
+          __all_sync(0xffffffffu, bounded_wait<0, 6>(bar_push, 0u, env, kErrEpilogueWait))) {
+        // the partial sums in split order, four columns per thread
+        for (int i = threadIdx.x; i < rows_mine * (R / 4); i += 32 * warps) {
+          const int r = i / (R / 4), q = i - r * (R / 4);
+          const uint32_t at = pushed + 16 * i, pitch = rows_each * (R * 4);
+          float4 t = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll 4
+          for (uint32_t c = 0; c < gridDim.y; ++c) {
+            const float4 v = lds_f32x4(at + c * pitch);
+            t.x += v.x, t.y += v.y, t.z += v.z, t.w += v.w;
+          }
+          uint16_t* dst = p.t_hilo + static_cast<size_t>(row0 + blockIdx.y * rows_each + r) * (2 * R);
+          store_t_pair(dst, R, 4 * q, t.x, t.y);
+          store_t_pair(dst, R, 4 * q + 2, t.z, t.w);
+        }
+      }
+      cluster_wait();   // nobody leaves while its shared memory may still be written
+    }
+    tc_fence_before_sync();
     __syncthreads();
-    {
-      int pstage = stage + kStages - 1;
-      if (pstage >= kStages) pstage -= kStages;
-      if (g + kStages - 1 < g_end) issue(g + kStages - 1, pstage);
-      asm volatile("cp.async.commit_group;" ::: "memory");
-    }
-    const uint4* slot = &xring[warp][stage][0][lane];
-    const uint4 ca0 = slot[0], ca1 = slot[32], cb0 = slot[64], cb1 = slot[96];
-    const float4* rl = reinterpret_cast<const float4*>(&lring[stage][coff]);
-    const float4 l0 = rl[0], l1 = rl[1], l4 = rl[4], l5 = rl[5];
-    float xhA[16], xhB[16];
-    smooth8(ca0, l0, l1, xhA);
-    smooth8(ca1, l4, l5, xhA + 8);
-    smooth8(cb0, l0, l1, xhB);
-    smooth8(cb1, l4, l5, xhB + 8);
-
-    if constexpr (FORMAT == kCodesMxfp4) {
-      // `scales` is the scale-byte workspace here: per 128-row block and per 4 scale blocks (128 channels) one
-      // 512-byte atom, byte (row % 32) * 16 + (row % 128 / 32) * 4 + (scale block % 4); scales_ld = atoms per row block.
-      uint32_t loA, hiA, loB, hiB;
-      const uint32_t exA = mxfp4_block16(xhA, rho, loA, hiA), exB = mxfp4_block16(xhB, rho, loB, hiB);
-      uint8_t* ca = codes + static_cast<size_t>(rowA) * (K >> 1) + 32 * g + (coff >> 1);
-      uint8_t* cb = codes + static_cast<size_t>(rowB) * (K >> 1) + 32 * g + (coff >> 1);
-      if (okA) {
-        *reinterpret_cast<uint32_t*>(ca) = loA;
-        *reinterpret_cast<uint32_t*>(ca + 8) = hiA;
-      }
-      if (okB) {
-        *reinterpret_cast<uint32_t*>(cb) = loB;
-        *reinterpret_cast<uint32_t*>(cb + 8) = hiB;
-      }
-      if ((qj & 1) == 0) {
-        uint8_t* sf = reinterpret_cast<uint8_t*>(scales);
-        const int sb = 2 * g + (qj >> 1);  // scale block of this lane's channels
-        const size_t atom_col = static_cast<size_t>(sb >> 2) * 512 + (sb & 3);
-        if (okA) sf[(static_cast<size_t>(rowA >> 7) * scales_ld) * 512 + atom_col + (rowA & 31) * 16 + ((rowA & 127) >> 5) * 4] = static_cast<uint8_t>(exA);
-        if (okB) sf[(static_cast<size_t>(rowB >> 7) * scales_ld) * 512 + atom_col + (rowB & 31) * 16 + ((rowB & 127) >> 5) * 4] = static_cast<uint8_t>(exB);
-      }
-    } else {
-    // Even lanes of the quad derive row A's scale, odd lanes row B's; one shuffle shares the reciprocals.
-    const float aA = quad_absmax16(xhA), aB = quad_absmax16(xhB);
-    float s_mine, is_mine;
-    group_scale(rho, (qj & 1) ? aB : aA, s_mine, is_mine);
-    const float is_other = __shfl_xor_sync(0xffffffffu, is_mine, 1);
-    const float isA = (qj & 1) ? is_other : is_mine, isB = (qj & 1) ? is_mine : is_other;
-    if constexpr (FORMAT == kCodesE4M3) {
-      const uint4 bA = quantize16_bytes(xhA, isA);
-      const uint4 bB = quantize16_bytes(xhB, isB);
-      uint8_t* ca = codes + static_cast<size_t>(rowA) * K + 64 * g + coff;
-      uint8_t* cb = codes + static_cast<size_t>(rowB) * K + 64 * g + coff;
-      if (okA) {
-        *reinterpret_cast<uint2*>(ca) = make_uint2(bA.x, bA.y);
-        *reinterpret_cast<uint2*>(ca + 16) = make_uint2(bA.z, bA.w);
-      }
-      if (okB) {
-        *reinterpret_cast<uint2*>(cb) = make_uint2(bB.x, bB.y);
-        *reinterpret_cast<uint2*>(cb + 16) = make_uint2(bB.z, bB.w);
-      }
-    } else {
-      const uint2 wA = quantize16(xhA, isA);
-      const uint2 wB = quantize16(xhB, isB);
-      const size_t cpitch = static_cast<size_t>(K >> 1);
-      if (okA) *reinterpret_cast<uint2*>(codes + rowA * cpitch + 32 * g + 8 * qj) = wA;
-      if (okB) *reinterpret_cast<uint2*>(codes + rowB * cpitch + 32 * g + 8 * qj) = wB;
-    }
-    // Scales are stored group-major ([G][scales_ld]): kernel 2 fetches a (2 groups x 128 rows) block by TMA.
-    if (qj == 0 && okA) scales[static_cast<size_t>(g) * scales_ld + rowA] = s_mine;
-    if (qj == 1 && okB) scales[static_cast<size_t>(g) * scales_ld + rowB] = s_mine;
-    if (a_sop != nullptr && ((qj == 0 && okA) || (qj == 1 && okB))) {
-      // The scale once more, as four BF16 slots of the operand from which the GEMM's tensor core forms sx * sw:
-      // 2 KiB shared-memory images per (128 rows, 2 groups), [8-row group][8 rows][group parity][8 bytes].
-      const int row = qj == 0 ? rowA : rowB;
-      const size_t image = static_cast<size_t>(row >> 7) * ((G + 1) >> 1) + (g >> 1);
-      a_sop[image * 256 + ((row & 127) >> 3) * 16 + (row & 7) * 2 + (g & 1)] = sop_slots_activation(s_mine);
-    }
-    }
-
-    if constexpr (NT > 0) {
-      // Fragment storage: [i][n-tile pair][lane] as uint4 = (b0, b1) of n-tile 2p, (b0, b1) of n-tile 2p + 1.
-      const uint4* lf = &fring[stage][lane];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        uint32_t a[4];
-        a[0] = pack_bf16x2(xhA[4 * i], xhA[4 * i + 1]);
-        a[1] = pack_bf16x2(xhB[4 * i], xhB[4 * i + 1]);
-        a[2] = pack_bf16x2(xhA[4 * i + 2], xhA[4 * i + 3]);
-        a[3] = pack_bf16x2(xhB[4 * i + 2], xhB[4 * i + 3]);
-#pragma unroll
-        for (int np = 0; np < NT / 2; ++np) {
-          const uint4 b = lf[(i * (NT / 2) + np) * 32];
-          mma_bf16_16816(acc[2 * np], a, b.x, b.y);
-          mma_bf16_16816(acc[2 * np + 1], a, b.z, b.w);
-        }
-      }
-    }
-    if (++stage == kStages) stage = 0;
-  }
-
-  // The GEMM's CTAs may come in now, as room allows.  (Letting them in from the start takes shared memory from nobody but
-  // measured the same; the GEMM itself lets nobody in before its end: the next forward's activation CTAs then sat beside
-  // it, 78 -> 84 us at 1560 x 5120 -> 13824 MXFP4.)
-  grid_dependency_launch();
-  if constexpr (NT > 0) {
-    // Each warp owns its 16 rows over all of K (or over its split of K): T, or its partial sum, is complete in
-    // the accumulators.  Unsplit: store it as a BF16 high part and the BF16 rounding of the remainder
-    // ([T_hi | T_lo], two values per 32-bit store).
-    if (gridDim.y == 1) {
-#pragma unroll
-      for (int nt = 0; nt < NT; ++nt) {
-        const int c = 8 * nt + 2 * qj;
-        if (okA) store_t_pair(t_hilo + static_cast<size_t>(rowA) * (2 * R), R, c, acc[nt][0], acc[nt][1]);
-        if (okB) store_t_pair(t_hilo + static_cast<size_t>(rowB) * (2 * R), R, c, acc[nt][2], acc[nt][3]);
-      }
-    } else {
-      // Split: the CTA's partial sums replace the rings in shared memory, then every CTA of the cluster adds up its
-      // share of the tile over all splits, in split order.
-      float* tile = reinterpret_cast<float*>(quant_smem);   // [16 WARPS rows][R]
-      static_assert(16 * R * 4 <= kStages * 4 * 32 * 16, "a warp's partial sums fit its activation ring");
-      __syncthreads();
-#pragma unroll
-      for (int nt = 0; nt < NT; ++nt) {
-        const int c = 8 * nt + 2 * qj;
-        *reinterpret_cast<float2*>(tile + (16 * warp + qi) * R + c) = make_float2(acc[nt][0], acc[nt][1]);
-        *reinterpret_cast<float2*>(tile + (16 * warp + qi + 8) * R + c) = make_float2(acc[nt][2], acc[nt][3]);
-      }
-      cluster_sync_all();
-      const uint32_t tile_addr = smem_u32(tile);
-      const int rows = min(16 * WARPS, M - static_cast<int>(blockIdx.x) * 16 * WARPS);
-      for (int i = blockIdx.y * (32 * WARPS) + threadIdx.x; i < rows * (R / 2); i += gridDim.y * (32 * WARPS)) {
-        float t0 = 0.0f, t1 = 0.0f;
-        for (uint32_t s = 0; s < gridDim.y; ++s) {
-          const float2 v = ld_cluster_f32x2(map_to_cta(tile_addr + 8 * i, s));
-          t0 += v.x;
-          t1 += v.y;
-        }
-        const int row = i / (R / 2), c = 2 * (i - row * (R / 2));
-        store_t_pair(t_hilo + (static_cast<size_t>(blockIdx.x) * (16 * WARPS) + row) * (2 * R), R, c, t0, t1);
-      }
-      cluster_sync_all();   // nobody leaves while its shared memory is still being read
+    drain_after_abort(&s_abort_word);
+    if (warp == warps) {
+      tc_fence_after_sync();
+      tmem_dealloc(tmem, kTmemCols);
     }
   }
 }
@@ -504,15 +657,47 @@ static __global__ void t_split_kernel(const float* __restrict__ t32, int M, int 
   t_hilo[row * 2 * r + r + c] = *reinterpret_cast<const uint16_t*>(&lo);
 }
 
-// Number of K splits for a launch of `row_ctas` row blocks over G groups on a device with `sms` SMs: enough CTAs
-// for about three per SM, at most kMaxKSplits (the portable cluster size).
-constexpr int kMaxKSplits = 8;
-inline int quantize_k_splits(int row_ctas, int G, int sms) {
-  if (row_ctas >= 2 * sms) return 1;
-  int s = (3 * sms + row_ctas - 1) / row_ctas;
-  if (s > kMaxKSplits) s = kMaxKSplits;
-  if (s > G) s = G;
-  return s < 1 ? 1 : s;
+// How a launch divides M rows x G groups.  fitting_clusters[k]: clusters of k CTAs that run at a time, one CTA to an SM.
+struct QuantizePlan {
+  int steps, warps, splits;   // a CTA owns 4 steps warps rows and a 1 / splits share of the groups
+};
+constexpr int kMaxKSplits = 16;
+inline QuantizePlan quantize_plan(int M, int G, int r, int sms, const int* fitting_clusters, bool expand) {
+  const int few = 448;   // rows up to which 2 steps per warp beat 4
+  if (r == 0) {
+    // The splits are independent CTAs.  About five to an SM at any size, so that no SM is left with a CTA more than others:
+    // 32760 x 5120 in 256 CTAs of 128 rows 105.7 us, in 768 95.1 us.
+    const int steps = M <= few ? 2 : 4, per_warp = 4 * steps;
+    const int warps = M < kQuantWarps * per_warp ? (M + per_warp - 1) / per_warp : kQuantWarps;
+    const int splits = (expand ? sms + sms / 4 : 5 * sms) / ((M + per_warp * warps - 1) / (per_warp * warps));
+    return {steps, warps, splits < 1 || G < 4 ? 1 : (splits > G / 2 ? G / 2 : splits)};
+  }
+  // Beside an expansion, which takes longer than the activations and wants its share of the machine from the start: smaller
+  // CTAs, two to an SM, about one per SM in all.  Forwards of 5120 -> 5120: 700 rows, r = 64 60.0 -> 51.2 us; 1560, r = 64
+  // 96.8 -> 90.3; 4097, r = 96 204 -> 194.
+  if (expand && M > few && M <= 34 * 128) {
+    const int k = M <= 1024 ? 8 : 4, clusters = k == 8 ? 16 : 33, warps = (M + 8 * clusters - 1) / (8 * clusters);
+    if (k <= G / 2) return {2, warps < kQuantWarps ? warps : kQuantWarps, k};
+  }
+  // The splits of a row block form a cluster; with the partial sums of T a CTA's shared memory leaves room for one per SM,
+  // and a cluster stays within a GPC (of 16 SMs at least).  The most splits that still run all row blocks at once, and
+  // the fewest warps that cover the rows: 1560 x 5120, r = 32, in 14 clusters of 8 CTAs of 7 warps 12.0 us, of 4 CTAs 15.9 us,
+  // not split 57 us; 32760 x 5120 split in two 152 us, not split 115 us.
+  for (int k = kMaxKSplits; k > 1; k = k > 8 ? 8 : k - 1) {
+    const int clusters = k > 8 ? 7 : fitting_clusters[k];
+    const int steps = k > 8 && M <= few ? 2 : 4, per_warp = 4 * steps;
+    if (clusters > 0 && k <= G / 2 && M <= clusters * kQuantWarps * per_warp)
+      return {steps, (M + clusters * per_warp - 1) / (clusters * per_warp), k};
+  }
+  // Not split, two CTAs per SM: the number of warps for which the busiest SM has the fewest rows.  32760 rows: 256 CTAs of 8
+  // warps leave 40 SMs with one, 293 of 7 fill 146.5: 120.3 -> 114.7 us at K = 5120, r = 32.
+  QuantizePlan best = {4, kQuantWarps, 1};
+  int least = 1 << 30;
+  for (int w = kQuantWarps; w >= 4; --w) {
+    const int ctas = (M + 16 * w - 1) / (16 * w), rows = (ctas + sms - 1) / sms * w;
+    if (rows < least) least = rows, best.warps = w;
+  }
+  return best;
 }
 
 }  // namespace w4a4

@@ -46,27 +46,13 @@ __global__ void pack_weight_kernel(const int8_t* __restrict__ q, uint8_t* __rest
   *reinterpret_cast<uint4*>(out + static_cast<size_t>(n) * (K >> 1) + 16 * c) = make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-// L1 [K, r] BF16 -> B fragments of mma.sync m16n8k16 in the K order the activation kernel uses,
-// stored [group][i][n-tile pair][lane][n-tile of the pair] so that one 16-byte load feeds two MMAs.
-__global__ void l1_fragment_kernel(const uint16_t* __restrict__ L1, uint2* __restrict__ out, int K, int r) {
-  const int NT = r / 8;
-  const size_t total = static_cast<size_t>(K / 64) * 4 * NT * 32;
+// L1 [K, r] BF16 -> [r, K]: the K-major B operand of the down-projection's tensor-core product; `xh_order`: each group's channels
+// in the order of kernel 1's A operand.
+__global__ void transpose_l1_kernel(const uint16_t* __restrict__ l1, uint16_t* __restrict__ out, int K, int r, bool xh_order) {
   const size_t idx = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (idx >= total) return;
-  const int sub = idx & 1;             // n-tile inside the pair
-  const int lane = (idx >> 1) & 31;
-  const int np = (idx >> 6) % (NT / 2);
-  const int i = ((idx >> 6) / (NT / 2)) & 3;
-  const int g = (idx >> 6) / (NT / 2) / 4;
-  const int nt = 2 * np + sub;
-  const int j = lane & 3, n = 8 * nt + (lane >> 2);
-  uint16_t v[4];
-  for (int e = 0; e < 4; ++e) {
-    const int ch = 64 * g + l1_fragment_channel(j, 4 * i + e);
-    v[e] = L1[static_cast<size_t>(ch) * r + n];
-  }
-  out[idx] = make_uint2(static_cast<uint32_t>(v[0]) | (static_cast<uint32_t>(v[1]) << 16),
-                        static_cast<uint32_t>(v[2]) | (static_cast<uint32_t>(v[3]) << 16));
+  if (idx >= static_cast<size_t>(K) * r) return;
+  const int k = static_cast<int>(idx / r), c = static_cast<int>(idx % r);
+  out[static_cast<size_t>(c) * K + (xh_order ? (k & ~63) + xh_position(k & 63) : k)] = l1[idx];
 }
 
 // L2 [r, N] BF16 -> [N, 2r]: the transposed factor twice, matching the [T_hi | T_lo] split of T.
@@ -126,10 +112,10 @@ struct ExpertData {
   float* wscale = nullptr;     // [G, N]
   uint8_t* b_sop = nullptr;    // weight scale operands of the scale MMA: [N/128][ceil(G/2)][4096]
   float* rlam = nullptr;       // [K]
-  uint2* l1frag = nullptr;
+  uint16_t* l1q = nullptr;     // L1 transposed, BF16 [r, K], each group in the order of kernel 1's operand
   uint16_t* l2dup = nullptr;   // [N, 2r]
   float* bias = nullptr;       // [N] or null
-  CUtensorMap tmL2, tmSopB;
+  CUtensorMap tmL2, tmSopB, tmL1;
 };
 
 struct w4a4_layer {
@@ -148,7 +134,7 @@ void free_expert(ExpertData& e) {
   cudaFree(e.wscale);
   cudaFree(e.b_sop);
   cudaFree(e.rlam);
-  cudaFree(e.l1frag);
+  cudaFree(e.l1q);
   cudaFree(e.l2dup);
   cudaFree(e.bias);
   e = ExpertData();
@@ -169,20 +155,32 @@ w4a4_status_t check_forward_args(w4a4_handle_t h, const void* X, int M, int expe
   return W4A4_OK;
 }
 
-// Kernel 1's launch: row blocks x K splits (a cluster per row block when K is split), plus the CTAs that expand weights.
+// Kernel 1's launch: row blocks x K splits (a cluster per row block when K is split and there is a low-rank branch), plus
+// the CTAs that expand weights.
+template <int R, int FORMAT, int STEPS, int MINB>
+cudaError_t launch_quantize_steps(int num_sms, cudaStream_t stream, const CUtensorMap& tmL1, QuantizeParams p, const QuantizePlan& plan) {
+  const int warps = plan.warps, splits = plan.splits;
+  const int threads = quantize_threads(R, warps), cta_rows = quantize_rows(STEPS, warps);
+  const int row_ctas = (p.M + cta_rows - 1) / cta_rows;
+  const size_t smem = quantize_smem_bytes(R, STEPS, warps, splits);
+  p.expand.first_cta = row_ctas;
+  if (smem > 48 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(quantize_kernel<R, FORMAT, STEPS, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    if (e != cudaSuccess) return e;
+  }
+  if (R > 0 && splits > 8) {
+    const cudaError_t e = cudaFuncSetAttribute(quantize_kernel<R, FORMAT, STEPS, MINB>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+  }
+  const OverlappedLaunch l(dim3(row_ctas + (expand_ctas(p.expand.chunks, threads, num_sms) + splits - 1) / splits, splits), dim3(threads), smem, stream,
+                           dim3(1, R > 0 ? splits : 1));
+  return cudaLaunchKernelEx(&l.cfg, quantize_kernel<R, FORMAT, STEPS, MINB>, tmL1, p);
+}
 template <int R, int FORMAT>
-cudaError_t launch_quantize_kernel(int num_sms, cudaStream_t stream, const uint16_t* x, int M, int K, const float* rlam,
-                                   const float* clip_table, int clip_index, const uint2* l1frag, uint8_t* codes,
-                                   float* scales, int scales_ld, uint16_t* t_hilo, uint2* a_sop, ExpandJob job) {
-  constexpr int kWarps = quantize_warps(R);
-  const int row_ctas = (M + kQuantRows * kWarps - 1) / (kQuantRows * kWarps);
-  const int splits = quantize_k_splits(row_ctas, K / 64, num_sms);
-  const uint32_t per_cta = 32 * kWarps * kExpandUnroll * splits;
-  job.first_cta = row_ctas;
-  const OverlappedLaunch l(dim3(row_ctas + (job.chunks + per_cta - 1) / per_cta, splits), dim3(32 * kWarps), quantize_smem_bytes(R),
-                           stream, dim3(1, splits));
-  return cudaLaunchKernelEx(&l.cfg, quantize_kernel<R, kWarps, FORMAT>, x, M, K, rlam, clip_table, clip_index, l1frag, codes,
-                            scales, scales_ld, t_hilo, a_sop, job);
+cudaError_t launch_quantize_kernel(const w4a4_ctx* ctx, cudaStream_t stream, const CUtensorMap& tmL1, const QuantizeParams& p) {
+  const QuantizePlan plan = quantize_plan(p.M, p.K / 64, R, ctx->num_sms, ctx->gemm_clusters, p.expand.chunks > 0);
+  if (plan.steps == 4) return launch_quantize_steps<R, FORMAT, 4, 2>(ctx->num_sms, stream, tmL1, p, plan);
+  return launch_quantize_steps<R, FORMAT, 2, 2>(ctx->num_sms, stream, tmL1, p, plan);
 }
 
 // Index of (expert, this layer, bin) in a clip table (Sec. III-C: one ratio per expert, layer and timestep bin).
@@ -198,19 +196,30 @@ ExpandJob expand_job(const w4a4_layer* h, int expert_id) {
 
 // Kernel 1 with the ratio read from clip_table[clip_index]; with `expand`, its launch also rewrites the context's byte
 // image with the expert's weights.
+// `scales`: also store the FP32 group scales (the parity tap; the GEMM reads them from the scale operands).
 w4a4_status_t launch_quantize_at(w4a4_handle_t h, const void* X, int M, int expert_id, const float* clip_table,
-                                 int clip_index, bool expand, cudaStream_t stream) {
+                                 int clip_index, bool expand, cudaStream_t stream, float* scales = nullptr) {
   if (M == 0) return W4A4_OK;
   w4a4_ctx* ctx = h->ctx;
   const ExpertData& e = h->experts[expert_id];
   ExpandJob job;
   if (expand) job = expand_job(h, expert_id);
-  const uint16_t* x = static_cast<const uint16_t*>(X);
-  uint2* a_sop = reinterpret_cast<uint2*>(ctx->a_sop);
+  QuantizeParams p = {};
+  p.X = static_cast<const uint16_t*>(X);
+  p.M = M;
+  p.K = h->K;
+  p.rlam = e.rlam;
+  p.clip_table = clip_table;
+  p.clip_index = clip_index;
+  p.codes = ctx->codes;
+  p.scales = scales;
+  p.scales_ld = ctx->scales_ld;
+  p.t_hilo = ctx->t_hilo;
+  p.a_sop = reinterpret_cast<uint2*>(ctx->a_sop);
+  p.expand = job;
+  p.err = ctx->d_err;
   cudaError_t le;
-#define W4A4_LAUNCH_Q(R)                                                                                          \
-  le = launch_quantize_kernel<R, kCodesE4M3>(ctx->num_sms, stream, x, M, h->K, e.rlam, clip_table, clip_index, e.l1frag, \
-                                             ctx->codes, ctx->scales, ctx->scales_ld, ctx->t_hilo, a_sop, job)
+#define W4A4_LAUNCH_Q(R) le = launch_quantize_kernel<R, kCodesE4M3>(ctx, stream, h->r > 0 ? e.tmL1 : h->tmSopA, p)
   switch (h->r) {
     case 0: W4A4_LAUNCH_Q(0); break;
     case 16: W4A4_LAUNCH_Q(16); break;
@@ -225,8 +234,8 @@ w4a4_status_t launch_quantize_at(w4a4_handle_t h, const void* X, int M, int expe
 }
 
 w4a4_status_t launch_quantize(w4a4_handle_t h, const void* X, int M, int expert_id, int bin, const float* clip_table,
-                              bool expand, cudaStream_t stream) {
-  return launch_quantize_at(h, X, M, expert_id, clip_table, clip_table_index(h, expert_id, bin), expand, stream);
+                              bool expand, cudaStream_t stream, float* scales = nullptr) {
+  return launch_quantize_at(h, X, M, expert_id, clip_table, clip_table_index(h, expert_id, bin), expand, stream, scales);
 }
 
 // Kernel 2; `expand`: preceded by the expansion of the expert's 4-bit weights (false: the context's byte image already
@@ -280,8 +289,7 @@ w4a4_status_t launch_gemm(w4a4_handle_t h, int M, int expert_id, void* Y, cudaSt
   }
   if (expand) {
     const ExpandJob job = expand_job(h, expert_id);
-    const uint32_t per_cta = 256 * kExpandUnroll;
-    expand_weight_kernel<<<(job.chunks + per_cta - 1) / per_cta, 256, 0, stream>>>(job);
+    expand_weight_kernel<<<expand_ctas(job.chunks, 256, ctx->num_sms), 256, 0, stream>>>(job);
   }
   // Persistent: one CTA per SM walks the 128 x 128 tiles.
   const int num_tiles = p.tiles_m * p.tiles_n;
@@ -374,10 +382,6 @@ w4a4_status_t w4a4_ctx_create(int device, int max_M, int max_K, int max_r, w4a4_
       cudaMemset(ctx->t_hilo, 0, static_cast<size_t>(max_M) * 2 * (max_r > 0 ? max_r : 8) * sizeof(uint16_t)) != cudaSuccess)
     st = W4A4_ERR_CUDA;
   if (st == W4A4_OK) {
-    cudaFuncSetAttribute(quantize_kernel<64, quantize_warps(64), kCodesE4M3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         static_cast<int>(quantize_smem_bytes(64)));
-    cudaFuncSetAttribute(quantize_kernel<96, quantize_warps(96), kCodesE4M3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         static_cast<int>(quantize_smem_bytes(96)));
     // The GEMM redistributes its launch's registers: it must have been compiled with as many as it hands out.
     auto prepare_gemm = [](auto* kernel) {
       cudaFuncAttributes a;
@@ -496,7 +500,7 @@ w4a4_status_t w4a4_pack_weights(w4a4_ctx_t ctx, const w4a4_weight_desc_t* d, w4a
     st = dev_alloc(&e.bpacked, static_cast<size_t>(N) * (K / 2), &h->bytes);
     if (st == W4A4_OK) st = dev_alloc(&e.wscale, static_cast<size_t>(G) * N, &h->bytes);
     if (st == W4A4_OK) st = dev_alloc(&e.rlam, static_cast<size_t>(K), &h->bytes);
-    if (st == W4A4_OK && r > 0) st = dev_alloc(&e.l1frag, static_cast<size_t>(G) * 4 * (r / 8) * 32, &h->bytes);
+    if (st == W4A4_OK && r > 0) st = dev_alloc(&e.l1q, static_cast<size_t>(r) * K, &h->bytes);
     if (st == W4A4_OK && r > 0) st = dev_alloc(&e.l2dup, static_cast<size_t>(N) * 2 * r, &h->bytes);
     const float* bias_src = d->bias ? d->bias[ei] : nullptr;
     if (st == W4A4_OK && bias_src) st = dev_alloc(&e.bias, static_cast<size_t>(N), &h->bytes);
@@ -530,8 +534,8 @@ w4a4_status_t w4a4_pack_weights(w4a4_ctx_t ctx, const w4a4_weight_desc_t* d, w4a
       reciprocal_kernel<<<(K + 255) / 256, 256>>>(lam_dev, e.rlam, K);
       pack_weight_kernel<<<dim3((N + 127) / 128, K / 32), 128>>>(q_dev, e.bpacked, K, N, d_bad);
       if (r > 0) {
-        const size_t nf = static_cast<size_t>(G) * 4 * (r / 8) * 32;
-        l1_fragment_kernel<<<static_cast<unsigned>((nf + 255) / 256), 256>>>(l1_dev, e.l1frag, K, r);
+        const size_t nt = static_cast<size_t>(K) * r;
+        transpose_l1_kernel<<<static_cast<unsigned>((nt + 255) / 256), 256>>>(l1_dev, e.l1q, K, r, true);
         const size_t nl = static_cast<size_t>(N) * 2 * r;
         l2_dup_kernel<<<static_cast<unsigned>((nl + 255) / 256), 256>>>(l2_dev, e.l2dup, r, N);
       }
@@ -546,6 +550,10 @@ w4a4_status_t w4a4_pack_weights(w4a4_ctx_t ctx, const w4a4_weight_desc_t* d, w4a
     // Scale operand images as rows of 32-bit words (one row per 128 output channels), fetched in boxes of 1 KiB.
     if (!encode_2d(ctx->encode, &e.tmSopB, CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, e.b_sop, static_cast<uint64_t>((G + 1) / 2) * (kSopBTile / 4),
                    N / kBN, static_cast<uint64_t>((G + 1) / 2) * kSopBTile, 256, 1, CU_TENSOR_MAP_SWIZZLE_NONE))
+      st = W4A4_ERR_CUDA;
+    if (st == W4A4_OK && r > 0 &&
+        !encode_2d(ctx->encode, &e.tmL1, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, e.l1q, K, r, 2 * static_cast<uint64_t>(K), 64, r,
+                   CU_TENSOR_MAP_SWIZZLE_128B))
       st = W4A4_ERR_CUDA;
     if (st == W4A4_OK && r > 0 &&
         !encode_2d(ctx->encode, &e.tmL2, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, e.l2dup, 2 * r, N, 4 * r, 64, kBN,
@@ -750,7 +758,7 @@ w4a4_status_t w4a4_debug_quantize(w4a4_handle_t h, const void* X, int M, int exp
   if (M > 0 && (!codes || !scales)) return W4A4_ERR_INVALID_ARG;
   DeviceGuard guard(h->ctx->device);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  st = launch_quantize(h, X, M, expert_id, timestep_bin, clip_table, false, s);
+  st = launch_quantize(h, X, M, expert_id, timestep_bin, clip_table, false, s, h->ctx->scales);
   if (st != W4A4_OK || M == 0) return st;
   const size_t nc = static_cast<size_t>(M) * h->K;
   decode_codes_kernel<<<static_cast<unsigned>((nc + 255) / 256), 256, 0, s>>>(h->ctx->codes, codes, M, h->K);

@@ -8,14 +8,13 @@ struct MxExpertData {
   uint8_t* bpacked = nullptr;  // [N, K/2] two E2M1 codes per byte
   uint8_t* sfb = nullptr;      // weight scale atoms [N/128][K/128][512]
   float* rlam = nullptr;       // [K]
-  uint2* l1frag = nullptr;
   uint16_t* l2dup = nullptr;   // [N, 2r]
   float* bias = nullptr;       // [N] or null
   CUtensorMap tmB, tmL2;
   CUtensorMap tmBhalf, tmL2half;   // 128-row boxes: what one CTA of a pair fetches (mx_gemm2_kernel)
   CUtensorMap tmSFB;               // scale atoms as 32-bit words: [N/128] rows of K words, boxes of 1 KiB
-  uint16_t* l1t = nullptr;         // L1 transposed, BF16 [r, K]: B operand of the fused producer's T MMA
-  CUtensorMap tmL1T;               // boxes of 64 channels x r/2 rows
+  uint16_t *l1q = nullptr, *l1t = nullptr;   // L1 transposed, BF16 [r, K]: in the order of kernel 1's operand, and as it is
+  CUtensorMap tmL1, tmL1T;         // boxes of 64 channels x r rows (kernel 1), x r/2 rows (the fused producer)
 };
 
 struct w4a4_mx_layer {
@@ -34,9 +33,9 @@ void mx_free_expert(MxExpertData& e) {
   cudaFree(e.bpacked);
   cudaFree(e.sfb);
   cudaFree(e.rlam);
-  cudaFree(e.l1frag);
   cudaFree(e.l2dup);
   cudaFree(e.bias);
+  cudaFree(e.l1q);
   cudaFree(e.l1t);
   e = MxExpertData();
 }
@@ -61,12 +60,20 @@ w4a4_status_t mx_launch_quantize_at(w4a4_mx_handle_t h, const void* X, int M, in
   if (M == 0) return W4A4_OK;
   w4a4_ctx* ctx = h->ctx;
   const MxExpertData& e = h->experts[expert_id];
-  const uint16_t* x = static_cast<const uint16_t*>(X);
-  float* sf = reinterpret_cast<float*>(ctx->mx_sfa);
+  QuantizeParams p = {};
+  p.X = static_cast<const uint16_t*>(X);
+  p.M = M;
+  p.K = h->K;
+  p.rlam = e.rlam;
+  p.clip_table = clip_table;
+  p.clip_index = clip_index;
+  p.codes = ctx->codes;
+  p.scales = reinterpret_cast<float*>(ctx->mx_sfa);
+  p.scales_ld = h->K / 128;
+  p.t_hilo = ctx->t_hilo;
+  p.err = ctx->d_err;
   cudaError_t le;
-#define W4A4_LAUNCH_MXQ(R)                                                                                        \
-  le = launch_quantize_kernel<R, kCodesMxfp4>(ctx->num_sms, stream, x, M, h->K, e.rlam, clip_table, clip_index, e.l1frag, \
-                                              ctx->codes, sf, h->K / 128, ctx->t_hilo, nullptr, ExpandJob())
+#define W4A4_LAUNCH_MXQ(R) le = launch_quantize_kernel<R, kCodesMxfp4>(ctx, stream, h->r > 0 ? e.tmL1 : h->tmA, p)
   switch (h->r) {
     case 0: W4A4_LAUNCH_MXQ(0); break;
     case 16: W4A4_LAUNCH_MXQ(16); break;
@@ -207,7 +214,7 @@ w4a4_status_t w4a4_mx_pack_weights(w4a4_ctx_t ctx, const w4a4_mx_weight_desc_t* 
   h->layer_id = d->layer_id;
   h->act = d->output_activation;
   h->experts.resize(d->num_experts);
-  const int K = d->K, N = d->N, r = d->r, G = K / 64;
+  const int K = d->K, N = d->N, r = d->r;
   const bool dev = d->pointers_on_device != 0;
   w4a4_status_t st = W4A4_OK;
 
@@ -237,9 +244,6 @@ w4a4_status_t w4a4_mx_pack_weights(w4a4_ctx_t ctx, const w4a4_mx_weight_desc_t* 
     if (st == W4A4_OK) st = dev_alloc(&ctx->t_hilo2, static_cast<size_t>(ctx->max_M) * 2 * rr, &ctx->bytes);
     if (st == W4A4_OK && cudaMemset(ctx->t_hilo2, 0, sizeof(uint16_t) * ctx->max_M * 2 * rr) != cudaSuccess) st = W4A4_ERR_CUDA;
 
-    if (st == W4A4_OK)
-      cudaFuncSetAttribute(quantize_kernel<64, quantize_warps(64), kCodesMxfp4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           static_cast<int>(quantize_smem_bytes(64)));
   }
   int* d_bad = nullptr;
   if (st == W4A4_OK) st = dev_alloc(&d_bad, 1, nullptr);
@@ -250,8 +254,8 @@ w4a4_status_t w4a4_mx_pack_weights(w4a4_ctx_t ctx, const w4a4_mx_weight_desc_t* 
     st = dev_alloc(&e.bpacked, static_cast<size_t>(N) * (K / 2), &h->bytes);
     if (st == W4A4_OK) st = dev_alloc(&e.sfb, static_cast<size_t>(N / 128) * (K / 128) * 512, &h->bytes);
     if (st == W4A4_OK) st = dev_alloc(&e.rlam, static_cast<size_t>(K), &h->bytes);
-    if (st == W4A4_OK && r > 0) st = dev_alloc(&e.l1frag, static_cast<size_t>(G) * 4 * (r / 8) * 32, &h->bytes);
     if (st == W4A4_OK && r > 0) st = dev_alloc(&e.l2dup, static_cast<size_t>(N) * 2 * r, &h->bytes);
+    if (st == W4A4_OK && r > 0) st = dev_alloc(&e.l1q, static_cast<size_t>(r) * K, &h->bytes);
     if (st == W4A4_OK && r > 0) st = dev_alloc(&e.l1t, static_cast<size_t>(r) * K, &h->bytes);
     const float* bias_src = d->bias ? d->bias[ei] : nullptr;
     if (st == W4A4_OK && bias_src) st = dev_alloc(&e.bias, static_cast<size_t>(N), &h->bytes);
@@ -277,12 +281,11 @@ w4a4_status_t w4a4_mx_pack_weights(w4a4_ctx_t ctx, const w4a4_mx_weight_desc_t* 
       const size_t ns = static_cast<size_t>(K / 32) * N;
       mx_pack_wscale_kernel<<<static_cast<unsigned>((ns + 255) / 256), 256>>>(x_dev, e.sfb, K, N, d_bad);
       if (r > 0) {
-        const size_t nf = static_cast<size_t>(G) * 4 * (r / 8) * 32;
-        l1_fragment_kernel<<<static_cast<unsigned>((nf + 255) / 256), 256>>>(l1_dev, e.l1frag, K, r);
         const size_t nl = static_cast<size_t>(N) * 2 * r;
         l2_dup_kernel<<<static_cast<unsigned>((nl + 255) / 256), 256>>>(l2_dev, e.l2dup, r, N);
         const size_t nt = static_cast<size_t>(K) * r;
-        mx_transpose_l1_kernel<<<static_cast<unsigned>((nt + 255) / 256), 256>>>(l1_dev, e.l1t, K, r);
+        transpose_l1_kernel<<<static_cast<unsigned>((nt + 255) / 256), 256>>>(l1_dev, e.l1q, K, r, true);
+        transpose_l1_kernel<<<static_cast<unsigned>((nt + 255) / 256), 256>>>(l1_dev, e.l1t, K, r, false);
       }
       if (cudaGetLastError() != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) st = W4A4_ERR_CUDA;
     }
@@ -302,6 +305,10 @@ w4a4_status_t w4a4_mx_pack_weights(w4a4_ctx_t ctx, const w4a4_mx_weight_desc_t* 
     if (st == W4A4_OK &&
         !encode_2d(ctx->encode, &e.tmSFB, CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, e.sfb, K, N / 128, 4 * static_cast<uint64_t>(K), 256,
                    1, CU_TENSOR_MAP_SWIZZLE_NONE))
+      st = W4A4_ERR_CUDA;
+    if (st == W4A4_OK && r > 0 &&
+        !encode_2d(ctx->encode, &e.tmL1, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, e.l1q, K, r, 2 * static_cast<uint64_t>(K), 64, r,
+                   CU_TENSOR_MAP_SWIZZLE_128B))
       st = W4A4_ERR_CUDA;
     if (st == W4A4_OK && r > 0 &&
         !encode_2d(ctx->encode, &e.tmL1T, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, e.l1t, K, r, 2 * static_cast<uint64_t>(K), 64, r / 2,

@@ -451,3 +451,43 @@ def test_shared_tiles_in_the_clip_search():
         assert abs(e - ref) <= 128 * 2.0 ** -24 * ref
     L.close()
     ctx.close()
+
+
+@pytest.mark.parametrize("M,K,r", [
+    (33, 64, 16),        # one group, CTAs of one warp, the last one with one row
+    (448, 2112, 64),     # most rows at two steps per warp; 33 groups over 16 CTAs: the last ones have none
+    (449, 2048, 32),     # fewest rows at four steps per warp
+    (1029, 576, 96),     # nine groups over four CTAs, ragged last row block
+    (1029, 1024, 0),     # no low-rank branch: splits without clusters
+    (9300, 128, 64),     # not split: fewer warps per CTA than eight, T straight from TMEM
+])
+def test_row_and_group_shares_of_the_quantizer(M, K, r):
+    x = gen.make_activations(M, K, outlier_idx=gen.outlier_channels(K, 0.02, 5), outlier_gain=40.0, seed=M)
+    layer = gen.make_layer_direct(K, 128, r, seed=K)
+    rng = np.random.default_rng(M)
+    rows = sorted({0, 1, M // 2, M - 2, M - 1, *range(28, 33), *rng.choice(M, min(M, 200), replace=False).tolist()})
+    run_case(x, [layer], torch.full((1, 1, 1), 0.8, dtype=torch.float32), 0, 0, rows=rows, max_M=M + 3)
+
+
+@pytest.mark.parametrize("rho", [1.0, 0.75, 2.0 ** -11])   # the last one: codes far outside [-8, 7] before the clamp
+def test_groups_outside_the_ordinary_scale_range(rho):
+    # Zero groups, magnitudes near both ends of FP32 and ordinary ones, in one warp and alone: codes and scales bit for bit.
+    M, K = 160, 256
+    x, layer = tiny_inputs(M, K, 128, 0, seed=8)
+    x = x.clone()
+    x[1::8] *= 1e-32
+    x[2::8] *= 1e32
+    x[3::8, 64:128] = 0
+    x[96:128] *= 1e-33
+    x[128:] = 0
+    clip = torch.full((1, 1, 1), rho, dtype=torch.float32)
+    ctx = w4.Context(0, M, K, 0)
+    L = w4.Layer(ctx, [layer.to(DEV)], num_bins=1)
+    codes = torch.empty(M, K, dtype=torch.int8, device=DEV)
+    scales = torch.empty(M, K // G, device=DEV)
+    w4.w4a4_debug_quantize(L.ptr, x.to(DEV), M, 0, 0, clip.to(DEV), codes, scales, None)
+    ctx.check()
+    with np.errstate(all="ignore"):
+        ref = oracle_rows(x, layer, rho)
+    assert np.array_equal(codes.cpu().numpy(), ref["q"])
+    assert np.array_equal(scales.cpu().numpy().view(np.uint32), ref["s"].view(np.uint32))

@@ -149,3 +149,16 @@ def test_mx_full_size_sampled_rows(name):
 def test_mx_tiles_shared_by_a_cluster(M, K, N, r):
     x = gen.make_activations(M, K, outlier_idx=gen.outlier_channels(K, 0.02, 4), outlier_gain=50.0, seed=M)
     run_mx_case(x, [gen.make_layer_mx_direct(K, N, r, seed=K)], torch.full((1, 1, 1), 0.85), 0, 0, max_M=M + 5)
+
+
+@pytest.mark.parametrize("M,K,r", [
+    (33, 256, 16),       # two steps per warp, CTAs of one warp, two splits
+    (449, 2048, 32),     # four steps per warp, clusters of 16
+    (1029, 768, 64),     # clusters of six, ragged last row block
+    (9300, 256, 0),      # no low-rank branch, many row blocks
+])
+def test_mx_row_and_block_shares_of_the_quantizer(M, K, r):
+    x = gen.make_activations(M, K, outlier_idx=gen.outlier_channels(K, 0.02, 4), outlier_gain=50.0, seed=M)
+    rng = np.random.default_rng(M)
+    rows = sorted({0, 1, M // 2, M - 2, M - 1, *range(28, 33), *rng.choice(M, min(M, 200), replace=False).tolist()})
+    run_mx_case(x, [gen.make_layer_mx_direct(K, 128, r, seed=K)], torch.full((1, 1, 1), 0.85), 0, 0, rows=rows, max_M=M + 5)
