@@ -134,8 +134,13 @@ w4a4_status_t mx_launch_gemm(w4a4_mx_handle_t h, int M, int expert_id, void* Y, 
     }
     return W4A4_OK;
   }
-  // CTA pairs (cta_group::2) need at least two row tiles and an even number of CTAs.
-  if (p.tiles_m >= 2 && ctx->num_sms >= 2) {
+  // CTA pairs (cta_group::2) need at least two row tiles and an even number of CTAs.  A wave of pairs takes less time than one of
+  // single CTAs, but single CTAs win where a tile each is about all there is (900 x 5120 -> 5120 25.1 -> 20.7 us, 700 17.6 -> 15.9)
+  // and where they need two waves and pairs three (600 x 5120 -> 13824 31.1 -> 25.1); at 1.22 waves and K = 13824 they lose (43.6 | 45.1),
+  // and with two row tiles the pairs' shared weight reads count (200 x 13824 -> 13824 30.7 | 35.0).
+  const int pair_tiles = (p.tiles_m + 1) / 2 * p.tiles_n, sms = ctx->num_sms;
+  const bool singles = !next && p.tiles_m > 2 && (num_tiles <= sms + sms / 8 || (num_tiles <= 2 * sms && pair_tiles > 2 * (sms / 2)));
+  if (p.tiles_m >= 2 && sms >= 2 && !singles) {
     const int runs = ((p.tiles_m + 1) / 2) * ((p.tiles_n + p.run - 1) / p.run);
     const int ctas = 2 * runs < ctx->num_sms ? 2 * runs : (ctx->num_sms & ~1);
     OverlappedLaunch l(dim3(ctas), block, next ? kMx2FuseSmemBytes : kMx2SmemBytes, stream, dim3(2));

@@ -162,3 +162,13 @@ def test_mx_row_and_block_shares_of_the_quantizer(M, K, r):
     rng = np.random.default_rng(M)
     rows = sorted({0, 1, M // 2, M - 2, M - 1, *range(28, 33), *rng.choice(M, min(M, 200), replace=False).tolist()})
     run_mx_case(x, [gen.make_layer_mx_direct(K, 128, r, seed=K)], torch.full((1, 1, 1), 0.85), 0, 0, rows=rows, max_M=M + 5)
+
+
+@pytest.mark.parametrize("M,K,N,r", [
+    (300, 256, 13824, 32),   # 162 tiles: one of single CTAs each, a few get a second
+    (515, 512, 13824, 0),    # 270 tiles: two waves of single CTAs where pairs would need three
+])
+def test_mx_single_ctas_over_many_row_tiles(M, K, N, r):
+    x = gen.make_activations(M, K, seed=M)
+    rows = sorted({0, 127, 128, 255, 256, M - 1, *range(290, 300)})
+    run_mx_case(x, [gen.make_layer_mx_direct(K, N, r, seed=K)], torch.full((1, 1, 1), 0.85), 0, 0, rows=rows, max_M=M + 5)
