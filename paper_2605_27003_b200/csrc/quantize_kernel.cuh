@@ -122,10 +122,11 @@ __device__ __forceinline__ float absmax_lanes(float a) {
   return a;
 }
 
-// Eq. 8-9 / Eq. 4: s = x / 7 with x = rho * a, and is = 1 / s, both correctly rounded (IEEE); a == 0 -> 0, 0.
-__device__ __forceinline__ void group_scale(float x, float& s, float& is) {
-  s = x > 0.0f ? __fdiv_rn(x, 7.0f) : 0.0f;
-  is = s > 0.0f ? __frcp_rn(s) : 0.0f;
+// Eq. 8-9 / Eq. 4: s = x / 7 with x = rho * a, and is = 1 / s, both correctly rounded (IEEE); a == 0 -> 0, 0.  A threshold that
+// vanishes although the group does not (underflow) has is = inf: the codes are the ends of the range.
+__device__ __forceinline__ void group_scale(float rho, float a, float& s, float& is) {
+  s = a > 0.0f ? __fdiv_rn(__fmul_rn(rho, a), 7.0f) : 0.0f;
+  is = a > 0.0f ? __frcp_rn(s) : 0.0f;
 }
 // The same for kOrdinaryMin <= x <= kOrdinaryMax, where nothing under- or overflows: an approximation corrected by its exact
 // remainder (Markstein, IBM J. Res. Dev. 34, 1990) is the correctly rounded quotient; compared with the two functions above
@@ -539,7 +540,7 @@ quantize_kernel(const __grid_constant__ CUtensorMap tmL1, const QuantizeParams p
           for (int s = 0; s < STEPS; ++s) a[s] = absmax_lanes<8, false>(absmax8<false>(xh[s]));
 #pragma unroll
           for (int s = 0; s < STEPS; s += 2)
-            group_scale(__fmul_rn(rho, STEPS > 1 && (j & 1) ? a[s + 1 < STEPS ? s + 1 : s] : a[s]), s_mine[s], is_mine[s]);
+            group_scale(rho, STEPS > 1 && (j & 1) ? a[s + 1 < STEPS ? s + 1 : s] : a[s], s_mine[s], is_mine[s]);
           share();
 #pragma unroll
           for (int s = 0; s < STEPS; ++s) quantize8(xh[s], is[s], u[s]);

@@ -491,3 +491,33 @@ def test_groups_outside_the_ordinary_scale_range(rho):
         ref = oracle_rows(x, layer, rho)
     assert np.array_equal(codes.cpu().numpy(), ref["q"])
     assert np.array_equal(scales.cpu().numpy().view(np.uint32), ref["s"].view(np.uint32))
+
+
+@pytest.mark.parametrize("rho", [0.75, 0.0, -0.5])
+def test_scales_that_are_no_positive_numbers(rho):
+    # Thresholds that vanish although the group does not (underflow of rho * max / 7, or a ratio of zero) have the reciprocal
+    # 1 / 0 = inf and codes at the ends of the range; a negative ratio mirrors the codes.  Bit for bit, through the handle's
+    # tap and through the entry point without one.
+    M, K = 40, 128
+    x, layer = tiny_inputs(M, K, 128, 0, seed=9)
+    x = torch.where(x == 0, torch.ones_like(x), x)                                              # 0 * inf is no number
+    layer.lam = torch.where(torch.arange(K) < 64, 2.0 ** 27, 1.0).float()
+    x[1::3, :64] = torch.sign(x[1::3, :64]) * (1 + torch.arange(64) % 3) * 2.0 ** -122          # 1 to 3 of FP32's smallest steps
+    ctx = w4.Context(0, M, K, 0)
+    L = w4.Layer(ctx, [layer.to(DEV)], num_bins=1)
+    clip = torch.full((1, 1, 1), rho, dtype=torch.float32, device=DEV)
+    with np.errstate(all="ignore"):
+        ref = oracle_rows(x, layer, rho)
+    assert rho < 0 or ((ref["s"] == 0).any() and np.all(ref["q"][np.repeat(ref["s"] == 0, G, axis=1)] != 0))
+    for call in ("tap", "noalloc"):
+        codes = torch.empty(M, K, dtype=torch.int8, device=DEV)
+        scales = torch.empty(M, K // G, device=DEV)
+        if call == "tap":
+            w4.w4a4_debug_quantize(L.ptr, x.to(DEV), M, 0, 0, clip, codes, scales, None)
+        else:
+            w4.w4a4_quantize_noalloc(x.to(DEV), M, K, layer.lam.to(DEV), clip, 0, codes, scales)
+        ctx.check()
+        assert np.array_equal(codes.cpu().numpy(), ref["q"]), call
+        assert np.array_equal(scales.cpu().numpy().view(np.uint32), ref["s"].view(np.uint32)), call
+    L.close()
+    ctx.close()
