@@ -155,6 +155,31 @@ w4a4_status_t check_forward_args(w4a4_handle_t h, const void* X, int M, int expe
   return W4A4_OK;
 }
 
+// Kernel 1's limits for every plan of a layer, once where the layer is packed.  They belong to the kernel on the device, not to
+// a launch: set per launch, one thread's smaller size would meet another thread's larger launch.
+template <int R, int FORMAT, int STEPS, int MINB>
+bool prepare_quantize_steps() {
+  auto* const kernel = quantize_kernel<R, FORMAT, STEPS, MINB>;
+  const size_t most = quantize_smem_bytes(R, STEPS, kQuantWarps, kMaxKSplits);   // grows with the warps and with the splits
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(most)) == cudaSuccess &&
+         (R == 0 || cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess);
+}
+template <int R, int FORMAT>
+bool prepare_quantize_rank() { return prepare_quantize_steps<R, FORMAT, 4, 2>() && prepare_quantize_steps<R, FORMAT, 2, 2>(); }
+template <int FORMAT>
+w4a4_status_t prepare_quantize(int r) {
+  bool ok = false;
+  switch (r) {
+    case 0: ok = prepare_quantize_rank<0, FORMAT>(); break;
+    case 16: ok = prepare_quantize_rank<16, FORMAT>(); break;
+    case 32: ok = prepare_quantize_rank<32, FORMAT>(); break;
+    case 64: ok = prepare_quantize_rank<64, FORMAT>(); break;
+    case 96: if constexpr (FORMAT == kCodesE4M3) ok = prepare_quantize_rank<96, FORMAT>(); break;
+  }
+  if (!ok) cudaGetLastError();
+  return ok ? W4A4_OK : W4A4_ERR_CUDA;
+}
+
 // Kernel 1's launch: row blocks x K splits (a cluster per row block when K is split and there is a low-rank branch), plus
 // the CTAs that expand weights.
 template <int R, int FORMAT, int STEPS, int MINB>
@@ -162,18 +187,9 @@ cudaError_t launch_quantize_steps(int num_sms, cudaStream_t stream, const CUtens
   const int warps = plan.warps, splits = plan.splits;
   const int threads = quantize_threads(R, warps), cta_rows = quantize_rows(STEPS, warps);
   const int row_ctas = (p.M + cta_rows - 1) / cta_rows;
-  const size_t smem = quantize_smem_bytes(R, STEPS, warps, splits);
   p.expand.first_cta = row_ctas;
-  if (smem > 48 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(quantize_kernel<R, FORMAT, STEPS, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
-  }
-  if (R > 0 && splits > 8) {
-    const cudaError_t e = cudaFuncSetAttribute(quantize_kernel<R, FORMAT, STEPS, MINB>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
-  }
-  const OverlappedLaunch l(dim3(row_ctas + (expand_ctas(p.expand.chunks, threads, num_sms) + splits - 1) / splits, splits), dim3(threads), smem, stream,
-                           dim3(1, R > 0 ? splits : 1));
+  const OverlappedLaunch l(dim3(row_ctas + (expand_ctas(p.expand.chunks, threads, num_sms) + splits - 1) / splits, splits), dim3(threads),
+                           quantize_smem_bytes(R, STEPS, warps, splits), stream, dim3(1, R > 0 ? splits : 1));
   return cudaLaunchKernelEx(&l.cfg, quantize_kernel<R, FORMAT, STEPS, MINB>, tmL1, p);
 }
 template <int R, int FORMAT>
@@ -491,6 +507,7 @@ w4a4_status_t w4a4_pack_weights(w4a4_ctx_t ctx, const w4a4_weight_desc_t* d, w4a
       if (st == W4A4_OK) ctx->b8_bytes = b8_need;
     }
   }
+  if (st == W4A4_OK) st = prepare_quantize<kCodesE4M3>(r);
   int* d_bad = nullptr;
   if (st == W4A4_OK) st = dev_alloc(&d_bad, 1, nullptr);
   if (st == W4A4_OK && cudaMemset(d_bad, 0, sizeof(int)) != cudaSuccess) st = W4A4_ERR_CUDA;

@@ -250,6 +250,7 @@ w4a4_status_t w4a4_mx_pack_weights(w4a4_ctx_t ctx, const w4a4_mx_weight_desc_t* 
     if (st == W4A4_OK && cudaMemset(ctx->t_hilo2, 0, sizeof(uint16_t) * ctx->max_M * 2 * rr) != cudaSuccess) st = W4A4_ERR_CUDA;
 
   }
+  if (st == W4A4_OK) st = prepare_quantize<kCodesMxfp4>(r);
   int* d_bad = nullptr;
   if (st == W4A4_OK) st = dev_alloc(&d_bad, 1, nullptr);
   if (st == W4A4_OK && cudaMemset(d_bad, 0, sizeof(int)) != cudaSuccess) st = W4A4_ERR_CUDA;
