@@ -49,32 +49,11 @@
 #include "fp8_codes.cuh"
 #include "pipeline.cuh"
 #include "ptx.cuh"
+#include "quantize_plan.h"
 
 namespace w4a4 {
 
 constexpr int kCodesInt8 = 0, kCodesE4M3 = 1, kCodesMxfp4 = 2;
-constexpr int kQuantWarps = 8;                               // element-wise warps at most
-constexpr int quantize_rows(int steps, int warps = kQuantWarps) { return 4 * warps * steps; }
-constexpr int quantize_threads(int R, int warps = kQuantWarps) { return 32 * (warps + (R > 0 ? 1 : 0)); }
-constexpr int kL1Stages = 3, kXhBuffers = 2;
-constexpr uint32_t xh_tile_bytes(int steps, int warps) { return quantize_rows(steps, warps) * 128u; }   // rows x 64 channels in BF16
-
-// One stage of the activation ring: what the element-wise warps read for one group, 16 bytes per lane and step and the
-// group's 64 reciprocals once per warp.
-constexpr uint32_t x_stage_bytes(int steps, int warps) { return warps * (steps * 512u + 256u); }
-constexpr int kXStages(int R, int steps) { return steps == 2 ? (R >= 96 ? 3 : 4) : (R == 0 ? 5 : (R <= 64 ? 3 : 2)); }
-
-// Dynamic shared memory: alignment slack, L1 ring, x_hat tiles, activation ring (and what the 128-row operand reads behind
-// the last x_hat tile), and in a K-split launch this CTA's share of all partial sums of T.
-constexpr uint32_t x_ring_bytes(int R, int steps, int warps) {
-  const uint32_t ring = kXStages(R, steps) * x_stage_bytes(steps, warps), behind = 128 * 128 - xh_tile_bytes(steps, warps);
-  return R == 0 || ring > behind ? ring : behind;
-}
-constexpr size_t quantize_smem_bytes(int R, int steps, int warps, int splits) {
-  return (R == 0 ? 0 : 1024 + kL1Stages * R * 128 + kXhBuffers * xh_tile_bytes(steps, warps)) + x_ring_bytes(R, steps, warps) +
-         (splits > 1 ? (quantize_rows(steps, warps) + splits) * R * 4 : 0);
-}
-
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<uint32_t*>(&v);
@@ -656,53 +635,6 @@ static __global__ void t_split_kernel(const float* __restrict__ t32, int M, int 
   const __nv_bfloat16 lo = __float2bfloat16_rn(t - __bfloat162float(hi));
   t_hilo[row * 2 * r + c] = *reinterpret_cast<const uint16_t*>(&hi);
   t_hilo[row * 2 * r + r + c] = *reinterpret_cast<const uint16_t*>(&lo);
-}
-
-// How a launch divides M rows x G groups.  fitting_clusters[k]: clusters of k CTAs that run at a time, one CTA to an SM.
-// `expand`: the layer's forwards carry an expansion in this launch.  With a low-rank branch every launch for such a layer
-// passes it, also one that carries none (a stage called alone, a search's later candidates, later chunks of a host forward):
-// the K split is the summation order of T, and the same rows have to give the same bits.  The plan made for a launch without
-// an expansion would take such a launch from 13.8 to 12.0 us at 1560 x 5120, r = 32.
-struct QuantizePlan {
-  int steps, warps, splits;   // a CTA owns 4 steps warps rows and a 1 / splits share of the groups
-};
-constexpr int kMaxKSplits = 16;
-inline QuantizePlan quantize_plan(int M, int G, int r, int sms, const int* fitting_clusters, bool expand) {
-  const int few = 448;   // rows up to which 2 steps per warp beat 4
-  if (r == 0) {
-    // The splits are independent CTAs.  About five to an SM at any size, so that no SM is left with a CTA more than others:
-    // 32760 x 5120 in 256 CTAs of 128 rows 105.7 us, in 768 95.1 us.
-    const int steps = M <= few ? 2 : 4, per_warp = 4 * steps;
-    const int warps = M < kQuantWarps * per_warp ? (M + per_warp - 1) / per_warp : kQuantWarps;
-    const int splits = (expand ? sms + sms / 4 : 5 * sms) / ((M + per_warp * warps - 1) / (per_warp * warps));
-    return {steps, warps, splits < 1 || G < 4 ? 1 : (splits > G / 2 ? G / 2 : splits)};
-  }
-  // Beside an expansion, which takes longer than the activations and wants its share of the machine from the start: smaller
-  // CTAs, two to an SM, about one per SM in all.  Forwards of 5120 -> 5120: 700 rows, r = 64 60.0 -> 51.2 us; 1560, r = 64
-  // 96.8 -> 90.3; 4097, r = 96 204 -> 194.
-  if (expand && M > few && M <= 34 * 128) {
-    const int k = M <= 1024 ? 8 : 4, clusters = k == 8 ? 16 : 33, warps = (M + 8 * clusters - 1) / (8 * clusters);
-    if (k <= G / 2) return {2, warps < kQuantWarps ? warps : kQuantWarps, k};
-  }
-  // The splits of a row block form a cluster; with the partial sums of T a CTA's shared memory leaves room for one per SM,
-  // and a cluster stays within a GPC (of 16 SMs at least).  The most splits that still run all row blocks at once, and
-  // the fewest warps that cover the rows: 1560 x 5120, r = 32, in 14 clusters of 8 CTAs of 7 warps 12.0 us, of 4 CTAs 15.9 us,
-  // not split 57 us; 32760 x 5120 split in two 152 us, not split 115 us.
-  for (int k = kMaxKSplits; k > 1; k = k > 8 ? 8 : k - 1) {
-    const int clusters = k > 8 ? 7 : fitting_clusters[k];
-    const int steps = k > 8 && M <= few ? 2 : 4, per_warp = 4 * steps;
-    if (clusters > 0 && k <= G / 2 && M <= clusters * kQuantWarps * per_warp)
-      return {steps, (M + clusters * per_warp - 1) / (clusters * per_warp), k};
-  }
-  // Not split, two CTAs per SM: the number of warps for which the busiest SM has the fewest rows.  32760 rows: 256 CTAs of 8
-  // warps leave 40 SMs with one, 293 of 7 fill 146.5: 120.3 -> 114.7 us at K = 5120, r = 32.
-  QuantizePlan best = {4, kQuantWarps, 1};
-  int least = 1 << 30;
-  for (int w = kQuantWarps; w >= 4; --w) {
-    const int ctas = (M + 16 * w - 1) / (16 * w), rows = (ctas + sms - 1) / sms * w;
-    if (rows < least) least = rows, best.warps = w;
-  }
-  return best;
 }
 
 }  // namespace w4a4

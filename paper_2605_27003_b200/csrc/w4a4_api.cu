@@ -124,6 +124,7 @@ struct w4a4_layer {
   std::vector<ExpertData> experts;
   CUtensorMap tmA, tmSopA, tmT, tmB;
   const uint8_t* tmB_base = nullptr;  // the context's weight-byte scratch this handle's tmB was encoded for
+  int wide_clusters = 0;              // clusters of kMaxKSplits CTAs of kernel 1 that run at a time on the device
   size_t bytes = 0;
 };
 
@@ -156,25 +157,38 @@ w4a4_status_t check_forward_args(w4a4_handle_t h, const void* X, int M, int expe
 }
 
 // Kernel 1's limits for every plan of a layer, once where the layer is packed.  They belong to the kernel on the device, not to
-// a launch: set per launch, one thread's smaller size would meet another thread's larger launch.
+// a launch: set per launch, one thread's smaller size would meet another thread's larger launch.  wide_clusters: how many
+// clusters of kMaxKSplits CTAs, a size that not every device can launch, run at a time.
 template <int R, int FORMAT, int STEPS, int MINB>
-bool prepare_quantize_steps() {
+bool prepare_quantize_steps(int* wide_clusters) {
   auto* const kernel = quantize_kernel<R, FORMAT, STEPS, MINB>;
   const size_t most = quantize_smem_bytes(R, STEPS, kQuantWarps, kMaxKSplits);   // grows with the warps and with the splits
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(most)) == cudaSuccess &&
-         (R == 0 || cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess);
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(most)) != cudaSuccess) return false;
+  if (R == 0) return true;   // no clusters
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return false;
+  int fitting = 0;
+  const OverlappedLaunch l(dim3(1, kMaxKSplits), dim3(quantize_threads(R)), most, nullptr, dim3(1, kMaxKSplits));
+  if (cudaOccupancyMaxActiveClusters(&fitting, kernel, &l.cfg) != cudaSuccess) {
+    cudaGetLastError();
+    fitting = 0;
+  }
+  if (fitting < *wide_clusters) *wide_clusters = fitting;
+  return true;
 }
 template <int R, int FORMAT>
-bool prepare_quantize_rank() { return prepare_quantize_steps<R, FORMAT, 4, 2>() && prepare_quantize_steps<R, FORMAT, 2, 2>(); }
+bool prepare_quantize_rank(int* wide_clusters) {
+  return prepare_quantize_steps<R, FORMAT, 4, 2>(wide_clusters) && prepare_quantize_steps<R, FORMAT, 2, 2>(wide_clusters);
+}
 template <int FORMAT>
-w4a4_status_t prepare_quantize(int r) {
+w4a4_status_t prepare_quantize(int r, int* wide_clusters) {
   bool ok = false;
+  *wide_clusters = 1 << 30;
   switch (r) {
-    case 0: ok = prepare_quantize_rank<0, FORMAT>(); break;
-    case 16: ok = prepare_quantize_rank<16, FORMAT>(); break;
-    case 32: ok = prepare_quantize_rank<32, FORMAT>(); break;
-    case 64: ok = prepare_quantize_rank<64, FORMAT>(); break;
-    case 96: if constexpr (FORMAT == kCodesE4M3) ok = prepare_quantize_rank<96, FORMAT>(); break;
+    case 0: ok = prepare_quantize_rank<0, FORMAT>(wide_clusters); break;
+    case 16: ok = prepare_quantize_rank<16, FORMAT>(wide_clusters); break;
+    case 32: ok = prepare_quantize_rank<32, FORMAT>(wide_clusters); break;
+    case 64: ok = prepare_quantize_rank<64, FORMAT>(wide_clusters); break;
+    case 96: if constexpr (FORMAT == kCodesE4M3) ok = prepare_quantize_rank<96, FORMAT>(wide_clusters); break;
   }
   if (!ok) cudaGetLastError();
   return ok ? W4A4_OK : W4A4_ERR_CUDA;
@@ -193,9 +207,9 @@ cudaError_t launch_quantize_steps(int num_sms, cudaStream_t stream, const CUtens
   return cudaLaunchKernelEx(&l.cfg, quantize_kernel<R, FORMAT, STEPS, MINB>, tmL1, p);
 }
 template <int R, int FORMAT>
-cudaError_t launch_quantize_kernel(const w4a4_ctx* ctx, cudaStream_t stream, const CUtensorMap& tmL1, const QuantizeParams& p) {
+cudaError_t launch_quantize_kernel(const w4a4_ctx* ctx, int wide_clusters, cudaStream_t stream, const CUtensorMap& tmL1, const QuantizeParams& p) {
   const bool expand = R > 0 ? FORMAT == kCodesE4M3 : p.expand.chunks > 0;   // (without a low-rank branch nothing is summed over K)
-  const QuantizePlan plan = quantize_plan(p.M, p.K / 64, R, ctx->num_sms, ctx->gemm_clusters, expand);
+  const QuantizePlan plan = quantize_plan(p.M, p.K / 64, R, ctx->num_sms, ctx->gemm_clusters, wide_clusters, expand);
   if (plan.steps == 4) return launch_quantize_steps<R, FORMAT, 4, 2>(ctx->num_sms, stream, tmL1, p, plan);
   return launch_quantize_steps<R, FORMAT, 2, 2>(ctx->num_sms, stream, tmL1, p, plan);
 }
@@ -236,7 +250,7 @@ w4a4_status_t launch_quantize_at(w4a4_handle_t h, const void* X, int M, int expe
   p.expand = job;
   p.err = ctx->d_err;
   cudaError_t le;
-#define W4A4_LAUNCH_Q(R) le = launch_quantize_kernel<R, kCodesE4M3>(ctx, stream, h->r > 0 ? e.tmL1 : h->tmSopA, p)
+#define W4A4_LAUNCH_Q(R) le = launch_quantize_kernel<R, kCodesE4M3>(ctx, h->wide_clusters, stream, h->r > 0 ? e.tmL1 : h->tmSopA, p)
   switch (h->r) {
     case 0: W4A4_LAUNCH_Q(0); break;
     case 16: W4A4_LAUNCH_Q(16); break;
@@ -508,7 +522,7 @@ w4a4_status_t w4a4_pack_weights(w4a4_ctx_t ctx, const w4a4_weight_desc_t* d, w4a
       if (st == W4A4_OK) ctx->b8_bytes = b8_need;
     }
   }
-  if (st == W4A4_OK) st = prepare_quantize<kCodesE4M3>(r);
+  if (st == W4A4_OK) st = prepare_quantize<kCodesE4M3>(r, &h->wide_clusters);
   int* d_bad = nullptr;
   if (st == W4A4_OK) st = dev_alloc(&d_bad, 1, nullptr);
   if (st == W4A4_OK && cudaMemset(d_bad, 0, sizeof(int)) != cudaSuccess) st = W4A4_ERR_CUDA;

@@ -24,6 +24,7 @@ struct w4a4_mx_layer {
   CUtensorMap tmA, tmT;
   CUtensorMap tmSFA;               // activation scale atoms as 32-bit words: [max_M/128] rows of K words
   CUtensorMap tmA2, tmT2, tmSFA2;  // the same three on the context's second workspace (input written by a fused producer)
+  int wide_clusters = 0;              // clusters of kMaxKSplits CTAs of kernel 1 that run at a time on the device
   size_t bytes = 0;
 };
 
@@ -73,7 +74,7 @@ w4a4_status_t mx_launch_quantize_at(w4a4_mx_handle_t h, const void* X, int M, in
   p.t_hilo = ctx->t_hilo;
   p.err = ctx->d_err;
   cudaError_t le;
-#define W4A4_LAUNCH_MXQ(R) le = launch_quantize_kernel<R, kCodesMxfp4>(ctx, stream, h->r > 0 ? e.tmL1 : h->tmA, p)
+#define W4A4_LAUNCH_MXQ(R) le = launch_quantize_kernel<R, kCodesMxfp4>(ctx, h->wide_clusters, stream, h->r > 0 ? e.tmL1 : h->tmA, p)
   switch (h->r) {
     case 0: W4A4_LAUNCH_MXQ(0); break;
     case 16: W4A4_LAUNCH_MXQ(16); break;
@@ -250,7 +251,7 @@ w4a4_status_t w4a4_mx_pack_weights(w4a4_ctx_t ctx, const w4a4_mx_weight_desc_t* 
     if (st == W4A4_OK && cudaMemset(ctx->t_hilo2, 0, sizeof(uint16_t) * ctx->max_M * 2 * rr) != cudaSuccess) st = W4A4_ERR_CUDA;
 
   }
-  if (st == W4A4_OK) st = prepare_quantize<kCodesMxfp4>(r);
+  if (st == W4A4_OK) st = prepare_quantize<kCodesMxfp4>(r, &h->wide_clusters);
   int* d_bad = nullptr;
   if (st == W4A4_OK) st = dev_alloc(&d_bad, 1, nullptr);
   if (st == W4A4_OK && cudaMemset(d_bad, 0, sizeof(int)) != cudaSuccess) st = W4A4_ERR_CUDA;

@@ -1,0 +1,67 @@
+"""How kernel 1's launches are divided, for devices other than the one at hand: the plan is plain C++, compiled here.
+
+Cluster sizes above 8 are not portable: a device (or a partition of one) may be unable to launch them, and then a plan must not
+ask for one.  Whatever the plan, its shared memory stays within the limit that is set once per layer.
+"""
+import ctypes
+import os
+import subprocess
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2605_27003_b200", "csrc")
+SHIM = """
+#include "quantize_plan.h"
+extern "C" void plan(int M, int G, int r, int sms, const int* fitting, int wide, int expand, int* out) {
+  const w4a4::QuantizePlan p = w4a4::quantize_plan(M, G, r, sms, fitting, wide, expand != 0);
+  out[0] = p.steps, out[1] = p.warps, out[2] = p.splits;
+  out[3] = static_cast<int>(w4a4::quantize_smem_bytes(r, p.steps, p.warps, p.splits));
+  out[4] = static_cast<int>(w4a4::quantize_smem_bytes(r, p.steps, w4a4::kQuantWarps, w4a4::kMaxKSplits));
+  out[5] = w4a4::quantize_rows(p.steps, p.warps);
+}
+"""
+FULL = [0, 0, 74, 45, 33, 26, 22, 15, 15]   # clusters of 2 .. 8 that fit a whole B200, one CTA to an SM
+ROWS = [1, 7, 8, 9, 63, 64, 65, 200, 448, 449, 700, 896, 897, 1024, 1025, 1560, 2048, 4352, 4353, 9300, 32760, 75600]
+GROUPS = [1, 2, 3, 4, 8, 9, 16, 31, 32, 33, 80, 216, 256]
+
+
+@pytest.fixture(scope="module")
+def plan(tmp_path_factory):
+    d = tmp_path_factory.mktemp("plan")
+    src, lib = d / "plan.cpp", d / "plan.so"
+    src.write_text(SHIM)
+    subprocess.run(["g++", "-std=c++17", "-O1", "-Wall", "-Werror", "-shared", "-fPIC", "-I", CSRC, "-o", str(lib), str(src)], check=True)
+    fn = ctypes.CDLL(str(lib)).plan
+
+    def call(M, G, r, sms=148, fitting=FULL, wide=7, expand=False):
+        out = (ctypes.c_int * 6)()
+        fn(M, G, r, sms, (ctypes.c_int * 9)(*fitting), wide, int(expand), out)
+        return dict(zip(("steps", "warps", "splits", "smem", "limit", "rows"), out))
+    return call
+
+
+@pytest.mark.parametrize("fitting,wide,most", [
+    (FULL, 7, 16),
+    (FULL, 0, 8),                                    # no GPC offers 16 SMs
+    ([0, 0, 8, 4, 4, 0, 0, 0, 0], 0, 4),             # a partition with GPCs of four or five SMs
+    ([0] * 9, 0, 1),                                 # no clusters at all
+])
+def test_a_plan_asks_for_no_cluster_that_the_device_cannot_launch(plan, fitting, wide, most):
+    for M in ROWS:
+        for G in GROUPS:
+            for r in (16, 32, 64, 96):
+                for expand in (False, True):
+                    p = plan(M, G, r, fitting=fitting, wide=wide, expand=expand)
+                    assert 1 <= p["splits"] <= most and p["splits"] <= max(1, G // 2), (M, G, r, expand, p)
+                    assert p["splits"] == 1 or (wide if p["splits"] > 8 else fitting[p["splits"]]) > 0, (M, G, r, expand, p)
+
+
+def test_every_plan_stays_within_the_limits_set_at_pack_time(plan):
+    for M in ROWS:
+        for G in GROUPS:
+            for r in (0, 16, 32, 64, 96):
+                for expand in (False, True):
+                    p = plan(M, G, r, expand=expand)
+                    assert p["steps"] in (2, 4) and 1 <= p["warps"] <= 8 and 1 <= p["splits"] <= max(1, G), (M, G, r, expand, p)
+                    assert p["smem"] <= p["limit"] <= 232448, (M, G, r, expand, p)
+                    assert p["rows"] <= 128
