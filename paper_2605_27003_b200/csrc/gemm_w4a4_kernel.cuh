@@ -310,9 +310,9 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           ok = __all_sync(0xffffffffu, bounded_wait<64>(bar_op_empty + 8 * op.slot, op.parity ^ 1u, env, kErrProducerWait));
           if (!ok) break;
           if (DEBUG) {
-            // Test hook: one stage is never loaded, so its consumers' waits run into their limit and every role of
-            // the CTA leaves through the common tail (error word, drain, TMEM release).
-            if (stage_no++ == p.dbg_stall_stage) {
+            // Test hook: one stage is never loaded (of a cluster that shares K: by its first CTA), so its consumers' waits
+            // run into their limit and every role of the CTA leaves through the common tail (error word, drain, TMEM release).
+            if (stage_no++ == p.dbg_stall_stage && split == 0) {
               op.advance();
               continue;
             }
@@ -592,7 +592,7 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 
   if constexpr (SPLIT) {
     cluster_sync_all();   // all partial tiles are written
-    if (live && warp >= kEpiWarp0 && !*s_abort) {
+    if (live && warp >= kEpiWarp0 && !cluster_gave_up(s_abort, p.splits)) {
       int tm_e, tn_e;
       tile_coords(first_tile, p.order, tm_e, tn_e);
       float sq = 0.0f;

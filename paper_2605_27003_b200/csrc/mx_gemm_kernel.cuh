@@ -77,6 +77,8 @@ struct MxGemmParams {
   int act;              // output activation: 0 none, 1 GELU (tanh form)
   int splits;           // mx_gemm_kernel: CTAs of a cluster that share a tile's K (1: K is not split)
   int run;              // CTA-pair kernel: consecutive column tiles of a row pair that one cluster takes at a time
+  int dbg_stall_stage;  // DEBUG: the stage that the first CTA of a cluster never loads, and the limit of its waits
+  uint64_t dbg_wait_limit_ns;
 };
 
 // One lane of a converged warp.  The MMA warp runs its loop with all lanes (waits included) and only predicates
@@ -120,7 +122,7 @@ __device__ __forceinline__ void bulk_load(uint32_t dst_smem, const void* src, ui
                : "memory");
 }
 
-template <bool SPLIT>
+template <bool SPLIT, bool DEBUG = false>
 __global__ void __launch_bounds__(kMxThreads, 1)
 mx_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmT, const __grid_constant__ CUtensorMap tmL2, const MxGemmParams p) {
@@ -145,7 +147,7 @@ mx_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   const int first_tile = SPLIT ? blockIdx.x / p.splits : blockIdx.x, tile_step = SPLIT ? p.tiles_m * p.tiles_n : gridDim.x;
   const int atoms_k = p.K / 128;
   const int num_tiles = p.tiles_m * p.tiles_n;
-  const WaitEnv env{p.err, s_abort, kWaitLimitNs};
+  const WaitEnv env{p.err, s_abort, DEBUG ? p.dbg_wait_limit_ns : kWaitLimitNs};
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < kMxStages; ++i) {
@@ -189,6 +191,10 @@ mx_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       for (int st = 0; st < n_lr_stages + n_k_stages; ++st) {
         ok = __all_sync(0xffffffffu, bounded_wait<128>(bar_empty + 8 * rg.slot, rg.parity ^ 1u, env, kErrProducerWait));
         if (!ok) break;
+        if (DEBUG && st == p.dbg_stall_stage && split == 0) {   // test hook: never loaded
+          rg.advance();
+          continue;
+        }
         const uint32_t full = bar_full + 8 * rg.slot;
         const uint32_t dst = smem_base + rg.slot * kMxStageBytes;
         if (st < n_lr_stages) {
@@ -271,7 +277,7 @@ mx_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     for (int tile = first_tile; ok && tile < num_tiles; tile += tile_step) {
       const int m0 = (tile / p.tiles_n) * kBM, n0 = (tile % p.tiles_n) * kMxBN;
       const int row = m0 + 32 * quarter + lane;
-      ok = bounded_wait(bar_acc_full, ab.parity, env, kErrEpilogueWait);
+      ok = __all_sync(0xffffffffu, bounded_wait(bar_acc_full, ab.parity, env, kErrEpilogueWait));
       if (!ok) break;
       tc_fence_after_sync();
       const uint32_t t_row = tmem_base + (static_cast<uint32_t>(32 * quarter) << 16) + 64 * colblk;
@@ -351,7 +357,7 @@ mx_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 
   if constexpr (SPLIT) {
     cluster_sync_all();   // all partial tiles are written
-    if (live && warp >= kMxEpiWarp0 && !*s_abort) {
+    if (live && warp >= kMxEpiWarp0 && !cluster_gave_up(s_abort, p.splits)) {
       const int m0 = (first_tile / p.tiles_n) * kBM, n0 = (first_tile % p.tiles_n) * kMxBN;
       float sq = 0.0f;
       // A warp takes 128 channels of a row at a time, a lane four of them.
@@ -756,7 +762,7 @@ mx_gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(tab + 16 * lane), "f"(t4.x), "f"(t4.y), "f"(t4.z), "f"(t4.w) : "memory");
         __syncwarp();
       }
-      ok = bounded_wait(bar_acc_full, ab.parity, env, kErrEpilogueWait);
+      ok = __all_sync(0xffffffffu, bounded_wait(bar_acc_full, ab.parity, env, kErrEpilogueWait));
       if (!ok) break;
       tc_fence_after_sync();
       const uint32_t t_row = tmem_base + (static_cast<uint32_t>(32 * quarter) << 16) + 64 * colblk;

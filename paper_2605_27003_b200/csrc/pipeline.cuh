@@ -182,6 +182,14 @@ __device__ __forceinline__ void drain_after_abort(volatile int* s_abort) {
   }
 }
 
+// Has any CTA of the cluster given up?  By whole warps, after a cluster barrier behind the role loops (no flag changes any more);
+// `ctas` <= 32.
+__device__ __forceinline__ bool cluster_gave_up(volatile int* s_abort, int ctas) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t word = smem_u32(const_cast<int*>(s_abort));
+  return __any_sync(0xffffffffu, lane < ctas && ld_cluster_u32(map_to_cta(word, lane)) != 0u);
+}
+
 // Exercises the give-up path of bounded_wait without any pipeline around it: one warp waits for a phase of an
 // mbarrier that nobody ever completes.  No copy, tensor-core operation or TMEM allocation is involved, so there is
 // nothing to drain: after limit_ns the wait records kErrProbeWait in *err and the kernel returns normally.

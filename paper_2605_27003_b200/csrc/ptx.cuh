@@ -202,9 +202,9 @@ __device__ __forceinline__ void st_async_u32x4(uint32_t cluster_addr, const uint
                "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(cluster_bar)
                : "memory");
 }
-__device__ __forceinline__ float2 ld_cluster_f32x2(uint32_t cluster_addr) {
-  float2 v;
-  asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(cluster_addr) : "memory");
+__device__ __forceinline__ uint32_t ld_cluster_u32(uint32_t cluster_addr) {
+  uint32_t v;
+  asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(cluster_addr) : "memory");
   return v;
 }
 __device__ __forceinline__ float4 ld_cluster_f32x4(uint32_t cluster_addr) {

@@ -274,7 +274,7 @@ w4a4_status_t launch_quantize(w4a4_handle_t h, const void* X, int M, int expert_
 // *sq_err instead of storing Y.
 w4a4_status_t launch_gemm(w4a4_handle_t h, int M, int expert_id, void* Y, cudaStream_t stream, int32_t* dbg_P,
                           int dbg_m0, int dbg_n0, const void* yref = nullptr, double* sq_err = nullptr,
-                          bool expand = false, int stall_stage = -1, uint64_t wait_limit_ns = kWaitLimitNs) {
+                          bool expand = false, int stall_stage = -1, uint64_t wait_limit_ns = kWaitLimitNs, bool stall_split = false) {
   if (M == 0) return W4A4_OK;
   w4a4_ctx* ctx = h->ctx;
   const ExpertData& e = h->experts[expert_id];
@@ -329,7 +329,8 @@ w4a4_status_t launch_gemm(w4a4_handle_t h, int M, int expert_id, void* Y, cudaSt
   const CUtensorMap& tmL2 = h->r > 0 ? e.tmL2 : h->tmB;
   // Few tiles: clusters of CTAs share a tile's K.  Four stages (eight groups) per CTA at least: the cluster's two barriers and
   // the exchange cost about as much as six groups.
-  p.splits = stall_stage >= 0 ? 1 : gemm_k_splits(num_tiles, (h->K / 64 + 1) / 2, 4, ctx->gemm_clusters);
+  p.splits = stall_stage >= 0 && !stall_split ? 1 : gemm_k_splits(num_tiles, (h->K / 64 + 1) / 2, 4, ctx->gemm_clusters);
+  if (stall_split && p.splits == 1) return W4A4_ERR_SHAPE;
   const OverlappedLaunch l(p.splits > 1 ? dim3(num_tiles * p.splits) : grid, block, kGemmSmemBytes, stream, dim3(p.splits));
   cudaError_t le;
   auto launch = [&](auto* kernel) { return cudaLaunchKernelEx(&l.cfg, kernel, h->tmA, h->tmB, tmT, tmL2, h->tmSopA, e.tmSopB, p); };
@@ -839,8 +840,8 @@ w4a4_status_t w4a4_debug_wait_probe(w4a4_ctx_t ctx, uint64_t limit_ns, void* str
   return cudaGetLastError() == cudaSuccess ? W4A4_OK : W4A4_ERR_CUDA;
 }
 
-w4a4_status_t w4a4_debug_stalled_gemm(w4a4_handle_t h, int M, int expert_id, void* Y, int stall_stage,
-                                      uint64_t limit_ns, void* stream) {
+static w4a4_status_t stalled_gemm(w4a4_handle_t h, int M, int expert_id, void* Y, int stall_stage, uint64_t limit_ns, void* stream,
+                                  bool split) {
   w4a4_status_t st = check_forward_args(h, nullptr, M, expert_id, 0, nullptr, false);
   if (st != W4A4_OK) return st;
   if (!Y || !aligned16(Y) || stall_stage < 0) return W4A4_ERR_INVALID_ARG;
@@ -848,7 +849,17 @@ w4a4_status_t w4a4_debug_stalled_gemm(w4a4_handle_t h, int M, int expert_id, voi
   DeviceGuard guard(h->ctx->device);
   if (!guard.ok) return W4A4_ERR_CUDA;
   return launch_gemm(h, M, expert_id, Y, static_cast<cudaStream_t>(stream), nullptr, 0, 0, nullptr, nullptr, true,
-                     stall_stage, limit_ns);
+                     stall_stage, limit_ns, split);
+}
+
+w4a4_status_t w4a4_debug_stalled_gemm(w4a4_handle_t h, int M, int expert_id, void* Y, int stall_stage,
+                                      uint64_t limit_ns, void* stream) {
+  return stalled_gemm(h, M, expert_id, Y, stall_stage, limit_ns, stream, false);
+}
+
+w4a4_status_t w4a4_debug_stalled_split_gemm(w4a4_handle_t h, int M, int expert_id, void* Y, int stall_stage,
+                                            uint64_t limit_ns, void* stream) {
+  return stalled_gemm(h, M, expert_id, Y, stall_stage, limit_ns, stream, true);
 }
 
 w4a4_status_t w4a4_debug_set_tile_order(w4a4_ctx_t ctx, int super_column_tiles) {

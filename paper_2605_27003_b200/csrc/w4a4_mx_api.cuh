@@ -96,7 +96,8 @@ w4a4_status_t mx_launch_quantize(w4a4_mx_handle_t h, const void* X, int M, int e
 // fused form, the epilogue quantizes the output for that layer into the second workspace instead of storing Y.
 w4a4_status_t mx_launch_gemm(w4a4_mx_handle_t h, int M, int expert_id, void* Y, cudaStream_t stream,
                              const void* yref = nullptr, double* sq_err = nullptr, bool second_ws = false,
-                             w4a4_mx_handle_t next = nullptr, const float* next_rho = nullptr) {
+                             w4a4_mx_handle_t next = nullptr, const float* next_rho = nullptr, int stall_stage = -1,
+                             uint64_t wait_limit_ns = kWaitLimitNs) {
   if (M == 0) return W4A4_OK;
   w4a4_ctx* ctx = h->ctx;
   const MxExpertData& e = h->experts[expert_id];
@@ -115,6 +116,8 @@ w4a4_status_t mx_launch_gemm(w4a4_mx_handle_t h, int M, int expert_id, void* Y, 
   p.yref = static_cast<const uint16_t*>(yref);
   p.sq_err = sq_err;
   p.act = h->act;
+  p.dbg_stall_stage = stall_stage;
+  p.dbg_wait_limit_ns = wait_limit_ns;
   // Runs of column tiles per cluster: 1 = interleave; the fused form takes six at a time (T stays in TMEM over a
   // run, and the 74 clusters of a wave then cover about a dozen row pairs whose A rows they share in L2).
   p.run = next ? (p.tiles_n < 6 ? p.tiles_n : 6) : 1;
@@ -129,12 +132,14 @@ w4a4_status_t mx_launch_gemm(w4a4_mx_handle_t h, int M, int expert_id, void* Y, 
   p.splits = next ? 1 : gemm_k_splits(num_tiles, h->K / kMxBK, 3, ctx->mx_gemm_clusters);
   if (p.splits > 1) {
     const OverlappedLaunch l(dim3(num_tiles * p.splits), block, kMxSmemBytes, stream, dim3(p.splits));
-    if (cudaLaunchKernelEx(&l.cfg, mx_gemm_kernel<true>, tmA, e.tmB, tmT, tmL2, p) != cudaSuccess) {
+    auto* const kernel = stall_stage >= 0 ? mx_gemm_kernel<true, true> : mx_gemm_kernel<true>;
+    if (cudaLaunchKernelEx(&l.cfg, kernel, tmA, e.tmB, tmT, tmL2, p) != cudaSuccess) {
       cudaGetLastError();
       return W4A4_ERR_CUDA;
     }
     return W4A4_OK;
   }
+  if (stall_stage >= 0) return W4A4_ERR_SHAPE;   // the test hook knows this form only
   // CTA pairs (cta_group::2) need at least two row tiles and an even number of CTAs.  A wave of pairs takes less time than one of
   // single CTAs, but single CTAs win where a tile each is about all there is (900 x 5120 -> 5120 25.1 -> 20.7 us, 700 17.6 -> 15.9)
   // and where they need two waves and pairs three (600 x 5120 -> 13824 31.1 -> 25.1); at 1.22 waves and K = 13824 they lose (43.6 | 45.1),
@@ -233,6 +238,7 @@ w4a4_status_t w4a4_mx_pack_weights(w4a4_ctx_t ctx, const w4a4_mx_weight_desc_t* 
     if (st == W4A4_OK) {
       cudaFuncSetAttribute(mx_gemm_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kMxSmemBytes));
       cudaFuncSetAttribute(mx_gemm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kMxSmemBytes));
+      cudaFuncSetAttribute(mx_gemm_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kMxSmemBytes));
       count_clusters(ctx->mx_gemm_clusters, mx_gemm_kernel<true>, kMxThreads, kMxSmemBytes);
     }
     if (st == W4A4_OK)
@@ -449,6 +455,18 @@ w4a4_status_t w4a4_mx_clip_search(w4a4_mx_handle_t h, const void* const* X_sampl
   cudaFree(d_best);
   if (st != W4A4_OK) cudaGetLastError();
   return st;
+}
+
+w4a4_status_t w4a4_mx_debug_stalled_split_gemm(w4a4_mx_handle_t h, int M, int expert_id, void* Y, int stall_stage,
+                                               uint64_t limit_ns, void* stream) {
+  w4a4_status_t st = mx_check_forward_args(h, nullptr, M, expert_id, 0, nullptr, false);
+  if (st != W4A4_OK) return st;
+  if (!Y || !aligned16(Y) || stall_stage < 0) return W4A4_ERR_INVALID_ARG;
+  if (limit_ns == 0 || limit_ns > 100000000ull) return W4A4_ERR_INVALID_ARG;  // at most 0.1 s
+  DeviceGuard guard(h->ctx->device);
+  if (!guard.ok) return W4A4_ERR_CUDA;
+  return mx_launch_gemm(h, M, expert_id, Y, static_cast<cudaStream_t>(stream), nullptr, nullptr, false, nullptr, nullptr, stall_stage,
+                        limit_ns);
 }
 
 w4a4_status_t w4a4_mx_debug_quantize(w4a4_mx_handle_t h, const void* X, int M, int expert_id, int timestep_bin,

@@ -8,7 +8,9 @@
    computes correct results afterwards.
    The same is then done to the real GEMM: `w4a4_debug_stalled_gemm` withholds one operand stage from every CTA, so
    that the producer, both MMA-issuing warps and the epilogue warps all run into a 1 ms limit and leave through the
-   kernel's common tail (drain of copies in flight, release of tensor memory).
+   kernel's common tail (drain of copies in flight, release of tensor memory).  In the form whose clusters share a tile's K
+   (`w4a4_debug_stalled_split_gemm`, both grids) one CTA of each cluster stalls, and the others must not store what they
+   add up from its part.
 2. Allocation failures.  A countdown hook makes the n-th device allocation fail as a refused cudaMalloc would.  Walking
    n over every allocation of w4a4_ctx_create and w4a4_pack_weights checks that each partial construction returns
    W4A4_ERR_ALLOC, leaks nothing (device memory in use returns to where it was) and leaves the library usable.
@@ -104,6 +106,42 @@ def test_a_stalled_gemm_pipeline_gives_up_cleans_up_and_the_context_recovers():
     assert w4.w4a4_query_status(ctx.ptr) == ERR_TIMEOUT
     assert w4.w4a4_query_status(ctx.ptr) == 0
     assert forward_matches_oracle(ctx, L, layer, M, seed=13)
+    ctx.check()
+    L.close()
+    ctx.close()
+
+
+@pytest.mark.parametrize("grid", ["int4", "mx"])
+@pytest.mark.parametrize("M,K,N,r,stage", [
+    (100, 2048, 640, 32, 2),    # the low-rank stage passes, an operand stage does not come
+    (300, 1792, 256, 0, 0),     # the very first stage; rows past M in the last row block
+])
+def test_a_stalled_member_of_a_cluster_keeps_the_others_from_storing(grid, M, K, N, r, stage):
+    # Its neighbours have their parts complete when the first CTA gives up after 1 ms: what they add up is no output.
+    pkg_build.build()
+    w4.load_library()
+    mx = grid == "mx"
+    layer = (gen.make_layer_mx_direct if mx else gen.make_layer_direct)(K, N, r, seed=6).to(DEV)
+    ctx = w4.Context(0, M, K, r)
+    L = (w4.MxLayer if mx else w4.Layer)(ctx, [layer], num_bins=1)
+    x = gen.make_activations(M, K, seed=12).to(DEV)
+    clip = torch.ones((1, 1, 1), dtype=torch.float32, device=DEV)
+    before = L.forward(x, 0, 0, clip)
+    y = torch.full_like(before, 7.0)
+    ev0, ev1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    ev0.record()
+    w4.w4a4_debug_stalled_split_gemm(L.ptr, M, 0, y, stage, 1_000_000, mx=mx)
+    ev1.record()
+    torch.cuda.synchronize()
+    assert ev0.elapsed_time(ev1) < 500.0, "the stalled kernel must end by itself shortly after its limit"
+    assert bool((y == 7.0).all()), "rows of a tile whose first part is missing were stored"
+    # a forward enqueued before the query stores nothing either
+    L.forward(x, 0, 0, clip, y)
+    torch.cuda.synchronize()
+    assert bool((y == 7.0).all())
+    assert w4.w4a4_query_status(ctx.ptr) == ERR_TIMEOUT
+    assert w4.w4a4_query_status(ctx.ptr) == 0
+    assert torch.equal(L.forward(x, 0, 0, clip), before)
     ctx.check()
     L.close()
     ctx.close()
