@@ -133,6 +133,7 @@ w4a4_status_t mx_launch_gemm(w4a4_mx_handle_t h, int M, int expert_id, void* Y, 
   if (p.splits > 1) {
     const OverlappedLaunch l(dim3(num_tiles * p.splits), block, kMxSmemBytes, stream, dim3(p.splits));
     auto* const kernel = stall_stage >= 0 ? mx_gemm_kernel<true, true> : mx_gemm_kernel<true>;
+    if (stall_stage >= 0) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kMxSmemBytes));
     if (cudaLaunchKernelEx(&l.cfg, kernel, tmA, e.tmB, tmT, tmL2, p) != cudaSuccess) {
       cudaGetLastError();
       return W4A4_ERR_CUDA;
@@ -238,7 +239,6 @@ w4a4_status_t w4a4_mx_pack_weights(w4a4_ctx_t ctx, const w4a4_mx_weight_desc_t* 
     if (st == W4A4_OK) {
       cudaFuncSetAttribute(mx_gemm_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kMxSmemBytes));
       cudaFuncSetAttribute(mx_gemm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kMxSmemBytes));
-      cudaFuncSetAttribute(mx_gemm_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kMxSmemBytes));
       count_clusters(ctx->mx_gemm_clusters, mx_gemm_kernel<true>, kMxThreads, kMxSmemBytes);
     }
     if (st == W4A4_OK)
