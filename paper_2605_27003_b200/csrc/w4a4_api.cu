@@ -518,16 +518,18 @@ w4a4_status_t w4a4_pack_weights(w4a4_ctx_t ctx, const w4a4_weight_desc_t* d, w4a
   const bool dev = d->pointers_on_device != 0;
   w4a4_status_t st = W4A4_OK;
   // The weight-byte scratch of the context must hold this layer's N x K image.  Growing it is safe between
-  // forwards only (synchronise first: a forward of another layer may still be reading the old one).
+  // forwards only (synchronise first: a forward of another layer may still be reading the old one).  The new one comes first:
+  // without memory for it, the context's other layers keep theirs.
   const size_t b8_need = static_cast<size_t>(N) * K;
   if (ctx->b8_bytes < b8_need) {
     if (cudaDeviceSynchronize() != cudaSuccess) st = W4A4_ERR_CUDA;
+    uint8_t* larger = nullptr;
+    if (st == W4A4_OK) st = dev_alloc(&larger, b8_need, &ctx->bytes);
     if (st == W4A4_OK) {
       cudaFree(ctx->b8);
       ctx->bytes -= ctx->b8_bytes;
-      ctx->b8_bytes = 0;
-      st = dev_alloc(&ctx->b8, b8_need, &ctx->bytes);
-      if (st == W4A4_OK) ctx->b8_bytes = b8_need;
+      ctx->b8 = larger;
+      ctx->b8_bytes = b8_need;
     }
   }
   if (st == W4A4_OK) st = prepare_quantize<kCodesE4M3>(r, &h->wide_clusters);

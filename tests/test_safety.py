@@ -207,6 +207,15 @@ def test_every_allocation_of_context_and_handle_construction_fails_cleanly():
         w4.w4a4_debug_fail_allocation_after(-1)
         assert L is not None and handle_allocs >= 6, "the hook must have reached every allocation of the handle"
 
+        # a layer whose weight image needs a larger scratch than the context has: the old one stays until the new one is there
+        held = w4.w4a4_ctx_bytes(ctx.ptr)
+        wide = gen.make_layer_direct(K, 4 * N, r, seed=5).to(DEV)
+        w4.w4a4_debug_fail_allocation_after(0)
+        with pytest.raises(w4.W4A4Error):
+            w4.Layer(ctx, [wide], num_bins=1)
+        w4.w4a4_debug_fail_allocation_after(-1)
+        assert w4.w4a4_ctx_bytes(ctx.ptr) == held
+
         # and the survivors work
         assert forward_matches_oracle(ctx, L, layer, M, seed=9)
         ctx.check()
