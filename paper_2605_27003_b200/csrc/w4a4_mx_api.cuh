@@ -233,6 +233,7 @@ w4a4_status_t w4a4_mx_pack_weights(w4a4_ctx_t ctx, const w4a4_mx_weight_desc_t* 
   // The activation scale atoms live in the context (zero-filled once: rows past M of the last row block are
   // read by the tensor core and must not hold E8M0's NaN byte).
   if (!ctx->mx_sfa) {
+    const size_t bytes_before = ctx->bytes;
     const size_t nb = mx_sfa_bytes(ctx->max_M, ctx->max_K);
     st = dev_alloc(&ctx->mx_sfa, nb, &ctx->bytes);
     if (st == W4A4_OK && cudaMemset(ctx->mx_sfa, 0, nb) != cudaSuccess) st = W4A4_ERR_CUDA;
@@ -255,7 +256,17 @@ w4a4_status_t w4a4_mx_pack_weights(w4a4_ctx_t ctx, const w4a4_mx_weight_desc_t* 
     if (st == W4A4_OK) st = dev_alloc(&ctx->mx_t32, static_cast<size_t>(ctx->max_M) * rr, &ctx->bytes);
     if (st == W4A4_OK) st = dev_alloc(&ctx->t_hilo2, static_cast<size_t>(ctx->max_M) * 2 * rr, &ctx->bytes);
     if (st == W4A4_OK && cudaMemset(ctx->t_hilo2, 0, sizeof(uint16_t) * ctx->max_M * 2 * rr) != cudaSuccess) st = W4A4_ERR_CUDA;
-
+    if (st != W4A4_OK) {   // all of them or none: the next layer starts over
+      cudaFree(ctx->mx_sfa);
+      cudaFree(ctx->mx_codes2);
+      cudaFree(ctx->mx_sfa2);
+      cudaFree(ctx->mx_t32);
+      cudaFree(ctx->t_hilo2);
+      ctx->mx_sfa = ctx->mx_codes2 = ctx->mx_sfa2 = nullptr;
+      ctx->mx_t32 = nullptr;
+      ctx->t_hilo2 = nullptr;
+      ctx->bytes = bytes_before;
+    }
   }
   if (st == W4A4_OK) st = prepare_quantize<kCodesMxfp4>(r, &h->wide_clusters);
   int* d_bad = nullptr;

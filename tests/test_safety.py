@@ -223,3 +223,36 @@ def test_every_allocation_of_context_and_handle_construction_fails_cleanly():
         ctx.close()
     finally:
         w4.w4a4_debug_fail_allocation_after(-1)
+
+
+def test_every_allocation_of_a_first_mxfp4_layer_fails_cleanly():
+    # The first MXFP4 layer of a context also makes the context's MXFP4 workspaces: all of them, or none.
+    pkg_build.build()
+    w4.load_library()
+    M, K, N, r = 200, 512, 256, 16
+    layer = gen.make_layer_mx_direct(K, N, r, seed=4).to(DEV)
+    try:
+        whole = w4.Context(0, M, K, r)
+        w4.MxLayer(whole, [layer], num_bins=1).close()
+        want = w4.w4a4_ctx_bytes(whole.ptr)
+        whole.close()
+        n, made = 0, False
+        while not made and n < 64:
+            ctx = w4.Context(0, M, K, r)
+            empty = w4.w4a4_ctx_bytes(ctx.ptr)
+            w4.w4a4_debug_fail_allocation_after(n)
+            try:
+                w4.MxLayer(ctx, [layer], num_bins=1).close()
+                made = True
+            except w4.W4A4Error as e:
+                assert e.status == ERR_ALLOC
+                assert w4.w4a4_ctx_bytes(ctx.ptr) in (empty, want), f"allocation {n}: the workspaces were left half made"
+            w4.w4a4_debug_fail_allocation_after(-1)
+            L = w4.MxLayer(ctx, [layer], num_bins=1)
+            assert w4.w4a4_ctx_bytes(ctx.ptr) == want, f"allocation {n}: the next layer found the workspaces half made"
+            L.close()
+            ctx.close()
+            n += 1
+        assert made and n > 8, "the hook must have reached every allocation"
+    finally:
+        w4.w4a4_debug_fail_allocation_after(-1)
