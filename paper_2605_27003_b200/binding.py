@@ -27,7 +27,7 @@ EXPORTED_SYMBOLS = (
     "w4a4_tile_shape", "w4a4_quantize_noalloc", "w4a4_clip_search",
     "w4a4_mx_pack_weights", "w4a4_mx_destroy", "w4a4_mx_handle_bytes", "w4a4_mx_linear_forward",
     "w4a4_mx_quantize_activations", "w4a4_mx_gemm_from_workspace", "w4a4_mx_debug_quantize", "w4a4_mx_clip_search",
-    "w4a4_mx_ffn_forward", "w4a4_mx_debug_fused_input", "w4a4_gptq_quantize", "w4a4_mx_gptq_quantize", "w4a4_gptq_accumulate", "w4a4_gptq_workspace_bytes", "w4a4_query_status", "w4a4_debug_wait_probe", "w4a4_debug_stalled_gemm", "w4a4_debug_stalled_split_gemm", "w4a4_mx_debug_stalled_split_gemm", "w4a4_debug_set_tile_order",
+    "w4a4_mx_ffn_forward", "w4a4_mx_debug_fused_input", "w4a4_gptq_quantize", "w4a4_mx_gptq_quantize", "w4a4_gptq_accumulate", "w4a4_gptq_workspace_bytes", "w4a4_query_status", "w4a4_debug_wait_probe", "w4a4_debug_stalled_gemm", "w4a4_debug_stalled_split_gemm", "w4a4_debug_stalled_quantize", "w4a4_mx_debug_stalled_split_gemm", "w4a4_debug_set_tile_order",
     "w4a4_debug_fail_allocation_after", "w4a4_handle_bytes", "w4a4_ctx_bytes", "w4a4_status_string",
 )
 
@@ -112,6 +112,7 @@ def _lib():
         lib.w4a4_query_status.argtypes = [vp]
         lib.w4a4_debug_wait_probe.argtypes = [vp, ctypes.c_uint64, vp]
         lib.w4a4_debug_stalled_gemm.argtypes = [vp, ci, ci, vp, ci, ctypes.c_uint64, vp]
+        lib.w4a4_debug_stalled_quantize.argtypes = [vp, vp, ci, ci, ci, vp, ci, ctypes.c_uint64, vp]
         lib.w4a4_debug_stalled_split_gemm.argtypes = lib.w4a4_debug_stalled_gemm.argtypes
         lib.w4a4_mx_debug_stalled_split_gemm.argtypes = lib.w4a4_debug_stalled_gemm.argtypes
         lib.w4a4_debug_fail_allocation_after.argtypes = [ci]
@@ -403,6 +404,13 @@ def w4a4_debug_stalled_split_gemm(handle, M: int, expert_id: int, Y, stall_stage
     """Test hook: the same for the form whose clusters share K, the stage withheld from the first CTA of each."""
     name = "w4a4_mx_debug_stalled_split_gemm" if mx else "w4a4_debug_stalled_split_gemm"
     _check(getattr(_lib(), name)(handle, M, expert_id, _ptr(Y), int(stall_stage), int(limit_ns), _stream(stream)), name)
+
+
+def w4a4_debug_stalled_quantize(handle, X, M: int, expert_id: int, timestep_bin: int, clip_table, stall_group: int, limit_ns: int,
+                                stream=None):
+    """Test hook: the activation pass with the low-rank factor of one group withheld and a short wait limit."""
+    _check(_lib().w4a4_debug_stalled_quantize(handle, _ptr(X), M, expert_id, timestep_bin, _ptr(clip_table), int(stall_group),
+                                              int(limit_ns), _stream(stream)), "w4a4_debug_stalled_quantize")
 
 
 def w4a4_debug_set_tile_order(ctx, super_column_tiles: int):

@@ -268,11 +268,13 @@ struct QuantizeParams {
   ExpandJob expand;
   int* err;                 // error word of the bounded waits (R > 0)
   float one = 1.0f;         // see quantize8_ordinary
+  int dbg_stall_group;      // STALL: the group (of the first CTA of a cluster) whose part of L1 is never loaded
+  uint64_t dbg_wait_limit_ns;
 };
 
-// MINB CTAs per SM: the register budget.
-template <int R, int FORMAT, int STEPS, int MINB>
-__global__ void __launch_bounds__(quantize_threads(R), MINB)
+// Two CTAs per SM.  STALL: test hook, one load is withheld, so that the waits for it run into their limit.
+template <int R, int FORMAT, int STEPS, bool STALL = false>
+__global__ void __launch_bounds__(quantize_threads(R), 2)
 quantize_kernel(const __grid_constant__ CUtensorMap tmL1, const QuantizeParams p) {
   const int warps = static_cast<int>(blockDim.x >> 5) - (R > 0 ? 1 : 0), cta_rows = quantize_rows(STEPS, warps);
   const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
@@ -305,8 +307,9 @@ quantize_kernel(const __grid_constant__ CUtensorMap tmL1, const QuantizeParams p
   const int rows = min(cta_rows, p.M - row0), rows_each = (rows + gridDim.y - 1) / gridDim.y;
   const int rows_mine = max(0, min(rows_each, rows - static_cast<int>(blockIdx.y) * rows_each));
   uint32_t tmem = 0;
-  const WaitEnv env{p.err, &s_abort_word, kWaitLimitNs};
+  const WaitEnv env{p.err, &s_abort_word, STALL ? p.dbg_wait_limit_ns : kWaitLimitNs};
   auto load_l1 = [&](int it) {   // by one lane
+    if (STALL && it == p.dbg_stall_group && blockIdx.y == 0) return;
     const uint32_t bar = bar_l1 + 8 * (it % kL1Stages);
     mbar_arrive_expect_tx(bar, R * 128);
     tma_load_2d(ring + (it % kL1Stages) * (R * 128), &tmL1, bar, 64 * (g_begin + it), 0);

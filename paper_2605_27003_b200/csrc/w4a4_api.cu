@@ -159,9 +159,9 @@ w4a4_status_t check_forward_args(w4a4_handle_t h, const void* X, int M, int expe
 // Kernel 1's limits for every plan of a layer, once where the layer is packed.  They belong to the kernel on the device, not to
 // a launch: set per launch, one thread's smaller size would meet another thread's larger launch.  wide_clusters: how many
 // clusters of kMaxKSplits CTAs, a size that not every device can launch, run at a time.
-template <int R, int FORMAT, int STEPS, int MINB>
+template <int R, int FORMAT, int STEPS, bool STALL = false>
 bool prepare_quantize_steps(int* wide_clusters) {
-  auto* const kernel = quantize_kernel<R, FORMAT, STEPS, MINB>;
+  auto* const kernel = quantize_kernel<R, FORMAT, STEPS, STALL>;
   const size_t most = quantize_smem_bytes(R, STEPS, kQuantWarps, kMaxKSplits);   // grows with the warps and with the splits
   if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(most)) != cudaSuccess) return false;
   if (R == 0) return true;   // no clusters
@@ -184,7 +184,7 @@ bool prepare_quantize_steps(int* wide_clusters) {
 }
 template <int R, int FORMAT>
 bool prepare_quantize_rank(int* wide_clusters) {
-  return prepare_quantize_steps<R, FORMAT, 4, 2>(wide_clusters) && prepare_quantize_steps<R, FORMAT, 2, 2>(wide_clusters);
+  return prepare_quantize_steps<R, FORMAT, 4>(wide_clusters) && prepare_quantize_steps<R, FORMAT, 2>(wide_clusters);
 }
 template <int FORMAT>
 w4a4_status_t prepare_quantize(int r, int* wide_clusters) {
@@ -203,7 +203,7 @@ w4a4_status_t prepare_quantize(int r, int* wide_clusters) {
 
 // Kernel 1's launch: row blocks x K splits (a cluster per row block when K is split and there is a low-rank branch), plus
 // the CTAs that expand weights.
-template <int R, int FORMAT, int STEPS, int MINB>
+template <int R, int FORMAT, int STEPS, bool STALL>
 cudaError_t launch_quantize_steps(int num_sms, cudaStream_t stream, const CUtensorMap& tmL1, QuantizeParams p, const QuantizePlan& plan) {
   const int warps = plan.warps, splits = plan.splits;
   const int threads = quantize_threads(R, warps), cta_rows = quantize_rows(STEPS, warps);
@@ -211,14 +211,14 @@ cudaError_t launch_quantize_steps(int num_sms, cudaStream_t stream, const CUtens
   p.expand.first_cta = row_ctas;
   const OverlappedLaunch l(dim3(row_ctas + (expand_ctas(p.expand.chunks, threads, num_sms) + splits - 1) / splits, splits), dim3(threads),
                            quantize_smem_bytes(R, STEPS, warps, splits), stream, dim3(1, R > 0 ? splits : 1));
-  return cudaLaunchKernelEx(&l.cfg, quantize_kernel<R, FORMAT, STEPS, MINB>, tmL1, p);
+  return cudaLaunchKernelEx(&l.cfg, quantize_kernel<R, FORMAT, STEPS, STALL>, tmL1, p);
 }
-template <int R, int FORMAT>
+template <int R, int FORMAT, bool STALL = false>
 cudaError_t launch_quantize_kernel(const w4a4_ctx* ctx, int wide_clusters, cudaStream_t stream, const CUtensorMap& tmL1, const QuantizeParams& p) {
   const bool expand = R > 0 ? FORMAT == kCodesE4M3 : p.expand.chunks > 0;   // (without a low-rank branch nothing is summed over K)
   const QuantizePlan plan = quantize_plan(p.M, p.K / 64, R, ctx->num_sms, ctx->gemm_clusters, wide_clusters, expand);
-  if (plan.steps == 4) return launch_quantize_steps<R, FORMAT, 4, 2>(ctx->num_sms, stream, tmL1, p, plan);
-  return launch_quantize_steps<R, FORMAT, 2, 2>(ctx->num_sms, stream, tmL1, p, plan);
+  if (plan.steps == 4) return launch_quantize_steps<R, FORMAT, 4, STALL>(ctx->num_sms, stream, tmL1, p, plan);
+  return launch_quantize_steps<R, FORMAT, 2, STALL>(ctx->num_sms, stream, tmL1, p, plan);
 }
 
 // Index of (expert, this layer, bin) in a clip table (Sec. III-C: one ratio per expert, layer and timestep bin).
@@ -236,7 +236,8 @@ ExpandJob expand_job(const w4a4_layer* h, int expert_id) {
 // image with the expert's weights.
 // `scales`: also store the FP32 group scales (the parity tap; the GEMM reads them from the scale operands).
 w4a4_status_t launch_quantize_at(w4a4_handle_t h, const void* X, int M, int expert_id, const float* clip_table,
-                                 int clip_index, bool expand, cudaStream_t stream, float* scales = nullptr) {
+                                 int clip_index, bool expand, cudaStream_t stream, float* scales = nullptr, int stall_group = -1,
+                                 uint64_t wait_limit_ns = kWaitLimitNs) {
   if (M == 0) return W4A4_OK;
   w4a4_ctx* ctx = h->ctx;
   const ExpertData& e = h->experts[expert_id];
@@ -256,7 +257,18 @@ w4a4_status_t launch_quantize_at(w4a4_handle_t h, const void* X, int M, int expe
   p.a_sop = reinterpret_cast<uint2*>(ctx->a_sop);
   p.expand = job;
   p.err = ctx->d_err;
+  p.dbg_stall_group = stall_group;
+  p.dbg_wait_limit_ns = wait_limit_ns;
   cudaError_t le;
+  if (stall_group >= 0) {   // the test hook exists at one rank
+    int clusters = 0;
+    if (h->r != 32) return W4A4_ERR_SHAPE;
+    if (!prepare_quantize_steps<32, kCodesE4M3, 4, true>(&clusters) || !prepare_quantize_steps<32, kCodesE4M3, 2, true>(&clusters))
+      return W4A4_ERR_CUDA;
+    le = launch_quantize_kernel<32, kCodesE4M3, true>(ctx, h->wide_clusters, stream, e.tmL1, p);
+    if (le != cudaSuccess) cudaGetLastError();
+    return le == cudaSuccess ? W4A4_OK : W4A4_ERR_CUDA;
+  }
 #define W4A4_LAUNCH_Q(R) le = launch_quantize_kernel<R, kCodesE4M3>(ctx, h->wide_clusters, stream, h->r > 0 ? e.tmL1 : h->tmSopA, p)
   switch (h->r) {
     case 0: W4A4_LAUNCH_Q(0); break;
@@ -869,6 +881,18 @@ w4a4_status_t w4a4_debug_stalled_gemm(w4a4_handle_t h, int M, int expert_id, voi
 w4a4_status_t w4a4_debug_stalled_split_gemm(w4a4_handle_t h, int M, int expert_id, void* Y, int stall_stage,
                                             uint64_t limit_ns, void* stream) {
   return stalled_gemm(h, M, expert_id, Y, stall_stage, limit_ns, stream, true);
+}
+
+w4a4_status_t w4a4_debug_stalled_quantize(w4a4_handle_t h, const void* X, int M, int expert_id, int timestep_bin,
+                                          const float* clip_table, int stall_group, uint64_t limit_ns, void* stream) {
+  w4a4_status_t st = check_forward_args(h, X, M, expert_id, timestep_bin, clip_table, true);
+  if (st != W4A4_OK) return st;
+  if (stall_group < 0) return W4A4_ERR_INVALID_ARG;
+  if (limit_ns == 0 || limit_ns > 100000000ull) return W4A4_ERR_INVALID_ARG;  // at most 0.1 s
+  DeviceGuard guard(h->ctx->device);
+  if (!guard.ok) return W4A4_ERR_CUDA;
+  return launch_quantize_at(h, X, M, expert_id, clip_table, clip_table_index(h, expert_id, timestep_bin), false,
+                            static_cast<cudaStream_t>(stream), nullptr, stall_group, limit_ns);
 }
 
 w4a4_status_t w4a4_debug_set_tile_order(w4a4_ctx_t ctx, int super_column_tiles) {

@@ -82,7 +82,7 @@ extern "C" w4a4_status_t w4a4_quantize_noalloc(const void* X, int M, int K, cons
   const int cta_rows = w4a4::quantize_rows(kSteps, plan.warps), row_ctas = (M + cta_rows - 1) / cta_rows;
   p.expand.first_cta = row_ctas;
   const CUtensorMap no_map = {};   // no low-rank branch
-  w4a4::quantize_kernel<0, w4a4::kCodesInt8, kSteps, 2>
+  w4a4::quantize_kernel<0, w4a4::kCodesInt8, kSteps>
       <<<dim3(row_ctas, plan.splits), w4a4::quantize_threads(0, plan.warps), w4a4::quantize_smem_bytes(0, kSteps, plan.warps, 1), s>>>(no_map, p);
   return cudaGetLastError() == cudaSuccess ? W4A4_OK : W4A4_ERR_CUDA;
 }

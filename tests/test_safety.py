@@ -10,7 +10,8 @@
    that the producer, both MMA-issuing warps and the epilogue warps all run into a 1 ms limit and leave through the
    kernel's common tail (drain of copies in flight, release of tensor memory).  In the form whose clusters share a tile's K
    (`w4a4_debug_stalled_split_gemm`, both grids) one CTA of each cluster stalls, and the others must not store what they
-   add up from its part.
+   add up from its part.  Kernel 1 (`w4a4_debug_stalled_quantize`) misses a part of its low-rank factor, alone and in the
+   clusters whose members push partial sums into one another's shared memory.
 2. Allocation failures.  A countdown hook makes the n-th device allocation fail as a refused cudaMalloc would.  Walking
    n over every allocation of w4a4_ctx_create and w4a4_pack_weights checks that each partial construction returns
    W4A4_ERR_ALLOC, leaks nothing (device memory in use returns to where it was) and leaves the library usable.
@@ -141,6 +142,43 @@ def test_a_stalled_member_of_a_cluster_keeps_the_others_from_storing(grid, M, K,
     assert bool((y == 7.0).all())
     assert w4.w4a4_query_status(ctx.ptr) == ERR_TIMEOUT
     assert w4.w4a4_query_status(ctx.ptr) == 0
+    assert torch.equal(L.forward(x, 0, 0, clip), before)
+    ctx.check()
+    L.close()
+    ctx.close()
+
+
+@pytest.mark.parametrize("M,K,group", [
+    (9600, 256, 1),     # K not split: one CTA per row block
+    (700, 1024, 0),     # clusters of 8, the first group
+    (200, 2112, 2),     # clusters of 16, the last members without groups; the last group of the first CTA's share
+])
+def test_a_stalled_activation_pass_gives_up_and_stores_no_t(M, K, group):
+    # With a residual of zeros the output is T L2 + bias.  A GEMM enqueued behind the failed pass stores nothing; one after the
+    # query finds T as the forward before left it.
+    pkg_build.build()
+    w4.load_library()
+    N, r = 256, 32
+    layer = gen.make_layer_direct(K, N, r, seed=6).to(DEV)
+    layer.qweight.zero_()
+    ctx = w4.Context(0, M, K, r)
+    L = w4.Layer(ctx, [layer], num_bins=1)
+    x = gen.make_activations(M, K, seed=12).to(DEV)
+    clip = torch.ones((1, 1, 1), dtype=torch.float32, device=DEV)
+    before = L.forward(x, 0, 0, clip)
+    y = torch.full_like(before, 7.0)
+    ev0, ev1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    ev0.record()
+    w4.w4a4_debug_stalled_quantize(L.ptr, -x, M, 0, 0, clip, group, 1_000_000)   # T of -x would be -T
+    w4.w4a4_gemm_from_workspace(L.ptr, M, 0, y)
+    ev1.record()
+    torch.cuda.synchronize()
+    assert ev0.elapsed_time(ev1) < 500.0, "the stalled kernel must end by itself shortly after its limit"
+    assert bool((y == 7.0).all()), "a GEMM behind a failed activation pass stored rows"
+    assert w4.w4a4_query_status(ctx.ptr) == ERR_TIMEOUT
+    assert w4.w4a4_query_status(ctx.ptr) == 0
+    w4.w4a4_gemm_from_workspace(L.ptr, M, 0, y)
+    assert torch.equal(y, before), "T was stored although a part of it is missing"
     assert torch.equal(L.forward(x, 0, 0, clip), before)
     ctx.check()
     L.close()
