@@ -324,6 +324,9 @@ w4a4_status_t w4a4_query_status(w4a4_ctx_t ctx);
  * w4a4_debug_stalled_quantize runs w4a4_quantize_activations (r = 32 only, else W4A4_ERR_SHAPE) with the low-rank factor of
  * one group (number stall_group >= 0 of the first CTA's share of K) never loaded: the tensor-core warp and the warps that
  * wait for it give up after limit_ns, the members of a cluster that wait for their partial sums follow, and T is not stored.
+ * w4a4_debug_scale_arithmetic compares, for the group thresholds whose FP32 bit patterns are first_bits .. first_bits + count
+ * - 1 (positive, finite), the short forms in which kernel 1 derives ordinary scales, reciprocals and codes with the general
+ * ones (IEEE division, conversion to integer), and adds the number of thresholds with any difference to *differ (device).
  * w4a4_debug_set_tile_order forces the width, in 128-channel column tiles, of the super-columns in which the INT4
  * GEMM walks its output tiles (all row blocks of one super-column before the next; the width is otherwise chosen so
  * that a super-column's weight bytes take about two ninths of the L2); 0 restores the automatic choice.  Results do
@@ -332,6 +335,7 @@ w4a4_status_t w4a4_debug_wait_probe(w4a4_ctx_t ctx, uint64_t limit_ns, void* str
 w4a4_status_t w4a4_debug_set_tile_order(w4a4_ctx_t ctx, int super_column_tiles);
 w4a4_status_t w4a4_debug_stalled_gemm(w4a4_handle_t h, int M, int expert_id, void* Y, int stall_stage,
                                       uint64_t limit_ns, void* stream);
+w4a4_status_t w4a4_debug_scale_arithmetic(w4a4_ctx_t ctx, uint32_t first_bits, uint32_t count, uint64_t* differ, void* stream);
 w4a4_status_t w4a4_debug_stalled_quantize(w4a4_handle_t h, const void* X, int M, int expert_id, int timestep_bin,
                                           const float* clip_table, int stall_group, uint64_t limit_ns, void* stream);
 w4a4_status_t w4a4_debug_stalled_split_gemm(w4a4_handle_t h, int M, int expert_id, void* Y, int stall_stage,

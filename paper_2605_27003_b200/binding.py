@@ -27,7 +27,7 @@ EXPORTED_SYMBOLS = (
     "w4a4_tile_shape", "w4a4_quantize_noalloc", "w4a4_clip_search",
     "w4a4_mx_pack_weights", "w4a4_mx_destroy", "w4a4_mx_handle_bytes", "w4a4_mx_linear_forward",
     "w4a4_mx_quantize_activations", "w4a4_mx_gemm_from_workspace", "w4a4_mx_debug_quantize", "w4a4_mx_clip_search",
-    "w4a4_mx_ffn_forward", "w4a4_mx_debug_fused_input", "w4a4_gptq_quantize", "w4a4_mx_gptq_quantize", "w4a4_gptq_accumulate", "w4a4_gptq_workspace_bytes", "w4a4_query_status", "w4a4_debug_wait_probe", "w4a4_debug_stalled_gemm", "w4a4_debug_stalled_split_gemm", "w4a4_debug_stalled_quantize", "w4a4_mx_debug_stalled_split_gemm", "w4a4_debug_set_tile_order",
+    "w4a4_mx_ffn_forward", "w4a4_mx_debug_fused_input", "w4a4_gptq_quantize", "w4a4_mx_gptq_quantize", "w4a4_gptq_accumulate", "w4a4_gptq_workspace_bytes", "w4a4_query_status", "w4a4_debug_wait_probe", "w4a4_debug_stalled_gemm", "w4a4_debug_stalled_split_gemm", "w4a4_debug_stalled_quantize", "w4a4_debug_scale_arithmetic", "w4a4_mx_debug_stalled_split_gemm", "w4a4_debug_set_tile_order",
     "w4a4_debug_fail_allocation_after", "w4a4_handle_bytes", "w4a4_ctx_bytes", "w4a4_status_string",
 )
 
@@ -113,6 +113,7 @@ def _lib():
         lib.w4a4_debug_wait_probe.argtypes = [vp, ctypes.c_uint64, vp]
         lib.w4a4_debug_stalled_gemm.argtypes = [vp, ci, ci, vp, ci, ctypes.c_uint64, vp]
         lib.w4a4_debug_stalled_quantize.argtypes = [vp, vp, ci, ci, ci, vp, ci, ctypes.c_uint64, vp]
+        lib.w4a4_debug_scale_arithmetic.argtypes = [vp, ctypes.c_uint32, ctypes.c_uint32, vp, vp]
         lib.w4a4_debug_stalled_split_gemm.argtypes = lib.w4a4_debug_stalled_gemm.argtypes
         lib.w4a4_mx_debug_stalled_split_gemm.argtypes = lib.w4a4_debug_stalled_gemm.argtypes
         lib.w4a4_debug_fail_allocation_after.argtypes = [ci]
@@ -411,6 +412,12 @@ def w4a4_debug_stalled_quantize(handle, X, M: int, expert_id: int, timestep_bin:
     """Test hook: the activation pass with the low-rank factor of one group withheld and a short wait limit."""
     _check(_lib().w4a4_debug_stalled_quantize(handle, _ptr(X), M, expert_id, timestep_bin, _ptr(clip_table), int(stall_group),
                                               int(limit_ns), _stream(stream)), "w4a4_debug_stalled_quantize")
+
+
+def w4a4_debug_scale_arithmetic(ctx, first_bits: int, count: int, differ, stream=None):
+    """Test hook: kernel 1's short scale and code arithmetic against the general forms; differ: int64 device tensor, added to."""
+    _check(_lib().w4a4_debug_scale_arithmetic(ctx, int(first_bits), int(count), _ptr(differ), _stream(stream)),
+           "w4a4_debug_scale_arithmetic")
 
 
 def w4a4_debug_set_tile_order(ctx, super_column_tiles: int):

@@ -108,8 +108,8 @@ __device__ __forceinline__ void group_scale(float rho, float a, float& s, float&
   is = a > 0.0f ? __frcp_rn(s) : 0.0f;
 }
 // The same for kOrdinaryMin <= x <= kOrdinaryMax, where nothing under- or overflows: an approximation corrected by its exact
-// remainder (Markstein, IBM J. Res. Dev. 34, 1990) is the correctly rounded quotient; compared with the two functions above
-// for every significand.  9 instructions instead of 27.
+// remainder (Markstein, IBM J. Res. Dev. 34, 1990) is the correctly rounded quotient; the tests compare both results with
+// group_scale's for every x of the range.  9 instructions instead of 27.
 constexpr float kOrdinaryMin = 1e-30f, kOrdinaryMax = 1e30f;
 __device__ __forceinline__ void group_scale_ordinary(float x, float& s, float& is) {
   const float seventh = 0.142857142857142857f;
@@ -142,6 +142,34 @@ __device__ __forceinline__ void quantize8_ordinary(const float* xh, float is, fl
     u[e >> 1] = __viaddmin_s16x2_relu(__byte_perm(__float_as_uint(m.x), __float_as_uint(m.y), 0x5410), 0x00080008u, 0x000f000fu);
   }
 }
+// Test hook: the two short forms above against the general ones, for every threshold whose bit pattern is in [first, first +
+// count).  Codes at, next to and far outside every rounding boundary.  *differ: thresholds with a difference.
+static __global__ void scale_arithmetic_kernel(uint32_t first, uint32_t count, float one, unsigned long long* differ) {
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) {
+    const float x = __uint_as_float(first + i);
+    if (!(x >= kOrdinaryMin && x <= kOrdinaryMax)) continue;
+    float s, is, s_general, is_general;
+    group_scale_ordinary(x, s, is);
+    group_scale(1.0f, x, s_general, is_general);
+    bool bad = __float_as_uint(s) != __float_as_uint(s_general) || __float_as_uint(is) != __float_as_uint(is_general);
+    for (int b = 0; b < 64; b += 8) {
+      float xh[8];
+      uint32_t u[4], u_general[4];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {   // boundary (b + e) / 3 and its neighbours below and above
+        const int n = (b + e) / 3;
+        const float z = n < 17 ? n - 8.5f : (n & 1 ? 7.0f : -7.0f) / (n < 19 ? kRhoOrdinary : 0.25f);
+        xh[e] = __uint_as_float(__float_as_uint(__fmul_rn(s, z)) + (b + e) % 3 - 1);
+      }
+      quantize8_ordinary(xh, is, one, u);
+      quantize8(xh, is, u_general);
+#pragma unroll
+      for (int w = 0; w < 4; ++w) bad = bad || u[w] != u_general[w];
+    }
+    if (bad) atomicAdd(differ, 1ull);
+  }
+}
+
 // Codes + 8, two to a word -> E4M3 bytes.  A half-word 0 .. 15 read as FP16 is u 2^-24: two exact FP16 steps make it u - 8,
 // and the conversion is exact too.
 __device__ __forceinline__ uint2 e4m3_of_codes(const uint32_t* u) {

@@ -895,6 +895,16 @@ w4a4_status_t w4a4_debug_stalled_quantize(w4a4_handle_t h, const void* X, int M,
                             static_cast<cudaStream_t>(stream), nullptr, stall_group, limit_ns);
 }
 
+w4a4_status_t w4a4_debug_scale_arithmetic(w4a4_ctx_t ctx, uint32_t first_bits, uint32_t count, uint64_t* differ, void* stream) {
+  if (!ctx || !differ) return W4A4_ERR_INVALID_ARG;
+  if (first_bits + static_cast<uint64_t>(count) > 0x7f800000ull) return W4A4_ERR_INVALID_ARG;   // positive and finite
+  DeviceGuard guard(ctx->device);
+  if (!guard.ok) return W4A4_ERR_CUDA;
+  scale_arithmetic_kernel<<<8 * ctx->num_sms, 256, 0, static_cast<cudaStream_t>(stream)>>>(
+      first_bits, count, 1.0f, reinterpret_cast<unsigned long long*>(differ));
+  return cudaGetLastError() == cudaSuccess ? W4A4_OK : W4A4_ERR_CUDA;
+}
+
 w4a4_status_t w4a4_debug_set_tile_order(w4a4_ctx_t ctx, int super_column_tiles) {
   if (!ctx || super_column_tiles < 0) return W4A4_ERR_INVALID_ARG;
   ctx->debug_sc_tiles = super_column_tiles;
