@@ -97,7 +97,6 @@ struct OverlappedLaunch {
   OverlappedLaunch(const OverlappedLaunch&) = delete;
 };
 
-constexpr int kMaxDevices = 64;     // devices whose answers are remembered
 constexpr int kMaxGemmSplits = 8;   // the portable cluster size
 // CTAs that share the K of one output tile: as many as still run all tiles at once, if each keeps `min_stages` of the tile's
 // operand stages.  `clusters[s]`: clusters of s CTAs that fit the device at a time (a cluster stays within one GPC).
