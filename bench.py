@@ -35,7 +35,7 @@ NOMINAL_INT8_TOPS = 4500.0
 NOMINAL_HBM_GBS = 7700.0
 # dram__bytes_read.sum + dram__bytes_write.sum per launch, each from one single-launch ncu capture of the kernel as
 # it stands (summaries under profiles/); None where no capture exists for that kernel and workload.
-NCU_TRAFFIC_BYTES = {("gemm", "attn_proj"): 545.9e6, ("quantize", "attn_proj"): 503.3e6}
+NCU_TRAFFIC_BYTES = {("gemm", "attn_proj"): 576.9e6, ("quantize", "attn_proj"): 495.7e6}
 
 
 def max_over_ranks(ms: float, dist, device="cpu") -> float:
@@ -403,7 +403,7 @@ def run_dit_step(args, w4, dev, local_rank, rank, world, dist, peaks, tp):
     if rank == 0:
         tops = whole_job_tops(d["ops"], world, ms_per_step)
         roof = tensor_roofline(tops / world, total_ms * 1e-3, peaks, tp)
-        roof.update(traffic=None, kernel="quantize + expand + gemm of every layer, whole step")
+        roof.update(traffic=None, kernel="quantize (with the weight expansion) + gemm of every layer, whole step")
         line = dict(metric=METRIC, value=tops, unit=UNIT, n_gpus=world, steps=args.steps, warmup=args.warmup,
                     ms_per_step=ms_per_step, higher_is_better=True, scaling="weak", vs_baseline=None, dtype="e4m3",
                     data="synthetic",
@@ -414,7 +414,7 @@ def run_dit_step(args, w4, dev, local_rank, rank, world, dist, peaks, tp):
                                 l2="inputs larger than L2: 3 rotating activation buffers per shape (335 / 906 MB)",
                                 parallelism="replicas" if world > 1 else "single"),
                     ms_per_dit_step=ms_per_step, roofline=roof, tensor_peaks=tp,
-                    gpu_launches=3 * d["linears"] * args.steps, clocks=d["clocks"])
+                    gpu_launches=2 * d["linears"] * args.steps, clocks=d["clocks"])
         print(json.dumps(line), flush=True)
     if dist is not None:
         dist.barrier()
@@ -607,7 +607,7 @@ def run_mxfp4_ffn(args, w4, dev, local_rank, rank, peaks, tp):
         roofline=roof,
         two_calls=dict(ms_per_step=ms_two, value=ops / (ms_two * 1e-3) / 1e12, unit=UNIT,
                        note="same layers as w4a4_mx_linear_forward twice (hidden activation stored and re-read)"),
-        e2e=None, gpu_launches=5 * args.steps, clocks=clocks)), flush=True)
+        e2e=None, gpu_launches=4 * args.steps, clocks=clocks)), flush=True)
     l_up.close()
     l_dn.close()
     ctx.close()
@@ -676,47 +676,29 @@ def run_clip_search(args, w4, dev, local_rank, rank, peaks):
         config=dict(workload="clip_search", M=M, K=K, N=N, r=r, candidates=cands, samples=n_samples,
                     l2="inputs larger than L2: activations and reference outputs of %.0f MB each" % (M * K * 2 / 1e6)),
         ms_per_forward=ms / forwards, best_candidate=cands[best], objective=errs,
-        gpu_launches=(2 * forwards + 2) * searches, clocks=clocks)), flush=True)
+        gpu_launches=(2 * forwards + 1) * searches, clocks=clocks)), flush=True)
     layer.close()
     ctx.close()
 
 
 def gptq_launch_count(K: int, nb: int = 64, band: int = 512, lazy: int = 256) -> int:
-    """Kernel launches of one w4a4_gptq_quantize call with calibration activations: the library's loop structure
-    (conversion, statistic, diagonal fix-ups, weight copy; banded factorization; banded triangular inverse; sweep in
-    lazy batches), counting only launches that have work."""
-    n = 5
+    """Kernel launches of one w4a4_gptq_quantize call with calibration activations: the library's loop structure (statistic,
+    banded factorization, sweep over lazy batches), counting only launches that have work."""
+    n = 3                                               # conversion, statistic, diagonal
     hi = K
-    while hi > 0:                                   # H = V V^T
+    while hi > 0:                                       # H = V V^T
         lo = max(0, hi - band)
-        for j0 in range(hi - nb, lo - 1, -nb):
-            n += 1                                  # diagonal block
-            if j0 == 0:
-                break
-            n += 1 + (1 if j0 > lo else 0)          # panel, in-band update
-        n += 1 if lo > 0 else 0
+        steps = (hi - lo) // nb
+        n += steps + (steps - 1) + (1 if lo > 0 else 0)     # block and panel, in-band update, update left of the band
         hi = lo
-    hi = K
-    while hi > 0:                                   # U = V^-1
-        lo = max(0, hi - band)
-        n += 1                                      # the band's diagonal inverses
-        n += 2 * len(range(hi - 2 * nb, lo - 1, -nb))
-        n += 2 if K - hi > 0 else 0
-        hi = lo
-    for b0 in range(0, K, lazy):                    # sweep
-        b1 = min(K, b0 + lazy)
-        for k0 in range(b0, b1, nb):
-            n += 1 + (1 if b1 - k0 - nb > 0 else 0)
-        if b1 < K:
-            b2 = min(K, b1 + lazy)
-            n += 1 + (1 if K - b2 > 0 else 0)       # next batch's rows, then the rest
-    return n
+    batches = -(-K // lazy)
+    return n + 1 + batches + (batches - 1)              # diagonal-block inverses; sweep, update of the later channels
 
 
 def run_gptq(args, w4, dev, local_rank, rank, peaks):
     """GPTQ on the residual branch (Sec. III-B) for one attention-projection layer: statistic from 2048 calibration
-    tokens, factorization, triangular inverse and the sweep, all FP64 on the device.  An offline step: the number is a
-    time per layer, with the FP64 rate it amounts to."""
+    tokens, factorization and the sweep, all FP64 on the device.  An offline step: the number is a time per layer, with the
+    FP64 rate it amounts to."""
     if rank != 0:
         return
     K, N = {"gptq": (5120, 5120), "gptq_mx": (5120, 5120), "gptq_ffn_up": (5120, 13824),
@@ -746,11 +728,11 @@ def run_gptq(args, w4, dev, local_rank, rank, peaks):
         torch.cuda.synchronize()
         per_call.append(e0.elapsed_time(e1))
     clocks = sampler.stop()
-    # A call is some 600 short launches from one host thread; when the host is disturbed a call takes up to twice
-    # as long with the same kernels.  The median says what the device does, the mean is reported beside it.
+    # A call is a chain of some 200 launches from one host thread; when the host is disturbed a call takes longer with the
+    # same kernels.  The median says what the device does, the mean is reported beside it.
     ms = statistics.median(per_call)
-    # FP64 operations the algorithm needs: upper triangle of X^T X, H = V V^T, U = V^-1, the error propagation
-    flops = M_cal * K * K + K ** 3 / 3 + K ** 3 / 3 + float(K) * K * N
+    # FP64 operations of the call: upper triangle of X^T X, H = V V^T, the error propagation
+    flops = M_cal * K * K + K ** 3 / 3 + float(K) * K * N
     sm_mhz = clocks.get("sm_max_mhz") or 1965
     peak = 148 * 64 * 2 * sm_mhz * 1e6 / 1e12      # 64 FP64 fused multiply-adds per SM and clock
     cpu = None
@@ -918,10 +900,10 @@ def main():
         roof.update(traffic=NCU_TRAFFIC_BYTES.get(("gemm", args.workload)),
                     kernel="gemm_w4a4_kernel (with the expand_weight_kernel in front of it)", ms=tg)
         # Bytes the activation step needs by its definition (X read; 4-bit codes, FP32 group scales and BF16 T written)
-        # and bytes this layout moves (one E4M3 byte per code, FP32 scales plus the 8-byte scale operand of the GEMM's
-        # scale MMA per (token, group), T as a BF16 high | low pair).
+        # and bytes this layout moves (one E4M3 byte per code, the 8-byte scale operand of the GEMM's scale MMA per (token,
+        # group), T as a BF16 high | low pair).
         q_alg = M * (2.0 * K + 0.5 * K + 4.0 * K / 64.0 + 2.0 * r)
-        q_layout = M * (2.0 * K + 1.0 * K + 4.0 * K / 64.0 + 8.0 * K / 64.0 + 4.0 * r)
+        q_layout = M * (2.0 * K + 1.0 * K + 8.0 * K / 64.0 + 4.0 * r)
         q_gbs = q_alg / (tq * 1e-3) / 1e9
         line = dict(
             metric=METRIC, value=value, unit=UNIT, n_gpus=world, steps=args.steps, warmup=args.warmup,

@@ -6,8 +6,8 @@
 // FP32 accumulators of tcgen05.mma kind::f8f6f4.  Feeding the codes as E4M3 bytes therefore yields the same
 // per-group partial sums P of Eq. 7, already in FP32.
 //
-// Both kernels translate "code + 8" (a nibble u in [0, 15]) to its E4M3 byte with the same byte-permute
-// lookup: two 8-entry tables held in two registers each, selected by the low three bits of every nibble,
+// The weight expansion translates "code + 8" (a nibble u in [0, 15]) to its E4M3 byte with a byte-permute
+// lookup (kernel 1 converts its codes by exact FP16 arithmetic): two 8-entry tables held in two registers each, selected by the low three bits of every nibble,
 // and a byte mask derived from the nibble's top bit that picks between them.
 #pragma once
 

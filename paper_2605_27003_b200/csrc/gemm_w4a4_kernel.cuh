@@ -18,7 +18,7 @@
 // zeros.  The epilogue then needs one fused multiply-add per partial sum, acc += P_g * S_g, on two TMEM fragments
 // and reads no scales from shared memory.  Operand tiles of the scale MMA live in global memory as ready-made
 // shared-memory images (no-swizzle K-major canonical layout: [8-row group][8 rows][16 bytes]); kernel 1 writes the
-// token side next to the FP32 scales, the channel side is built once at pack time.  The low-rank product T L2 goes
+// token side, the channel side is built once at pack time.  The low-rank product T L2 goes
 // through the same path as one more "group" that opens a tile: its P is the BF16 product [T_hi | T_lo] [L2 | L2]^T,
 // which the epilogue takes as the accumulators' first value.
 //
@@ -42,7 +42,8 @@
 //               another) were slower.
 // What bounds the kernel is the serial chain of an epilogue warp per group: wait, load, 8 multiply-adds, load, release, 8
 // multiply-adds (a stand-alone copy of the hand-over runs at 330-340 clocks per group with the MMAs and without them; the
-// loads and multiply-adds alone at 200; this kernel at ~355).  A lone warp's dependent instructions
+// loads and multiply-adds alone at 200; this kernel at 349, from its clocks per tile at 80 and 216 groups, plus about
+// 2600 per tile for the tile's end).  A lone warp's dependent instructions
 // cost 10-15 cycles each and a branch on a fresh mbarrier result ~70, so the hops are written as single instruction
 // sequences without branches: wait_issue_* (try_wait, then fence, MMAs and commit predicated on its answer),
 // wait_then_ld16 (try_wait, then fence and first TMEM load predicated on its answer), descriptors computed before the wait, and
@@ -54,7 +55,8 @@
 // Split K (SPLIT instantiation): where the tiles alone leave most SMs idle, the CTAs of a thread-block cluster share one
 // tile, each over its part of the operand stages (the first one with the low-rank product).  Their FP32 partial tiles meet
 // in shared memory (the operand ring's, idle by then), and every CTA adds its share of them over distributed shared
-// memory in split order, so results do not depend on timing.  One tile per CTA, no loop.
+// memory in split order, so results do not depend on timing; none does once a member has given up on a wait.  One tile per
+// CTA, no loop.
 // Every role loops warp-uniformly (waits are voted, only the TMA / tcgen05 instructions are predicated on one elected
 // lane), which keeps ring positions, addresses and descriptors in uniform registers.  All waits are bounded
 // (pipeline.cuh).  Finally + bias -> optional GELU -> BF16, or the squared error against a reference (clip search).

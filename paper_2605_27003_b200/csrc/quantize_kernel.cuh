@@ -13,19 +13,20 @@
 // tile, from which one more warp issues four tcgen05.mma per group (M = 128, N = r, K = 16 each; the rows past the CTA's own
 // read whatever lies behind the tile and only touch accumulator rows that nobody reads) against the group's r x 64 tile
 // of L1, which it fetches by TMA into a ring of its own.
-// The bound is instruction issue: 101 (MXFP4) to 115 instructions per 8 values and lane at r = 32, 57 to 65 % of the issue slots
-// of two CTAs per SM, DRAM at about 70 %.  So the loop's addresses are kept in registers (derived anew in every pass they
-// cost 15 of those instructions: 127 -> 94 us at 32760 x 5120 MXFP4) and the rare cases of the scale arithmetic have a branch
-// of their own.  The predecessor held 16 rows of a warp in mma.sync fragments, with r accumulators per row in registers.
-// 32760 x 5120, INT4 | MXFP4: r = 0 120 -> 100 | 93 -> 79 us, r = 32 148 -> 113 | 122 -> 92, r = 64 192 -> 120 | 158 -> 100, r = 96
-// 278 -> 140 (INT4); 32760 x 13824, r = 32 389 -> 290 | 320 -> 233.  (335 MB in and 168 | 89 MB out take 76 | 64 us.)
+// The bound is instruction issue and latency: 93 (MXFP4) to 123 warp instructions per 8 values and lane at r = 32 take 60 to
+// 67 % of the issue slots of two CTAs per SM; DRAM traffic is 60 % of what a copy reaches.  So the loop's addresses are kept in
+// registers (derived anew in every pass they cost 15 of those instructions: 127 -> 94 us at 32760 x 5120 MXFP4) and the rare cases
+// of the scale arithmetic have a branch of their own.  The predecessor held 16 rows of a warp in mma.sync fragments, with r
+// accumulators per row in registers.  Eight launches replayed from one graph, 32760 x 5120, INT4 | MXFP4: r = 0 120 -> 100 | 93 ->
+// 79 us, r = 32 148 -> 113.5 | 121 -> 93, r = 64 192 -> 120 | 158 -> 101, r = 96 278 -> 140 (INT4); 32760 x 13824, r = 32 390 -> 291 |
+// 320 -> 237.  (335 MB in and 168 | 89 MB out take 76 | 64 us.)
 //
 // K split (gridDim.y > 1): with few token rows there are too few row blocks to fill the machine, so the K groups are divided
 // among gridDim.y CTAs per row block, which form one thread-block cluster when there is a low-rank branch.  Codes and scales
 // of different groups are independent; of T every CTA adds up a share of the rows, for which the others push their partial
 // sums into its shared memory (st.async on an mbarrier there) and which it adds in split order.  Pulled over distributed
 // shared memory between two cluster barriers instead, the end of the kernel took 5000 clocks, pushed about 2000.
-// 100 x 5120, r = 32 12.9 -> 5.4 us INT4, 9.0 -> 5.1 MXFP4; 700 x 8192, r = 64 22.6 -> 11.6 | 15.9 -> 10.6.
+// 100 x 5120, r = 32 12.9 -> 5.4 us INT4, 9.0 -> 5.1 MXFP4; 700 x 8192, r = 64 23.1 -> 12.9 | 16.6 -> 10.7.
 //
 // Weight expansion (ExpandJob): the CTAs past the row blocks turn the layer's 4-bit weights into the byte image the
 // INT4 GEMM reads.  It is independent of the activations, so it shares their launch instead of being a kernel between

@@ -33,8 +33,8 @@ constexpr size_t quantize_smem_bytes(int R, int steps, int warps, int splits) {
 // that run at a time, one CTA to an SM, as the device answers (0: such a cluster cannot be launched there).
 // `expand`: the layer's forwards carry an expansion in this launch.  With a low-rank branch every launch for such a layer
 // passes it, also one that carries none (a stage called alone, a search's later candidates, later chunks of a host forward):
-// the K split is the summation order of T, and the same rows have to give the same bits.  (A search of 12 forwards of 1560 x
-// 5120 -> 5120, r = 32, takes 1194 us with it and 1173 with the split that suits launches without an expansion.)
+// the K split is the summation order of T, and the same rows have to give the same bits.  (Without an expansion the
+// launch takes 14.2 us with it and 12.9 with the plan below at 1560 x 5120, r = 32, a search of 12 forwards 1194 and 1173.)
 struct QuantizePlan {
   int steps, warps, splits;   // a CTA owns 4 steps warps rows and a 1 / splits share of the groups
 };
@@ -50,8 +50,10 @@ inline QuantizePlan quantize_plan(int M, int G, int r, int sms, const int* fitti
     return {steps, warps, splits < 1 || G < 4 ? 1 : (splits > G / 2 ? G / 2 : splits)};
   }
   // Beside an expansion, which takes longer than the activations and wants its share of the machine from the start: smaller
-  // CTAs, two to an SM, about one per SM in all.  Forwards of 5120 -> 5120: 700 rows, r = 64 60.0 -> 51.2 us; 1560, r = 64
-  // 96.8 -> 90.3; 4097, r = 96 204 -> 194.
+  // CTAs, two to an SM, about one per SM in all.  Eight forwards of 5120 -> 5120 replayed from one graph, each: 700 rows,
+  // r = 64 60.0 -> 51.2 us; 1560, r = 64 96.8 -> 90.3; 4097, r = 96 204 -> 194.   Above 34 x 128 rows
+  // it no longer pays: 4480 rows, r = 32 201.4 us with this plan and 200.0 with the general one, 4736 209.2 | 199.7; r = 96 209.7 |
+  // 210.6 and 215.2 | 213.0.
   if (expand && M > few && M <= 34 * 128) {
     const int k = M <= 1024 ? 8 : 4, clusters = k == 8 ? 16 : 33, warps = (M + 8 * clusters - 1) / (8 * clusters);
     if (k <= G / 2 && fitting_clusters[k] > 0) return {2, warps < kQuantWarps ? warps : kQuantWarps, k};

@@ -28,7 +28,7 @@
 
 namespace {
 
-constexpr int kNb = 64;     // block of the factorization = quantization group = lazy batch
+constexpr int kNb = 64;     // block of the factorization = quantization group
 constexpr int kBand = 512;  // columns per band of the factorization
 constexpr int kLazy = 256;  // input channels per lazy batch of the sweep
 
@@ -637,7 +637,7 @@ void launch_dgemm(cudaStream_t st, const GemmArgs& g) {
   const dim3 grid(g.N / kBN, (g.M + BM - 1) / BM);
   dgemm_kernel<BM, AK, BK><<<grid, 256, dgemm_smem_bytes(BM), st>>>(g);
 }
-// 128-row tiles where they fill the SMs; 64-row tiles (twice the blocks, 4/3 of the operand traffic) where they would not.
+// 128-row tiles where they fill the 148 SMs; 64-row tiles (twice the blocks, 4/3 of the operand traffic) where they would not.
 template <bool AK, bool BK>
 void dgemm(cudaStream_t st, const GemmArgs& g) {
   if (g.M <= 0 || g.N <= 0 || g.Kd <= 0) return;

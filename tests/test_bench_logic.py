@@ -59,6 +59,11 @@ def test_dit_step_layer_list_matches_the_workload_definition():
     assert sum(k * n for k, n, _ in packed) == sum(k * n for k, n, _ in shapes)
 
 
+def test_gptq_launch_count_follows_the_library():
+    assert bench.gptq_launch_count(64) == 6        # conversion, statistic, diagonal, one step, one inverse, one sweep
+    assert bench.gptq_launch_count(5120) == 202    # as listed by a profiler
+
+
 def test_reference_arm_prints_one_contract_line_on_the_tiny_workload():
     p = subprocess.run([sys.executable, os.path.join(ROOT, "bench.py"), "--impl", "reference", "--workload", "tiny",
                         "--steps", "2", "--warmup", "1"], capture_output=True, text=True, timeout=600, cwd=ROOT)
