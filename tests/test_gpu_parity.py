@@ -456,8 +456,9 @@ def test_shared_tiles_in_the_clip_search():
 @pytest.mark.parametrize("M,K,r", [
     (33, 64, 16),        # one group, CTAs of one warp, the last one with one row
     (448, 2112, 64),     # most rows at two steps per warp; 33 groups over 16 CTAs: the last ones have none
-    (449, 2048, 32),     # fewest rows at four steps per warp
+    (449, 2048, 32),     # fewest rows with the plan of launches beside an expansion, eight CTAs per row block
     (1029, 576, 96),     # nine groups over four CTAs, ragged last row block
+    (4353, 384, 32),     # fewest rows above that plan: four steps per warp, three CTAs per row block
     (1029, 1024, 0),     # no low-rank branch: splits without clusters
     (9300, 128, 64),     # not split: fewer warps per CTA than eight, T straight from TMEM
 ])
