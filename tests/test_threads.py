@@ -3,6 +3,9 @@
 Two threads, each with its own context, layer and stream, run the same instantiation of kernel 1 with row counts whose
 launches differ (CTA size, shared memory).  Outputs of every call have to be those of a run without the other thread.
 """
+import os
+import subprocess
+import sys
 import threading
 
 import pytest
@@ -57,3 +60,26 @@ def test_threads_with_contexts_of_their_own_do_not_meet(grid):
         ctx.check()
         L.close()
         ctx.close()
+
+
+FIRST_CALL = """
+import torch, paper_2605_27003_b200 as w4
+from workloads import generator as gen
+mx, K, N, r, M = {mx}, 2048, 256, 64, 1
+layer = (gen.make_layer_mx_direct if mx else gen.make_layer_direct)(K, N, r, seed=1).to("cuda:0")
+ctx = w4.Context(0, M, K, r)
+L = (w4.MxLayer if mx else w4.Layer)(ctx, [layer], num_bins=1)
+L.forward(gen.make_activations(M, K, seed=2).to("cuda:0"), 0, 0, torch.full((1, 1, 1), 0.9, device="cuda:0"))
+torch.cuda.synchronize()
+ctx.check()
+"""
+
+
+@pytest.mark.parametrize("mx", [False, True])
+def test_the_first_call_of_a_process_needs_no_larger_one_before_it(mx):
+    # This plan's dynamic shared memory is 48 KiB exactly: with the kernel's static part it is more than a launch may take
+    # unless the kernel's limit has been raised.
+    pkg_build.build()
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    p = subprocess.run([sys.executable, "-c", FIRST_CALL.format(mx=mx)], cwd=root, capture_output=True, text=True, timeout=300)
+    assert p.returncode == 0, p.stderr[-2000:]
