@@ -205,12 +205,28 @@ __host__ __device__ constexpr uint32_t xh_position(uint32_t c) {
 // Keeps an address that the loop needs from being derived again in every pass.
 __device__ __forceinline__ void keep_in_register(uint32_t& v) { asm volatile("" : "+r"(v)); }
 
-// Two neighbouring entries of a row of T as BF16 high parts (columns c, c + 1 of the row) and the BF16 rounding of the
-// remainders (columns R + c, R + c + 1).
-__device__ __forceinline__ void store_t_pair(uint16_t* row, int R, int c, float t0, float t1) {
+// Two entries of T as BF16 high parts and the BF16 rounding of the remainders.
+__device__ __forceinline__ uint2 split_t_pair(float t0, float t1) {
   const __nv_bfloat16 h0 = __float2bfloat16_rn(t0), h1 = __float2bfloat16_rn(t1);
-  *reinterpret_cast<uint32_t*>(row + c) = pack_bf16x2(__bfloat162float(h0), __bfloat162float(h1));
-  *reinterpret_cast<uint32_t*>(row + R + c) = pack_bf16x2(t0 - __bfloat162float(h0), t1 - __bfloat162float(h1));
+  return make_uint2(pack_bf16x2(__bfloat162float(h0), __bfloat162float(h1)), pack_bf16x2(t0 - __bfloat162float(h0), t1 - __bfloat162float(h1)));
+}
+// Four neighbouring entries of a row of T: high parts to columns c .. c + 3, remainders to R + c .. R + c + 3.
+__device__ __forceinline__ void store_t4(uint16_t* row, int R, int c, const float4& t) {
+  const uint2 a = split_t_pair(t.x, t.y), b = split_t_pair(t.z, t.w);
+  *reinterpret_cast<uint2*>(row + c) = make_uint2(a.x, b.x);
+  *reinterpret_cast<uint2*>(row + R + c) = make_uint2(a.y, b.y);
+}
+// Eight, 16 bytes each.  A lane stores a row of its own, so that every access touches as many sectors as there are rows: in 4-byte
+// pieces 20000 x 256, r = 96 INT4 took 21.1 us instead of 10.0, 32760 x 5120 138 instead of 124.
+__device__ __forceinline__ void store_t8(uint16_t* row, int R, int c, const uint32_t* t) {
+  uint32_t hi[4], lo[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const uint2 p = split_t_pair(__uint_as_float(t[2 * i]), __uint_as_float(t[2 * i + 1]));
+    hi[i] = p.x, lo[i] = p.y;
+  }
+  *reinterpret_cast<uint4*>(row + c) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+  *reinterpret_cast<uint4*>(row + R + c) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
 }
 
 // Eight FP32 values -> eight E2M1 codes (round to nearest even, saturating at +-6), element 0 in the lowest nibble.
@@ -608,8 +624,7 @@ quantize_kernel(const __grid_constant__ CUtensorMap tmL1, const QuantizeParams p
           if (gridDim.y == 1) {
             if (ok && r < rows) {
 #pragma unroll
-              for (int e = 0; e < 16; e += 2)
-                store_t_pair(p.t_hilo + static_cast<size_t>(row) * (2 * R), R, c + e, __uint_as_float(v[e]), __uint_as_float(v[e + 1]));
+              for (int e = 0; e < 16; e += 8) store_t8(p.t_hilo + static_cast<size_t>(row) * (2 * R), R, c + e, v + e);
             }
           } else if (ok && r < rows) {
             const uint32_t owner = r / rows_each, at = pushed + ((blockIdx.y * rows_each + r - owner * rows_each) * R + c) * 4;
@@ -639,8 +654,7 @@ quantize_kernel(const __grid_constant__ CUtensorMap tmL1, const QuantizeParams p
             t.x += v.x, t.y += v.y, t.z += v.z, t.w += v.w;
           }
           uint16_t* dst = p.t_hilo + static_cast<size_t>(row0 + blockIdx.y * rows_each + r) * (2 * R);
-          store_t_pair(dst, R, 4 * q, t.x, t.y);
-          store_t_pair(dst, R, 4 * q + 2, t.z, t.w);
+          store_t4(dst, R, 4 * q, t);
         }
       }
       cluster_wait();   // nobody leaves while its shared memory may still be written
