@@ -31,7 +31,7 @@ constexpr size_t quantize_smem_bytes(int R, int steps, int warps, int splits) {
 
 // How a launch divides M rows x G groups.  fitting_clusters[k], k <= 8, and wide_clusters: clusters of k and of kMaxKSplits CTAs
 // that run at a time, one CTA to an SM, as the device answers (0: such a cluster cannot be launched there).
-// `expand`: the layer's forwards carry an expansion in this launch.  With a low-rank branch every launch for such a layer
+// `int4`: an INT4 layer, whose codes take longer.  `expand`: the layer's forwards carry an expansion in this launch.  With a low-rank branch every launch for such a layer
 // passes it, also one that carries none (a stage called alone, a search's later candidates, later chunks of a host forward):
 // the K split is the summation order of T, and the same rows have to give the same bits.  (Without an expansion the
 // launch takes 14.2 us with it and 12.9 with the plan below at 1560 x 5120, r = 32, a search of 12 forwards 1194 and 1173.)
@@ -39,7 +39,22 @@ struct QuantizePlan {
   int steps, warps, splits;   // a CTA owns 4 steps warps rows and a 1 / splits share of the groups
 };
 constexpr int kMaxKSplits = 16;
-inline QuantizePlan quantize_plan(int M, int G, int r, int sms, const int* fitting_clusters, int wide_clusters, bool expand) {
+
+// Clocks that a launch of 16-row warps takes, as a model: a group takes an SM as long as its element-wise warps need to issue it, or
+// one warp's own chain; every CTA adds its start and the end with T.  `int4`: INT4 codes, else MXFP4.
+inline int quantize_clocks(int M, int G, int r, int fitting, int w, int k, bool int4) {
+  const int slots = quantize_smem_bytes(r, 4, w, k) <= 114688 ? 2 : 1;   // CTAs that share an SM
+  const int ctas = ((M + 16 * w - 1) / (16 * w) + fitting - 1) / fitting;     // CTAs that an SM takes in all
+  const int groups = (G + k - 1) / k;
+  auto wave = [&](int n) {   // n CTAs at a time
+    const int issue = (int4 ? 142 : 160) * w * n + 23 * n, chain = int4 ? 1300 : 1250;
+    return groups * (issue > chain ? issue : chain) + 4300 + 820 * n + (k > 1 ? 13 : 1) * r * w * n / 2;
+  };
+  const int last = ctas % slots;
+  return ctas / slots * wave(slots) + (last > 0 ? wave(last) : 0) + (k > 1 ? 2000 + 190 * k : 0);
+}
+
+inline QuantizePlan quantize_plan(int M, int G, int r, int sms, const int* fitting_clusters, int wide_clusters, bool int4, bool expand) {
   const int few = 448;   // rows up to which 2 steps per warp beat 4
   if (r == 0) {
     // The splits are independent CTAs.  About five to an SM at any size, so that no SM is left with a CTA more than others:
@@ -58,23 +73,28 @@ inline QuantizePlan quantize_plan(int M, int G, int r, int sms, const int* fitti
     const int k = M <= 1024 ? 8 : 4, clusters = k == 8 ? 16 : 33, warps = (M + 8 * clusters - 1) / (8 * clusters);
     if (k <= G / 2 && fitting_clusters[k] > 0) return {2, warps < kQuantWarps ? warps : kQuantWarps, k};
   }
-  // The splits of a row block form a cluster; with the partial sums of T a CTA's shared memory leaves room for one per SM,
-  // and a cluster stays within a GPC.  The most splits that still run all row blocks at once, and the fewest warps that cover
-  // the rows: 1560 x 5120, r = 32, in 14 clusters of 8 CTAs of 7 warps 12.0 us, of 4 CTAs 15.9 us,
-  // not split 57 us; 32760 x 5120 split in two 152 us, not split 115 us.
-  for (int k = kMaxKSplits; k > 1; k = k > 8 ? 8 : k - 1) {
+  // The splits of a row block form a cluster, which stays within a GPC.  With few rows: the most splits that still run all row
+  // blocks at once, one CTA to an SM, and the fewest warps that cover the rows.
+  if (M <= few) for (int k = kMaxKSplits; k > 1; k = k > 8 ? 8 : k - 1) {
     const int clusters = k > 8 ? wide_clusters : fitting_clusters[k];
     const int steps = k > 8 && M <= few ? 2 : 4, per_warp = 4 * steps;
     if (clusters > 0 && k <= G / 2 && M <= clusters * kQuantWarps * per_warp)
       return {steps, (M + clusters * per_warp - 1) / (clusters * per_warp), k};
   }
-  // Not split, two CTAs per SM: the number of warps for which the busiest SM has the fewest rows.  32760 rows: 256 CTAs of 8
-  // warps leave 40 SMs with one, 293 of 7 fill 146.5: 120.3 -> 114.7 us at K = 5120, r = 32.
+  // Otherwise what takes the fewest clocks.  The model's constants are fitted to 444 measured surfaces (449 to 32760 rows, K 256 to
+  // 13824, r 16 to 96, all warps and splits): its choice is 1.6 % (MXFP4) and 2.5 % (INT4) slower than the best one on average and
+  // 3 | 5 % faster than the rule before it (the most splits with one CTA to an SM, else none), nowhere by more than 3 % slower.
+  // That rule left the middle of the range half empty: 6000 x 13824, r = 16, MXFP4 73 -> 53 us, 9600 rows 135 -> 82.  32760 rows
+  // keep 293 CTAs of 7 warps.
   QuantizePlan best = {4, kQuantWarps, 1};
-  int least = 1 << 30;
-  for (int w = kQuantWarps; w >= 4; --w) {
-    const int ctas = (M + 16 * w - 1) / (16 * w), rows = (ctas + sms - 1) / sms * w;
-    if (rows < least) least = rows, best.warps = w;
+  int least = quantize_clocks(M, G, r, sms, kQuantWarps, 1, int4);
+  for (int k = 1; k <= kMaxKSplits; k = k == 8 ? kMaxKSplits : k + 1) {
+    const int clusters = k == 1 ? sms : (k > 8 ? wide_clusters : fitting_clusters[k]);
+    if (clusters == 0 || (k > 1 && k > G / 2)) continue;
+    for (int w = kQuantWarps; w >= (M <= 2048 ? 2 : 4); --w) {
+      const int clocks = quantize_clocks(M, G, r, clusters, w, k, int4);
+      if (clocks < least) least = clocks, best = {4, w, k};
+    }
   }
   return best;
 }

@@ -12,8 +12,8 @@ import pytest
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2605_27003_b200", "csrc")
 SHIM = """
 #include "quantize_plan.h"
-extern "C" void plan(int M, int G, int r, int sms, const int* fitting, int wide, int expand, int* out) {
-  const w4a4::QuantizePlan p = w4a4::quantize_plan(M, G, r, sms, fitting, wide, expand != 0);
+extern "C" void plan(int M, int G, int r, int sms, const int* fitting, int wide, int int4, int expand, int* out) {
+  const w4a4::QuantizePlan p = w4a4::quantize_plan(M, G, r, sms, fitting, wide, int4 != 0, expand != 0);
   out[0] = p.steps, out[1] = p.warps, out[2] = p.splits;
   out[3] = static_cast<int>(w4a4::quantize_smem_bytes(r, p.steps, p.warps, p.splits));
   out[4] = static_cast<int>(w4a4::quantize_smem_bytes(r, p.steps, w4a4::kQuantWarps, w4a4::kMaxKSplits));
@@ -33,9 +33,9 @@ def plan(tmp_path_factory):
     subprocess.run(["g++", "-std=c++17", "-O1", "-Wall", "-Werror", "-shared", "-fPIC", "-I", CSRC, "-o", str(lib), str(src)], check=True)
     fn = ctypes.CDLL(str(lib)).plan
 
-    def call(M, G, r, sms=148, fitting=FULL, wide=7, expand=False):
+    def call(M, G, r, sms=148, fitting=FULL, wide=7, expand=False, int4=None):
         out = (ctypes.c_int * 6)()
-        fn(M, G, r, sms, (ctypes.c_int * 9)(*fitting), wide, int(expand), out)
+        fn(M, G, r, sms, (ctypes.c_int * 9)(*fitting), wide, int(expand if int4 is None else int4), int(expand), out)
         return dict(zip(("steps", "warps", "splits", "smem", "limit", "rows"), out))
     return call
 
@@ -65,3 +65,19 @@ def test_every_plan_stays_within_the_limits_set_at_pack_time(plan):
                     assert p["steps"] in (2, 4) and 1 <= p["warps"] <= 8 and 1 <= p["splits"] <= max(1, G), (M, G, r, expand, p)
                     assert p["smem"] <= p["limit"] <= 232448, (M, G, r, expand, p)
                     assert p["rows"] <= 128
+
+
+@pytest.mark.parametrize("M", [6000, 9600, 12000, 14000])
+@pytest.mark.parametrize("int4", [False, True])
+def test_the_middle_of_the_range_fills_the_machine(plan, M, int4):
+    # A warp's chain takes about eight warps' issue time, so fewer than that per SM leave it waiting; two CTAs fit.
+    p = plan(M, 216, 16, int4=int4)
+    assert -(-M // p["rows"]) * p["splits"] * p["warps"] >= 8 * 148, p
+
+
+@pytest.mark.parametrize("r", [16, 32, 64, 96])
+def test_the_model_keeps_the_plan_of_full_launches(plan, r):
+    # 293 CTAs of seven warps, two to an SM, in one wave.
+    for int4 in (False, True):
+        p = plan(32760, 80, r, int4=int4)
+        assert (p["steps"], p["warps"], p["splits"]) == (4, 7, 1), p
