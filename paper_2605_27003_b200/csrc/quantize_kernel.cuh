@@ -312,6 +312,7 @@ struct QuantizeParams {
   uint2* a_sop;             // kCodesE4M3: token-side scale operands of the GEMM
   ExpandJob expand;
   int* err;                 // error word of the bounded waits (R > 0)
+  int row_warps;            // element-wise warps that a CTA has rows for; a launch may have spare ones, for the expansion
   float one = 1.0f;         // see quantize8_ordinary
   int dbg_stall_group;      // STALL: the group (of the first CTA of a cluster) whose part of L1 is never loaded
   uint64_t dbg_wait_limit_ns;
@@ -321,7 +322,8 @@ struct QuantizeParams {
 template <int R, int FORMAT, int STEPS, bool STALL = false>
 __global__ void __launch_bounds__(quantize_threads(R), 2)
 quantize_kernel(const __grid_constant__ CUtensorMap tmL1, const QuantizeParams p) {
-  const int warps = static_cast<int>(blockDim.x >> 5) - (R > 0 ? 1 : 0), cta_rows = quantize_rows(STEPS, warps);
+  const int warps = p.row_warps, cta_rows = quantize_rows(STEPS, warps);
+  const int tensor_warp = static_cast<int>(blockDim.x >> 5) - 1;   // R > 0: the last one
   const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   if (blockIdx.x >= p.expand.first_cta) {   // whole clusters: the cluster spans gridDim.y, never blockIdx.x
     grid_dependency_wait();
@@ -351,6 +353,7 @@ quantize_kernel(const __grid_constant__ CUtensorMap tmL1, const QuantizeParams p
   const uint32_t pushed = x_ring + x_ring_bytes(R, STEPS, warps);
   const int rows = min(cta_rows, p.M - row0), rows_each = (rows + gridDim.y - 1) / gridDim.y;
   const int rows_mine = max(0, min(rows_each, rows - static_cast<int>(blockIdx.y) * rows_each));
+  const int active = (rows + 4 * STEPS - 1) / (4 * STEPS);   // element-wise warps that have rows; the others skip the groups
   uint32_t tmem = 0;
   const WaitEnv env{p.err, &s_abort_word, STALL ? p.dbg_wait_limit_ns : kWaitLimitNs};
   auto load_l1 = [&](int it) {   // by one lane
@@ -368,7 +371,7 @@ quantize_kernel(const __grid_constant__ CUtensorMap tmL1, const QuantizeParams p
     }
   };
 
-  if (R > 0 && warp == warps) {
+  if (R > 0 && warp == tensor_warp) {
     // ------------------------------------------------------------------ L1 producer and MMA issuer (one lane issues)
     constexpr uint32_t idesc = umma_idesc(1, 1, 128, R > 0 ? R : 16);
     const bool issuer = elect_one_lane();
@@ -377,7 +380,7 @@ quantize_kernel(const __grid_constant__ CUtensorMap tmL1, const QuantizeParams p
     if (issuer) {
       for (int i = 0; i < kL1Stages; ++i) mbar_init(bar_l1 + 8 * i, 1);
       for (int i = 0; i < kXhBuffers; ++i) {
-        mbar_init(bar_xh_full + 8 * i, warps);
+        mbar_init(bar_xh_full + 8 * i, active);
         mbar_init(bar_xh_empty + 8 * i, 1);
       }
       mbar_init(bar_t, 1);
@@ -421,6 +424,7 @@ quantize_kernel(const __grid_constant__ CUtensorMap tmL1, const QuantizeParams p
     grid_dependency_wait();
     const int j = lane & 7;                                     // this lane's channels: 8 j .. 8 j + 7 of the group
     const int tile_row = warp * (4 * STEPS) + (lane >> 4) + 2 * (lane >> 3 & 1);   // and rows: + 4 per step
+    const int g_first = warp < active ? g_begin : g_end;
     const float rho = __ldg(p.clip_table + p.clip_index);
     const float x_min = rho >= kRhoOrdinary ? kOrdinaryMin : kOrdinaryMax * 2.0f;   // below it the general path is taken
     // 32-bit byte offsets from the CTA's first row (at most 128 rows of 16384 channels and a margin): half the address
@@ -469,11 +473,11 @@ quantize_kernel(const __grid_constant__ CUtensorMap tmL1, const QuantizeParams p
       cp_async_commit();
     };
 #pragma unroll
-    for (int i = 0; i < kStages - 1; ++i) load(g_begin + i, stage_bytes * i);
+    for (int i = 0; i < kStages - 1; ++i) load(g_first + i, stage_bytes * i);
     join_setup();   // its microsecond passes beside the first loads
     uint32_t slot = 0, slot_before = stage_bytes * (kStages - 1);   // this group's and the previous group's
     bool ok = true;
-    for (int g = g_begin; g < g_end; ++g) {
+    for (int g = g_first; g < g_end; ++g) {
       float xh[STEPS][8];
       cp_async_wait<kStages - 2>();
       __syncwarp();
@@ -662,7 +666,7 @@ quantize_kernel(const __grid_constant__ CUtensorMap tmL1, const QuantizeParams p
     tc_fence_before_sync();
     __syncthreads();
     drain_after_abort(&s_abort_word);
-    if (warp == warps) {
+    if (warp == tensor_warp) {
       tc_fence_after_sync();
       tmem_dealloc(tmem, kTmemCols);
     }

@@ -31,12 +31,13 @@ constexpr size_t quantize_smem_bytes(int R, int steps, int warps, int splits) {
 
 // How a launch divides M rows x G groups.  fitting_clusters[k], k <= 8, and wide_clusters: clusters of k and of kMaxKSplits CTAs
 // that run at a time, one CTA to an SM, as the device answers (0: such a cluster cannot be launched there).
-// `int4`: an INT4 layer, whose codes take longer.  `expand`: the layer's forwards carry an expansion in this launch.  With a low-rank branch every launch for such a layer
+// `image`: bytes of an INT4 layer's weight image (0: MXFP4), whose codes take longer.  `expand`: the layer's forwards carry an expansion in this launch.  With a low-rank branch every launch for such a layer
 // passes it, also one that carries none (a stage called alone, a search's later candidates, later chunks of a host forward):
 // the K split is the summation order of T, and the same rows have to give the same bits.  (Without an expansion the
 // launch takes 14.2 us with it and 12.9 with the plan below at 1560 x 5120, r = 32, a search of 12 forwards 1194 and 1173.)
 struct QuantizePlan {
   int steps, warps, splits;   // a CTA owns 4 steps warps rows and a 1 / splits share of the groups
+  int spare = 0;              // warps without rows for a launch whose other CTAs expand weights
 };
 constexpr int kMaxKSplits = 16;
 
@@ -54,7 +55,8 @@ inline int quantize_clocks(int M, int G, int r, int fitting, int w, int k, bool 
   return ctas / slots * wave(slots) + (last > 0 ? wave(last) : 0) + (k > 1 ? 2000 + 190 * k : 0);
 }
 
-inline QuantizePlan quantize_plan(int M, int G, int r, int sms, const int* fitting_clusters, int wide_clusters, bool int4, bool expand) {
+inline QuantizePlan quantize_plan(int M, int G, int r, int sms, const int* fitting_clusters, int wide_clusters, size_t image, bool expand) {
+  const bool int4 = image > 0;
   const int few = 448;   // rows up to which 2 steps per warp beat 4
   if (r == 0) {
     // The splits are independent CTAs.  About five to an SM at any size, so that no SM is left with a CTA more than others:
@@ -74,12 +76,18 @@ inline QuantizePlan quantize_plan(int M, int G, int r, int sms, const int* fitti
     if (k <= G / 2 && fitting_clusters[k] > 0) return {2, warps < kQuantWarps ? warps : kQuantWarps, k};
   }
   // The splits of a row block form a cluster, which stays within a GPC.  With few rows: the most splits that still run all row
-  // blocks at once, one CTA to an SM, and the fewest warps that cover the rows.
-  if (M <= few) for (int k = kMaxKSplits; k > 1; k = k > 8 ? 8 : k - 1) {
+  // blocks at once, one CTA to an SM, and the fewest warps that cover the rows.  Above a byte image of 2^24 (5120 x 5120 is 1.6 of
+  // that) its expansion is what the launch takes long for, on CTAs of the same form: clusters of 8 at most, which leave fewer SMs
+  // out than those of 16, and six warps.  1 x 5120 -> 13824, r = 16: one warp in clusters of 16 111 us, six 57, six in clusters of 8 48;
+  // 1 x 5120 -> 5120 35, 22.4 and 22.0.  Smaller layers lose by it: 64 x 13824 -> 1024 22.5 us in clusters of 16, 28.6 of 8.
+  const bool large = image > (1u << 24);
+  if (M <= few) for (int k = large ? 8 : kMaxKSplits; k > 1; k = k > 8 ? 8 : k - 1) {
     const int clusters = k > 8 ? wide_clusters : fitting_clusters[k];
-    const int steps = k > 8 && M <= few ? 2 : 4, per_warp = 4 * steps;
-    if (clusters > 0 && k <= G / 2 && M <= clusters * kQuantWarps * per_warp)
-      return {steps, (M + clusters * per_warp - 1) / (clusters * per_warp), k};
+    const int steps = k > 8 || large ? 2 : 4, per_warp = 4 * steps;
+    if (clusters > 0 && k <= G / 2 && M <= clusters * kQuantWarps * per_warp) {
+      const int warps = (M + clusters * per_warp - 1) / (clusters * per_warp);
+      return {steps, warps, k, large && warps < 6 ? 6 - warps : 0};
+    }
   }
   // Otherwise what takes the fewest clocks.  The model's constants are fitted to 444 measured surfaces (449 to 32760 rows, K 256 to
   // 13824, r 16 to 96, all warps and splits): its choice is 1.6 % (MXFP4) and 2.5 % (INT4) slower than the best one on average and

@@ -199,17 +199,18 @@ w4a4_status_t prepare_quantize(int r, int* wide_clusters) {
 template <int R, int FORMAT, int STEPS, bool STALL>
 cudaError_t launch_quantize_steps(int num_sms, cudaStream_t stream, const CUtensorMap& tmL1, QuantizeParams p, const QuantizePlan& plan) {
   const int warps = plan.warps, splits = plan.splits;
-  const int threads = quantize_threads(R, warps), cta_rows = quantize_rows(STEPS, warps);
+  const int threads = quantize_threads(R, warps + (p.expand.chunks > 0 ? plan.spare : 0)), cta_rows = quantize_rows(STEPS, warps);
   const int row_ctas = (p.M + cta_rows - 1) / cta_rows;
+  p.row_warps = warps;
   p.expand.first_cta = row_ctas;
   const OverlappedLaunch l(dim3(row_ctas + (expand_ctas(p.expand.chunks, threads, num_sms) + splits - 1) / splits, splits), dim3(threads),
                            quantize_smem_bytes(R, STEPS, warps, splits), stream, dim3(1, R > 0 ? splits : 1));
   return cudaLaunchKernelEx(&l.cfg, quantize_kernel<R, FORMAT, STEPS, STALL>, tmL1, p);
 }
 template <int R, int FORMAT, bool STALL = false>
-cudaError_t launch_quantize_kernel(const w4a4_ctx* ctx, int wide_clusters, cudaStream_t stream, const CUtensorMap& tmL1, const QuantizeParams& p) {
+cudaError_t launch_quantize_kernel(const w4a4_ctx* ctx, int wide_clusters, size_t image, cudaStream_t stream, const CUtensorMap& tmL1, const QuantizeParams& p) {
   const bool expand = R > 0 ? FORMAT == kCodesE4M3 : p.expand.chunks > 0;   // (without a low-rank branch nothing is summed over K)
-  const QuantizePlan plan = quantize_plan(p.M, p.K / 64, R, ctx->num_sms, ctx->gemm_clusters, wide_clusters, FORMAT == kCodesE4M3, expand);
+  const QuantizePlan plan = quantize_plan(p.M, p.K / 64, R, ctx->num_sms, ctx->gemm_clusters, wide_clusters, image, expand);
   if (plan.steps == 4) return launch_quantize_steps<R, FORMAT, 4, STALL>(ctx->num_sms, stream, tmL1, p, plan);
   return launch_quantize_steps<R, FORMAT, 2, STALL>(ctx->num_sms, stream, tmL1, p, plan);
 }
@@ -236,6 +237,7 @@ w4a4_status_t launch_quantize_at(w4a4_handle_t h, const void* X, int M, int expe
   const ExpertData& e = h->experts[expert_id];
   ExpandJob job;
   if (expand) job = expand_job(h, expert_id);
+  const size_t image = static_cast<size_t>(h->N) * h->K;
   QuantizeParams p = {};
   p.X = static_cast<const uint16_t*>(X);
   p.M = M;
@@ -258,11 +260,11 @@ w4a4_status_t launch_quantize_at(w4a4_handle_t h, const void* X, int M, int expe
     if (h->r != 32) return W4A4_ERR_SHAPE;
     if (!prepare_quantize_steps<32, kCodesE4M3, 4, true>(&clusters) || !prepare_quantize_steps<32, kCodesE4M3, 2, true>(&clusters))
       return W4A4_ERR_CUDA;
-    le = launch_quantize_kernel<32, kCodesE4M3, true>(ctx, h->wide_clusters, stream, e.tmL1, p);
+    le = launch_quantize_kernel<32, kCodesE4M3, true>(ctx, h->wide_clusters, image, stream, e.tmL1, p);
     if (le != cudaSuccess) cudaGetLastError();
     return le == cudaSuccess ? W4A4_OK : W4A4_ERR_CUDA;
   }
-#define W4A4_LAUNCH_Q(R) le = launch_quantize_kernel<R, kCodesE4M3>(ctx, h->wide_clusters, stream, h->r > 0 ? e.tmL1 : h->tmSopA, p)
+#define W4A4_LAUNCH_Q(R) le = launch_quantize_kernel<R, kCodesE4M3>(ctx, h->wide_clusters, image, stream, h->r > 0 ? e.tmL1 : h->tmSopA, p)
   switch (h->r) {
     case 0: W4A4_LAUNCH_Q(0); break;
     case 16: W4A4_LAUNCH_Q(16); break;

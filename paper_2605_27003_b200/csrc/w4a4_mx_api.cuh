@@ -74,7 +74,7 @@ w4a4_status_t mx_launch_quantize_at(w4a4_mx_handle_t h, const void* X, int M, in
   p.t_hilo = ctx->t_hilo;
   p.err = ctx->d_err;
   cudaError_t le;
-#define W4A4_LAUNCH_MXQ(R) le = launch_quantize_kernel<R, kCodesMxfp4>(ctx, h->wide_clusters, stream, h->r > 0 ? e.tmL1 : h->tmA, p)
+#define W4A4_LAUNCH_MXQ(R) le = launch_quantize_kernel<R, kCodesMxfp4>(ctx, h->wide_clusters, 0, stream, h->r > 0 ? e.tmL1 : h->tmA, p)
   switch (h->r) {
     case 0: W4A4_LAUNCH_MXQ(0); break;
     case 16: W4A4_LAUNCH_MXQ(16); break;

@@ -76,10 +76,11 @@ extern "C" w4a4_status_t w4a4_quantize_noalloc(const void* X, int M, int K, cons
   p.clip_index = clip_index;
   p.codes = reinterpret_cast<uint8_t*>(codes);
   p.scales = scales;
-  w4a4::QuantizePlan plan = w4a4::quantize_plan(M, K / 64, 0, 148, nullptr, 0, true, false);
+  w4a4::QuantizePlan plan = w4a4::quantize_plan(M, K / 64, 0, 148, nullptr, 0, 0, false);
   constexpr int kSteps = 2;
   if (plan.steps != kSteps) plan.splits = (plan.splits + 1) / 2;
   const int cta_rows = w4a4::quantize_rows(kSteps, plan.warps), row_ctas = (M + cta_rows - 1) / cta_rows;
+  p.row_warps = plan.warps;
   p.expand.first_cta = row_ctas;
   const CUtensorMap no_map = {};   // no low-rank branch
   w4a4::quantize_kernel<0, w4a4::kCodesInt8, kSteps>

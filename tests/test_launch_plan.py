@@ -12,12 +12,12 @@ import pytest
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2605_27003_b200", "csrc")
 SHIM = """
 #include "quantize_plan.h"
-extern "C" void plan(int M, int G, int r, int sms, const int* fitting, int wide, int int4, int expand, int* out) {
-  const w4a4::QuantizePlan p = w4a4::quantize_plan(M, G, r, sms, fitting, wide, int4 != 0, expand != 0);
+extern "C" void plan(int M, int G, int r, int sms, const int* fitting, int wide, int image, int expand, int* out) {
+  const w4a4::QuantizePlan p = w4a4::quantize_plan(M, G, r, sms, fitting, wide, static_cast<size_t>(image), expand != 0);
   out[0] = p.steps, out[1] = p.warps, out[2] = p.splits;
   out[3] = static_cast<int>(w4a4::quantize_smem_bytes(r, p.steps, p.warps, p.splits));
   out[4] = static_cast<int>(w4a4::quantize_smem_bytes(r, p.steps, w4a4::kQuantWarps, w4a4::kMaxKSplits));
-  out[5] = w4a4::quantize_rows(p.steps, p.warps);
+  out[5] = w4a4::quantize_rows(p.steps, p.warps), out[6] = p.spare;
 }
 """
 FULL = [0, 0, 74, 45, 33, 26, 22, 15, 15]   # clusters of 2 .. 8 that fit a whole B200, one CTA to an SM
@@ -33,10 +33,10 @@ def plan(tmp_path_factory):
     subprocess.run(["g++", "-std=c++17", "-O1", "-Wall", "-Werror", "-shared", "-fPIC", "-I", CSRC, "-o", str(lib), str(src)], check=True)
     fn = ctypes.CDLL(str(lib)).plan
 
-    def call(M, G, r, sms=148, fitting=FULL, wide=7, expand=False, int4=None):
-        out = (ctypes.c_int * 6)()
-        fn(M, G, r, sms, (ctypes.c_int * 9)(*fitting), wide, int(expand if int4 is None else int4), int(expand), out)
-        return dict(zip(("steps", "warps", "splits", "smem", "limit", "rows"), out))
+    def call(M, G, r, sms=148, fitting=FULL, wide=7, expand=False, int4=None, image=1 << 22):
+        out = (ctypes.c_int * 7)()
+        fn(M, G, r, sms, (ctypes.c_int * 9)(*fitting), wide, image if (expand if int4 is None else int4) else 0, int(expand), out)
+        return dict(zip(("steps", "warps", "splits", "smem", "limit", "rows", "spare"), out))
     return call
 
 
@@ -62,7 +62,7 @@ def test_every_plan_stays_within_the_limits_set_at_pack_time(plan):
             for r in (0, 16, 32, 64, 96):
                 for expand in (False, True):
                     p = plan(M, G, r, expand=expand)
-                    assert p["steps"] in (2, 4) and 1 <= p["warps"] <= 8 and 1 <= p["splits"] <= max(1, G), (M, G, r, expand, p)
+                    assert p["steps"] in (2, 4) and 1 <= p["warps"] <= p["warps"] + p["spare"] <= 8 and 1 <= p["splits"] <= max(1, G), (M, G, r, expand, p)
                     assert p["smem"] <= p["limit"] <= 232448, (M, G, r, expand, p)
                     assert p["rows"] <= 128
 
@@ -81,3 +81,12 @@ def test_the_model_keeps_the_plan_of_full_launches(plan, r):
     for int4 in (False, True):
         p = plan(32760, 80, r, int4=int4)
         assert (p["steps"], p["warps"], p["splits"]) == (4, 7, 1), p
+
+
+@pytest.mark.parametrize("G", [8, 16, 80, 216])
+def test_few_rows_leave_enough_warps_for_the_weight_expansion(plan, G):
+    # The CTAs that expand weights have the plan's warps: with one or two each, a large layer's expansion took twice its time.
+    for M in (1, 8, 16, 64, 130, 300, 448):
+        p = plan(M, G, 16, expand=True, image=5120 * 5120)
+        assert 6 <= p["warps"] + p["spare"] <= 8 and p["splits"] <= 8
+        assert plan(M, G, 16, expand=True, image=1024 * 1024)["spare"] == 0
