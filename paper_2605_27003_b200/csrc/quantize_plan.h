@@ -31,10 +31,11 @@ constexpr size_t quantize_smem_bytes(int R, int steps, int warps, int splits) {
 
 // How a launch divides M rows x G groups.  fitting_clusters[k], k <= 8, and wide_clusters: clusters of k and of kMaxKSplits CTAs
 // that run at a time, one CTA to an SM, as the device answers (0: such a cluster cannot be launched there).
-// `image`: bytes of an INT4 layer's weight image (0: MXFP4), whose codes take longer.  `expand`: the layer's forwards carry an expansion in this launch.  With a low-rank branch every launch for such a layer
-// passes it, also one that carries none (a stage called alone, a search's later candidates, later chunks of a host forward):
-// the K split is the summation order of T, and the same rows have to give the same bits.  (Without an expansion the
-// launch takes 14.2 us with it and 12.9 with the plan below at 1560 x 5120, r = 32, a search of 12 forwards 1194 and 1173.)
+// `image`: bytes of an INT4 layer's weight image, which its forwards expand in this launch and whose codes take longer (0: MXFP4).
+// With a low-rank branch every launch for a layer has the same K split, also one without the expansion (a stage called alone, a
+// search's later candidates, later chunks of a host forward): the split is the summation order of T, and the same rows have to
+// give the same bits.  (Without an expansion 1560 x 5120, r = 32, takes 14.2 us with it and 12.9 with one of its own, a search of
+// 12 forwards 1194 and 1173.)
 struct QuantizePlan {
   int steps, warps, splits;   // a CTA owns 4 steps warps rows and a 1 / splits share of the groups
   int spare = 0;              // warps without rows for a launch whose other CTAs expand weights
@@ -55,15 +56,16 @@ inline int quantize_clocks(int M, int G, int r, int fitting, int w, int k, bool 
   return ctas / slots * wave(slots) + (last > 0 ? wave(last) : 0) + (k > 1 ? 2000 + 190 * k : 0);
 }
 
-inline QuantizePlan quantize_plan(int M, int G, int r, int sms, const int* fitting_clusters, int wide_clusters, size_t image, bool expand) {
+inline QuantizePlan quantize_plan(int M, int G, int r, int sms, const int* fitting_clusters, int wide_clusters, size_t image) {
   const bool int4 = image > 0;
   const int few = 448;   // rows up to which 2 steps per warp beat 4
   if (r == 0) {
     // The splits are independent CTAs.  About five to an SM at any size, so that no SM is left with a CTA more than others:
-    // 32760 x 5120 in 256 CTAs of 128 rows 105.7 us, in 768 95.1 us.
+    // 32760 x 5120 in 256 CTAs of 128 rows 105.7 us, in 768 95.1 us.  Beside an expansion too: with 1.25 per SM there, forwards of
+    // 20000 x 13824 -> 1024 took 664 us instead of 612, of 6000 x 13824 -> 1024 211 instead of 182.
     const int steps = M <= few ? 2 : 4, per_warp = 4 * steps;
     const int warps = M < kQuantWarps * per_warp ? (M + per_warp - 1) / per_warp : kQuantWarps;
-    const int splits = (expand ? sms + sms / 4 : 5 * sms) / ((M + per_warp * warps - 1) / (per_warp * warps));
+    const int splits = 5 * sms / ((M + per_warp * warps - 1) / (per_warp * warps));
     return {steps, warps, splits < 1 || G < 4 ? 1 : (splits > G / 2 ? G / 2 : splits)};
   }
   // Beside an expansion, which takes longer than the activations and wants its share of the machine from the start: smaller
@@ -71,17 +73,18 @@ inline QuantizePlan quantize_plan(int M, int G, int r, int sms, const int* fitti
   // r = 64 60.0 -> 51.2 us; 1560, r = 64 96.8 -> 90.3; 4097, r = 96 204 -> 194.   Above 34 x 128 rows
   // it no longer pays: 4480 rows, r = 32 201.4 us with this plan and 200.0 with the general one, 4736 209.2 | 199.7; r = 96 209.7 |
   // 210.6 and 215.2 | 213.0.
-  if (expand && M > few && M <= 34 * 128) {
+  if (int4 && M > few && M <= 34 * 128) {
     const int k = M <= 1024 ? 8 : 4, clusters = k == 8 ? 16 : 33, warps = (M + 8 * clusters - 1) / (8 * clusters);
     if (k <= G / 2 && fitting_clusters[k] > 0) return {2, warps < kQuantWarps ? warps : kQuantWarps, k};
   }
   // The splits of a row block form a cluster, which stays within a GPC.  With few rows: the most splits that still run all row
   // blocks at once, one CTA to an SM, and the fewest warps that cover the rows.  Above a byte image of 2^24 (5120 x 5120 is 1.6 of
-  // that) its expansion is what the launch takes long for, on CTAs of the same form: clusters of 8 at most, which leave fewer SMs
-  // out than those of 16, and six warps.  1 x 5120 -> 13824, r = 16: one warp in clusters of 16 111 us, six 57, six in clusters of 8 48;
-  // 1 x 5120 -> 5120 35, 22.4 and 22.0.  Smaller layers lose by it: 64 x 13824 -> 1024 22.5 us in clusters of 16, 28.6 of 8.
+  // that) its expansion is what the launch takes long for, on CTAs of the same form, so these get six warps: 1 x 5120 -> 13824, r = 16
+  // 107 us with one, 53 with six; 1 x 5120 -> 5120 33.8 and 22.5.  Where many row blocks would make many clusters of 16, which
+  // leave more SMs out, clusters of 8 do: 448 x 5120 -> 13824 94 and 85.  Smaller layers lose by either: 64 x 13824 -> 1024 22.5 us in
+  // clusters of 16, 28.6 of 8.
   const bool large = image > (1u << 24);
-  if (M <= few) for (int k = large ? 8 : kMaxKSplits; k > 1; k = k > 8 ? 8 : k - 1) {
+  if (M <= few) for (int k = large && M > 256 ? 8 : kMaxKSplits; k > 1; k = k > 8 ? 8 : k - 1) {
     const int clusters = k > 8 ? wide_clusters : fitting_clusters[k];
     const int steps = k > 8 || large ? 2 : 4, per_warp = 4 * steps;
     if (clusters > 0 && k <= G / 2 && M <= clusters * kQuantWarps * per_warp) {

@@ -209,8 +209,7 @@ cudaError_t launch_quantize_steps(int num_sms, cudaStream_t stream, const CUtens
 }
 template <int R, int FORMAT, bool STALL = false>
 cudaError_t launch_quantize_kernel(const w4a4_ctx* ctx, int wide_clusters, size_t image, cudaStream_t stream, const CUtensorMap& tmL1, const QuantizeParams& p) {
-  const bool expand = R > 0 ? FORMAT == kCodesE4M3 : p.expand.chunks > 0;   // (without a low-rank branch nothing is summed over K)
-  const QuantizePlan plan = quantize_plan(p.M, p.K / 64, R, ctx->num_sms, ctx->gemm_clusters, wide_clusters, image, expand);
+  const QuantizePlan plan = quantize_plan(p.M, p.K / 64, R, ctx->num_sms, ctx->gemm_clusters, wide_clusters, image);
   if (plan.steps == 4) return launch_quantize_steps<R, FORMAT, 4, STALL>(ctx->num_sms, stream, tmL1, p, plan);
   return launch_quantize_steps<R, FORMAT, 2, STALL>(ctx->num_sms, stream, tmL1, p, plan);
 }

@@ -76,7 +76,7 @@ extern "C" w4a4_status_t w4a4_quantize_noalloc(const void* X, int M, int K, cons
   p.clip_index = clip_index;
   p.codes = reinterpret_cast<uint8_t*>(codes);
   p.scales = scales;
-  w4a4::QuantizePlan plan = w4a4::quantize_plan(M, K / 64, 0, 148, nullptr, 0, 0, false);
+  w4a4::QuantizePlan plan = w4a4::quantize_plan(M, K / 64, 0, 148, nullptr, 0, 0);
   constexpr int kSteps = 2;
   if (plan.steps != kSteps) plan.splits = (plan.splits + 1) / 2;
   const int cta_rows = w4a4::quantize_rows(kSteps, plan.warps), row_ctas = (M + cta_rows - 1) / cta_rows;

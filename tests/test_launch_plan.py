@@ -12,8 +12,8 @@ import pytest
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2605_27003_b200", "csrc")
 SHIM = """
 #include "quantize_plan.h"
-extern "C" void plan(int M, int G, int r, int sms, const int* fitting, int wide, int image, int expand, int* out) {
-  const w4a4::QuantizePlan p = w4a4::quantize_plan(M, G, r, sms, fitting, wide, static_cast<size_t>(image), expand != 0);
+extern "C" void plan(int M, int G, int r, int sms, const int* fitting, int wide, int image, int* out) {
+  const w4a4::QuantizePlan p = w4a4::quantize_plan(M, G, r, sms, fitting, wide, static_cast<size_t>(image));
   out[0] = p.steps, out[1] = p.warps, out[2] = p.splits;
   out[3] = static_cast<int>(w4a4::quantize_smem_bytes(r, p.steps, p.warps, p.splits));
   out[4] = static_cast<int>(w4a4::quantize_smem_bytes(r, p.steps, w4a4::kQuantWarps, w4a4::kMaxKSplits));
@@ -33,9 +33,9 @@ def plan(tmp_path_factory):
     subprocess.run(["g++", "-std=c++17", "-O1", "-Wall", "-Werror", "-shared", "-fPIC", "-I", CSRC, "-o", str(lib), str(src)], check=True)
     fn = ctypes.CDLL(str(lib)).plan
 
-    def call(M, G, r, sms=148, fitting=FULL, wide=7, expand=False, int4=None, image=1 << 22):
+    def call(M, G, r, sms=148, fitting=FULL, wide=7, int4=True, image=1 << 22):
         out = (ctypes.c_int * 7)()
-        fn(M, G, r, sms, (ctypes.c_int * 9)(*fitting), wide, image if (expand if int4 is None else int4) else 0, int(expand), out)
+        fn(M, G, r, sms, (ctypes.c_int * 9)(*fitting), wide, image if int4 else 0, out)
         return dict(zip(("steps", "warps", "splits", "smem", "limit", "rows", "spare"), out))
     return call
 
@@ -50,20 +50,20 @@ def test_a_plan_asks_for_no_cluster_that_the_device_cannot_launch(plan, fitting,
     for M in ROWS:
         for G in GROUPS:
             for r in (16, 32, 64, 96):
-                for expand in (False, True):
-                    p = plan(M, G, r, fitting=fitting, wide=wide, expand=expand)
-                    assert 1 <= p["splits"] <= most and p["splits"] <= max(1, G // 2), (M, G, r, expand, p)
-                    assert p["splits"] == 1 or (wide if p["splits"] > 8 else fitting[p["splits"]]) > 0, (M, G, r, expand, p)
+                for int4 in (False, True):
+                    p = plan(M, G, r, fitting=fitting, wide=wide, int4=int4)
+                    assert 1 <= p["splits"] <= most and p["splits"] <= max(1, G // 2), (M, G, r, int4, p)
+                    assert p["splits"] == 1 or (wide if p["splits"] > 8 else fitting[p["splits"]]) > 0, (M, G, r, int4, p)
 
 
 def test_every_plan_stays_within_the_limits_set_at_pack_time(plan):
     for M in ROWS:
         for G in GROUPS:
             for r in (0, 16, 32, 64, 96):
-                for expand in (False, True):
-                    p = plan(M, G, r, expand=expand)
-                    assert p["steps"] in (2, 4) and 1 <= p["warps"] <= p["warps"] + p["spare"] <= 8 and 1 <= p["splits"] <= max(1, G), (M, G, r, expand, p)
-                    assert p["smem"] <= p["limit"] <= 232448, (M, G, r, expand, p)
+                for int4 in (False, True):
+                    p = plan(M, G, r, int4=int4)
+                    assert p["steps"] in (2, 4) and 1 <= p["warps"] <= p["warps"] + p["spare"] <= 8 and 1 <= p["splits"] <= max(1, G), (M, G, r, int4, p)
+                    assert p["smem"] <= p["limit"] <= 232448, (M, G, r, int4, p)
                     assert p["rows"] <= 128
 
 
@@ -87,6 +87,12 @@ def test_the_model_keeps_the_plan_of_full_launches(plan, r):
 def test_few_rows_leave_enough_warps_for_the_weight_expansion(plan, G):
     # The CTAs that expand weights have the plan's warps: with one or two each, a large layer's expansion took twice its time.
     for M in (1, 8, 16, 64, 130, 300, 448):
-        p = plan(M, G, 16, expand=True, image=5120 * 5120)
-        assert 6 <= p["warps"] + p["spare"] <= 8 and p["splits"] <= 8
-        assert plan(M, G, 16, expand=True, image=1024 * 1024)["spare"] == 0
+        p = plan(M, G, 16, image=5120 * 5120)
+        assert 6 <= p["warps"] + p["spare"] <= 8 and (M <= 256 or p["splits"] <= 8)
+        assert plan(M, G, 16, image=1024 * 1024)["spare"] == 0
+
+
+@pytest.mark.parametrize("M", [2000, 6000, 12000, 20000])
+def test_without_a_low_rank_branch_every_sm_gets_several_ctas(plan, M):
+    p = plan(M, 216, 0)
+    assert -(-M // p["rows"]) * p["splits"] >= 4 * 148, p
