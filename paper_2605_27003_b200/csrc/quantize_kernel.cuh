@@ -17,16 +17,16 @@
 // 67 % of the issue slots of two CTAs per SM; DRAM traffic is 60 % of what a copy reaches.  So the loop's addresses are kept in
 // registers (derived anew in every pass they cost 15 of those instructions: 127 -> 94 us at 32760 x 5120 MXFP4) and the rare cases
 // of the scale arithmetic have a branch of their own.  The predecessor held 16 rows of a warp in mma.sync fragments, with r
-// accumulators per row in registers.  Eight launches replayed from one graph, 32760 x 5120, INT4 | MXFP4: r = 0 120 -> 100 | 93 ->
-// 79 us, r = 32 148 -> 113.5 | 121 -> 93, r = 64 192 -> 120 | 158 -> 101, r = 96 278 -> 140 (INT4); 32760 x 13824, r = 32 390 -> 291 |
-// 320 -> 237.  (335 MB in and 168 | 89 MB out take 76 | 64 us.)
+// accumulators per row in registers.  Eight launches replayed from one graph, 32760 x 5120, INT4 | MXFP4: r = 0 120 -> 99 | 93 ->
+// 78 us, r = 32 148 -> 114 | 121 -> 90, r = 64 191 -> 117 | 158 -> 95, r = 96 278 -> 125 (INT4); 32760 x 13824, r = 32 390 -> 300 |
+// 320 -> 236.  (335 MB in and 168 | 89 MB out take 76 | 64 us.)
 //
 // K split (gridDim.y > 1): with few token rows there are too few row blocks to fill the machine, so the K groups are divided
 // among gridDim.y CTAs per row block, which form one thread-block cluster when there is a low-rank branch.  Codes and scales
 // of different groups are independent; of T every CTA adds up a share of the rows, for which the others push their partial
 // sums into its shared memory (st.async on an mbarrier there) and which it adds in split order.  Pulled over distributed
 // shared memory between two cluster barriers instead, the end of the kernel took 5000 clocks, pushed about 2000.
-// 100 x 5120, r = 32 12.9 -> 5.4 us INT4, 9.0 -> 5.1 MXFP4; 700 x 8192, r = 64 23.1 -> 12.9 | 16.6 -> 10.7.
+// 100 x 5120, r = 32 12.9 -> 5.4 us INT4, 9.0 -> 5.1 MXFP4; 700 x 8192, r = 64 23.2 -> 13.2 | 16.5 -> 10.8.
 //
 // Weight expansion (ExpandJob): the CTAs past the row blocks turn the layer's 4-bit weights into the byte image the
 // INT4 GEMM reads.  It is independent of the activations, so it shares their launch instead of being a kernel between
@@ -424,7 +424,6 @@ quantize_kernel(const __grid_constant__ CUtensorMap tmL1, const QuantizeParams p
     grid_dependency_wait();
     const int j = lane & 7;                                     // this lane's channels: 8 j .. 8 j + 7 of the group
     const int tile_row = warp * (4 * STEPS) + (lane >> 4) + 2 * (lane >> 3 & 1);   // and rows: + 4 per step
-    const int g_first = warp < active ? g_begin : g_end;
     const float rho = __ldg(p.clip_table + p.clip_index);
     const float x_min = rho >= kRhoOrdinary ? kOrdinaryMin : kOrdinaryMax * 2.0f;   // below it the general path is taken
     // 32-bit byte offsets from the CTA's first row (at most 128 rows of 16384 channels and a margin): half the address
@@ -472,12 +471,14 @@ quantize_kernel(const __grid_constant__ CUtensorMap tmL1, const QuantizeParams p
       }
       cp_async_commit();
     };
+    // Warps without rows neither load nor walk the groups.  (A branch around the loop: bounds of their own made the loop 3 % longer.)
 #pragma unroll
-    for (int i = 0; i < kStages - 1; ++i) load(g_first + i, stage_bytes * i);
+    for (int i = 0; i < kStages - 1; ++i)
+      if (warp < active) load(g_begin + i, stage_bytes * i);
     join_setup();   // its microsecond passes beside the first loads
     uint32_t slot = 0, slot_before = stage_bytes * (kStages - 1);   // this group's and the previous group's
     bool ok = true;
-    for (int g = g_first; g < g_end; ++g) {
+    if (warp < active) for (int g = g_begin; g < g_end; ++g) {
       float xh[STEPS][8];
       cp_async_wait<kStages - 2>();
       __syncwarp();
