@@ -27,28 +27,37 @@
 // columns 0..127 P_g, columns 128..255 S_g.  Warp roles:
 //   warp 0      producer: per stage of 128 K-codes (two groups) TMA loads of the A and B code tiles (16 KiB each,
 //               128-byte swizzle) and of the two scale-operand images, all onto the stage's mbarrier;
-//   warp 1      code-MMA issuer: per group two tcgen05.mma kind::f8f6f4 (K = 32) into the slot's P columns, then a
-//               commit onto tmem_full[slot];
+//   warps 1, 2  code-MMA issuers, warp 1 for the first group of every stage (and the low-rank entry), warp 2 for the second:
+//               per group two tcgen05.mma kind::f8f6f4 (K = 32) into the slot's P columns, then a commit onto
+//               tmem_full[slot];
 //   warp 3      scale-MMA issuer: per group one tcgen05.mma kind::f16 (K = 16) into the slot's S columns and a commit
-//               onto the same barrier (it counts two arrivals).  Two issuing threads because the issue of a
-//               tcgen05.mma waits for room in the tensor pipe's queue: one thread would put all of that on the
-//               hand-over path of every slot;
-//   warp 2      TMEM allocation;
+//               onto the same barrier (it counts two arrivals).  The issue of a tcgen05.mma waits for room in the tensor
+//               pipe's queue and the loop around it costs as much again, so that one thread with everything to issue is
+//               late for every slot: with one code-MMA warp the slot had been free for 200 clocks when its issue was
+//               through, with two 98 (410 -> 402 clocks per group; a fourth issuing warp for the scale MMAs, or both
+//               products of a group from one warp, gained nothing: 405 and 420);
+//   warp 2      also TMEM allocation;
 //   warps 4-19  epilogue: a thread owns one token row and 32 output channels.  Per group two round trips of two
 //               tcgen05.ld.32x32b.x16 (P and S of 16 columns) with the eight packed multiply-adds of the first half
 //               in between; the slot goes back to the issuing warps (tmem_empty[slot], 16 arrivals) as soon as the
 //               second half is in registers.  Measured alternatives (all four loads in one round trip; the second
 //               half's loads issued ahead of the first half's arithmetic; warps of a scheduler skewed against one
 //               another) were slower.
-// What bounds the kernel is the serial chain of an epilogue warp per group: wait, load, 8 multiply-adds, load, release, 8
-// multiply-adds (a stand-alone copy of the hand-over runs at 330-340 clocks per group with the MMAs and without them; the
-// loads and multiply-adds alone at 200; this kernel at 349, from its clocks per tile at 80 and 216 groups, plus about
-// 2600 per tile for the tile's end).  A lone warp's dependent instructions
+// What bounds the kernel is the round trip of a TMEM slot, of which there are two: release, issue, MMAs, commit, wait, loads
+// (4736 x 5120, slope over K = 2560 and 10240 with the weight expansion's share of 20, clocks per group: 402; without any
+// operand loads the same, with an epilogue that loads 16 columns and adds nothing 336, and with one MMA instead of three 300).
+// Epilogue warps that form the scale products themselves leave room for three or four slots, but their broadcast reads of the
+// channel scales alone cost 190 clocks per group (651 with two CTAs per SM, 16 warps with 8 of 32 channels' products from the
+// tensor core 800).  A lone warp's dependent instructions
 // cost 10-15 cycles each and a branch on a fresh mbarrier result ~70, so the hops are written as single instruction
 // sequences without branches: wait_issue_* (try_wait, then fence, MMAs and commit predicated on its answer),
 // wait_then_ld16 (try_wait, then fence and first TMEM load predicated on its answer), descriptors computed before the wait, and
 // predicated instead of branched single-lane instructions (umma_*_if, mbar_arrive_if).  A wait that outlasts the
-// try_wait falls back to the bounded wait of pipeline.cuh and the same instructions issued from C++.
+// try_wait falls back to the bounded wait of pipeline.cuh and the same instructions issued from C++.  The slots' addresses are
+// toggled, not derived from a counter (423 -> 410 clocks per group).  The vote on the answer stays: a barrier that completes
+// during a try_wait can answer the lanes differently.
+// The tile's end: outputs in BF16 through a swizzled tile in shared memory and out by one TMA store per warp, which the next
+// tile does not wait for.  16-byte stores from registers held the warps for 1150 of the tile change's 2600 clocks.
 // Tile order: column tiles are walked in super-columns (GemmParams::order, all row blocks of a
 // super-column before the next) sized so that the weight bytes a wave of CTAs touches stay in L2; with the plain
 // row-major order the 71 MB weight image of the FFN shapes streamed from DRAM once per 1.4 row blocks.
@@ -86,19 +95,19 @@ static_assert(kGemmSmemBytes <= 232448, "shared memory budget of one CTA");
 static_assert(kStageBytes % 1024 == 0, "operand tiles must stay 1024-byte aligned");
 
 // Register budgets.  640 threads are launched with 96 registers each; the control warpgroup gives most of its share to the
-// epilogue's four.  What the compiler makes of the epilogue's loop decides the kernel (clocks per 128 x 128 tile at K = 5120
-// | 13824, the same on every SM and at every clock): ring position as slot + parity with a wrap, 96 registers 34261 |
-// 88083; as a counter whose bits are slot and parity 31314 | 79971; with 112 registers 30529 | 78045.
+// epilogue's four.  What the compiler makes of the epilogue's loop decides the kernel (clocks per 128 x 128 tile at K = 5120:
+// 96 registers 31314, 112 30529).
 constexpr int kGemmRegs = 96, kControlRegs = 32, kEpilogueRegs = 112;
 static_assert((kGemmThreads - 32 * kEpiWarps) * kControlRegs + 32 * kEpiWarps * kEpilogueRegs <= kGemmThreads * kGemmRegs,
               "a larger sum would wait forever for registers that the launch does not have");
 
-// Uses of the TMEM slots, counted: use u takes slot u % kTmemSlots.
+// The epilogue's position in the two TMEM slots: the current slot's column address and full barrier, and its phase.
 struct SlotUse {
-  uint32_t u = 0;
-  static_assert(kTmemSlots == 2, "slot and parity are bits 0 and 1 of the counter");
-  __device__ __forceinline__ uint32_t slot() const { return u & 1u; }
-  __device__ __forceinline__ uint32_t parity() const { return (u >> 1) & 1u; }
+  uint32_t t, full, phase = 0;
+  static_assert(kTmemSlots == 2, "the slots differ in one bit of each address");
+  __device__ __forceinline__ SlotUse(uint32_t t0, uint32_t full0) : t(t0), full(full0) {}
+  __device__ __forceinline__ uint32_t empty() const { return full + 8 * kTmemSlots; }
+  __device__ __forceinline__ void next() { t ^= 2 * kBN, full ^= 8u, phase ^= (~full >> 3) & 1u; }
 };
 
 // Wait for a TMEM slot and issue its MMAs in one branch-free instruction sequence: one try_wait (it blocks in hardware
@@ -228,15 +237,16 @@ template <bool DEBUG, bool SPLIT>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                  const __grid_constant__ CUtensorMap tmT, const __grid_constant__ CUtensorMap tmL2,
-                 const __grid_constant__ CUtensorMap tmSopA, const __grid_constant__ CUtensorMap tmSopB, const GemmParams p) {
+                 const __grid_constant__ CUtensorMap tmSopA, const __grid_constant__ CUtensorMap tmSopB,
+                 const __grid_constant__ CUtensorMap tmY, const GemmParams p) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* smem = smem_raw + (smem_base - smem_u32(smem_raw));
   // Above every operand tile so that the descriptors' chunk distances are positive.
   const uint32_t zero_base = smem_base + kGemmStages * kStageBytes;   // second K chunk of every scale MMA
-  const uint32_t out_base = zero_base + kZeroTile;                    // the epilogue warps' output tiles
+  const uint32_t out_base = zero_base + kZeroTile;                    // the epilogue warps' output tiles (512-byte aligned: 64-byte swizzle)
   const uint32_t bar_base = out_base + kEpiWarps * kOutTile;
-  const uint32_t bar_op_full = bar_base;
+  const uint32_t bar_op_full = bar_base;   // 16-byte aligned; so is bar_tmem_full, behind an even number of barriers
   const uint32_t bar_op_empty = bar_op_full + 8 * kGemmStages;
   const uint32_t bar_tmem_full = bar_op_empty + 8 * kGemmStages;
   const uint32_t bar_tmem_empty = bar_tmem_full + 8 * kTmemSlots;
@@ -260,10 +270,10 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   if (threadIdx.x == 0) {
     for (int i = 0; i < kGemmStages; ++i) {
       mbar_init(bar_op_full + 8 * i, 1);
-      mbar_init(bar_op_empty + 8 * i, 2);    // the code-MMA warp and the scale-MMA warp
+      mbar_init(bar_op_empty + 8 * i, 3);    // the code-MMA warps and the scale-MMA warp
     }
     for (int i = 0; i < kTmemSlots; ++i) {
-      mbar_init(bar_tmem_full + 8 * i, 2);   // the code-MMA warp and the scale-MMA warp
+      mbar_init(bar_tmem_full + 8 * i, 2);   // a code-MMA warp and the scale-MMA warp
       mbar_init(bar_tmem_empty + 8 * i, kEpiWarps);
     }
     mbar_fence_init();
@@ -272,6 +282,7 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     tma_prefetch_desc(&tmB);
     tma_prefetch_desc(&tmSopA);
     tma_prefetch_desc(&tmSopB);
+    if (!SPLIT && p.yref == nullptr) tma_prefetch_desc(&tmY);
     if (p.r > 0) {
       tma_prefetch_desc(&tmT);
       tma_prefetch_desc(&tmL2);
@@ -342,10 +353,11 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           op.advance();
         }
       }
-    } else if (live && warp == 1) {
+    } else if (live && (warp == 1 || warp == 2)) {
       // ------------------------------------------------------------------ code-MMA issuer (all lanes loop, one issues)
       constexpr uint32_t idesc_f8 = umma_idesc(1, 0, kBM, kBN);
       constexpr uint32_t idesc_bf16 = umma_idesc(1, 1, kBM, kBN);
+      const int v = warp - 1;
       const bool issuer = elect_one_lane();
       const uint32_t go = issuer ? 1u : 0u;
       const int issue_lane = __ffs(__ballot_sync(0xffffffffu, issuer)) - 1;   // the decision below is the issuing lane's
@@ -353,9 +365,13 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       Ring<kTmemSlots> tm;
       bool ok = true;
       for (int tile = first_tile; ok && tile < num_tiles; tile += tile_step) {
+        // Both warps wait for the tile's first use.  Each waits for every other use within a tile; the uses of a tile may be odd in
+        // number, and a warp that has not seen the use before the last one of a slot released would take an older phase of the
+        // same parity for the one it waits for.
+        ok = __all_sync(0xffffffffu, bounded_wait<0, 1>(bar_tmem_empty + 8 * tm.slot, tm.parity ^ 1u, env, kErrMmaWait));
+        if (!ok) break;
+        tc_fence_after_sync();
         if (n_lr_stages > 0) {
-          ok = __all_sync(0xffffffffu, bounded_wait<0, 1>(bar_tmem_empty + 8 * tm.slot, tm.parity ^ 1u, env, kErrMmaWait));
-          if (ok) tc_fence_after_sync();
           const uint32_t d = tmem_base + tm.slot * 2 * kBN;
           const uint32_t full_bar = bar_tmem_full + 8 * tm.slot;
           tm.advance();
@@ -363,23 +379,26 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             ok = __all_sync(0xffffffffu, bounded_wait<0, 1>(bar_op_full + 8 * op.slot, op.parity, env, kErrMmaWait));
             if (!ok) break;
             const uint32_t a = smem_base + op.slot * kStageBytes, b = a + kOpATile;
-            if (issuer) {
+            if (issuer && v == 0) {
 #pragma unroll
               for (int kk = 0; kk < 4; ++kk)
                 umma_f16(d, umma_desc_k_sw128(a, 32 * kk), umma_desc_k_sw128(b, 32 * kk), idesc_bf16, (l > 0 || kk > 0) ? 1u : 0u);
               umma_commit(bar_op_empty + 8 * op.slot);
+            } else if (issuer) {
+              mbar_arrive(bar_op_empty + 8 * op.slot);
             }
             op.advance();
           }
           if (!ok) break;
-          if (issuer) umma_commit(full_bar);
+          if (issuer && v == 0) umma_commit(full_bar);
         }
         for (int st = st_begin; ok && st < st_end; ++st) {
           ok = __all_sync(0xffffffffu, bounded_wait<0, 1>(bar_op_full + 8 * op.slot, op.parity, env, kErrMmaWait));
           if (!ok) break;
           const uint32_t a = smem_base + op.slot * kStageBytes, b = a + kOpATile;
           const int groups = (2 * st + 1 < G) ? 2 : 1;
-          for (int v = 0; v < groups; ++v) {
+          if (v == 1) tm.advance();
+          if (v < groups) {
             // everything the issue needs is ready before the wait that sits on the slot's round trip
             const uint32_t d = tmem_base + tm.slot * 2 * kBN;
             const uint32_t full_bar = bar_tmem_full + 8 * tm.slot;
@@ -395,14 +414,14 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             }
             tm.advance();
           }
-          if (!ok) break;
+          if (v == 0 && groups == 2) tm.advance();
           umma_commit_if(go, bar_op_empty + 8 * op.slot);
           op.advance();
         }
       }
     } else if (live && warp == 3) {
       // ------------------------------------------------------------------ scale-MMA issuer
-      // Walks the same slot uses as the code-MMA warp.
+      // Walks the same slot uses as the code-MMA warps.
       constexpr uint32_t idesc_bf16 = umma_idesc(1, 1, kBM, kBN);
       const bool issuer = elect_one_lane();
       const uint32_t go = issuer ? 1u : 0u;
@@ -460,7 +479,7 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       const int quarter = ew & 3, colblk = ew >> 2;
       const uint32_t t_lane = tmem_base + (static_cast<uint32_t>(32 * quarter) << 16) + kEpiCols * colblk;
       const uint32_t out_tile = out_base + kOutTile * ew;
-      SlotUse use;
+      SlotUse use(t_lane, bar_tmem_full);
       bool ok = true;
       for (int tile = first_tile; ok && tile < num_tiles; tile += tile_step) {
         int tm_e, tn_e;
@@ -471,9 +490,9 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         const float bias_lane = p.bias ? __ldg(p.bias + n0 + kEpiCols * colblk + lane) : 0.0f;
         float2 acc[16];  // pair k: channels ch0 + 2 k, ch0 + 2 k + 1
         if (n_lr_stages > 0) {   // the low-rank entry opens the tile: the accumulators start as T L2
-          const uint32_t t = t_lane + use.slot() * 2 * kBN;
+          const uint32_t t = use.t;
           uint32_t pv[16], qv[16];
-          ok = __all_sync(0xffffffffu, bounded_wait(bar_tmem_full + 8 * use.slot(), use.parity(), env, kErrEpilogueWait));
+          ok = __all_sync(0xffffffffu, bounded_wait(use.full, use.phase, env, kErrEpilogueWait));
           if (!ok) break;
           tc_fence_after_sync();
           tmem_ld_32x32b_x16(t, pv);
@@ -482,8 +501,8 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           tie_fragment(pv);
           tie_fragment(qv);
           tc_fence_before_sync();
-          mbar_arrive_if(lane == 0 ? 1u : 0u, bar_tmem_empty + 8 * use.slot());
-          ++use.u;
+          mbar_arrive_if(lane == 0 ? 1u : 0u, use.empty());
+          use.next();
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
             acc[j] = make_float2(__uint_as_float(pv[2 * j]), __uint_as_float(pv[2 * j + 1]));
@@ -494,10 +513,10 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           for (int j = 0; j < 16; ++j) acc[j] = make_float2(0.0f, 0.0f);
         }
         for (int g = g_begin; g < g_end; ++g) {
-          const uint32_t t = t_lane + use.slot() * 2 * kBN;
+          const uint32_t t = use.t;
           uint32_t pv[16], sv[16];
-          if (!__all_sync(0xffffffffu, wait_then_ld16(bar_tmem_full + 8 * use.slot(), use.parity(), t, pv) != 0)) {
-            ok = __all_sync(0xffffffffu, bounded_wait(bar_tmem_full + 8 * use.slot(), use.parity(), env, kErrEpilogueWait));
+          if (!__all_sync(0xffffffffu, wait_then_ld16(use.full, use.phase, t, pv) != 0)) {   // lanes can differ
+            ok = __all_sync(0xffffffffu, bounded_wait(use.full, use.phase, env, kErrEpilogueWait));
             if (!ok) break;
             tc_fence_after_sync();
             tmem_ld_32x32b_x16(t, pv);
@@ -518,8 +537,8 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           tie_fragment(sv);
           // The whole slot is in registers (loads and waits are warp-wide): hand it back to the MMA warps.
           tc_fence_before_sync();
-          mbar_arrive_if(lane == 0 ? 1u : 0u, bar_tmem_empty + 8 * use.slot());
-          ++use.u;
+          mbar_arrive_if(lane == 0 ? 1u : 0u, use.empty());
+          use.next();
           fma_fragment<DEBUG>(pv, sv, acc + 8, DEBUG && d0 ? d0 + 16 : nullptr);
         }
         if (!ok) break;
@@ -535,6 +554,7 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         }
         // The tile's end: bias, activation, BF16, then through shared memory so that a warp's 16-byte accesses to Y (or to
         // the reference) cover eight rows x 64 bytes instead of 32 rows x 16.
+        if (!SPLIT && lane == 0) bulk_store_wait_read();   // the previous tile has left the staging tile
         __syncwarp();
         sts_f32(out_tile + 4 * lane, bias_lane);
         __syncwarp();
@@ -556,31 +576,30 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           sts_u32x4(out_tile + 64 * lane + 16 * (c ^ ((lane >> 1) & 3)), o);
         }
         __syncwarp();
-        const int row = m0 + 32 * quarter + (lane >> 2);   // and rows + 8, + 16, + 24
-        const size_t at = static_cast<size_t>(row) * p.N + n0 + kEpiCols * colblk + 8 * (lane & 3);
-        const size_t step = 8 * static_cast<size_t>(p.N);
-        uint4 y[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          y[j] = lds_u32x4(out_tile + 512 * j + 64 * (lane >> 2) + 16 * ((lane ^ (lane >> 3)) & 3));
         if (p.yref == nullptr) {
-          uint16_t* yp = p.Y + at;
-#pragma unroll
-          for (int j = 0; j < 4; ++j)
-            if (row + 8 * j < p.M) *reinterpret_cast<uint4*>(yp + j * step) = y[j];
+          fence_proxy_async_smem();
+          __syncwarp();
+          if (lane == 0 && m0 + 32 * quarter < p.M) {
+            tma_store_2d(&tmY, out_tile, n0 + kEpiCols * colblk, m0 + 32 * quarter);
+            bulk_store_commit();
+          }
         } else {
           // Eq. 10's objective: || Y_ref - Y_hat ||^2 over the tile, with Y_hat rounded to BF16 exactly as the
           // forward would store it.  FP32 within the thread and the warp, FP64 across warps and tiles.
+          __syncwarp();
+          const int row = m0 + 32 * quarter + (lane >> 2);   // and rows + 8, + 16, + 24
+          const size_t step = 8 * static_cast<size_t>(p.N);
+          const uint16_t* rp = p.yref + static_cast<size_t>(row) * p.N + n0 + kEpiCols * colblk + 8 * (lane & 3);
           float sq = 0.0f;
-          const uint16_t* rp = p.yref + at;
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
             if (row + 8 * j < p.M) {
+              const uint4 y = lds_u32x4(out_tile + 512 * j + 64 * (lane >> 2) + 16 * ((lane ^ (lane >> 3)) & 3));
               const uint4 ref = __ldg(reinterpret_cast<const uint4*>(rp + j * step));
-              sq = sq_diff_bf16x2(ref.x, y[j].x, sq);
-              sq = sq_diff_bf16x2(ref.y, y[j].y, sq);
-              sq = sq_diff_bf16x2(ref.z, y[j].z, sq);
-              sq = sq_diff_bf16x2(ref.w, y[j].w, sq);
+              sq = sq_diff_bf16x2(ref.x, y.x, sq);
+              sq = sq_diff_bf16x2(ref.y, y.y, sq);
+              sq = sq_diff_bf16x2(ref.z, y.z, sq);
+              sq = sq_diff_bf16x2(ref.w, y.w, sq);
             }
           }
 #pragma unroll
@@ -589,6 +608,7 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         }
       }
       tmem_wait_ld();   // a role that gave up may still have loads in flight
+      if (!SPLIT && lane == 0) bulk_store_wait_read();   // stores still read the staging tile
     }
   }
 
