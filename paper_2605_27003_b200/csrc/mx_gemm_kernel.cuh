@@ -57,7 +57,9 @@ constexpr uint32_t kMxBTile = kMxBN * 128;       // 32 KiB
 constexpr uint32_t kMxSfTile = 2 * 512;          // scale bytes of 128 rows x 8 blocks: two atoms
 constexpr uint32_t kMxStageBytes = kMxATile + kMxBTile + 3 * kMxSfTile;   // A, B, scales of A and of both halves of B
 constexpr uint32_t kMxNumBarriers = 2 * kMxStages + 2;
-constexpr uint32_t kMxSmemBytes = 1024 + kMxStages * kMxStageBytes + kMxNumBarriers * 8 + 16;
+constexpr int kMxOutCols = 16;                        // channels of one TMA store of an epilogue warp
+constexpr uint32_t kMxOutTile = 32 * 2 * kMxOutCols;  // and its 32 rows in BF16
+constexpr uint32_t kMxSmemBytes = 1024 + kMxStages * kMxStageBytes + kMxEpiWarps * kMxOutTile + kMxNumBarriers * 8 + 16;
 constexpr uint32_t kMxTmemSfA = 256, kMxTmemSfB = 264;   // columns: accumulator 0..255, then 8 + 16 scale columns
 static_assert(kBM == 128, "the scale-factor atoms and the TMEM layout assume 128-row tiles");
 static_assert(kMxStageBytes % 1024 == 0, "operand tiles must stay 1024-byte aligned");
@@ -122,14 +124,55 @@ __device__ __forceinline__ void bulk_load(uint32_t dst_smem, const void* src, ui
                : "memory");
 }
 
+// A warp's 32 x 64 outputs: bias, activation, BF16, and out by TMA stores of 16 channels through a swizzled tile in shared memory,
+// which the warp only waits for before it writes the tile again.  (A thread's own 16-byte stores, a row each, took longer than a
+// K = 5120 main loop: 9472 x 2560 -> 5120 81.7 -> 51 us, K = 5120 102.6 -> 84, 10240 156 -> 153; stores of 32 channels with five
+// operand stages instead of six 54, 87, 157.)
+__device__ __forceinline__ void mx_store_tile(const uint32_t (&v)[4][16], const MxGemmParams& p, const CUtensorMap* tmY, uint32_t out_tile,
+                                              int ch0, int row0, int lane) {
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    if (lane == 0) bulk_store_wait_read();
+    __syncwarp();
+    const int ch = ch0 + 16 * c;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      uint32_t o[4];
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const float4 b4 = p.bias ? __ldg(reinterpret_cast<const float4*>(p.bias + ch) + 2 * h + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+        const uint32_t* w = v[c] + 8 * h + 4 * i;
+        float2 y0 = make_float2(__uint_as_float(w[0]) + b4.x, __uint_as_float(w[1]) + b4.y);
+        float2 y1 = make_float2(__uint_as_float(w[2]) + b4.z, __uint_as_float(w[3]) + b4.w);
+        if (p.act != 0) {  // uniform over the grid: the plain layer pays one predicate per four outputs
+          y0 = make_float2(apply_activation(y0.x, p.act), apply_activation(y0.y, p.act));
+          y1 = make_float2(apply_activation(y1.x, p.act), apply_activation(y1.y, p.act));
+        }
+        o[2 * i] = bf16x2_bits(y0);
+        o[2 * i + 1] = bf16x2_bits(y1);
+      }
+      // 32-byte rows, 16-byte half h at h ^ (row / 4 % 2): the map's 32-byte swizzle, conflict free.
+      sts_u32x4(out_tile + 32 * lane + 16 * (h ^ ((lane >> 2) & 1)), make_uint4(o[0], o[1], o[2], o[3]));
+    }
+    fence_proxy_async_smem();
+    __syncwarp();
+    if (lane == 0) {
+      tma_store_2d(tmY, out_tile, ch, row0);
+      bulk_store_commit();
+    }
+  }
+}
+
 template <bool SPLIT, bool DEBUG = false>
 __global__ void __launch_bounds__(kMxThreads, 1)
 mx_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-               const __grid_constant__ CUtensorMap tmT, const __grid_constant__ CUtensorMap tmL2, const MxGemmParams p) {
+               const __grid_constant__ CUtensorMap tmT, const __grid_constant__ CUtensorMap tmL2,
+               const __grid_constant__ CUtensorMap tmY, const MxGemmParams p) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* smem = smem_raw + (smem_base - smem_u32(smem_raw));
-  const uint32_t bar_base = smem_base + kMxStages * kMxStageBytes;
+  const uint32_t out_base = smem_base + kMxStages * kMxStageBytes;   // the epilogue warps' output tiles
+  const uint32_t bar_base = out_base + kMxEpiWarps * kMxOutTile;
   const uint32_t bar_full = bar_base;
   const uint32_t bar_empty = bar_full + 8 * kMxStages;
   const uint32_t bar_acc_full = bar_empty + 8 * kMxStages;
@@ -272,6 +315,7 @@ mx_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     // the MMA warp as soon as the warp's part of it is in registers, before it is converted and stored.
     const int ew = warp - kMxEpiWarp0;
     const int quarter = ew & 3, colblk = ew >> 2;
+    const uint32_t out_tile = out_base + kMxOutTile * ew;
     Ring<1> ab;
     bool ok = true;
     for (int tile = first_tile; ok && tile < num_tiles; tile += tile_step) {
@@ -324,37 +368,14 @@ mx_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
         if (lane == 0) atomicAdd(p.sq_err, static_cast<double>(e));
-      } else if (row < p.M && ch0 < p.N) {
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const int ch = ch0 + 16 * c;
-          uint4 o[2];
-          uint32_t* ow = reinterpret_cast<uint32_t*>(o);
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const float4 b4 = p.bias ? __ldg(reinterpret_cast<const float4*>(p.bias + ch) + i) : make_float4(0.f, 0.f, 0.f, 0.f);
-            float y0 = __uint_as_float(v[c][4 * i]) + b4.x, y1 = __uint_as_float(v[c][4 * i + 1]) + b4.y;
-            float y2 = __uint_as_float(v[c][4 * i + 2]) + b4.z, y3 = __uint_as_float(v[c][4 * i + 3]) + b4.w;
-            if (p.act != 0) {  // uniform over the grid: the plain layer pays one predicate per four outputs
-              y0 = apply_activation(y0, p.act);
-              y1 = apply_activation(y1, p.act);
-              y2 = apply_activation(y2, p.act);
-              y3 = apply_activation(y3, p.act);
-            }
-            __nv_bfloat162 lo = __floats2bfloat162_rn(y0, y1);
-            __nv_bfloat162 hi = __floats2bfloat162_rn(y2, y3);
-            ow[2 * i] = *reinterpret_cast<uint32_t*>(&lo);
-            ow[2 * i + 1] = *reinterpret_cast<uint32_t*>(&hi);
-          }
-          uint4* y = reinterpret_cast<uint4*>(p.Y + static_cast<size_t>(row) * p.N + ch);
-          y[0] = o[0];
-          y[1] = o[1];
-        }
+      } else if (m0 + 32 * quarter < p.M && ch0 < p.N) {
+        mx_store_tile(v, p, &tmY, out_tile, ch0, m0 + 32 * quarter, lane);
       }
       ab.advance();
     }
   }
 
+  if (!SPLIT && warp >= kMxEpiWarp0 && lane == 0) bulk_store_wait_read();   // stores still read the output tiles
   if constexpr (SPLIT) {
     cluster_sync_all();   // all partial tiles are written
     if (live && warp >= kMxEpiWarp0 && !cluster_gave_up(s_abort, p.splits)) {
@@ -441,7 +462,8 @@ constexpr int kMx2Stages = 6;
 constexpr uint32_t kMx2BHalf = kMxBTile / 2;                                  // 16 KiB: this CTA's 128 rows of B
 constexpr uint32_t kMx2StageBytes = kMxATile + kMx2BHalf + 3 * kMxSfTile;      // 35 KiB
 constexpr uint32_t kMx2NumBarriers = 2 * kMx2Stages + 2;
-constexpr uint32_t kMx2SmemBytes = 1024 + kMx2Stages * kMx2StageBytes + kMx2NumBarriers * 8 + 16;
+constexpr uint32_t kMx2SmemBytes = kMx2Stages * kMx2StageBytes + kMxEpiWarps * kMxOutTile + kMx2NumBarriers * 8 + 16;
+static_assert(kMx2SmemBytes <= 232448 && kMxSmemBytes <= 232448, "shared memory budget of one CTA");
 static_assert(kMx2StageBytes % 1024 == 0, "operand tiles must stay 1024-byte aligned");
 
 // ---- Fused form (FUSE = true): the epilogue does not store the layer's output but quantizes it for the NEXT layer
@@ -462,7 +484,7 @@ constexpr int kMx2FuseStages = 4;
 constexpr uint32_t kMx2XhBytes = 4 * kMxATile;       // 128 rows x 256 channels BF16: four K slices of 64 channels
 constexpr uint32_t kMx2L1SliceBytes = 4096;           // up to 32 rows (r' / 2 <= 32) x 128 bytes
 constexpr uint32_t kMx2FuseBarriers = 2 * kMx2FuseStages + 2 + 7;
-constexpr uint32_t kMx2FuseSmemBytes = 1024 + kMx2FuseStages * kMx2StageBytes + kMx2XhBytes + 4 * kMx2L1SliceBytes +
+constexpr uint32_t kMx2FuseSmemBytes = kMx2FuseStages * kMx2StageBytes + kMx2XhBytes + 4 * kMx2L1SliceBytes +
                                        kMx2FuseBarriers * 8 + 16;
 static_assert(kMx2FuseSmemBytes <= 232448, "shared memory budget of one CTA");
 constexpr uint32_t kMxTmemT = 320;                    // two T buffers of 64 columns: 320..447
@@ -510,14 +532,17 @@ __global__ void __launch_bounds__(kMxThreads, 1)
 mx_gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmBhalf,
                 const __grid_constant__ CUtensorMap tmT, const __grid_constant__ CUtensorMap tmL2half,
                 const __grid_constant__ CUtensorMap tmSFA, const __grid_constant__ CUtensorMap tmSFB,
-                const __grid_constant__ CUtensorMap tmL1T, const MxGemmParams p, const MxNextParams nx) {
+                const __grid_constant__ CUtensorMap tmL1T, const __grid_constant__ CUtensorMap tmY, const MxGemmParams p,
+                const MxNextParams nx) {
   constexpr int STAGES = FUSE ? kMx2FuseStages : kMx2Stages;
-  extern __shared__ uint8_t smem_raw[];
-  const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-  uint8_t* smem = smem_raw + (smem_base - smem_u32(smem_raw));
+  // Declared with the alignment the operand tiles need: the unfused form has no room for slack.
+  extern __shared__ __align__(1024) uint8_t smem_aligned[];
+  uint8_t* const smem = smem_aligned;
+  const uint32_t smem_base = smem_u32(smem);
   const uint32_t xh_base = smem_base + STAGES * kMx2StageBytes;          // FUSE only: x_hat tile, then the L1' tile
   const uint32_t l1_base = xh_base + kMx2XhBytes;
-  const uint32_t bar_base = FUSE ? l1_base + 4 * kMx2L1SliceBytes : xh_base;
+  const uint32_t out_base = xh_base;                                      // !FUSE: the epilogue warps' output tiles
+  const uint32_t bar_base = FUSE ? l1_base + 4 * kMx2L1SliceBytes : out_base + kMxEpiWarps * kMxOutTile;
   const uint32_t bar_full = bar_base;
   const uint32_t bar_empty = bar_full + 8 * STAGES;
   const uint32_t bar_acc_full = bar_empty + 8 * STAGES;
@@ -738,6 +763,7 @@ mx_gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     // ------------------------------------------------------------------ epilogue (both CTAs, own rows)
     const int ew = warp - kMxEpiWarp0;
     const int quarter = ew & 3, colblk = ew >> 2;
+    const uint32_t out_tile = out_base + kMxOutTile * ew;
     const uint32_t acc_empty_leader = map_to_cta(bar_acc_empty, 0);
     Ring<1> ab;
     uint32_t kq = 0, tb = 0, t_uses0 = 0, t_uses1 = 0;   // FUSE: items done, T buffer, drains per buffer
@@ -893,37 +919,14 @@ mx_gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
         if (lane == 0) atomicAdd(p.sq_err, static_cast<double>(e));
-      } else if (row < p.M && ch0 < p.N) {
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const int ch = ch0 + 16 * c;
-          uint4 o[2];
-          uint32_t* ow = reinterpret_cast<uint32_t*>(o);
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const float4 b4 = p.bias ? __ldg(reinterpret_cast<const float4*>(p.bias + ch) + i) : make_float4(0.f, 0.f, 0.f, 0.f);
-            float y0 = __uint_as_float(v[c][4 * i]) + b4.x, y1 = __uint_as_float(v[c][4 * i + 1]) + b4.y;
-            float y2 = __uint_as_float(v[c][4 * i + 2]) + b4.z, y3 = __uint_as_float(v[c][4 * i + 3]) + b4.w;
-            if (p.act != 0) {
-              y0 = apply_activation(y0, p.act);
-              y1 = apply_activation(y1, p.act);
-              y2 = apply_activation(y2, p.act);
-              y3 = apply_activation(y3, p.act);
-            }
-            __nv_bfloat162 lo = __floats2bfloat162_rn(y0, y1);
-            __nv_bfloat162 hi = __floats2bfloat162_rn(y2, y3);
-            ow[2 * i] = *reinterpret_cast<uint32_t*>(&lo);
-            ow[2 * i + 1] = *reinterpret_cast<uint32_t*>(&hi);
-          }
-          uint4* y = reinterpret_cast<uint4*>(p.Y + static_cast<size_t>(row) * p.N + ch);
-          y[0] = o[0];
-          y[1] = o[1];
-        }
+      } else if (m0 + 32 * quarter < p.M && ch0 < p.N) {
+        mx_store_tile(v, p, &tmY, out_tile, ch0, m0 + 32 * quarter, lane);
       }
       ab.advance();
     }
   }
 
+  if (!FUSE && warp >= kMxEpiWarp0 && lane == 0) bulk_store_wait_read();   // stores still read the output tiles
   // ---------------------------------------------------------------------- common tail
   tc_fence_before_sync();
   __syncthreads();

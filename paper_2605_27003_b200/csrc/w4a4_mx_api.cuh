@@ -130,11 +130,12 @@ w4a4_status_t mx_launch_gemm(w4a4_mx_handle_t h, int M, int expert_id, void* Y, 
   // Few tiles: clusters of single CTAs share a tile's K, at least three 256-deep stages each (a CTA pair per tile would leave
   // half of the SMs or more without work).
   p.splits = next ? 1 : gemm_k_splits(num_tiles, h->K / kMxBK, 3, ctx->mx_gemm_clusters);
+  CUtensorMap tmY = tmA;   // unused where K is split and where nothing is stored
   if (p.splits > 1) {
     const OverlappedLaunch l(dim3(num_tiles * p.splits), block, kMxSmemBytes, stream, dim3(p.splits));
     auto* const kernel = stall_stage >= 0 ? mx_gemm_kernel<true, true> : mx_gemm_kernel<true>;
     if (stall_stage >= 0) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kMxSmemBytes));
-    if (cudaLaunchKernelEx(&l.cfg, kernel, tmA, e.tmB, tmT, tmL2, p) != cudaSuccess) {
+    if (cudaLaunchKernelEx(&l.cfg, kernel, tmA, e.tmB, tmT, tmL2, tmY, p) != cudaSuccess) {
       cudaGetLastError();
       return W4A4_ERR_CUDA;
     }
@@ -147,7 +148,13 @@ w4a4_status_t mx_launch_gemm(w4a4_mx_handle_t h, int M, int expert_id, void* Y, 
   // and with two row tiles the pairs' shared weight reads count (200 x 13824 -> 13824 30.7 | 35.0).
   const int pair_tiles = (p.tiles_m + 1) / 2 * p.tiles_n, sms = ctx->num_sms;
   const bool singles = !next && p.tiles_m > 2 && (num_tiles <= sms + sms / 8 || (num_tiles <= 2 * sms && pair_tiles > 2 * (sms / 2)));
-  if (p.tiles_m >= 2 && sms >= 2 && !singles) {
+  const bool pairs = p.tiles_m >= 2 && sms >= 2 && !singles;
+  // Y in boxes of 32 rows x kMxOutCols channels (encoded for every call: nothing is kept by a caller's address).
+  if (!next && yref == nullptr &&
+      !encode_2d(ctx->encode, &tmY, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Y, h->N, M, 2 * static_cast<uint64_t>(h->N),
+                 kMxOutCols, 32, CU_TENSOR_MAP_SWIZZLE_32B))
+    return W4A4_ERR_CUDA;
+  if (pairs) {
     const int runs = ((p.tiles_m + 1) / 2) * ((p.tiles_n + p.run - 1) / p.run);
     const int ctas = 2 * runs < ctx->num_sms ? 2 * runs : (ctx->num_sms & ~1);
     OverlappedLaunch l(dim3(ctas), block, next ? kMx2FuseSmemBytes : kMx2SmemBytes, stream, dim3(2));
@@ -163,9 +170,9 @@ w4a4_status_t mx_launch_gemm(w4a4_mx_handle_t h, int M, int expert_id, void* Y, 
       nx.t32 = ctx->mx_t32;
       nx.r2 = next->r;
       const CUtensorMap& tmL1T = next->r > 0 ? ne.tmL1T : e.tmBhalf;
-      le = cudaLaunchKernelEx(&l.cfg, mx_gemm2_kernel<true>, tmA, e.tmBhalf, tmT, tmL2h, tmSFA, e.tmSFB, tmL1T, p, nx);
+      le = cudaLaunchKernelEx(&l.cfg, mx_gemm2_kernel<true>, tmA, e.tmBhalf, tmT, tmL2h, tmSFA, e.tmSFB, tmL1T, tmY, p, nx);
     } else {
-      le = cudaLaunchKernelEx(&l.cfg, mx_gemm2_kernel<false>, tmA, e.tmBhalf, tmT, tmL2h, tmSFA, e.tmSFB, e.tmBhalf, p, nx);
+      le = cudaLaunchKernelEx(&l.cfg, mx_gemm2_kernel<false>, tmA, e.tmBhalf, tmT, tmL2h, tmSFA, e.tmSFB, e.tmBhalf, tmY, p, nx);
     }
     if (le != cudaSuccess) {
       cudaGetLastError();
@@ -175,7 +182,7 @@ w4a4_status_t mx_launch_gemm(w4a4_mx_handle_t h, int M, int expert_id, void* Y, 
   }
   if (next) return W4A4_ERR_SHAPE;   // the fused form runs on CTA pairs only
   const OverlappedLaunch l(grid, block, kMxSmemBytes, stream);
-  if (cudaLaunchKernelEx(&l.cfg, mx_gemm_kernel<false>, tmA, e.tmB, tmT, tmL2, p) != cudaSuccess) {
+  if (cudaLaunchKernelEx(&l.cfg, mx_gemm_kernel<false>, tmA, e.tmB, tmT, tmL2, tmY, p) != cudaSuccess) {
     cudaGetLastError();
     return W4A4_ERR_CUDA;
   }
