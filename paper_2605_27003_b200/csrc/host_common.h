@@ -8,6 +8,7 @@
 #include <atomic>
 
 #include "../../include/w4a4.h"
+#include "pipeline.cuh"
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
@@ -97,18 +98,17 @@ struct OverlappedLaunch {
   OverlappedLaunch(const OverlappedLaunch&) = delete;
 };
 
-constexpr int kMaxGemmSplits = 8;   // the portable cluster size
 // CTAs that share the K of one output tile: as many as still run all tiles at once, if each keeps `min_stages` of the tile's
 // operand stages.  `clusters[s]`: clusters of s CTAs that fit the device at a time (a cluster stays within one GPC).
 inline int gemm_k_splits(int tiles, int stages, int min_stages, const int* clusters) {
-  for (int s = kMaxGemmSplits; s > 1; --s)
+  for (int s = w4a4::kMaxGemmSplits; s > 1; --s)
     if (tiles <= clusters[s] && stages / s >= min_stages) return s;
   return 1;
 }
 
 template <typename Kernel>
 void count_clusters(int* clusters, Kernel* kernel, int threads, size_t smem) {
-  for (int s = 2; s <= kMaxGemmSplits; ++s) {
+  for (int s = 2; s <= w4a4::kMaxGemmSplits; ++s) {
     const OverlappedLaunch l(dim3(s), dim3(threads), smem, nullptr, dim3(s));
     if (cudaOccupancyMaxActiveClusters(&clusters[s], kernel, &l.cfg) != cudaSuccess) {
       cudaGetLastError();

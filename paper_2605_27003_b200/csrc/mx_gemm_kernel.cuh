@@ -387,11 +387,15 @@ mx_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         if (m0 + row >= p.M) break;
         if (ch >= p.N) continue;
         const uint32_t at = smem_base + 1024 * row + 16 * ((32 * (i & 1) + lane) ^ (row & 7));
+        // All loads on their way before the first addition (100 x 5120 -> 5120 12.1 -> 11.5 us).
+        float4 part[kMaxGemmSplits];
+#pragma unroll
+        for (int c = 0; c < kMaxGemmSplits; ++c)
+          if (c < p.splits) part[c] = ld_cluster_f32x4(map_to_cta(at, c));
         float4 y = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        for (int c = 0; c < p.splits; ++c) {
-          const float4 a = ld_cluster_f32x4(map_to_cta(at, c));
-          y.x += a.x, y.y += a.y, y.z += a.z, y.w += a.w;
-        }
+#pragma unroll
+        for (int c = 0; c < kMaxGemmSplits; ++c)
+          if (c < p.splits) y.x += part[c].x, y.y += part[c].y, y.z += part[c].z, y.w += part[c].w;
         const float4 b = p.bias ? __ldg(reinterpret_cast<const float4*>(p.bias + ch)) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         y.x += b.x, y.y += b.y, y.z += b.z, y.w += b.w;
         if (p.act != 0)

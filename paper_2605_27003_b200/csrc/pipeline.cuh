@@ -190,6 +190,8 @@ __device__ __forceinline__ bool cluster_gave_up(volatile int* s_abort, int ctas)
   return __any_sync(0xffffffffu, lane < ctas && ld_cluster_u32(map_to_cta(word, lane)) != 0u);
 }
 
+constexpr int kMaxGemmSplits = 8;   // CTAs that share a tile's K at most: the portable cluster size
+
 // Exercises the give-up path of bounded_wait without any pipeline around it: one warp waits for a phase of an
 // mbarrier that nobody ever completes.  No copy, tensor-core operation or TMEM allocation is involved, so there is
 // nothing to drain: after limit_ns the wait records kErrProbeWait in *err and the kernel returns normally.

@@ -476,6 +476,10 @@ quantize_kernel(const __grid_constant__ CUtensorMap tmL1, const QuantizeParams p
     for (int i = 0; i < kStages - 1; ++i)
       if (warp < active) load(g_begin + i, stage_bytes * i);
     join_setup();   // its microsecond passes beside the first loads
+    // The GEMM's CTAs may come in now, as room allows: this CTA has its TMEM (a GEMM's CTA takes all that an SM has left of it, and
+    // waits for this kernel's end).  After the loop instead of here, 1 x 5120 -> 1024 MXFP4 took 8.1 us, 7.5 now.  (The GEMM itself
+    // lets nobody in before its end: the next forward's activation CTAs then sat beside it, 78 -> 84 us at 1560 x 5120 -> 13824 MXFP4.)
+    grid_dependency_launch();
     uint32_t slot = 0, slot_before = stage_bytes * (kStages - 1);   // this group's and the previous group's
     bool ok = true;
     if (warp < active) for (int g = g_begin; g < g_end; ++g) {
@@ -605,9 +609,6 @@ quantize_kernel(const __grid_constant__ CUtensorMap tmL1, const QuantizeParams p
       }
     }
     cp_async_wait<0>();
-    // The GEMM's CTAs may come in now, as room allows.  (The GEMM itself lets nobody in before its end: the next forward's
-    // activation CTAs then sat beside it, 78 -> 84 us at 1560 x 5120 -> 13824 MXFP4.)
-    grid_dependency_launch();
     if constexpr (R > 0) {
       // T: TMEM lane = row of the tile; warp w reads lanes 32 w .. 32 w + 31.
       if (32 * warp < cta_rows && warp < 4) {
