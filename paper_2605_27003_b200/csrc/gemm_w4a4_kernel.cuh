@@ -44,8 +44,9 @@
 //               half's loads issued ahead of the first half's arithmetic; warps of a scheduler skewed against one
 //               another) were slower.
 // What bounds the kernel is the round trip of a TMEM slot, of which there are two: release, issue, MMAs, commit, wait, loads
-// (4736 x 5120, slope over K = 2560 and 10240 with the weight expansion's share of 20, clocks per group: 402; without any
-// operand loads the same, with an epilogue that loads 16 columns and adds nothing 336, and with one MMA instead of three 300).
+// (4736 x 5120, slope over K = 2560 and 10240 with the weight expansion's share of 20, clocks per group: 402.  One code-MMA warp and
+// slots from a counter: 421; of that kernel without any operand loads the same, with an epilogue that loads 16 columns and adds
+// nothing 336, and with one MMA instead of three beside that 300).
 // Epilogue warps that form the scale products themselves leave room for three or four slots, but their broadcast reads of the
 // channel scales alone cost 190 clocks per group (651 with two CTAs per SM, 16 warps with 8 of 32 channels' products from the
 // tensor core 800).  A lone warp's dependent instructions

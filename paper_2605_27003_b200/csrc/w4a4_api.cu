@@ -344,7 +344,7 @@ w4a4_status_t launch_gemm(w4a4_handle_t h, int M, int expert_id, void* Y, cudaSt
   // the exchange cost about as much as six groups.
   p.splits = stall_stage >= 0 && !stall_split ? 1 : gemm_k_splits(num_tiles, (h->K / 64 + 1) / 2, 4, ctx->gemm_clusters);
   if (stall_split && p.splits == 1) return W4A4_ERR_SHAPE;
-  // Y in boxes of an epilogue warp's 32 x 32 outputs.  (Encoded for every call: 0.1 us; nothing is kept by a caller's address.)
+  // Y in boxes of an epilogue warp's 32 x 32 outputs.  (Encoded for every call: nothing is kept by a caller's address.)
   CUtensorMap tmY = h->tmA;
   if (p.splits == 1 && yref == nullptr &&
       !encode_2d(ctx->encode, &tmY, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Y, h->N, M, 2 * static_cast<uint64_t>(h->N), kEpiCols, 32,
