@@ -478,6 +478,9 @@ static_assert(kMx2StageBytes % 1024 == 0, "operand tiles must stay 1024-byte ali
 // matching 256 rows of L1' (tcgen05.mma kind::f16, M = 256 over the pair, N = r') into a small TMEM accumulator
 // that stays resident while the cluster walks a run of column tiles of one row pair (work is dealt to clusters in
 // such runs), and is added into an FP32 [M, r'] array when the run ends.
+// Every lane of an epilogue warp writes a row of its own, so a store or a sum costs a transaction per lane whatever its width:
+// codes leave 32 bytes at a time and T is added four sums at a time (3000 x 5120 -> 13824 -> 5120, r' = 32 | 64, whole
+// call: 236 | 258 us with 16-byte stores and single sums, 230 | 246 so; 32760 rows, r' = 32, in short runs 1806 and 1779).
 // Shared memory: four stages instead of six, the 64 KiB x_hat tile, 16 KiB for the L1' tile (four K slices of
 // r'/2 rows, packed at whole swizzle atoms; for r' <= 32 they fill the lower half and the upper half holds one
 // 512-byte table per epilogue warp: the bias and the next layer's 1/lambda of the warp's 64 channels).
@@ -863,9 +866,7 @@ mx_gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
           uint4 w0, w1;
           const uint32_t ex0 = mxfp4_block32(v[0], v[1], rho2, w0);
           const uint32_t ex1 = mxfp4_block32(v[2], v[3], rho2, w1);
-          uint4* cdst = reinterpret_cast<uint4*>(nx.codes + static_cast<size_t>(row) * (p.N >> 1) + (ch0 >> 1));
-          cdst[0] = w0;
-          cdst[1] = w1;
+          st_global_32b(nx.codes + static_cast<size_t>(row) * (p.N >> 1) + (ch0 >> 1), w0, w1);   // N % 128 == 0: a whole sector
           const int sb = ch0 >> 5;   // even: the two exponent bytes are neighbours inside the atom
           uint8_t* sdst = nx.sfa + (static_cast<size_t>(row >> 7) * (p.N >> 7) + (sb >> 2)) * 512 + (row & 31) * 16 +
                           ((row & 127) >> 5) * 4 + (sb & 3);
@@ -886,7 +887,7 @@ mx_gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                 tmem_wait_ld();
                 if (row_ok) {
 #pragma unroll
-                  for (int j = 0; j < 16; ++j) atomicAdd(nx.t32 + static_cast<size_t>(row) * nx.r2 + 16 * cc + j, __uint_as_float(tv[j]));
+                  for (int j = 0; j < 16; j += 4) red_add_f32x4(nx.t32 + static_cast<size_t>(row) * nx.r2 + 16 * cc + j, tv + j);
                 }
               }
               tc_fence_before_sync();
