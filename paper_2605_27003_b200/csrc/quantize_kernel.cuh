@@ -476,10 +476,11 @@ quantize_kernel(const __grid_constant__ CUtensorMap tmL1, const QuantizeParams p
     for (int i = 0; i < kStages - 1; ++i)
       if (warp < active) load(g_begin + i, stage_bytes * i);
     join_setup();   // its microsecond passes beside the first loads
-    // The GEMM's CTAs may come in now, as room allows: this CTA has its TMEM (a GEMM's CTA takes all that an SM has left of it, and
-    // waits for this kernel's end).  After the loop instead of here, 1 x 5120 -> 1024 MXFP4 took 8.1 us, 7.5 now.  (The GEMM itself
+    // The MXFP4 GEMM's CTAs may come in now, as room allows: this CTA has its TMEM (a GEMM's CTA takes all that an SM has left of it,
+    // and waits for this kernel's end).  After the loop instead of here, 1 x 5120 -> 1024 took 8.1 us, 7.5 now.  The INT4 GEMM's
+    // come after the loop: at 256 x 512 -> 512 a forward takes 9.40 us that way and 9.57 this way.  (The GEMM itself
     // lets nobody in before its end: the next forward's activation CTAs then sat beside it, 78 -> 84 us at 1560 x 5120 -> 13824 MXFP4.)
-    grid_dependency_launch();
+    if constexpr (FORMAT == kCodesMxfp4) grid_dependency_launch();
     uint32_t slot = 0, slot_before = stage_bytes * (kStages - 1);   // this group's and the previous group's
     bool ok = true;
     if (warp < active) for (int g = g_begin; g < g_end; ++g) {
@@ -609,6 +610,7 @@ quantize_kernel(const __grid_constant__ CUtensorMap tmL1, const QuantizeParams p
       }
     }
     cp_async_wait<0>();
+    if constexpr (FORMAT != kCodesMxfp4) grid_dependency_launch();
     if constexpr (R > 0) {
       // T: TMEM lane = row of the tile; warp w reads lanes 32 w .. 32 w + 31.
       if (32 * warp < cta_rows && warp < 4) {
