@@ -318,6 +318,9 @@ w4a4_status_t w4a4_query_status(w4a4_ctx_t ctx);
  * leaves through the kernel's common tail (error word, a drain period for copies in flight, release of tensor
  * memory), and Y is left partly written.  The next w4a4_query_status returns W4A4_ERR_TIMEOUT, and the context must
  * compute correctly afterwards.  Nothing faults or traps.
+ * w4a4_debug_late_gemm runs the GEMM of w4a4_gemm_from_workspace (the same instantiation) with one of the three warps that
+ * issue its tensor-core products (late_warp 1 .. 3) idle for late_ns (at most 1e6) in front of every output tile: Y must
+ * come out as ever.
  * w4a4_debug_stalled_split_gemm and w4a4_mx_debug_stalled_split_gemm do the same to the forms of the two GEMMs in which the
  * CTAs of a cluster share a tile's K (W4A4_ERR_SHAPE for a call that does not take that form): the first CTA of every
  * cluster never loads the stage, the others complete theirs, and nothing is stored to Y.
@@ -335,6 +338,7 @@ w4a4_status_t w4a4_debug_wait_probe(w4a4_ctx_t ctx, uint64_t limit_ns, void* str
 w4a4_status_t w4a4_debug_set_tile_order(w4a4_ctx_t ctx, int super_column_tiles);
 w4a4_status_t w4a4_debug_stalled_gemm(w4a4_handle_t h, int M, int expert_id, void* Y, int stall_stage,
                                       uint64_t limit_ns, void* stream);
+w4a4_status_t w4a4_debug_late_gemm(w4a4_handle_t h, int M, int expert_id, void* Y, int late_warp, uint64_t late_ns, void* stream);
 w4a4_status_t w4a4_debug_scale_arithmetic(w4a4_ctx_t ctx, uint32_t first_bits, uint32_t count, uint64_t* differ, void* stream);
 w4a4_status_t w4a4_debug_stalled_quantize(w4a4_handle_t h, const void* X, int M, int expert_id, int timestep_bin,
                                           const float* clip_table, int stall_group, uint64_t limit_ns, void* stream);

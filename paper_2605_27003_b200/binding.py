@@ -27,7 +27,7 @@ EXPORTED_SYMBOLS = (
     "w4a4_tile_shape", "w4a4_quantize_noalloc", "w4a4_clip_search",
     "w4a4_mx_pack_weights", "w4a4_mx_destroy", "w4a4_mx_handle_bytes", "w4a4_mx_linear_forward",
     "w4a4_mx_quantize_activations", "w4a4_mx_gemm_from_workspace", "w4a4_mx_debug_quantize", "w4a4_mx_clip_search",
-    "w4a4_mx_ffn_forward", "w4a4_mx_debug_fused_input", "w4a4_gptq_quantize", "w4a4_mx_gptq_quantize", "w4a4_gptq_accumulate", "w4a4_gptq_workspace_bytes", "w4a4_query_status", "w4a4_debug_wait_probe", "w4a4_debug_stalled_gemm", "w4a4_debug_stalled_split_gemm", "w4a4_debug_stalled_quantize", "w4a4_debug_scale_arithmetic", "w4a4_mx_debug_stalled_split_gemm", "w4a4_debug_set_tile_order",
+    "w4a4_mx_ffn_forward", "w4a4_mx_debug_fused_input", "w4a4_gptq_quantize", "w4a4_mx_gptq_quantize", "w4a4_gptq_accumulate", "w4a4_gptq_workspace_bytes", "w4a4_query_status", "w4a4_debug_wait_probe", "w4a4_debug_stalled_gemm", "w4a4_debug_late_gemm", "w4a4_debug_stalled_split_gemm", "w4a4_debug_stalled_quantize", "w4a4_debug_scale_arithmetic", "w4a4_mx_debug_stalled_split_gemm", "w4a4_debug_set_tile_order",
     "w4a4_debug_fail_allocation_after", "w4a4_handle_bytes", "w4a4_ctx_bytes", "w4a4_status_string",
 )
 
@@ -114,6 +114,7 @@ def _lib():
         lib.w4a4_debug_stalled_gemm.argtypes = [vp, ci, ci, vp, ci, ctypes.c_uint64, vp]
         lib.w4a4_debug_stalled_quantize.argtypes = [vp, vp, ci, ci, ci, vp, ci, ctypes.c_uint64, vp]
         lib.w4a4_debug_scale_arithmetic.argtypes = [vp, ctypes.c_uint32, ctypes.c_uint32, vp, vp]
+        lib.w4a4_debug_late_gemm.argtypes = lib.w4a4_debug_stalled_gemm.argtypes
         lib.w4a4_debug_stalled_split_gemm.argtypes = lib.w4a4_debug_stalled_gemm.argtypes
         lib.w4a4_mx_debug_stalled_split_gemm.argtypes = lib.w4a4_debug_stalled_gemm.argtypes
         lib.w4a4_debug_fail_allocation_after.argtypes = [ci]
@@ -399,6 +400,12 @@ def w4a4_debug_stalled_gemm(handle, M: int, expert_id: int, Y, stall_stage: int,
     """Test hook: the GEMM on the current workspace with one operand stage withheld and a short wait limit."""
     _check(_lib().w4a4_debug_stalled_gemm(handle, M, expert_id, _ptr(Y), int(stall_stage), int(limit_ns),
                                           _stream(stream)), "w4a4_debug_stalled_gemm")
+
+
+def w4a4_debug_late_gemm(handle, M: int, expert_id: int, Y, late_warp: int, late_ns: int, stream=None):
+    """Test hook: the GEMM on the current workspace with one issuing warp (1 .. 3) idle for late_ns in front of every tile."""
+    _check(_lib().w4a4_debug_late_gemm(handle, M, expert_id, _ptr(Y), int(late_warp), int(late_ns), _stream(stream)),
+           "w4a4_debug_late_gemm")
 
 
 def w4a4_debug_stalled_split_gemm(handle, M: int, expert_id: int, Y, stall_stage: int, limit_ns: int, stream=None, mx: bool = False):

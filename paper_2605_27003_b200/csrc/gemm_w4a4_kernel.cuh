@@ -27,9 +27,8 @@
 // columns 0..127 P_g, columns 128..255 S_g.  Warp roles:
 //   warp 0      producer: per stage of 128 K-codes (two groups) TMA loads of the A and B code tiles (16 KiB each,
 //               128-byte swizzle) and of the two scale-operand images, all onto the stage's mbarrier;
-//   warps 1, 2  code-MMA issuers, warp 1 for the first group of every stage (and the low-rank entry), warp 2 for the second:
-//               per group two tcgen05.mma kind::f8f6f4 (K = 32) into the slot's P columns, then a commit onto
-//               tmem_full[slot];
+//   warps 1, 2  code-MMA issuers, one per TMEM slot (CodeSlotWalk): per group two tcgen05.mma kind::f8f6f4 (K = 32) into the
+//               slot's P columns, then a commit onto tmem_full[slot]; the low-rank entry is its slot's warp's;
 //   warp 3      scale-MMA issuer: per group one tcgen05.mma kind::f16 (K = 16) into the slot's S columns and a commit
 //               onto the same barrier (it counts two arrivals).  The issue of a tcgen05.mma waits for room in the tensor
 //               pipe's queue and the loop around it costs as much again, so that one thread with everything to issue is
@@ -77,11 +76,11 @@
 
 #include "pipeline.cuh"
 #include "ptx.cuh"
+#include "tmem_slots.h"
 
 namespace w4a4 {
 
 constexpr int kGemmStages = 5;
-constexpr int kTmemSlots = 2;       // TMEM slots of 2 x kBN columns: one per group in flight
 constexpr uint32_t kOpATile = kBM * kBK;              // 16 KiB: 128 token rows x 128 codes
 constexpr uint32_t kOpBTile = kBN * kBK;              // 16 KiB: 128 weight rows x 128 codes
 constexpr uint32_t kSopATile = kBM * 16;              // 2 KiB: 128 token rows x one 16-byte chunk (two groups)
@@ -234,6 +233,13 @@ __global__ void sop_weight_kernel(const float* __restrict__ wscale, uint4* __res
   out[image * 256 + (g & 1) * 128 + ((n & 127) >> 3) * 8 + (n & 7)] = (g & 1) ? make_uint4(0u, 0u, w, w) : make_uint4(w, w, 0u, 0u);
 }
 
+// Test hook of the tap instantiation: one issuing warp comes late to every tile.
+__device__ __forceinline__ void late_start(const GemmParams& p, int warp) {
+  if (warp != p.dbg_late_warp) return;
+  const uint64_t t0 = global_timer_ns();
+  while (global_timer_ns() - t0 < p.dbg_late_ns) __nanosleep(200);
+}
+
 template <bool DEBUG, bool SPLIT>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
@@ -306,8 +312,8 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   const bool live = __all_sync(0xffffffffu, *s_abort == 0);
 
   // Shared-memory stage: A codes | B codes | token scale operand (two groups) | channel scale operand (two groups).
-  // Per tile the issuing warps and the epilogue walk the same list of TMEM slot uses: [the low-rank entry, if r > 0]
-  // followed by one entry per group.
+  // Per tile the scale-MMA warp and the epilogue walk the same list of TMEM slot uses: [the low-rank entry, if r > 0]
+  // followed by one entry per group.  The code-MMA warps take the list's uses of one slot each.
   if (warp < kEpiWarp0) {
     setmaxnreg_dec<kControlRegs>();
     if (live && warp == 0) {
@@ -358,29 +364,27 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       // ------------------------------------------------------------------ code-MMA issuer (all lanes loop, one issues)
       constexpr uint32_t idesc_f8 = umma_idesc(1, 0, kBM, kBN);
       constexpr uint32_t idesc_bf16 = umma_idesc(1, 1, kBM, kBN);
-      const int v = warp - 1;
       const bool issuer = elect_one_lane();
       const uint32_t go = issuer ? 1u : 0u;
       const int issue_lane = __ffs(__ballot_sync(0xffffffffu, issuer)) - 1;   // the decision below is the issuing lane's
+      CodeSlotWalk walk(warp - 1);
+      const uint32_t d = tmem_base + walk.own * 2 * kBN, full_bar = bar_tmem_full + 8 * walk.own, empty_bar = bar_tmem_empty + 8 * walk.own;
       Ring<kGemmStages> op;
-      Ring<kTmemSlots> tm;
       bool ok = true;
       for (int tile = first_tile; ok && tile < num_tiles; tile += tile_step) {
-        // Both warps wait for the tile's first use.  Each waits for every other use within a tile; the uses of a tile may be odd in
-        // number, and a warp that has not seen the use before the last one of a slot released would take an older phase of the
-        // same parity for the one it waits for.
-        ok = __all_sync(0xffffffffu, bounded_wait<0, 1>(bar_tmem_empty + 8 * tm.slot, tm.parity ^ 1u, env, kErrMmaWait));
-        if (!ok) break;
-        tc_fence_after_sync();
+        if (DEBUG) late_start(p, warp);
         if (n_lr_stages > 0) {
-          const uint32_t d = tmem_base + tm.slot * 2 * kBN;
-          const uint32_t full_bar = bar_tmem_full + 8 * tm.slot;
-          tm.advance();
+          const bool mine = walk.owns_next();
+          if (mine) {
+            ok = __all_sync(0xffffffffu, bounded_wait<0, 1>(empty_bar, walk.free_parity(), env, kErrMmaWait));
+            if (!ok) break;
+            tc_fence_after_sync();
+          }
           for (int l = 0; ok && l < n_lr_stages; ++l) {
             ok = __all_sync(0xffffffffu, bounded_wait<0, 1>(bar_op_full + 8 * op.slot, op.parity, env, kErrMmaWait));
             if (!ok) break;
             const uint32_t a = smem_base + op.slot * kStageBytes, b = a + kOpATile;
-            if (issuer && v == 0) {
+            if (issuer && mine) {
 #pragma unroll
               for (int kk = 0; kk < 4; ++kk)
                 umma_f16(d, umma_desc_k_sw128(a, 32 * kk), umma_desc_k_sw128(b, 32 * kk), idesc_bf16, (l > 0 || kk > 0) ? 1u : 0u);
@@ -391,38 +395,40 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             op.advance();
           }
           if (!ok) break;
-          if (issuer && v == 0) umma_commit(full_bar);
+          if (mine) {
+            if (issuer) umma_commit(full_bar);
+            walk.issued();
+          }
+          walk.pass(1);
         }
+        const int v = walk.group();   // the same one in all of the tile's stages
         for (int st = st_begin; ok && st < st_end; ++st) {
           ok = __all_sync(0xffffffffu, bounded_wait<0, 1>(bar_op_full + 8 * op.slot, op.parity, env, kErrMmaWait));
           if (!ok) break;
           const uint32_t a = smem_base + op.slot * kStageBytes, b = a + kOpATile;
           const int groups = (2 * st + 1 < G) ? 2 : 1;
-          if (v == 1) tm.advance();
           if (v < groups) {
             // everything the issue needs is ready before the wait that sits on the slot's round trip
-            const uint32_t d = tmem_base + tm.slot * 2 * kBN;
-            const uint32_t full_bar = bar_tmem_full + 8 * tm.slot;
             const uint64_t da0 = umma_desc_k_sw128(a, 64 * v), db0 = umma_desc_k_sw128(b, 64 * v);
             const uint64_t da1 = umma_desc_k_sw128(a, 64 * v + 32), db1 = umma_desc_k_sw128(b, 64 * v + 32);
-            if (__shfl_sync(0xffffffffu, wait_issue_f8x2(go, bar_tmem_empty + 8 * tm.slot, tm.parity ^ 1u, d, da0, db0, da1, db1, idesc_f8, full_bar), issue_lane) == 0) {
-              ok = __all_sync(0xffffffffu, bounded_wait<0, 1>(bar_tmem_empty + 8 * tm.slot, tm.parity ^ 1u, env, kErrMmaWait));
+            if (__shfl_sync(0xffffffffu, wait_issue_f8x2(go, empty_bar, walk.free_parity(), d, da0, db0, da1, db1, idesc_f8, full_bar), issue_lane) == 0) {
+              ok = __all_sync(0xffffffffu, bounded_wait<0, 1>(empty_bar, walk.free_parity(), env, kErrMmaWait));
               if (!ok) break;
               tc_fence_after_sync();
               umma_f8_if(go, d, da0, db0, idesc_f8, 0u);
               umma_f8_if(go, d, da1, db1, idesc_f8, 1u);
               umma_commit_if(go, full_bar);
             }
-            tm.advance();
+            walk.issued();
           }
-          if (v == 0 && groups == 2) tm.advance();
           umma_commit_if(go, bar_op_empty + 8 * op.slot);
           op.advance();
         }
+        walk.pass(g_end - g_begin);
       }
     } else if (live && warp == 3) {
       // ------------------------------------------------------------------ scale-MMA issuer
-      // Walks the same slot uses as the code-MMA warps.
+      // Walks the slot uses of both code-MMA warps.
       constexpr uint32_t idesc_bf16 = umma_idesc(1, 1, kBM, kBN);
       const bool issuer = elect_one_lane();
       const uint32_t go = issuer ? 1u : 0u;
@@ -431,6 +437,7 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       Ring<kTmemSlots> tm;
       bool ok = true;
       for (int tile = first_tile; ok && tile < num_tiles; tile += tile_step) {
+        if (DEBUG) late_start(p, warp);
         if (n_lr_stages > 0) {
           ok = __all_sync(0xffffffffu, bounded_wait<0, 1>(bar_tmem_empty + 8 * tm.slot, tm.parity ^ 1u, env, kErrMmaWait));
           if (!ok) break;

@@ -287,7 +287,8 @@ w4a4_status_t launch_quantize(w4a4_handle_t h, const void* X, int M, int expert_
 // *sq_err instead of storing Y.
 w4a4_status_t launch_gemm(w4a4_handle_t h, int M, int expert_id, void* Y, cudaStream_t stream, int32_t* dbg_P,
                           int dbg_m0, int dbg_n0, const void* yref = nullptr, double* sq_err = nullptr,
-                          bool expand = false, int stall_stage = -1, uint64_t wait_limit_ns = kWaitLimitNs, bool stall_split = false) {
+                          bool expand = false, int stall_stage = -1, uint64_t wait_limit_ns = kWaitLimitNs, bool stall_split = false,
+                          int late_warp = -1, uint64_t late_ns = 0) {
   if (M == 0) return W4A4_OK;
   w4a4_ctx* ctx = h->ctx;
   const ExpertData& e = h->experts[expert_id];
@@ -318,6 +319,8 @@ w4a4_status_t launch_gemm(w4a4_handle_t h, int M, int expert_id, void* Y, cudaSt
   p.err = ctx->d_err;
   p.wait_limit_ns = wait_limit_ns;
   p.dbg_stall_stage = stall_stage;
+  p.dbg_late_warp = late_warp;
+  p.dbg_late_ns = late_ns;
   p.dbg_P = dbg_P;
   p.dbg_m0 = dbg_m0;
   p.dbg_n0 = dbg_n0;
@@ -353,7 +356,7 @@ w4a4_status_t launch_gemm(w4a4_handle_t h, int M, int expert_id, void* Y, cudaSt
   const OverlappedLaunch l(p.splits > 1 ? dim3(num_tiles * p.splits) : grid, block, kGemmSmemBytes, stream, dim3(p.splits));
   cudaError_t le;
   auto launch = [&](auto* kernel) { return cudaLaunchKernelEx(&l.cfg, kernel, h->tmA, h->tmB, tmT, tmL2, h->tmSopA, e.tmSopB, tmY, p); };
-  if (dbg_P || stall_stage >= 0) le = p.splits > 1 ? launch(gemm_w4a4_kernel<true, true>) : launch(gemm_w4a4_kernel<true, false>);
+  if (dbg_P || stall_stage >= 0 || late_warp >= 0) le = p.splits > 1 ? launch(gemm_w4a4_kernel<true, true>) : launch(gemm_w4a4_kernel<true, false>);
   else le = p.splits > 1 ? launch(gemm_w4a4_kernel<false, true>) : launch(gemm_w4a4_kernel<false, false>);
   if (le != cudaSuccess) cudaGetLastError();
   return le == cudaSuccess ? W4A4_OK : W4A4_ERR_CUDA;
@@ -881,6 +884,17 @@ w4a4_status_t w4a4_debug_stalled_gemm(w4a4_handle_t h, int M, int expert_id, voi
 w4a4_status_t w4a4_debug_stalled_split_gemm(w4a4_handle_t h, int M, int expert_id, void* Y, int stall_stage,
                                             uint64_t limit_ns, void* stream) {
   return stalled_gemm(h, M, expert_id, Y, stall_stage, limit_ns, stream, true);
+}
+
+w4a4_status_t w4a4_debug_late_gemm(w4a4_handle_t h, int M, int expert_id, void* Y, int late_warp, uint64_t late_ns, void* stream) {
+  w4a4_status_t st = check_forward_args(h, nullptr, M, expert_id, 0, nullptr, false);
+  if (st != W4A4_OK) return st;
+  if (!Y || !aligned16(Y) || late_warp < 1 || late_warp > 3) return W4A4_ERR_INVALID_ARG;
+  if (late_ns > 1000000ull) return W4A4_ERR_INVALID_ARG;  // at most 1 ms a tile
+  DeviceGuard guard(h->ctx->device);
+  if (!guard.ok) return W4A4_ERR_CUDA;
+  return launch_gemm(h, M, expert_id, Y, static_cast<cudaStream_t>(stream), nullptr, 0, 0, nullptr, nullptr, true, -1, kWaitLimitNs,
+                     false, late_warp, late_ns);
 }
 
 w4a4_status_t w4a4_debug_stalled_quantize(w4a4_handle_t h, const void* X, int M, int expert_id, int timestep_bin,
