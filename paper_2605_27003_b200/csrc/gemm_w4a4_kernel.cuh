@@ -51,11 +51,10 @@
 // tensor core 800).  A lone warp's dependent instructions
 // cost 10-15 cycles each and a branch on a fresh mbarrier result ~70, so the hops are written as single instruction
 // sequences without branches: wait_issue_* (try_wait, then fence, MMAs and commit predicated on its answer),
-// wait_then_ld16 (try_wait, then fence and first TMEM load predicated on its answer), descriptors computed before the wait, and
+// wait_then_ld16 (try_wait, a vote, then fence and first TMEM load predicated on it), descriptors computed before the wait, and
 // predicated instead of branched single-lane instructions (umma_*_if, mbar_arrive_if).  A wait that outlasts the
 // try_wait falls back to the bounded wait of pipeline.cuh and the same instructions issued from C++.  The slots' addresses are
-// toggled, not derived from a counter (423 -> 410 clocks per group).  The vote on the answer stays: a barrier that completes
-// during a try_wait can answer the lanes differently.
+// toggled, not derived from a counter (423 -> 410 clocks per group).
 // The tile's end: outputs in BF16 through a swizzled tile in shared memory and out by one TMA store per warp, which the next
 // tile does not wait for.  16-byte stores from registers held the warps for 1150 of the tile change's 2600 clocks.
 // Tile order: column tiles are walked in super-columns (GemmParams::order, all row blocks of a
@@ -155,14 +154,17 @@ __device__ __forceinline__ uint32_t wait_issue_f16(uint32_t go, uint32_t bar, ui
   return done;
 }
 
-// Wait for a full TMEM slot and start its first load in one branch-free instruction sequence.  Returns 0 if the barrier
-// did not complete within the try_wait (nothing was loaded then).
+// Wait for a full TMEM slot and start its first load in one branch-free instruction sequence.  The load is the whole warp's
+// (.sync.aligned, undefined where the lanes' predicates differ), and a barrier that completes during a try_wait may answer the lanes
+// differently: hence the vote in front of it, which behind the load would be hidden (32760 x 5120 -> 13824 3954 -> 3980 us).
+// Returns 0, to all lanes, if the barrier did not complete within the try_wait of every lane (nothing was loaded then).
 __device__ __forceinline__ uint32_t wait_then_ld16(uint32_t bar, uint32_t parity, uint32_t taddr, uint32_t (&v)[16]) {
   uint32_t done;
   asm volatile(
       "{\n"
       ".reg .pred p;\n"
       "mbarrier.try_wait.parity.shared::cta.b64 p, [%17], %18;\n"
+      "vote.sync.all.pred p, p, 0xffffffff;\n"
       "@p tcgen05.fence::after_thread_sync;\n"
       "@p tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%19];\n"
       "selp.u32 %16, 1, 0, p;\n"
@@ -523,7 +525,7 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         for (int g = g_begin; g < g_end; ++g) {
           const uint32_t t = use.t;
           uint32_t pv[16], sv[16];
-          if (!__all_sync(0xffffffffu, wait_then_ld16(use.full, use.phase, t, pv) != 0)) {   // lanes can differ
+          if (wait_then_ld16(use.full, use.phase, t, pv) == 0) {
             ok = __all_sync(0xffffffffu, bounded_wait(use.full, use.phase, env, kErrEpilogueWait));
             if (!ok) break;
             tc_fence_after_sync();

@@ -7,6 +7,7 @@ state that the five of them can reach together is visited.
 """
 import ctypes
 import os
+import re
 import subprocess
 
 import pytest
@@ -161,6 +162,24 @@ def test_the_model_finds_a_warp_that_only_watches(slots, lr_stages, groups):
 def test_the_model_finds_a_wait_for_an_older_phase(slots, lr_stages, groups):
     # Without that wait an odd number of uses per tile moves a warp to the other slot, one phase of which it has not seen.
     assert slots(4, lr_stages, groups, 5, 2) in (1, 2)
+
+
+def test_no_warp_wide_instruction_hangs_on_a_lanes_own_answer():
+    # PTX: a .sync.aligned instruction under a predicate that the lanes of a warp see differently is undefined.  So in each inline
+    # assembly block the predicate's last writer in front of such an instruction is a vote.
+    guarded = 0
+    for name in sorted(n for n in os.listdir(CSRC) if n.endswith((".cu", ".cuh", ".h"))):
+        for block in re.findall(r"asm\s*(?:volatile)?\s*\((.*?)\);", open(os.path.join(CSRC, name)).read(), flags=re.S):
+            code = re.sub(r"//[^\n]*", "", "".join(re.findall(r'"((?:[^"\\]|\\.)*)"', block))).replace("\\n", "\n")
+            lines = [line.strip() for line in re.split(r"[;\n]", code) if line.strip()]
+            for i, line in enumerate(lines):
+                m = re.match(r"@!?(\w+)\s+\S*\.sync\.aligned", line)
+                if m is None:
+                    continue
+                guarded += 1
+                writers = [w for w in lines[:i] if re.match(rf"(?!@|\.reg)\S+\s+{m.group(1)}\b", w)]
+                assert writers and writers[-1].startswith("vote.sync.all.pred"), (name, line)
+    assert guarded > 0
 
 
 @pytest.mark.gpu
