@@ -3,6 +3,7 @@
 #pragma once
 
 #include "mx_gemm_kernel.cuh"
+#include "mx_gemm_plan.h"
 
 struct MxExpertData {
   uint8_t* bpacked = nullptr;  // [N, K/2] two E2M1 codes per byte
@@ -142,13 +143,7 @@ w4a4_status_t mx_launch_gemm(w4a4_mx_handle_t h, int M, int expert_id, void* Y, 
     return W4A4_OK;
   }
   if (stall_stage >= 0) return W4A4_ERR_SHAPE;   // the test hook knows this form only
-  // CTA pairs (cta_group::2) need at least two row tiles and an even number of CTAs.  A wave of pairs takes less time than one of
-  // single CTAs, but single CTAs win where a tile each is about all there is (900 x 5120 -> 5120 25.1 -> 20.7 us, 700 17.6 -> 15.9)
-  // and where they need two waves and pairs three (600 x 5120 -> 13824 31.1 -> 25.1); at 1.22 waves and K = 13824 they lose (43.6 | 45.1),
-  // and with two row tiles the pairs' shared weight reads count (200 x 13824 -> 13824 30.7 | 35.0).
-  const int pair_tiles = (p.tiles_m + 1) / 2 * p.tiles_n, sms = ctx->num_sms;
-  const bool singles = !next && p.tiles_m > 2 && (num_tiles <= sms + sms / 8 || (num_tiles <= 2 * sms && pair_tiles > 2 * (sms / 2)));
-  const bool pairs = p.tiles_m >= 2 && sms >= 2 && !singles;
+  const bool pairs = mx_gemm_pairs(p.tiles_m, p.tiles_n, ctx->num_sms, next != nullptr);
   // Y in boxes of 32 rows x kMxOutCols channels (encoded for every call: nothing is kept by a caller's address).
   if (!next && yref == nullptr &&
       !encode_2d(ctx->encode, &tmY, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Y, h->N, M, 2 * static_cast<uint64_t>(h->N),
