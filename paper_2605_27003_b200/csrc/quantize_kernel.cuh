@@ -476,9 +476,13 @@ quantize_kernel(const __grid_constant__ CUtensorMap tmL1, const QuantizeParams p
     for (int i = 0; i < kStages - 1; ++i)
       if (warp < active) load(g_begin + i, stage_bytes * i);
     join_setup();   // its microsecond passes beside the first loads
-    // The MXFP4 GEMM's CTAs may come in now, as room allows: this CTA has its TMEM (a GEMM's CTA takes all that an SM has left of it,
-    // and waits for this kernel's end).  After the loop instead of here, 1 x 5120 -> 1024 took 8.1 us, 7.5 now.  The INT4 GEMM's
-    // come after the loop: at 256 x 512 -> 512 a forward takes 9.40 us that way and 9.57 this way.  (The GEMM itself
+    // The MXFP4 GEMM's CTAs may come in now: every CTA of this grid has started by the time the last one passes here.  They come to SMs
+    // that this grid leaves free or is done with, since their shared memory leaves no room beside a CTA that has TMEM (asserted in
+    // w4a4_mx_api.cuh): a GEMM's CTA, which takes all of an SM's TMEM and keeps it until this grid has ended, never stands in front of
+    // one that this grid waits for.  After the loop instead of here, 1 x 5120 -> 1024 took 8.1 us, 7.5 now.  The INT4 GEMM's CTAs come
+    // after the loop.  From here it makes no difference where the launch expands much (forwards replayed from one graph, after the loop
+    // | from here: 1 x 5120 -> 5120 26.8 | 26.7 us, 100 x 5120 -> 5120 24.4 | 24.4, 448 x 5120 -> 13824 80.6 | 80.7); of small layers 64 x 512 ->
+    // 512, r = 0, gains (7.1 | 6.8) and 256 x 512 -> 512, r = 16, does not (9.2 | 9.2; called one by one 9.40 | 9.57).  (The GEMM itself
     // lets nobody in before its end: the next forward's activation CTAs then sat beside it, 78 -> 84 us at 1560 x 5120 -> 13824 MXFP4.)
     if constexpr (FORMAT == kCodesMxfp4) grid_dependency_launch();
     uint32_t slot = 0, slot_before = stage_bytes * (kStages - 1);   // this group's and the previous group's

@@ -31,6 +31,16 @@ struct w4a4_mx_layer {
 
 namespace {
 
+// No kernel of this library ever waits for TMEM.  A GEMM's CTA takes all 512 columns, may come in while kernel 1 runs and then keeps them
+// until kernel 1 has ended: it must not share an SM with a CTA of kernel 1 that has TMEM (r > 0; the smallest form), neither of its own
+// forward nor of another stream's, or clusters of the two could wait for each other.  Kernel 1's CTAs have room for all that fit.
+constexpr size_t kSmSharedBytes = 228 * 1024, kCtaReservedBytes = 1024;
+constexpr size_t smallest_quantize_cta(int r) { return quantize_smem_bytes(r, 2, 1, 1) + kCtaReservedBytes; }
+constexpr bool alone_on_its_sm(size_t gemm_bytes) { return gemm_bytes + kCtaReservedBytes + smallest_quantize_cta(16) > kSmSharedBytes; }
+static_assert(alone_on_its_sm(kGemmSmemBytes) && alone_on_its_sm(kMxSmemBytes) && alone_on_its_sm(kMx2SmemBytes) && alone_on_its_sm(kMx2FuseSmemBytes));
+static_assert(kSmSharedBytes / smallest_quantize_cta(96) * 128 <= 512 && kSmSharedBytes / smallest_quantize_cta(64) * 64 <= 512 &&
+              kSmSharedBytes / smallest_quantize_cta(16) * 32 <= 512);
+
 void mx_free_expert(MxExpertData& e) {
   cudaFree(e.bpacked);
   cudaFree(e.sfb);
