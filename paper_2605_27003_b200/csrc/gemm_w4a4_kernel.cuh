@@ -32,9 +32,8 @@
 //   warp 3      scale-MMA issuer: per group one tcgen05.mma kind::f16 (K = 16) into the slot's S columns and a commit
 //               onto the same barrier (it counts two arrivals).  The issue of a tcgen05.mma waits for room in the tensor
 //               pipe's queue and the loop around it costs as much again, so that one thread with everything to issue is
-//               late for every slot: with one code-MMA warp the slot had been free for 200 clocks when its issue was
-//               through, with two 98 (410 -> 402 clocks per group; a fourth issuing warp for the scale MMAs, or both
-//               products of a group from one warp, gained nothing: 405 and 420);
+//               late for every slot: with one code-MMA warp a group takes 330 clocks, with two 321 (a fourth issuing warp for the
+//               scale MMAs gained nothing, both products of a group from one warp lost 4 %);
 //   warp 2      also TMEM allocation;
 //   warps 4-19  epilogue: a thread owns one token row and 32 output channels.  Per group two round trips of two
 //               tcgen05.ld.32x32b.x16 (P and S of 16 columns) with the eight packed multiply-adds of the first half
@@ -42,19 +41,19 @@
 //               second half is in registers.  Measured alternatives (all four loads in one round trip; the second
 //               half's loads issued ahead of the first half's arithmetic; warps of a scheduler skewed against one
 //               another) were slower.
-// What bounds the kernel is the round trip of a TMEM slot, of which there are two: release, issue, MMAs, commit, wait, loads
-// (4736 x 5120, slope over K = 2560 and 10240 with the weight expansion's share of 20, clocks per group: 402.  One code-MMA warp and
-// slots from a counter: 421; of that kernel without any operand loads the same, with an epilogue that loads 16 columns and adds
-// nothing 336, and with one MMA instead of three beside that 300).
+// What bounds the kernel is the round trip of a TMEM slot, of which there are two: release, issue, MMAs, commit, wait, loads.
+// 321 clocks per group and 2.7 thousand per tile beside its groups (sm__cycles_active at 4736 rows -> 5120, K = 2560 and 10240).
+// Without any operand loads it took as long, with an epilogue that loads 16 columns and adds nothing 0.80 of that, with one MMA
+// instead of three beside that 0.71 (measured with one code-MMA warp).
 // Epilogue warps that form the scale products themselves leave room for three or four slots, but their broadcast reads of the
-// channel scales alone cost 190 clocks per group (651 with two CTAs per SM, 16 warps with 8 of 32 channels' products from the
-// tensor core 800).  A lone warp's dependent instructions
+// channel scales made a group take 1.6 times as long (two CTAs per SM) or twice (16 warps with 8 of 32 channels' products from
+// the tensor core).  A lone warp's dependent instructions
 // cost 10-15 cycles each and a branch on a fresh mbarrier result ~70, so the hops are written as single instruction
 // sequences without branches: wait_issue_* (try_wait, then fence, MMAs and commit predicated on its answer),
 // wait_then_ld16 (try_wait, a vote, then fence and first TMEM load predicated on it), descriptors computed before the wait, and
 // predicated instead of branched single-lane instructions (umma_*_if, mbar_arrive_if).  A wait that outlasts the
 // try_wait falls back to the bounded wait of pipeline.cuh and the same instructions issued from C++.  The slots' addresses are
-// toggled, not derived from a counter (423 -> 410 clocks per group).
+// toggled, not derived from a counter (342 clocks per group -> 318, before the vote in wait_then_ld16, which costs three).
 // The tile's end: outputs in BF16 through a swizzled tile in shared memory and out by one TMA store per warp, which the next
 // tile does not wait for.  16-byte stores from registers held the warps for 1150 of the tile change's 2600 clocks.
 // Tile order: column tiles are walked in super-columns (GemmParams::order, all row blocks of a
@@ -94,8 +93,8 @@ static_assert(kGemmSmemBytes <= 232448, "shared memory budget of one CTA");
 static_assert(kStageBytes % 1024 == 0, "operand tiles must stay 1024-byte aligned");
 
 // Register budgets.  640 threads are launched with 96 registers each; the control warpgroup gives most of its share to the
-// epilogue's four.  What the compiler makes of the epilogue's loop decides the kernel (clocks per 128 x 128 tile at K = 5120:
-// 96 registers 31314, 112 30529).
+// epilogue's four.  What the compiler makes of the epilogue's loop decides the kernel (clocks per 128 x 128 tile at K = 5120, before
+// TMA stores and a second code-MMA warp: 96 registers 31314, 112 30529; 28.4 thousand now).
 constexpr int kGemmRegs = 96, kControlRegs = 32, kEpilogueRegs = 112;
 static_assert((kGemmThreads - 32 * kEpiWarps) * kControlRegs + 32 * kEpiWarps * kEpilogueRegs <= kGemmThreads * kGemmRegs,
               "a larger sum would wait forever for registers that the launch does not have");
@@ -562,8 +561,8 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                                  __float_as_uint(acc[2 * c + 1].y)));
           break;
         }
-        // The tile's end: bias, activation, BF16, then through shared memory so that a warp's 16-byte accesses to Y (or to
-        // the reference) cover eight rows x 64 bytes instead of 32 rows x 16.
+        // The tile's end: bias, activation, BF16, then a swizzled tile in shared memory: the source of the TMA store to Y, and where the
+        // clip search reads outputs beside the reference so that a warp's 16-byte reads of that cover eight rows x 64 bytes.
         if (!SPLIT && lane == 0) bulk_store_wait_read();   // the previous tile has left the staging tile
         __syncwarp();
         sts_f32(out_tile + 4 * lane, bias_lane);
@@ -632,6 +631,8 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       for (int row = 16 * split + warp - kEpiWarp0; row < kBM; row += 16 * p.splits) {
         if (tm_e * kBM + row >= p.M) break;
         const uint32_t at = smem_base + 512 * row + 16 * (lane ^ (row & 7));
+        // One remote load after the other: with all of them on their way first, as in the MXFP4 GEMM, this kernel's 96 registers
+        // spill (100 x 5120 -> 5120 21.7 us and 28.0 so, 300 x 1024 -> 1024 14.3 and 23.1).
         float4 y = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         for (int i = 0; i < p.splits; ++i) {
           const float4 v = ld_cluster_f32x4(map_to_cta(at, i));

@@ -20,8 +20,8 @@ __device__ __forceinline__ uint64_t global_timer_ns() {
 
 // Programmatic dependent launch: a kernel launched with that attribute may start while the kernel before it on the
 // stream still runs.  grid_dependency_wait() returns once that kernel has completed and its writes are visible: nothing
-// that an earlier kernel wrote (or still reads) may be touched before it.  At 256 x 512 -> 512 the overlap takes a forward
-// from 14.3 to 11.1 us.  grid_dependency_launch() lets the next kernel
+// that an earlier kernel wrote (or still reads) may be touched before it.  The overlap takes a forward of
+// 256 x 512 -> 512 from 14.4 to 9.3 us, one of 100 x 5120 -> 5120 MXFP4 from 16.4 to 11.5.  grid_dependency_launch() lets the next kernel
 // start its own prologue once every CTA of this grid has called it or left.
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dependency_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

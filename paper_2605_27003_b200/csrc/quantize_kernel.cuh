@@ -13,8 +13,8 @@
 // tile, from which one more warp issues four tcgen05.mma per group (M = 128, N = r, K = 16 each; the rows past the CTA's own
 // read whatever lies behind the tile and only touch accumulator rows that nobody reads) against the group's r x 64 tile
 // of L1, which it fetches by TMA into a ring of its own.
-// The bound is instruction issue and latency: 93 (MXFP4) to 123 warp instructions per 8 values and lane at r = 32 take 60 to
-// 67 % of the issue slots of two CTAs per SM; DRAM traffic is 60 % of what a copy reaches.  So the loop's addresses are kept in
+// The bound is instruction issue and latency: 93 (MXFP4) to 127 warp instructions per 8 values and lane at r = 32 take 60 to
+// 68 % of the issue slots of two CTAs per SM; DRAM traffic is 60 % of what a copy reaches.  So the loop's addresses are kept in
 // registers (derived anew in every pass they cost 15 of those instructions: 127 -> 94 us at 32760 x 5120 MXFP4) and the rare cases
 // of the scale arithmetic have a branch of their own.  The predecessor held 16 rows of a warp in mma.sync fragments, with r
 // accumulators per row in registers.  Eight launches replayed from one graph, 32760 x 5120, INT4 | MXFP4: r = 0 120 -> 99 | 93 ->
